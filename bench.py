@@ -60,7 +60,7 @@ WORKLOADS = {
 # same kernels on the same workload with the same launch settings ("tuned":
 # the cached lc_autotune choice); a class whose kernels changed since has none
 # (null).
-TRAFFIC_PER_STEP = {("rmat22", "move", "tuned"): 46_775_339_264}
+TRAFFIC_PER_STEP = {}
 
 
 def make_graph(name: str, scale_override: int | None = None):

@@ -20,6 +20,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "lc_constraint.cuh"
+#include "lc_coop.cuh"
 #include "lc_contract.cuh"
 #include "lc_leiden.cuh"
 #include "lc_internal.cuh"
@@ -177,17 +178,15 @@ struct Run {
   Arena ar;
   Prof prof;
   // scratch sized for G_0
-  int32_t *C = nullptr, *D = nullptr, *C_out = nullptr, *freelist = nullptr, *used = nullptr,
-          *newid = nullptr, *cnt = nullptr, *scan32 = nullptr, *freepos = nullptr, *mrank = nullptr,
-          *Cprev = nullptr, *dirty = nullptr, *dirty_list = nullptr, *movers = nullptr;
+  int32_t *C = nullptr, *C_out = nullptr, *freelist = nullptr, *used = nullptr,
+          *newid = nullptr, *cnt = nullptr, *scan32 = nullptr, *emovers = nullptr,
+          *dirty = nullptr, *dirty_list = nullptr, *movers = nullptr;
   int64_t *W = nullptr, *delta = nullptr, *bound = nullptr, *off = nullptr, *scan64 = nullptr;
-  uint8_t *M = nullptr, *E = nullptr;
+  uint8_t *M = nullptr;  // survivors of the last pass (trace only)
   AbRec *ab = nullptr;
-  uint32_t *inL = nullptr;    // afterburner candidate bitmap
-  AbWork *ab_list = nullptr;  // afterburner candidates by group, with their work records
+  unsigned long long *eblocks = nullptr;  // per-block counts of the new-cluster ids
   int2 *upd_list = nullptr;
   unsigned long long *gtab = nullptr;
-  long long *gself = nullptr;
   Scalars *sc = nullptr;
   // per graph
   long long *phi_acc = nullptr, *phi_out = nullptr, *phi_trace = nullptr;
@@ -195,7 +194,7 @@ struct Run {
   long long *phi_final = nullptr;  // [G] Phi of C_out after each graph's last LocalMovePasses call
   long long *Tg = nullptr, *Vg = nullptr, *sw2g = nullptr;
   int *improved = nullptr;
-  int32_t *gstart = nullptr;
+  int32_t *gstart = nullptr, *gfree = nullptr, *gmover = nullptr;
   uint8_t *keep = nullptr;
   GraphStats *st = nullptr;
   std::vector<long long> hT, hV, hsw2;
@@ -246,6 +245,8 @@ static int alloc_per_graph(Run &r) {
   LC_TRY(r.ar.get(&r.sw2g, G));
   LC_TRY(r.ar.get(&r.improved, G));
   LC_TRY(r.ar.get(&r.gstart, G));
+  LC_TRY(r.ar.get(&r.gfree, G));
+  LC_TRY(r.ar.get(&r.gmover, G));
   LC_TRY(r.ar.get(&r.keep, G));
   LC_CK(cudaMemsetAsync(r.Tg, 0, 8 * (size_t)G, r.s));
   LC_CK(cudaMemsetAsync(r.Vg, 0, 8 * (size_t)G, r.s));
@@ -255,15 +256,12 @@ static int alloc_per_graph(Run &r) {
 
 static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.C, n0));
-  LC_TRY(r.ar.get(&r.D, n0));
   LC_TRY(r.ar.get(&r.C_out, n0));
   LC_TRY(r.ar.get(&r.freelist, n0));
   LC_TRY(r.ar.get(&r.used, n0));
   LC_TRY(r.ar.get(&r.newid, n0));
   LC_TRY(r.ar.get(&r.cnt, n0));
-  LC_TRY(r.ar.get(&r.freepos, n0));
-  LC_TRY(r.ar.get(&r.mrank, n0));
-  LC_TRY(r.ar.get(&r.Cprev, n0));
+  LC_TRY(r.ar.get(&r.emovers, n0));
   LC_TRY(r.ar.get(&r.movers, n0));
   if (r.o.tables == 1) {  // kept tables only
     LC_TRY(r.ar.get(&r.dirty, n0));
@@ -276,15 +274,12 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.W, n0));
   LC_TRY(r.ar.get(&r.delta, n0));
   LC_TRY(r.ar.get(&r.ab, n0));
-  LC_TRY(r.ar.get(&r.inL, (n0 + 31) / 32));
-  LC_TRY(r.ar.get(&r.ab_list, n0));
+  LC_TRY(r.ar.get(&r.eblocks, kCoopBlocks));
   LC_TRY(r.ar.get(&r.bound, n0 + 1));
   LC_TRY(r.ar.get(&r.off, n0 + 1));
   LC_TRY(r.ar.get(&r.scan64, scan_scratch(n0 + 1)));
-  LC_TRY(r.ar.get(&r.M, n0));
-  LC_TRY(r.ar.get(&r.E, n0));
+  if (r.o.event_cb) LC_TRY(r.ar.get(&r.M, n0));
   LC_TRY(r.ar.get(&r.gtab, 2 * nnz0));
-  if (r.G > 1) LC_TRY(r.ar.get(&r.gself, n0));
   LC_TRY(r.ar.get(&r.sc, 1));
   LC_CK(cudaMemsetAsync(r.gtab, 0, sizeof(unsigned long long) * (size_t)(2 * nnz0 > 0 ? 2 * nnz0 : 1), r.s));
   LC_CK(cudaMemsetAsync(r.sc, 0, sizeof(Scalars), r.s));
@@ -326,15 +321,15 @@ static int resolve_plan(const lc_opts &o, BinPlan *out) {
 // upload_params, compact_level, contract_level), for the footprint below.
 static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tables) {
   const int64_t n = n0 > 0 ? n0 : 1, big = 2 * nnz0 > n0 + 1 ? 2 * nnz0 : n0 + 1;
-  int64_t b = G * (11 * 8 + 4 + 4 + 1);                     // alloc_per_graph
-  b += 11 * 4 * n;                                           // C .. movers
+  int64_t b = G * (11 * 8 + 4 * 4 + 1);                     // alloc_per_graph
+  b += 8 * 4 * n;                                            // C .. movers
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
   b += 4 * scan_scratch(big);                                // scan32
   b += 2 * 8 * n + (int64_t)sizeof(AbRec) * n;               // W, delta, ab
-  b += 4 * ((n0 + 31) / 32 + 1) + (int64_t)sizeof(AbWork) * n;  // inL, ab_list
-  b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + 2 * n;  // bound, off, scan64, M, E
+  b += 8 * kCoopBlocks;                                      // eblocks
+  b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + n;      // bound, off, scan64, M
   b += 8 * (2 * nnz0 > 0 ? 2 * nnz0 : 1);                    // gtab
-  if (G > 1) b += 8 * n + 8 * (G + 1) + 4 * n;               // gself, graph_ptr, gid
+  if (G > 1) b += 8 * (G + 1) + 4 * n;                       // graph_ptr, gid
   return b + (int64_t)sizeof(Scalars) + (int64_t)sizeof(GraphStats);
 }
 static int64_t level_bytes(int64_t n, int64_t nnz, int64_t G, const BinPlan &p) {
@@ -441,27 +436,21 @@ static PassArgs pass_args(Run &r, const Level &L) {
   a.gid = L.gid;
   a.gp = L.gp;
   a.G = r.G;
-  a.gself = r.G > 1 ? r.gself : nullptr;
   a.phi_acc = r.phi_acc;
   a.phi_out = r.phi_out;
   a.improved = r.improved;
   a.C = r.C;
   a.W = r.W;
-  a.D = r.D;
   a.delta = r.delta;
   a.ab = r.ab;
-  a.M = r.M;
   a.sc = r.sc;
   a.gtab = r.gtab;
   a.hub = L.hub;
-  a.Cprev = r.Cprev;
   a.dirty = r.dirty;
   a.dirty_list = r.dirty_list;
   a.obj = r.obj;
   a.hub_min = r.plan.hub_min();
-  a.inL = r.inL;
-  a.ab_list = r.ab_list;
-  set_ab_groups(a, L.bins, r.plan);
+  for (int g = 0; g < kAbGroups; ++g) a.ab_gs[g] = r.plan.ab_gs[g];
   return a;
 }
 
@@ -479,14 +468,14 @@ static int emit_pass_event(Run &r, const Level &L, int level, int phase, int pas
   a.phi_acc = r.phi_trace;
   LC_CK(cudaMemsetAsync(r.phi_trace, 0, 8 * (size_t)r.G, r.s));
   launch_objective(a, L.bins, r.s);
-  launch_graph_sums(a, r.s);
+  launch_destinations(a, r.newid, r.s);  // newid is free during the passes
   LC_TRY(launch_check());
   std::vector<int32_t> C(n > 0 ? n : 1), D(n > 0 ? n : 1);
   std::vector<uint8_t> M(n > 0 ? n : 1);
   long long phi = 0;
   Scalars sc;
   LC_CK(cudaMemcpyAsync(C.data(), r.C, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaMemcpyAsync(D.data(), r.D, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, r.s));
+  LC_CK(cudaMemcpyAsync(D.data(), r.newid, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaMemcpyAsync(M.data(), r.M, n, cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaMemcpyAsync(&phi, r.phi_trace, 8, cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaMemcpyAsync(&sc, r.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, r.s));
@@ -512,7 +501,7 @@ static int emit_pass_event(Run &r, const Level &L, int level, int phase, int pas
 // singletons nor the last of its call (move step, best-of test, afterburner,
 // update; the temperature comes from the device schedule) into an
 // executable CUDA graph.  counts: kernels per class in one replay.
-static int capture_pass(Run &r, Level &L, const PassArgs &a, const ApplyScratch &w, cudaGraphExec_t *out,
+static int capture_pass(Run &r, Level &L, const PassArgs &a, const EmptyScratch &w, cudaGraphExec_t *out,
                         int64_t counts[LC_K_COUNT]) {
   *out = nullptr;
   cudaStream_t cs = capture_stream();
@@ -524,9 +513,9 @@ static int capture_pass(Run &r, Level &L, const PassArgs &a, const ApplyScratch 
   for (int k = 0; k < LC_K_COUNT; ++k) counts[k] = 0;
   launch_pass_begin(r.sc, cs, 1);
   counts[LC_K_MOVE] += launch_move(a, L.bins, cs);
-  counts[LC_K_APPLY] += launch_graph_sums(a, cs) + launch_bestof(a, r.C_out, cs);
+  counts[LC_K_APPLY] += launch_bestof(a, r.C_out, cs);
   counts[LC_K_AFTERBURNER] += launch_afterburner(a, L.bins, cs);
-  counts[LC_K_APPLY] += launch_apply(a, w, cs) + 1;
+  counts[LC_K_APPLY] += launch_assign_empty(a, w, cs) + 1;
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(cs, &g);
   if (e != cudaSuccess || !g) {
@@ -553,7 +542,8 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
   const int64_t n = L.g.n, nnz = L.g.nnz;
   LC_TRY(upload_params(r, L, active));
   PassArgs a = pass_args(r, L);
-  ApplyScratch w{r.E, r.used, r.freelist, r.freepos, r.mrank, r.scan32};
+  a.M = r.M;
+  EmptyScratch w{r.used, r.freelist, r.emovers, r.gfree, r.gmover, r.eblocks};
   if (singleton) {
     launch_iota(r.C, n, r.s);
     launch_iota(r.C_out, n, r.s);
@@ -644,7 +634,6 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
         a.tab_build = 0;
       }
       r.prof.begin(LC_K_APPLY);
-      r.res->kernel_launches[LC_K_APPLY] += launch_graph_sums(a, r.s);
       // Phi entering the last pass, per graph, before the best-of test resets it
       if (incremental && last) r.res->kernel_launches[LC_K_OBJECTIVE] += launch_save_phi_enter(a, r.s);
       r.res->kernel_launches[LC_K_APPLY] += launch_bestof(a, r.C_out, r.s);
@@ -656,10 +645,11 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
     else  // ablations: no filter, or the minimum label heuristic in odd passes
       r.res->kernel_launches[LC_K_AFTERBURNER] +=
           launch_symmetry_ablation(a, r.o.symmetry == 2 && i % 2 == 1, r.cnt, r.s);
-    r.prof.end(32.0 * n);  // + 24 B per candidate edge, added from sc->cand_edges at the end
+    // records, vertices and labels (+ 24 B per candidate edge, added from sc->cand_edges at the end)
+    r.prof.end(56.0 * n);
     r.prof.begin(LC_K_APPLY);
-    r.res->kernel_launches[LC_K_APPLY] += launch_apply(a, w, r.s);
-    r.prof.end(14.0 * n);
+    r.res->kernel_launches[LC_K_APPLY] += launch_assign_empty(a, w, r.s);
+    r.prof.end(0.0);
     LC_TRY(launch_check());
     r.res->passes_total++;
     r.res->edges_local_move += nnz;
@@ -674,7 +664,7 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
     r.prof.end(17.0 * n);  // W, w(v) and M per vertex (+ 13 B per mover edge, added at the end)
   } else {
     r.res->kernel_launches[LC_K_OBJECTIVE] +=
-        launch_objective(a, L.bins, r.s) + launch_graph_sums(a, r.s) + launch_bestof(a, r.C_out, r.s);
+        launch_objective(a, L.bins, r.s) + launch_bestof(a, r.C_out, r.s);
     r.prof.end(12.0 * nnz + 32.0 * n);
   }
   r.res->kernel_launches[LC_K_OTHER] += launch_keep_phi(a, r.phi_final, r.s);
@@ -962,7 +952,7 @@ static int objective_of(Run &r, Level &L, const int32_t *labels, std::vector<lon
   PassArgs a = pass_args(r, L);
   LC_CK(cudaMemsetAsync(r.phi_acc, 0, 8 * (size_t)r.G, r.s));
   r.prof.begin(LC_K_OBJECTIVE);
-  r.res->kernel_launches[LC_K_OBJECTIVE] += launch_objective(a, L.bins, r.s) + launch_graph_sums(a, r.s) + 1;
+  r.res->kernel_launches[LC_K_OBJECTIVE] += launch_objective(a, L.bins, r.s) + 1;
   r.prof.end(12.0 * L.g.nnz + 32.0 * n);
   phi.assign(r.G, 0);
   LC_CK(cudaMemcpyAsync(phi.data(), r.phi_acc, 8 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
@@ -1265,7 +1255,7 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
       r.res->kernel_launches[LC_K_MOVE] += launch_move(a, L.bins, r.s);
       r.prof.end(12.0 * L.g.nnz + 48.0 * n);
       r.prof.begin(LC_K_ALT);
-      launch_local_move_alt(L.g, L.gp, r.C, r.D, r.delta, r.W, ls, &r.sc->error, r.s);
+      launch_local_move_alt(L.g, L.gp, r.C, r.ab, r.delta, r.W, ls, &r.sc->error, r.s);
       r.prof.end(24.0 * n);
       r.res->kernel_launches[LC_K_ALT] += 6;
       LC_CK(cudaMemcpyAsync(r.C_out, r.C, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, r.s));

@@ -57,6 +57,22 @@ struct Grp {
   }
 };
 
+// acc[g] += x from every lane (warp-uniform call; g < 0 adds nothing).  When
+// all contributing lanes share a graph, as almost always, one atomic per warp.
+__device__ __forceinline__ void graph_add(long long *acc, int g, long long x) {
+  const bool on = g >= 0 && x != 0;
+  const unsigned act = __ballot_sync(0xFFFFFFFFu, on);
+  if (!act) return;
+  const int leader = __ffs(act) - 1;
+  const int g0 = __shfl_sync(0xFFFFFFFFu, g, leader);
+  if (__all_sync(0xFFFFFFFFu, !on || g == g0)) {
+    const long long t = warp_sum(on ? x : 0ll);
+    if ((int)(threadIdx.x & 31) == leader) atomicAdd((unsigned long long *)(acc + g0), (unsigned long long)t);
+  } else if (on) {
+    atomicAdd((unsigned long long *)(acc + g), (unsigned long long)x);
+  }
+}
+
 // Calls body(i, active) for every index i of a bin list of `count` entries,
 // uniformly over each warp (GS <= 32) or block (GS > 32).
 template <int GS, typename Body>

@@ -133,23 +133,14 @@ struct __align__(16) VRec {
   long long w;
 };
 
-// Afterburner record of a vertex for one pass: its cluster, destination and
-// priority bucket packed into one 16-byte load.
+// What a pass decided for a vertex, written by the move step for every vertex
+// of the level: the cluster it is in, its destination (kNone: no candidate)
+// and its priority bucket, one 16-byte load for the afterburner's neighbour
+// gathers.  It stays as written until the next pass, so after the update step
+// C is the vertex's previous cluster.
 struct __align__(16) AbRec {
   int32_t C, D;
   long long q;
-};
-
-// Everything the afterburner needs about one listed candidate v itself, written
-// by the record pass beside its list entry so that the group kernels read it
-// in one coalesced 64-byte load instead of a chain of gathers: its id,
-// cluster, destination, degree, hash and graph base, ordering bucket,
-// mu w(v), Lambda, row start and delta_v.
-struct __align__(16) AbWork {
-  int32_t v, C, D, deg;
-  uint32_t hv;
-  int32_t vbase;
-  long long q, muw, Lam, beg, delta;
 };
 
 // Device-resident counters of one call (all graphs of a batch together).
@@ -170,9 +161,10 @@ struct Scalars {
   int pad3;
   long long distinct_x;  // (vertex, adjacent cluster) pairs whose W(X) the move step read,
                          // summed over the call (the argmax's gathers, for the profile)
-  // candidates listed per afterburner group in this pass: per-warp atomics
-  // of the record pass, on a line of their own
-  alignas(128) int ab_count[8];
+  // barrier of the cooperative kernels: arrivals and blocks that have left,
+  // both zero between launches; on a line of their own
+  alignas(128) unsigned bar_arrived;
+  unsigned bar_left;
   // device-side temperature schedule (graph replays): k_pass_begin loads
   // phi_live from phi_tab[pass_idx] and advances pass_idx
   int pass_idx;
@@ -322,6 +314,20 @@ __device__ __forceinline__ void group_argmax(long long &g, int32_t &x) {
       x = x2;
     }
   }
+}
+
+// Argmax (gain, id) over a full warp by integer reductions: the high words'
+// maximum, the low words' among its holders, the smallest id among the
+// holders of both.  Three REDUX (1.6 clocks each per SM, measured) against
+// fifteen shuffles and as many selects.
+__device__ __forceinline__ void warp_argmax(long long &g, int32_t &x) {
+  constexpr unsigned full = 0xFFFFFFFFu;
+  const int hi = (int)(g >> 32);
+  const int mh = __reduce_max_sync(full, hi);
+  const unsigned ml = __reduce_max_sync(full, hi == mh ? (unsigned)g : 0u);
+  const bool win = hi == mh && (unsigned)g == ml;
+  x = (int32_t)__reduce_min_sync(full, win ? (unsigned)x : 0xFFFFFFFFu);
+  g = (long long)(((unsigned long long)(unsigned)mh << 32) | ml);
 }
 
 // ------------------------------------------------------------- launch

@@ -25,9 +25,9 @@ unsigned ld_grid(int64_t n, int per_block) {
 // ------------------------------------------------------- LocalMoveAlt
 
 struct AltIn {
-  const int32_t *D;
+  const AbRec *ab;
   const int64_t *delta;
-  __device__ int64_t operator()(int64_t v) const { return D[v] != kNone && delta[v] > 0; }
+  __device__ int64_t operator()(int64_t v) const { return ab[v].D != kNone && delta[v] > 0; }
 };
 struct AltOut {
   int32_t *list;
@@ -50,7 +50,7 @@ constexpr int kAltThreads = 1024;
 // empty cluster takes the smallest unused id (a vertex already alone keeps
 // its id).  At the end the moves after the best prefix are undone.
 __global__ void __launch_bounds__(kAltThreads) k_local_move_alt(LevelGraph g, const GraphParam *gp,
-                                                               int32_t *C, const int32_t *D,
+                                                               int32_t *C, const AbRec *ab,
                                                                int64_t *W, int32_t *size,
                                                                const int32_t *list, const int64_t *m_ptr,
                                                                int32_t *to, int32_t *old,
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kAltThreads) k_local_move_alt(LevelGraph g, co
   __syncthreads();
   for (int64_t k = 0; k < m; ++k) {
     const int32_t v = list[k];
-    const int32_t Dv = D[v], Cv = C[v];
+    const int32_t Dv = ab[v].D, Cv = C[v];
     long long sc = 0, sd = 0;
     for (int64_t e = g.rp[v] + threadIdx.x; e < g.rp[v + 1]; e += kAltThreads) {
       const int32_t X = C[g.col[e]];
@@ -528,14 +528,14 @@ __global__ void k_downsample(const int32_t *__restrict__ Cd, const int32_t *__re
 
 }  // namespace
 
-void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C, const int32_t *D,
+void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C, const AbRec *ab,
                            const int64_t *delta, int64_t *W, LeidenScratch &ls, int *error,
                            cudaStream_t s) {
   if (g.n == 0) return;
-  scan_apply<int64_t>(g.n, AltIn{D, delta}, AltOut{ls.list}, ls.scan64, s);
+  scan_apply<int64_t>(g.n, AltIn{ab, delta}, AltOut{ls.list}, ls.scan64, s);
   cudaMemsetAsync(ls.size, 0, sizeof(int32_t) * (size_t)g.n, s);
   k_sizes<<<ld_grid(g.n, 256), 256, 0, s>>>(C, ls.size, g.n);
-  k_local_move_alt<<<1, kAltThreads, 0, s>>>(g, gp, C, D, W, ls.size, ls.list,
+  k_local_move_alt<<<1, kAltThreads, 0, s>>>(g, gp, C, ab, W, ls.size, ls.list,
                                               ls.scan64 + scan_tiles(g.n), ls.to, ls.list2, ls.scal,
                                               error);
 }

@@ -64,10 +64,10 @@ struct LeidenScratch {
 // Elements of hist / scan64 the radix sort of n keys needs.
 int64_t radix_hist_len(int64_t n);
 
-// LocalMoveAlt (Section V-A) on labels C (in place), given D and delta of a
+// LocalMoveAlt (Section V-A) on labels C (in place), given the records and delta of a
 // pass with phi = 0 (D = kNone: no move with gD >= gC).  W: cluster weights
 // of C (modified).  Leaves the number of committed moves in scal[1].
-void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C, const int32_t *D,
+void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C, const AbRec *ab,
                            const int64_t *delta, int64_t *W, LeidenScratch &ls, int *error,
                            cudaStream_t s);
 // pLeidenR (Algorithm 6) with constraint B (dense labels in [0, n)): refined

@@ -12,16 +12,14 @@ struct PassArgs {
   const int32_t *gid;     // graph of each vertex of a packed batch (nullptr: one graph)
   const GraphParam *gp;   // [G] per-graph lambda, vertex base, active flag
   int32_t G;
-  long long *gself;       // batch only: per-vertex g(v, C[v]) for the per-graph objective
   long long *phi_acc;     // [G] objective of the clustering entering the pass
   long long *phi_out;     // [G] objective of C_out
   int *improved;          // [G] last best-of test
   int32_t *C;       // clustering entering the pass (updated by the apply step)
   int64_t *W;       // W(X) for X in [0, n)
-  int32_t *D;       // destination of candidates; kNone for non-candidates
+  AbRec *ab;        // per pass: {C, D, epsilon bucket of delta} (Section IV-A-1 order)
   int64_t *delta;   // g(v, D[v]) - g(v, C[v]) of candidates
-  AbRec *ab;        // per-pass {C, D, epsilon bucket of delta} (Section IV-A-1 order)
-  uint8_t *M;       // afterburner survivors
+  uint8_t *M;       // afterburner survivors (trace only, else nullptr)
   Scalars *sc;
   unsigned long long *gtab;  // clean global hash scratch, >= 2 nnz slots
   int32_t phi_n, phi_d;      // temperature of this pass
@@ -30,7 +28,6 @@ struct PassArgs {
   // kept tables: each vertex's S(v, .) in its gtab region (tab_cap slots)
   int32_t tab_build;         // this aggregation pass also writes the tables out
   int32_t tab_reset;         // this table pass clears the tables as it reads them
-  int32_t *Cprev;            // [n] label before the last apply, of its movers
   int32_t *dirty;            // [n] 1: the table overflowed and is rebuilt (zero between passes)
   int32_t *dirty_list;       // [n] those vertices, sc->tab_dirty of them
   int2 *upd_list;            // chunks {mover, chunk} of the movers' rows, listed by the
@@ -40,12 +37,6 @@ struct PassArgs {
   long long *obj;            // [4 G] per graph: Phi entering the last pass, Q entering it,
                              // Q after it, change of IN by its moves (objective update)
   int64_t hub_min;           // rows longer than this are hubs (BinPlan::hub_min)
-  // afterburner: candidate bitmap (bit v of word v / 32) and the candidates
-  // of each group, listed by the record pass into ab_list[ab_off[g] ...)
-  uint32_t *inL;
-  AbWork *ab_list;
-  int64_t ab_off[kAbGroups];  // start of group g (the offset of its first bin)
-  int64_t ab_max[kAbGroups];  // largest degree in group g (BinPlan)
   int32_t ab_gs[kAbGroups];   // threads per candidate in group g (BinPlan)
 };
 
@@ -86,8 +77,8 @@ void launch_hub_rows(const int64_t *rp, const int32_t *vtx, int H, int64_t *out,
 void launch_pass_begin(Scalars *sc, cudaStream_t s, int advance = 0);
 int launch_first_pass(const PassArgs &a, const Bins &b, cudaStream_t s);
 int launch_move(const PassArgs &a, const Bins &b, cudaStream_t s);
-// Fills the afterburner groups' list offsets and degree bounds of a level.
-void set_ab_groups(PassArgs &a, const Bins &b, const BinPlan &plan);
+// Afterburner and update: survivors move (Algorithm 2, Update), except that
+// movers to a new empty cluster are left at C[v] = kEmpty for launch_assign_empty.
 int launch_afterburner(const PassArgs &a, const Bins &b, cudaStream_t s);
 // Ablations of the afterburner: every candidate moves, or (mlh) all but a
 // vertex alone in its cluster whose destination is another one-vertex
@@ -111,15 +102,16 @@ int launch_table_pass(const PassArgs &a, const Bins &b, cudaStream_t s);
 // Entries of PassArgs::upd_list a level of n vertices and nnz stored edges
 // may need.
 inline int64_t upd_list_size(int64_t n, int64_t nnz) { return n + nnz / kUpdChunk + 1; }
-// Scratch of the update step (all [n] of the level).
-struct ApplyScratch {
-  uint8_t *E;
-  int32_t *used, *freelist, *freepos, *mrank, *scan_tmp;
+// Scratch of the new-cluster ids (used, freelist, movers: [n]; blocks: one
+// entry per block; gfree, gmover: [G]).
+struct EmptyScratch {
+  int32_t *used, *freelist, *movers, *gfree, *gmover;
+  unsigned long long *blocks;
 };
-// Update step: moves, W, then ids for movers to new empty clusters.
-int launch_apply(const PassArgs &a, const ApplyScratch &w, cudaStream_t s);
-// Batch only: per-graph sums of the recorded g(v, C[v]) into phi_acc.
-int launch_graph_sums(const PassArgs &a, cudaStream_t s);
+// Ids for this pass's movers to new empty clusters (nothing to do without any).
+int launch_assign_empty(const PassArgs &a, const EmptyScratch &w, cudaStream_t s);
+// Splits the records into destinations (for the trace).
+void launch_destinations(const PassArgs &a, int32_t *D, cudaStream_t s);
 // Per-graph best-of test and copy of improved graphs' labels into C_out.
 int launch_bestof(const PassArgs &a, int32_t *C_out, cudaStream_t s);
 // phi_final[g] = phi_out[g] for every graph active in the call (gp[g].active).
