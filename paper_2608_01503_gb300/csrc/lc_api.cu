@@ -21,6 +21,7 @@
 
 #include "lc_constraint.cuh"
 #include "lc_coop.cuh"
+#include "lc_fused.cuh"
 #include "lc_contract.cuh"
 #include "lc_leiden.cuh"
 #include "lc_internal.cuh"
@@ -81,6 +82,7 @@ static void configure_device() {
   std::lock_guard<std::mutex> lock(mtx);
   if (done_mask & bit) return;
   configure_kernels();
+  configure_fused();
   cudaGetLastError();
   done_mask |= bit;
 }
@@ -158,6 +160,7 @@ struct Level {
   LevelGraph g{};
   Bins bins{};
   Hubs hub{};
+  int64_t max_deg = 0;               // longest hub row (0: no hub)
   int32_t *gid = nullptr;            // [n] graph of each vertex (nullptr: one graph)
   GraphParam *gp = nullptr;          // [G] device
   std::vector<int64_t> vbase, nv;    // [G] host
@@ -191,6 +194,7 @@ struct Run {
   // per graph
   long long *phi_acc = nullptr, *phi_out = nullptr, *phi_trace = nullptr;
   long long *obj = nullptr;  // [4 G] objective update after a call's last pass
+  long long *fused = nullptr;  // [6 G] accumulators of the fused passes (FusedArgs)
   long long *phi_final = nullptr;  // [G] Phi of C_out after each graph's last LocalMovePasses call
   long long *Tg = nullptr, *Vg = nullptr, *sw2g = nullptr;
   int *improved = nullptr;
@@ -238,6 +242,7 @@ static int alloc_per_graph(Run &r) {
   LC_TRY(r.ar.get(&r.phi_out, G));
   LC_TRY(r.ar.get(&r.phi_trace, G));
   LC_TRY(r.ar.get(&r.obj, 4 * (int64_t)G));
+  LC_TRY(r.ar.get(&r.fused, 6 * (int64_t)G));
   LC_TRY(r.ar.get(&r.phi_final, G));
   LC_CK(cudaMemsetAsync(r.phi_final, 0, 8 * (size_t)G, r.s));  // a graph with no vertices: Phi = 0
   LC_TRY(r.ar.get(&r.Tg, G));
@@ -321,7 +326,7 @@ static int resolve_plan(const lc_opts &o, BinPlan *out) {
 // upload_params, compact_level, contract_level), for the footprint below.
 static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tables) {
   const int64_t n = n0 > 0 ? n0 : 1, big = 2 * nnz0 > n0 + 1 ? 2 * nnz0 : n0 + 1;
-  int64_t b = G * (11 * 8 + 4 * 4 + 1);                     // alloc_per_graph
+  int64_t b = G * (17 * 8 + 4 * 4 + 1);                     // alloc_per_graph
   b += 8 * 4 * n;                                            // C .. movers
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
   b += 4 * scan_scratch(big);                                // scan32
@@ -361,6 +366,7 @@ static int bins_for(Run &r, Level &L) {
   finish_bins(L.bins, h);
   r.res->kernel_launches[LC_K_OTHER] += 4 * kBins + 1;
   L.hub = Hubs{};
+  L.max_deg = 0;
   const int H = (int)L.bins.count[kHubBin];
   if (H > 0) {
     int64_t *rows = nullptr;
@@ -373,6 +379,7 @@ static int bins_for(Run &r, Level &L) {
     std::vector<int32_t> hub_of, c0(H + 1);
     std::vector<int64_t> e0, e1;
     for (int k = 0; k < H; ++k) {
+      L.max_deg = std::max(L.max_deg, hrows[2 * k + 1] - hrows[2 * k]);
       c0[k] = (int32_t)hub_of.size();
       const int64_t ch = r.plan.hub_chunk;
       for (int64_t b = hrows[2 * k]; b < hrows[2 * k + 1]; b += ch) {
@@ -533,6 +540,20 @@ static int capture_pass(Run &r, Level &L, const PassArgs &a, const EmptyScratch 
   return LC_OK;
 }
 
+// Whether a level's passes run as one cooperative kernel (lc_fused.cu): the
+// plain passes of a level small enough that the separate launches, not their
+// work, set the time.  Measured by moving the line (ms per call, separate
+// kernels / line at 2 M / 4 M / 16 M / 40 M vertices and stored edges): 256^3
+// lattice 64.0 / 64.0 / 60.1 / 61.0 / 66.6, 512-graph batch 79.2 / 78.3 /
+// 77.8 / 78.4 / 80.7, an SBM of 100,000 vertices and 2 M stored edges 8.4 /
+// 6.8 / 6.5 / 6.5 / 6.5, one of 1 M vertices and 16 M stored edges 3.2 / 3.2 /
+// 3.2 / 3.2 / 3.8: a large level wants the separate kernels' occupancy.
+constexpr int64_t kFusedMaxSize = 4000000;
+static bool use_fused(const Run &r, const Level &L) {
+  return r.o.pass_limit >= 1 && r.o.tables == 0 && r.o.symmetry == 0 && !r.prof.on && !r.o.event_cb &&
+         L.g.n + L.g.nnz <= kFusedMaxSize;
+}
+
 // Algorithm 2: `pass_limit` synchronous passes from r.C for the graphs with
 // active[g]; leaves C_out (the best clustering seen, strict improvement) in
 // r.C_out and Phi(C_out) per graph in r.phi_out.
@@ -544,6 +565,31 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
   PassArgs a = pass_args(r, L);
   a.M = r.M;
   EmptyScratch w{r.used, r.freelist, r.emovers, r.gfree, r.gmover, r.eblocks};
+  if (use_fused(r, L)) {
+    FusedArgs f{};
+    f.rec = L.bins.recs;
+    for (int k = 0; k < kBins; ++k) f.off[k] = L.bins.list[k] - L.bins.list[0];
+    f.off[kBins] = n;
+    f.C_out = r.C_out;
+    f.acc = r.fused;
+    f.best = r.fused + 3 * (int64_t)r.G;
+    f.fin = r.fused + 5 * (int64_t)r.G;
+    f.phi_final = r.phi_final;
+    f.empties = r.sc->fused_empties;
+    f.next = r.sc->fused_next;
+    f.empty = w;
+    f.passes = r.o.pass_limit;
+    f.singleton = singleton;
+    f.big = L.max_deg > fused_row_max();
+    for (int k = 0; k < f.passes; ++k) {
+      f.phi[k][0] = r.o.phi_num[k];
+      f.phi[k][1] = r.o.phi_den[k];
+    }
+    r.res->kernel_launches[LC_K_MOVE] += launch_fused_passes(a, f, r.s);
+    r.res->passes_total += f.passes;
+    r.res->edges_local_move += f.passes * nnz;
+    return launch_check();
+  }
   if (singleton) {
     launch_iota(r.C, n, r.s);
     launch_iota(r.C_out, n, r.s);
@@ -695,6 +741,7 @@ static int constrained_passes(Run &r, Level &L, int level, const std::vector<uin
   const LevelGraph full = L.g;
   const Bins full_bins = L.bins;
   const Hubs full_hub = L.hub;
+  const int64_t full_max_deg = L.max_deg;
   int64_t *rp_f = nullptr;
   LC_TRY(r.ar.get(&rp_f, full.n + 1));
   r.prof.begin(LC_K_OTHER);
@@ -717,6 +764,7 @@ static int constrained_passes(Run &r, Level &L, int level, const std::vector<uin
   L.g = full;
   L.bins = full_bins;
   L.hub = full_hub;
+  L.max_deg = full_max_deg;
   if (rc == LC_OK) {
     r.ar.release(col_f);
     r.ar.release(ew_f);

@@ -33,20 +33,23 @@ __device__ __forceinline__ unsigned long long coop_scan(unsigned long long x, un
 
 // Labels the `total` > 0 vertices with C[v] = kEmpty.  Free ids and movers
 // are counted and listed together: packed as free << 32 | movers (both below
-// 2^31).  False if a barrier ran out.
-__device__ __forceinline__ bool assign_empty(const PassArgs &a, const EmptyScratch &w, int total,
+// 2^31).  marked: w.used already marks the ids in use.  False if a barrier
+// ran out.
+__device__ __forceinline__ bool assign_empty(const PassArgs &a, const EmptyScratch &w, int total, bool marked,
                                              GridBarrier &bar) {
   __shared__ unsigned long long red[kCoopThreads / 32];
   const int64_t n = a.g.n;
   const int64_t tid = (int64_t)blockIdx.x * kCoopThreads + threadIdx.x;
   const int64_t nt = (int64_t)gridDim.x * kCoopThreads;
-  for (int64_t x = tid; x < n; x += nt) w.used[x] = 0;
-  if (!bar.sync()) return false;
-  for (int64_t v = tid; v < n; v += nt) {
-    const int32_t x = a.C[v];
-    if (x >= 0) w.used[x] = 1;
+  if (!marked) {
+    for (int64_t x = tid; x < n; x += nt) w.used[x] = 0;
+    if (!bar.sync()) return false;
+    for (int64_t v = tid; v < n; v += nt) {
+      const int32_t x = a.C[v];
+      if (x >= 0) w.used[x] = 1;
+    }
+    if (!bar.sync()) return false;
   }
-  if (!bar.sync()) return false;
   // each block its own run of ids
   const int64_t per = ((n + gridDim.x - 1) / gridDim.x + kCoopThreads - 1) / kCoopThreads * kCoopThreads;
   const int64_t lo = (int64_t)blockIdx.x * per, hi = lo + per < n ? lo + per : n;

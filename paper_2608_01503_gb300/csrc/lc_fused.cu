@@ -1,0 +1,595 @@
+// lc_fused.cu — one LocalMovePasses call (Algorithm 2) as one kernel.
+//
+// A level of a few thousand to about a million vertices keeps the chip busy
+// for tens of microseconds per pass, while the separate kernels of a pass
+// (up to nine move kernels, the best-of test and copy, up to seven
+// afterburner kernels, the counters and the new-cluster ids) cost 2-4 us each
+// whatever they find to do.  Here all passes of a call run in one cooperative
+// launch of one 1,024-thread block per SM; the phases of a pass are separated
+// by grid barriers (1.2 us over 152 blocks, measured):
+//
+//   move:    gains, argmax, candidate test of every vertex; records written
+//   barrier
+//   update:  best-of test and copy (from the records), afterburner, moves
+//   barrier  (then the new-cluster ids if the pass has such movers)
+//
+// The work inside a phase is the separate kernels' own device code
+// (lc_move.cuh), so the results are identical.  Rows are taken by a thread
+// (bin 0), 16 lanes, a warp (bins 2-4), four warps (bins 5-6) or the block
+// (bins 7-8 and hubs of up to kRowSlots / 2 edges); longer hub rows go by
+// chunks over the global table, with two more barriers per pass.
+#include "lc_coop.cuh"
+#include "lc_empty.cuh"
+#include "lc_fused.cuh"
+#include "lc_move.cuh"
+
+namespace lc {
+
+namespace {
+
+constexpr int kT = kCoopThreads, kW = kT / 32;
+constexpr int kWarpSlots = 512;                 // shared table of a warp (bins 3-4)
+constexpr int kTeam = 128;                      // threads of a team (bins 5-6)
+constexpr int kTeamSlots = kWarpSlots * kTeam / 32;
+constexpr int kRowSlots = kWarpSlots * kW;      // the whole block's table
+constexpr int64_t kRowMaxDeg = kRowSlots / 2;   // rows above go by chunks
+
+// Per-warp staging; the move and update phases never hold theirs at once.
+union Stage {
+  struct {
+    MoveStage st;
+    LaneTags tags;
+  } move;
+  AbStage ab;
+};
+constexpr size_t kSmemBytes = sizeof(uint32_t) * 2 * kRowSlots + sizeof(Stage) * kW;
+
+// Barrier of one team of kTeam threads (ids 1 .. kT / kTeam; 0 is the block's).
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeam) : "memory");
+}
+
+// Work of a phase is handed out in order of cost: the first piece of a block,
+// team or warp by its place in the grid (warps in turn over SMs, so a short
+// list reaches every SM), every later piece from a counter, which evens out
+// the blocks that had long rows.  Pieces are fetched one ahead.
+enum { kNextRow = 0, kNextTeam = 1, kNextChunk = 2, kNextCount = 3 };
+
+// A run of bins cut into chunks for warps.
+struct ChunkList {
+  const VRec *rec;
+  int64_t count, chunks;
+  int c;
+};
+// One chunk of a list per warp, of at most `most` vertices (fewer where rows
+// are long, so that the last ones even out); a thread per vertex takes 32.
+__device__ __forceinline__ ChunkList chunk_list(const FusedArgs &f, int lo, int hi, int most) {
+  ChunkList l;
+  l.rec = f.rec + f.off[lo];
+  l.count = f.off[hi + 1] - f.off[lo];
+  const int64_t nw = (int64_t)gridDim.x * kW;
+  const int64_t c = (l.count + nw - 1) / nw;
+  l.c = lo == 0 ? 32 : c >= most ? most : c < 1 ? 1 : (int)c;
+  l.chunks = (l.count + l.c - 1) / l.c;
+  return l;
+}
+
+// Calls body(list, rec, base, m) for the warp's chunks of lists[0 .. N).
+template <int N, typename Body>
+__device__ __forceinline__ void for_chunks(const ChunkList (&lists)[N], unsigned *next, Body body) {
+  int64_t total = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) total += lists[k].chunks;
+  const unsigned nw = gridDim.x * kW;
+  const int lane = threadIdx.x & 31;
+  unsigned j = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  while (j < total) {  // chunks < 2^31: n is an int32 range
+    unsigned after = 0;
+    if (total > nw && lane == 0) after = nw + atomicAdd(next, 1u);
+    int64_t at = j;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      if (at >= 0 && at < lists[k].chunks) {
+        const int64_t base = at * lists[k].c, left = lists[k].count - base;
+        body(k, lists[k].rec, base, (int)(left < lists[k].c ? left : lists[k].c));
+      }
+      at -= lists[k].chunks;
+    }
+    if (total <= nw) break;
+    j = __shfl_sync(0xFFFFFFFFu, after, 0);
+  }
+}
+
+// Rows for whole blocks, longest bins first: the hubs up to kRowMaxDeg edges
+// and bins 8-7.  body must pass a block barrier.
+template <typename Body>
+__device__ __forceinline__ void block_rows(const FusedArgs &f, unsigned *next, Body body) {
+  __shared__ unsigned s_next;
+  const unsigned n = (unsigned)(f.off[kBins] - f.off[7]);
+  const VRec *last = f.rec + f.off[kBins] - 1;
+  for (unsigned i = blockIdx.x; i < n;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_next = n > gridDim.x ? gridDim.x + atomicAdd(next, 1u) : n;
+    const VRec vr = last[-(int64_t)i];
+    if (vr.deg <= kRowMaxDeg) body(vr);
+    __syncthreads();
+    i = s_next;
+  }
+}
+
+// Rows for teams of kTeam threads (bins 6-5).
+template <typename Body>
+__device__ __forceinline__ void team_rows(const FusedArgs &f, unsigned *next, Body body) {
+  constexpr int teams = kT / kTeam;
+  __shared__ unsigned s_next[teams];
+  const int team = threadIdx.x / kTeam;
+  const unsigned n = (unsigned)(f.off[7] - f.off[5]);
+  const VRec *last = f.rec + f.off[7] - 1;
+  const unsigned nteams = gridDim.x * teams;
+  for (unsigned i = team * gridDim.x + blockIdx.x; i < n;) {
+    team_sync(team);
+    if (threadIdx.x % kTeam == 0) s_next[team] = n > nteams ? nteams + atomicAdd(next, 1u) : n;
+    body(last[-(int64_t)i]);
+    team_sync(team);
+    i = s_next[team];
+  }
+}
+
+// Best (gain, cluster) and sum of S over `nw` warps' partials; every thread
+// of them has called it, `first` combines.
+struct RowPart {
+  long long g[kW];
+  int32_t x[kW], S[kW];
+};
+
+// Move step of one row of up to GS N edges by GS threads of rank r with
+// `slots` table slots.
+template <int GS, int N, typename Sync>
+__device__ __forceinline__ void row_move(const PassArgs &a, const VRec &vr, SplitTab tab, uint32_t slots, int r,
+                                         RowPart &part, Sync sync, MoveState &ms) {
+  const int32_t v = vr.v;
+  const int32_t Cv = LC_IDX(a.C[v], a.g.n, kDbgLabel);
+  const GraphParam P = a.gp[vr.g];
+  const long long muw = P.mu * vr.w;
+  bool ok = true;
+  int32_t slot[N];
+  const int32_t self = claim_row<GS, N>(a, vr.beg, vr.deg, Cv, tab, slots, r, slot, ok);
+  if (!ok) {
+    a.sc->error = 1;
+    LC_DBG_FAIL(kDbgProbe, v, a.g.n);
+  }
+  sync();
+  long long gb = LLONG_MIN;
+  int32_t xb = kNone;
+  claim_argmax<N>(a, P.Lam, muw, tab, slot, gb, xb, ms.nX);
+  warp_argmax(gb, xb);
+  int32_t S = (int32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)self);
+  const int w0 = (threadIdx.x - r) >> 5;  // the row's first warp
+  if ((threadIdx.x & 31) == 0) {
+    part.g[threadIdx.x >> 5] = gb;
+    part.x[threadIdx.x >> 5] = xb;
+    part.S[threadIdx.x >> 5] = S;
+  }
+  sync();
+  if (r == 0) {
+    for (int w = 1; w < GS / 32; ++w) {
+      S += part.S[w0 + w];
+      if (better(part.g[w0 + w], part.x[w0 + w], gb, xb)) {
+        gb = part.g[w0 + w];
+        xb = part.x[w0 + w];
+      }
+    }
+    const long long gC = gain_self(P, S, vr.w, a.W[Cv]);
+    phi_add_one(a, ms.acc, vr.g, gC, ms.phi);
+    decide(a, P, v, Cv, gC, xb, gb, ms);
+  }
+  // part is written again only after the next row's first sync
+}
+
+// First pass (singleton start) of one row by GS threads.
+template <int GS, typename Sync>
+__device__ __forceinline__ void row_first(const PassArgs &a, const VRec &vr, int r, RowPart &part, Sync sync,
+                                          MoveState &ms) {
+  const GraphParam P = a.gp[vr.g];
+  const long long muw = P.mu * vr.w;
+  long long gb = LLONG_MIN;
+  int32_t xb = kNone;
+#pragma unroll 4
+  for (int64_t e = vr.beg + r; e < vr.beg + vr.deg; e += GS) first_edge(a, P.Lam, muw, e, gb, xb);
+  warp_argmax(gb, xb);
+  const int w0 = (threadIdx.x - r) >> 5;
+  sync();  // the last row's partials have been read
+  if ((threadIdx.x & 31) == 0) {
+    part.g[threadIdx.x >> 5] = gb;
+    part.x[threadIdx.x >> 5] = xb;
+  }
+  sync();
+  if (r == 0) {
+    for (int w = 1; w < GS / 32; ++w)
+      if (better(part.g[w0 + w], part.x[w0 + w], gb, xb)) {
+        gb = part.g[w0 + w];
+        xb = part.x[w0 + w];
+      }
+    decide(a, P, vr.v, vr.v, 0, xb, gb, ms);
+  }
+}
+
+// Sum of x over the block (every thread; the result in thread 0).
+__device__ __forceinline__ long long block_total(long long x, long long *red) {
+  x = warp_sum(x);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  if (threadIdx.x >= 32) return 0;
+  return warp_sum(red[threadIdx.x]);
+}
+
+// The chunks of the hubs above kRowMaxDeg edges.
+template <typename Body>
+__device__ __forceinline__ void big_chunks(const PassArgs &a, Body body) {
+  for (int c = blockIdx.x; c < a.hub.Q; c += gridDim.x) {
+    const int h = a.hub.hub_of[c];
+    const int32_t v = a.hub.vtx[h];
+    if (a.g.rp[v + 1] - a.g.rp[v] > kRowMaxDeg) body(c, h, v);
+  }
+}
+
+__global__ void __launch_bounds__(kT, 1)
+    k_passes(const __grid_constant__ PassArgs a, const __grid_constant__ FusedArgs f) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  uint32_t *keys = reinterpret_cast<uint32_t *>(smem);
+  int32_t *vals = reinterpret_cast<int32_t *>(keys + kRowSlots);
+  Stage &stage = reinterpret_cast<Stage *>(vals + kRowSlots)[threadIdx.x >> 5];
+  __shared__ RowPart part;
+  __shared__ long long red[kW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, team = threadIdx.x / kTeam;
+  const SplitTab wtab{keys + wid * kWarpSlots, vals + wid * kWarpSlots};
+  const SplitTab ttab{keys + team * kTeamSlots, vals + team * kTeamSlots};
+  const SplitTab btab{keys, vals};
+  auto bsync = [] { __syncthreads(); };
+  auto tsync = [team] { team_sync(team); };
+  const int64_t n = a.g.n;
+  const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
+  const int64_t wbase = tid - lane;  // whole-warp loops start here
+  const int G = a.G;
+  GridBarrier bar(a.sc);
+
+  for (int s = threadIdx.x; s < kRowSlots; s += kT) {
+    keys[s] = 0u;
+    vals[s] = 0;
+  }
+  // clustering, cluster weights, accumulators of the call
+  for (int64_t v = tid; v < n; v += nt) {
+    if (f.singleton) {
+      a.C[v] = (int32_t)v;
+      f.C_out[v] = (int32_t)v;
+      a.W[v] = a.g.vw[v];
+    } else {
+      a.W[v] = 0;
+    }
+  }
+  for (int64_t g = tid; g < G; g += nt) {
+    f.acc[g] = f.acc[G + g] = f.acc[2 * G + g] = 0;
+    f.fin[g] = 0;
+    f.best[g] = f.singleton ? 0 : LLONG_MIN;  // Phi(singletons) = 0
+  }
+  if (tid < 6) f.empties[tid] = 0;
+  if (tid < 2 * kNextCount) f.next[tid] = 0;
+  if (!bar.sync()) return;
+  if (!f.singleton) {
+    for (int64_t v0 = wbase; v0 < n; v0 += nt) {
+      const int64_t v = v0 + lane;
+      add_weights(a.W, v < n, v < n ? a.C[v] : 0, v < n ? a.g.vw[v] : 0);
+    }
+    if (!bar.sync()) return;
+  }
+
+  for (int i = 0; i < f.passes; ++i) {
+    const bool first = f.singleton && i == 0, last = i + 1 == f.passes;
+    long long *acc = f.acc + (int64_t)(i % 3) * G;       // Phi entering this pass
+    const long long *best = f.best + (int64_t)(i & 1) * G;
+    long long *best_next = f.best + (int64_t)((i & 1) ^ 1) * G;
+    MoveState ms;
+    ms.acc = acc;
+    ms.num = f.phi[i][0];
+    ms.den = f.phi[i][1];
+    if (tid == 0) f.empties[(i + 1) % 3] = f.empties[3 + (i + 1) % 3] = 0;
+    for (int64_t x = tid; x < n; x += nt) f.empty.used[x] = 0;
+
+    // ------------------------------------------------------------ move
+    unsigned *next = f.next + (i % 3) * 2 * kNextCount;
+    if (tid < 2 * kNextCount) f.next[((i + 1) % 3) * 2 * kNextCount + tid] = 0;
+    {
+      if (first) {
+        block_rows(f, next + kNextRow, [&](const VRec &vr) { row_first<kT>(a, vr, threadIdx.x, part, bsync, ms); });
+        if (f.big)
+          big_chunks(a, [&](int c, int h, int32_t v) {
+            const GraphParam P = a.gp[graph_of(a, v)];
+            const long long muw = P.mu * a.g.vw[v];
+            long long gb = LLONG_MIN;
+            int32_t xb = kNone;
+            for (int64_t e = a.hub.e0[c] + threadIdx.x; e < a.hub.e1[c]; e += kT)
+              first_edge(a, P.Lam, muw, e, gb, xb);
+            Grp<kT>::argmax(gb, xb, part.g, part.x);
+            if (threadIdx.x == 0) {
+              a.hub.part_g[c] = gb;
+              a.hub.part_x[c] = xb;
+            }
+          });
+        const ChunkList lists[4] = {chunk_list(f, 5, 6, 1), chunk_list(f, 2, 4, 8), chunk_list(f, 1, 1, 32),
+                                    chunk_list(f, 0, 0, 32)};
+        for_chunks(lists, next + kNextChunk, [&](int k, const VRec *rec, int64_t b, int m) {
+          if (k <= 1)
+            first_chunk<32>(a, rec, b, m, stage.move.st, ms);
+          else if (k == 2)
+            first_chunk<16>(a, rec, b, m, stage.move.st, ms);
+          else if (lane < m)
+            first_thread(a, rec, b + lane, ms);
+        });
+      } else {
+        if (f.big)
+          big_chunks(a, [&](int c, int h, int32_t v) {
+            const long long s = block_total(hub_insert<kT>(a, c, stage.move.tags), red);
+            if (threadIdx.x == 0 && s != 0)
+              atomicAdd((unsigned long long *)&a.hub.acc[h], (unsigned long long)s);
+          });
+        block_rows(f, next + kNextRow, [&](const VRec &vr) {
+          row_move<kT, (int)(kRowMaxDeg / kT)>(a, vr, btab, kRowSlots, threadIdx.x, part, bsync, ms);
+        });
+        __syncthreads();
+        team_rows(f, next + kNextTeam, [&](const VRec &vr) {
+          row_move<kTeam, kTeamSlots / 2 / kTeam>(a, vr, ttab, kTeamSlots, threadIdx.x % kTeam, part, tsync, ms);
+        });
+        __syncthreads();  // the teams' tables are clean and their partials read
+        const ChunkList lists[4] = {chunk_list(f, 3, 4, 8), chunk_list(f, 2, 2, 32), chunk_list(f, 1, 1, 32),
+                                    chunk_list(f, 0, 0, 32)};
+        for_chunks(lists, next + kNextChunk, [&](int k, const VRec *rec, int64_t b, int m) {
+          if (k == 0)
+            warp_chunk(a, rec, b, m, stage.move.st, wtab, kWarpSlots, ms);
+          else if (k == 1)
+            lanes_chunk<32>(a, rec, b, m, stage.move.st, stage.move.tags, ms);
+          else if (k == 2)
+            lanes_chunk<16>(a, rec, b, m, stage.move.st, stage.move.tags, ms);
+          else
+            move_thread(a, lane < m, rec, b + lane, ms);
+        });
+      }
+      if (last)  // Q of W before the last update (see launch_final_objective)
+        for (int64_t x0 = wbase; x0 < n; x0 += nt) {
+          const int64_t x = x0 + lane;
+          const int g = x < n ? graph_of(a, (int32_t)x) : -1;
+          const unsigned long long W = x < n ? (unsigned long long)a.W[x] : 0ull;
+          graph_add(f.fin, g, g >= 0 ? (long long)((unsigned long long)a.gp[g].mu * W * W) : 0ll);
+        }
+    }
+    if (f.big) {
+      if (!bar.sync()) return;
+      if (!first) {
+        big_chunks(a, [&](int c, int h, int32_t v) {
+          const GraphParam P = a.gp[graph_of(a, v)];
+          const int64_t beg = a.g.rp[v];
+          long long gb = LLONG_MIN;
+          int32_t xb = kNone;
+          range_argmax<kT>(a, P.Lam, P.mu * a.g.vw[v], a.gtab + 2 * beg, (uint32_t)(2 * (a.hub.e0[c] - beg)),
+                           (uint32_t)(2 * (a.hub.e1[c] - beg)), threadIdx.x, gb, xb, ms.nX);
+          Grp<kT>::argmax(gb, xb, part.g, part.x);
+          if (threadIdx.x == 0) {
+            a.hub.part_g[c] = gb;
+            a.hub.part_x[c] = xb;
+          }
+        });
+        if (!bar.sync()) return;
+      }
+      for (int64_t h = tid; h < a.hub.H; h += nt) {
+        const int32_t v = a.hub.vtx[h];
+        if (a.g.rp[v + 1] - a.g.rp[v] <= kRowMaxDeg) continue;
+        const int g = graph_of(a, v);
+        const GraphParam P = a.gp[g];
+        long long gb = LLONG_MIN, gC = 0;
+        int32_t xb = kNone;
+        for (int c = a.hub.c0[h]; c < a.hub.c0[h + 1]; ++c)
+          if (better(a.hub.part_g[c], a.hub.part_x[c], gb, xb)) {
+            gb = a.hub.part_g[c];
+            xb = a.hub.part_x[c];
+          }
+        const int32_t Cv = a.C[v];
+        if (!first) {
+          gC = gain_self(P, a.hub.acc[h], a.g.vw[v], a.W[Cv]);
+          a.hub.acc[h] = 0;
+          phi_add_one(a, acc, g, gC, ms.phi);
+        }
+        decide(a, P, v, Cv, gC, xb, gb, ms);
+      }
+    }
+    {
+      const int e = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)ms.empties);
+      if (lane == 0 && e) atomicAdd(&f.empties[3 + i % 3], e);
+    }
+    if (!first && !a.gid) {
+      const long long t = block_total(ms.phi, red);
+      if (threadIdx.x == 0 && t != 0) atomicAdd((unsigned long long *)acc, (unsigned long long)t);
+    }
+    if (!bar.sync()) return;
+
+    // ---------------------------------------------------------- update
+    // best-of test (Algorithm 2) on the state entering the pass: its labels
+    // are in the records, which the moves below do not touch
+    if (!first) {
+      const bool all = !a.gid && acc[0] > best[0];
+      if (a.gid || all)
+        for (int64_t v = tid; v < n; v += nt) {
+          const int g = graph_of(a, (int32_t)v);
+          if (all || acc[g] > best[g]) f.C_out[v] = a.ab[v].C;
+        }
+    }
+    for (int64_t g = tid; g < G; g += nt) {
+      best_next[g] = !first && acc[g] > best[g] ? acc[g] : best[g];
+      f.acc[(int64_t)((i + 1) % 3) * G + g] = 0;
+    }
+    UpdateSums us;
+    // ids in use are marked if some candidate wants a new cluster (uniform)
+    int32_t *used = f.empties[3 + i % 3] > 0 ? f.empty.used : nullptr;
+    next += kNextCount;
+    {
+      if (f.big)
+        big_chunks(a, [&](int c, int h, int32_t v) {
+          const AbRec r = a.ab[v];
+          if (r.D == kNone) return;  // block-uniform
+          const AbCtx ctx = ab_ctx(a, v, r, a.gp[graph_of(a, v)], 0, 0, a.g.vw[v]);
+          const long long s = block_total(ab_edges<kT, 2>(a, ctx, a.hub.e0[c], a.hub.e1[c], threadIdx.x), red);
+          if (threadIdx.x == 0 && s != 0)
+            atomicAdd((unsigned long long *)&a.hub.acc[h], (unsigned long long)s);
+        });
+      block_rows(f, next + kNextRow, [&](const VRec &vr) {
+        const AbRec r = a.ab[vr.v];
+        bool keep = false;
+        if (r.D != kNone) {
+          const AbCtx ctx = ab_ctx(a, vr.v, r, a.gp[vr.g], vr.beg, vr.deg, vr.w);
+          const long long s = block_total(ab_edges<kT, 4>(a, ctx, vr.beg, vr.beg + vr.deg, threadIdx.x), red);
+          keep = a.delta[vr.v] + s >= 0;  // thread 0's
+        }
+        if (wid == 0) apply_lanes(a, lane == 0, vr.v, vr.deg, r, vr.w, keep, us, used);
+      });
+      const ChunkList lists[5] = {chunk_list(f, 5, 6, 1), chunk_list(f, 3, 4, 8), chunk_list(f, 2, 2, 32),
+                                  chunk_list(f, 1, 1, 32), chunk_list(f, 0, 0, 32)};
+      for_chunks(lists, next + kNextChunk, [&](int k, const VRec *rec, int64_t b, int m) {
+        if (k <= 1)
+          ab_chunk<32>(a, rec, b, m, stage.ab, us, used);
+        else if (k == 2)
+          ab_chunk<8>(a, rec, b, m, stage.ab, us, used);
+        else if (k == 3)
+          ab_chunk<4>(a, rec, b, m, stage.ab, us, used);
+        else
+          ab_thread(a, lane < m, rec, b + lane, us, used);
+      });
+    }
+    if (f.big) {
+      if (!bar.sync()) return;
+      for (int64_t h0 = wbase; h0 < a.hub.H; h0 += nt) {
+        const int64_t h = h0 + lane;
+        bool on = h < a.hub.H, keep = false;
+        int32_t v = 0;
+        int64_t deg = 0;
+        AbRec r{0, kNone, 0};
+        if (on) {
+          v = a.hub.vtx[h];
+          deg = a.g.rp[v + 1] - a.g.rp[v];
+          on = deg > kRowMaxDeg;
+        }
+        if (on) {
+          r = a.ab[v];
+          keep = r.D != kNone && a.delta[v] + a.hub.acc[h] >= 0;
+          a.hub.acc[h] = 0;
+        }
+        apply_lanes(a, on, v, deg, r, on ? a.g.vw[v] : 0, keep, us, used);
+      }
+    }
+    {
+      const int e = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)us.empties);
+      if (lane == 0 && e) atomicAdd(&f.empties[i % 3], e);
+    }
+    if (!bar.sync()) return;
+    const int total = f.empties[i % 3];
+    if (total > 0) {  // uniform over the grid
+      if (!assign_empty(a, f.empty, total, true, bar)) return;
+      if (!bar.sync()) return;
+    }
+  }
+
+  // ---------------------------------- objective of the final state
+  // Phi' = Phi + Lam dIN - mu (Q' - Q), from the last pass's movers' rows
+  // and W (lc_pass.cu, launch_final_objective); Q' - sum w^2 and Q - sum w^2
+  // differ by the same constant, so W^2 alone is summed.
+  const int p = f.passes;
+  {
+    long long dphi = 0;
+    auto add = [&](int g, long long d) {  // one thread
+      const long long x = a.gp[g].Lam * d;
+      if (!a.gid)
+        dphi += x;
+      else if (x != 0)
+        atomicAdd((unsigned long long *)&f.fin[g], (unsigned long long)x);
+    };
+    {
+      const VRec *rec = f.rec + f.off[7];
+      for (int64_t i = blockIdx.x; i < f.off[kBins] - f.off[7]; i += gridDim.x) {
+        const VRec vr = rec[i];
+        if (a.C[vr.v] == a.ab[vr.v].C) continue;  // not a mover
+        const long long d = block_total(delta_in_edges<kT>(a, vr.v, vr.beg, vr.beg + vr.deg, threadIdx.x), red);
+        if (threadIdx.x == 0) add(vr.g, d);
+      }
+    }
+    const ChunkList lists[3] = {chunk_list(f, 5, 6, 1), chunk_list(f, 1, 4, 8), chunk_list(f, 0, 0, 32)};
+    // the counters of the pass after the last were zeroed by it and not used
+    for_chunks(lists, f.next + (p % 3) * 2 * kNextCount, [&](int k, const VRec *rec, int64_t b, int m) {
+      VRec vr{};
+      bool mover = false;
+      if (lane < m) {
+        vr = rec[b + lane];
+        mover = a.C[vr.v] != a.ab[vr.v].C;
+      }
+      if (k == 2) {
+        if (mover) add(vr.g, delta_in_edges<1>(a, vr.v, vr.beg, vr.beg + vr.deg, 0));
+        __syncwarp();
+        return;
+      }
+      for (unsigned left = __ballot_sync(0xFFFFFFFFu, mover); left; left &= left - 1) {
+        const int j = __ffs(left) - 1;
+        const int32_t v = __shfl_sync(0xFFFFFFFFu, vr.v, j), deg = __shfl_sync(0xFFFFFFFFu, vr.deg, j);
+        const int64_t beg = __shfl_sync(0xFFFFFFFFu, vr.beg, j);
+        const long long d = warp_sum(delta_in_edges<32>(a, v, beg, beg + deg, lane));
+        if (lane == j) add(vr.g, d);
+      }
+    });
+    for (int64_t x0 = wbase; x0 < n; x0 += nt) {
+      const int64_t x = x0 + lane;
+      const int g = x < n ? graph_of(a, (int32_t)x) : -1;
+      const unsigned long long W = x < n ? (unsigned long long)a.W[x] : 0ull;
+      graph_add(f.fin, g, g >= 0 ? -(long long)((unsigned long long)a.gp[g].mu * W * W) : 0ll);
+    }
+    if (!a.gid) {
+      const long long t = block_total(dphi, red);
+      if (threadIdx.x == 0 && t != 0) atomicAdd((unsigned long long *)f.fin, (unsigned long long)t);
+    }
+  }
+  if (!bar.sync()) return;
+  const long long *acc = f.acc + (int64_t)((p - 1) % 3) * G;
+  const long long *best = f.best + (int64_t)(p & 1) * G;
+  {
+    const bool all = !a.gid && acc[0] + f.fin[0] > best[0];
+    if (a.gid || all)
+      for (int64_t v = tid; v < n; v += nt) {
+        const int g = graph_of(a, (int32_t)v);
+        if (all || acc[g] + f.fin[g] > best[g]) f.C_out[v] = a.C[v];
+      }
+  }
+  for (int64_t g = tid; g < G; g += nt) {
+    const long long now = acc[g] + f.fin[g];
+    const long long out = now > best[g] ? now : best[g];
+    a.phi_out[g] = out;
+    if (a.gp[g].active) f.phi_final[g] = out;
+  }
+  bar.leave();
+}
+
+}  // namespace
+
+void configure_fused() {
+  cudaFuncSetAttribute(k_passes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+}
+
+int64_t fused_row_max() { return kRowMaxDeg; }
+
+int launch_fused_passes(const PassArgs &a, const FusedArgs &f, cudaStream_t s) {
+  // a block per 64 vertices or 1,024 stored edges, at most one per SM
+  int64_t blocks = a.g.n / 64 > a.g.nnz / 1024 ? a.g.n / 64 : a.g.nnz / 1024;
+  if (blocks > coop_blocks()) blocks = coop_blocks();
+  if (blocks < 1) blocks = 1;
+  PassArgs pa = a;
+  FusedArgs fa = f;
+  void *args[] = {&pa, &fa};
+  cudaLaunchCooperativeKernel((const void *)k_passes, dim3((unsigned)blocks), dim3(kT), args, kSmemBytes, s);
+  return 1;
+}
+
+}  // namespace lc

@@ -165,6 +165,8 @@ struct Scalars {
   // both zero between launches; on a line of their own
   alignas(128) unsigned bar_arrived;
   unsigned bar_left;
+  int fused_empties[6];      // FusedArgs::empties
+  unsigned fused_next[18];   // FusedArgs::next
   // device-side temperature schedule (graph replays): k_pass_begin loads
   // phi_live from phi_tab[pass_idx] and advances pass_idx
   int pass_idx;

@@ -25,18 +25,41 @@ __device__ __forceinline__ int graph_of(const PassArgs &a, int32_t v) { return a
 // Adds x to the objective of graph g (whole warps; lanes with on = false add
 // nothing): one graph accumulates in a register that the kernel flushes once
 // per block, a batch adds warp sums to the graph's accumulator.
-__device__ __forceinline__ void phi_add(const PassArgs &a, bool on, int g, long long x, long long &phi) {
+__device__ __forceinline__ void phi_add(const PassArgs &a, long long *acc, bool on, int g, long long x,
+                                        long long &phi) {
   if (!a.gid)
     phi += on ? x : 0;
   else
-    graph_add(a.phi_acc, on ? g : -1, x);
+    graph_add(acc, on ? g : -1, x);
 }
 // The same from one thread of a block.
-__device__ __forceinline__ void phi_add_one(const PassArgs &a, int g, long long x, long long &phi) {
+__device__ __forceinline__ void phi_add_one(const PassArgs &a, long long *acc, int g, long long x,
+                                            long long &phi) {
   if (!a.gid)
     phi += x;
   else if (x != 0)
-    atomicAdd((unsigned long long *)&a.phi_acc[g], (unsigned long long)x);
+    atomicAdd((unsigned long long *)&acc[g], (unsigned long long)x);
+}
+
+// What a move step sums per thread, its temperature phi = num / den and the
+// per-graph objective accumulator it adds to.
+struct MoveState {
+  long long *acc;
+  int32_t num, den;
+  long long cntL = 0, phi = 0, nX = 0;
+  int empties = 0;  // candidates for a new empty cluster
+};
+__device__ __forceinline__ MoveState move_state(const PassArgs &a) {
+  MoveState m;
+  m.acc = a.phi_acc;
+  m.num = a.phi_live ? a.phi_live[0] : a.phi_n;
+  m.den = a.phi_live ? a.phi_live[1] : a.phi_d;
+  return m;
+}
+__device__ __forceinline__ void flush_move(const PassArgs &a, const MoveState &m) {
+  flush_block_sum(m.nX, &a.sc->distinct_x);
+  flush_block_sum(m.cntL, &a.sc->count_L);
+  flush_block_sum(m.phi, &m.acc[0]);
 }
 
 // ---------------------------------------------------- vertex decision
@@ -46,7 +69,7 @@ __device__ __forceinline__ void phi_add_one(const PassArgs &a, int g, long long 
 // temperature phi = phi_n / phi_d, delta_v and its epsilon bucket
 // (Algorithm 3's priority).  Writes the record of every vertex.
 __device__ __forceinline__ void decide(const PassArgs &a, const GraphParam &P, int32_t v, int32_t Cv,
-                                       long long gC, int32_t best, long long gbest, long long &cntL) {
+                                       long long gC, int32_t best, long long gbest, MoveState &ms) {
   AbRec r;
   r.C = Cv;
   r.D = kNone;
@@ -56,14 +79,13 @@ __device__ __forceinline__ void decide(const PassArgs &a, const GraphParam &P, i
       best = kEmpty;
       gbest = 0;
     }
-    const int32_t pn = a.phi_live ? a.phi_live[0] : a.phi_n;
-    const int32_t pd = a.phi_live ? a.phi_live[1] : a.phi_d;
-    if (best != kNone && (__int128)pd * gbest >= (__int128)(pd - pn) * (__int128)gC) {
+    if (best != kNone && (__int128)ms.den * gbest >= (__int128)(ms.den - ms.num) * (__int128)gC) {
       const long long delta = gbest - gC;
       r.D = best;
       r.q = eps_bucket(a.m, P.Lam, delta);
       a.delta[v] = delta;
-      cntL++;
+      ms.cntL++;
+      ms.empties += best == kEmpty;
     }
   }
   a.ab[v] = r;
@@ -110,12 +132,12 @@ __device__ __forceinline__ ChunkLane stage_move(const PassArgs &a, const VRec *_
 
 // Decides the chunk's vertices from the staged results (full warp).
 __device__ __forceinline__ void settle_move(const PassArgs &a, const ChunkLane &c, int m, int lane, bool first,
-                                            const MoveRes *res, long long &cntL, long long &phi) {
+                                            const MoveRes *res, MoveState &ms) {
   const bool on = lane < m;
   const MoveRes r = on ? res[lane] : MoveRes{0, kNone, 0};
   const long long gC = first ? 0 : gain_self(c.P, r.S, c.vr.w, c.WC);
-  if (!first) phi_add(a, on, c.vr.g, gC, phi);
-  if (on) decide(a, c.P, c.vr.v, c.Cv, gC, r.x, r.g, cntL);
+  if (!first) phi_add(a, ms.acc, on, c.vr.g, gC, ms.phi);
+  if (on) decide(a, c.P, c.vr.v, c.Cv, gC, r.x, r.g, ms);
 }
 
 // ------------------------------------------- first pass (Section IV-A-3)
@@ -144,7 +166,7 @@ __device__ __forceinline__ void lanes_argmax(long long &g, int32_t &x) {
 
 template <int G>
 __device__ __forceinline__ void first_chunk(const PassArgs &a, const VRec *__restrict__ rec, int64_t base, int m,
-                                            MoveStage &st, long long &cntL) {
+                                            MoveStage &st, MoveState &ms) {
   constexpr int V = 32 / G;
   const int lane = threadIdx.x & 31, grp = lane / G, sub = lane & (G - 1);
   const ChunkLane c = stage_move(a, rec, base, m, lane, true, st.ctx);
@@ -163,8 +185,7 @@ __device__ __forceinline__ void first_chunk(const PassArgs &a, const VRec *__res
     if (idx < m && sub == 0) st.res[idx] = MoveRes{gb, xb, 0};
   }
   __syncwarp();
-  long long phi = 0;
-  settle_move(a, c, m, lane, true, st.res, cntL, phi);
+  settle_move(a, c, m, lane, true, st.res, ms);
   __syncwarp();
 }
 
@@ -225,6 +246,36 @@ __device__ __forceinline__ long long thread_gains(const PassArgs &a, const VRec 
   return self;
 }
 
+// Bin 0: one thread per vertex (full warp, lanes with on = false idle).
+__device__ __forceinline__ void move_thread(const PassArgs &a, bool on, const VRec *__restrict__ rec, int64_t i,
+                                            MoveState &ms) {
+  VRec vr{};
+  long long gC = 0;
+  if (on) {
+    vr = rec[i];
+    const int32_t Cv = LC_IDX(a.C[vr.v], a.g.n, kDbgLabel);
+    const GraphParam P = a.gp[vr.g];
+    const long long WC = a.W[Cv];
+    long long gb;
+    int32_t xb;
+    const long long self = thread_gains(a, vr, Cv, P, gb, xb, ms.nX);
+    gC = gain_self(P, self, vr.w, WC);
+    decide(a, P, vr.v, Cv, gC, xb, gb, ms);
+  }
+  phi_add(a, ms.acc, on, vr.g, gC, ms.phi);
+}
+
+__device__ __forceinline__ void first_thread(const PassArgs &a, const VRec *__restrict__ rec, int64_t i,
+                                             MoveState &ms) {
+  const VRec vr = rec[i];
+  const GraphParam P = a.gp[vr.g];
+  long long gb = LLONG_MIN;
+  int32_t xb = kNone;
+#pragma unroll 4
+  for (int64_t e = vr.beg; e < vr.beg + vr.deg; ++e) first_edge(a, P.Lam, P.mu * vr.w, e, gb, xb);
+  decide(a, P, vr.v, vr.v, 0, xb, gb, ms);
+}
+
 // ------------------------------------ aggregation + argmax, bins 1-2 (lanes)
 
 // Shared scratch of a warp whose lanes hold one neighbour each: 1,024 byte
@@ -278,71 +329,77 @@ __device__ __forceinline__ int32_t lane_sums(LaneTags &t, int lane, bool on, int
   return S;
 }
 
+// A step takes the rows of two vertices (G = 32) or four (G = 16): their
+// label gathers are issued together, then their W gathers, while the next
+// step's columns and weights are on their way.
 template <int G>
 __device__ __forceinline__ void lanes_chunk(const PassArgs &a, const VRec *__restrict__ rec, int64_t base, int m,
-                                            MoveStage &st, LaneTags &tags, long long &cntL, long long &phi,
-                                            long long &nX) {
-  constexpr int V = 32 / G;
+                                            MoveStage &st, LaneTags &tags, MoveState &ms) {
+  constexpr int V = 32 / G, U = 2;
   const int lane = threadIdx.x & 31, grp = lane / G, sub = lane & (G - 1);
   const ChunkLane c = stage_move(a, rec, base, m, lane, false, st.ctx);
   __syncwarp();
-  // the next vertices' columns and weights are loaded while this one's
-  // clusters are gathered
-  auto load = [&](int k, int32_t &u, int32_t &w) {
+  auto load = [&](int idx, int32_t &u, int32_t &w) {
     u = -1;
     w = 0;
-    if (k + grp < m && sub < st.ctx[k + grp].deg) {
-      const int64_t e = st.ctx[k + grp].beg + sub;
+    if (idx < m && sub < st.ctx[idx].deg) {
+      const int64_t e = st.ctx[idx].beg + sub;
       u = LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn);
       w = __ldg(a.g.ew + e);
     }
   };
-  int32_t u, w;
-  load(0, u, w);
-  for (int k = 0; k < m; k += V) {
-    const int idx = k + grp;
-    const int32_t X = u >= 0 ? LC_IDX(a.C[u], a.g.n, kDbgLabel) : -1;
-    int32_t un, wn;
-    load(k + V, un, wn);
-    MoveCtx x{0, 0, -2, 0, 0};
-    if (idx < m) x = st.ctx[idx];
-    const bool self = u >= 0 && X == x.Cv;
-    const bool other = u >= 0 && !self;
-    const long long WX = other ? a.W[X] : 0;
-    int32_t S_self;
-    if constexpr (G == 32)
-      S_self = (int32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)(self ? w : 0));
-    else
-      S_self = group_sum<G>(self ? w : 0);
-    int leader;
-    const int32_t S = lane_sums<G>(tags, lane, other, X, w, leader);
-    long long g = LLONG_MIN;
-    int32_t xb = kNone;
-    if (other && leader == lane) {
-      g = x.Lam * (long long)S - x.muw * WX;
-      xb = X;
-      nX++;
+  int32_t u[U], w[U];
+#pragma unroll
+  for (int j = 0; j < U; ++j) load(j * V + grp, u[j], w[j]);
+  for (int k = 0; k < m; k += U * V) {
+    int32_t X[U], wk[U];
+    long long WX[U];
+    bool other[U], self[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) X[j] = u[j] >= 0 ? LC_IDX(a.C[u[j]], a.g.n, kDbgLabel) : -1;
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int idx = k + j * V + grp;
+      const int32_t Cv = idx < m ? st.ctx[idx].Cv : -2;
+      self[j] = u[j] >= 0 && X[j] == Cv;
+      other[j] = u[j] >= 0 && !self[j];
+      wk[j] = w[j];
     }
-    lanes_argmax<G>(g, xb);
-    if (idx < m && sub == 0) st.res[idx] = MoveRes{g, xb, S_self};
-    u = un;
-    w = wn;
+#pragma unroll
+    for (int j = 0; j < U; ++j) load(k + (U + j) * V + grp, u[j], w[j]);
+#pragma unroll
+    for (int j = 0; j < U; ++j) WX[j] = other[j] ? a.W[X[j]] : 0;
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      if (k + j * V >= m) break;  // uniform
+      const int idx = k + j * V + grp;
+      int32_t S_self;
+      if constexpr (G == 32)
+        S_self = (int32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)(self[j] ? wk[j] : 0));
+      else
+        S_self = group_sum<G>(self[j] ? wk[j] : 0);
+      int leader;
+      const int32_t S = lane_sums<G>(tags, lane, other[j], X[j], wk[j], leader);
+      long long g = LLONG_MIN;
+      int32_t xb = kNone;
+      if (other[j] && leader == lane) {
+        g = st.ctx[idx].Lam * (long long)S - st.ctx[idx].muw * WX[j];
+        xb = X[j];
+        ms.nX++;
+      }
+      lanes_argmax<G>(g, xb);
+      if (idx < m && sub == 0) st.res[idx] = MoveRes{g, xb, S_self};
+    }
   }
   __syncwarp();
-  settle_move(a, c, m, lane, false, st.res, cntL, phi);
+  settle_move(a, c, m, lane, false, st.res, ms);
   __syncwarp();
 }
 
 // ------------------------------------ shared-table aggregation, bins 3-5
 
-// Shared tables stay clean between vertices: a vertex's argmax scans the
-// slots [0, cap) it may have used and resets the occupied ones.  The warp
-// bins use 2 deg rounded up to 32 slots (load <= 1/2, whole warps of slots);
-// the block bins use tab_cap(deg), the layout of the kept tables.
-__device__ __forceinline__ uint32_t warp_table_cap(int64_t deg) {
-  return (uint32_t)((2 * deg + 31) & ~31ll);
-}
-
+// Shared tables stay clean between vertices: a vertex's argmax resets the
+// slots it used.
 // Best (gain, cluster) over slots [s0, s1) of a table (strided by GS),
 // resetting the slots it reads unless `keep` (a kept table being built).
 // g(v, X) = Lam S(v, X) - (mu w(v)) W(X), with mu w(v) formed once.
@@ -468,9 +525,9 @@ __device__ __forceinline__ long long split_insert_row(const PassArgs &a, int64_t
 }
 
 // Best (gain, cluster) over slots [0, cap) (strided by GS), resetting the
-// occupied ones.  g(v, X) = Lam S(v, X) - (mu w(v)) W(X).  BUILD: every
-// slot is also copied to the kept table gt (same layout, empties included).
-template <int GS, bool BUILD>
+// occupied ones.  g(v, X) = Lam S(v, X) - (mu w(v)) W(X).  Every slot is also
+// copied to the kept table gt (same layout, empties included).
+template <int GS>
 __device__ __forceinline__ void split_argmax(const PassArgs &a, long long Lam, long long muw, SplitTab t,
                                              uint32_t cap, int r, long long &gb, int32_t &xb,
                                              unsigned long long *gt, long long &nX) {
@@ -490,12 +547,10 @@ __device__ __forceinline__ void split_argmax(const PassArgs &a, long long Lam, l
         t.val[s] = 0;
       }
     }
-    if constexpr (BUILD) {
 #pragma unroll
-      for (int k = 0; k < U; ++k) {
-        const uint32_t s = base + k * GS;
-        if (s < cap) gt[s] = key[k] != 0u ? ((unsigned long long)key[k] << 32) | (uint32_t)S[k] : kEmptySlot;
-      }
+    for (int k = 0; k < U; ++k) {
+      const uint32_t s = base + k * GS;
+      if (s < cap) gt[s] = key[k] != 0u ? ((unsigned long long)key[k] << 32) | (uint32_t)S[k] : kEmptySlot;
     }
 #pragma unroll
     for (int k = 0; k < U; ++k) WX[k] = key[k] != 0u ? a.W[LC_IDX(key[k] - 1u, a.g.n, kDbgLabel)] : 0;
@@ -513,34 +568,194 @@ __device__ __forceinline__ void split_argmax(const PassArgs &a, long long Lam, l
   }
 }
 
-// Bins 3-4: a warp's chunk, one row after the other in its own shared table.
-template <int U>
+// ------------------------------------------------- claimed slots
+//
+// A thread remembers the slots its own edges claimed, so the argmax reads
+// and resets exactly the occupied slots and never scans the table: in passes
+// from singletons it saves the walk over the empty half, in uncoarsening,
+// where a row falls into a few clusters, nearly all of it, and the table may
+// be as sparse as shared memory allows (fewer probes).  N: edges per thread
+// at most, four at a time.
+template <int GS, int N>
+__device__ __forceinline__ int32_t claim_row(const PassArgs &a, int64_t beg, int deg, int32_t Cv, SplitTab t,
+                                             uint32_t cap, int r, int32_t (&slot)[N], bool &ok) {
+  constexpr int U = 4;
+  const int32_t *__restrict__ col = a.g.col + beg;
+  const int32_t *__restrict__ ew = a.g.ew + beg;
+  int32_t self = 0;
+#pragma unroll
+  for (int b = 0; b < N; b += U) {
+    int32_t u[U], w[U], X[U];
+    uint32_t cur[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int e = r + (b + k) * GS;
+      u[k] = -1;
+      w[k] = 0;
+      if (e < deg) {
+        u[k] = LC_IDX(__ldg(col + e), a.g.n, kDbgColumn);
+        w[k] = __ldg(ew + e);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) X[k] = u[k] >= 0 ? LC_IDX(a.C[u[k]], a.g.n, kDbgLabel) : -1;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (u[k] >= 0 && X[k] == Cv) {
+        self += w[k];
+        X[k] = -1;
+      }
+      slot[b + k] = X[k] >= 0 ? (int32_t)slot_of(X[k], cap) : -1;
+      cur[k] = X[k] >= 0 ? t.key[slot[b + k]] : 1u;
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (cur[k] == 0u) cur[k] = atomicCAS(&t.key[slot[b + k]], 0u, (uint32_t)X[k] + 1u);
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (X[k] < 0) continue;
+      const uint32_t tag = (uint32_t)X[k] + 1u;
+      uint32_t s = (uint32_t)slot[b + k];
+      if (cur[k] != 0u && cur[k] != tag) {  // another key's slot: probe on
+        uint32_t probe = 1;
+        do {
+          s = s + 1 == cap ? 0 : s + 1;
+          cur[k] = t.key[s];
+          if (cur[k] == 0u) cur[k] = atomicCAS(&t.key[s], 0u, tag);
+        } while (cur[k] != 0u && cur[k] != tag && ++probe < cap);
+        if (cur[k] != 0u && cur[k] != tag) {
+          ok = false;
+          slot[b + k] = -1;
+          continue;
+        }
+      }
+      atomicAdd(&t.val[s], w[k]);
+      slot[b + k] = cur[k] == 0u ? (int32_t)s : -1;  // claimed by this edge, or not
+    }
+  }
+  return self;
+}
+
+// Best (gain, cluster) over the thread's claimed slots, which it resets.
+template <int N>
+__device__ __forceinline__ void claim_argmax(const PassArgs &a, long long Lam, long long muw, SplitTab t,
+                                             const int32_t (&slot)[N], long long &gb, int32_t &xb,
+                                             long long &nX) {
+  constexpr int U = 4;
+#pragma unroll
+  for (int b = 0; b < N; b += U) {
+    int32_t X[U], S[U];
+    long long WX[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      X[k] = -1;
+      S[k] = 0;
+      if (slot[b + k] >= 0) {
+        X[k] = (int32_t)(t.key[slot[b + k]] - 1u);
+        S[k] = t.val[slot[b + k]];
+        t.key[slot[b + k]] = 0u;
+        t.val[slot[b + k]] = 0;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) WX[k] = X[k] >= 0 ? a.W[LC_IDX(X[k], a.g.n, kDbgLabel)] : 0;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (X[k] < 0) continue;
+      nX++;
+      const long long g = Lam * (long long)S[k] - muw * WX[k];
+      if (better(g, X[k], gb, xb)) {
+        gb = g;
+        xb = X[k];
+      }
+    }
+  }
+}
+
+// One row of up to 32 N edges by a warp.
+template <int N>
+__device__ __forceinline__ MoveRes warp_row(const PassArgs &a, const MoveCtx &x, int32_t v, SplitTab tab, uint32_t cap,
+                                            int lane, MoveState &ms) {
+  int32_t slot[N];
+  bool ok = true;
+  const int32_t self = claim_row<32, N>(a, x.beg, x.deg, x.Cv, tab, cap, lane, slot, ok);
+  if (!ok) {
+    a.sc->error = 1;
+    LC_DBG_FAIL(kDbgProbe, v, a.g.n);
+  }
+  __syncwarp();
+  long long gb = LLONG_MIN;
+  int32_t xb = kNone;
+  claim_argmax<N>(a, x.Lam, x.muw, tab, slot, gb, xb, ms.nX);
+  warp_argmax(gb, xb);
+  const int32_t S = (int32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)self);
+  return MoveRes{gb, xb, S};
+}
+
+// Bins 3-4: a warp's chunk, one row after the other in its own shared table
+// of `cap` slots (at least 512).
 __device__ __forceinline__ void warp_chunk(const PassArgs &a, const VRec *__restrict__ rec, int64_t base, int m,
-                                           MoveStage &st, SplitTab tab, long long &cntL, long long &phi,
-                                           long long &nX) {
+                                           MoveStage &st, SplitTab tab, uint32_t cap, MoveState &ms) {
   const int lane = threadIdx.x & 31;
   const ChunkLane c = stage_move(a, rec, base, m, lane, false, st.ctx);
   __syncwarp();
   for (int k = 0; k < m; ++k) {
     const MoveCtx x = st.ctx[k];
-    const uint32_t cap = warp_table_cap(x.deg);
-    bool ok = true;
-    const int32_t self = (int32_t)split_insert_row<32, U>(a, x.beg, x.beg + x.deg, x.Cv, tab, cap, lane, ok);
-    if (!ok) {
-      a.sc->error = 1;
-      LC_DBG_FAIL(kDbgProbe, base + k, a.g.n);
-    }
-    __syncwarp();
-    long long gb = LLONG_MIN;
-    int32_t xb = kNone;
-    split_argmax<32, false>(a, x.Lam, x.muw, tab, cap, lane, gb, xb, nullptr, nX);
-    warp_argmax(gb, xb);
-    const int32_t S = (int32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)self);
-    if (lane == 0) st.res[k] = MoveRes{gb, xb, S};
+    const MoveRes r = x.deg <= 128 ? warp_row<4>(a, x, (int32_t)(base + k), tab, cap, lane, ms)
+                                   : warp_row<8>(a, x, (int32_t)(base + k), tab, cap, lane, ms);
+    if (lane == 0) st.res[k] = r;
     __syncwarp();
   }
-  settle_move(a, c, m, lane, false, st.res, cntL, phi);
+  settle_move(a, c, m, lane, false, st.res, ms);
   __syncwarp();
+}
+
+// Inserts chunk c of a hub row into the hub's global table (GS threads, tg:
+// this warp's tags); returns this thread's part of S(v, C[v]).
+template <int GS>
+__device__ __forceinline__ long long hub_insert(const PassArgs &a, int c, LaneTags &tg) {
+  constexpr int U = GS > 512 ? 2 : 4;
+  const int h = a.hub.hub_of[c];
+  const int32_t v = a.hub.vtx[h];
+  const int64_t beg = a.g.rp[v], end = a.g.rp[v + 1];
+  const int32_t Cv = LC_IDX(a.C[v], a.g.n, kDbgLabel);
+  unsigned long long *tab = a.gtab + 2 * beg;
+  const uint32_t cap = (uint32_t)(2 * (end - beg));
+  const int lane = threadIdx.x & 31;
+  const int64_t e0 = a.hub.e0[c], e1 = a.hub.e1[c];
+  long long self = 0;
+  bool ok = true;
+  for (int64_t base = e0; base < e1; base += GS * U) {
+    int32_t u[U], w[U], X[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int64_t e = base + k * GS + threadIdx.x;
+      u[k] = -1;
+      w[k] = 0;
+      if (e < e1) {
+        u[k] = LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn);
+        w[k] = __ldg(a.g.ew + e);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) X[k] = u[k] >= 0 ? LC_IDX(a.C[u[k]], a.g.n, kDbgLabel) : -1;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const bool other = u[k] >= 0 && X[k] != Cv;
+      if (u[k] >= 0 && X[k] == Cv) self += w[k];
+      int leader;
+      const int32_t S = lane_sums<32>(tg, lane, other, X[k], w[k], leader);
+      if (other && lane == leader) {
+        bool fresh = false;
+        ok &= table_add(tab, cap, X[k], S, fresh);
+      }
+    }
+  }
+  if (!ok) {
+    a.sc->error = 1;
+    LC_DBG_FAIL(kDbgProbe, v, a.g.n);
+  }
+  return self;
 }
 
 // ------------------------------------------------ afterburner (Algorithm 3)
@@ -635,30 +850,52 @@ __device__ __forceinline__ void flush_update(const PassArgs &a, const UpdateSums
   if ((threadIdx.x & 31) == 0 && e) atomicAdd(&a.sc->empty_movers, e);
 }
 
+// W[X[lane]] += w[lane] over the lanes with on (full warp).  Many movers of
+// a warp often join the same cluster (a hub's), and atomics on one address
+// are served one after the other: the lanes that share the first two such
+// clusters are summed first.
+__device__ __forceinline__ void add_weights(int64_t *W, bool on, int32_t X, long long w) {
+  constexpr unsigned full = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  unsigned todo = __ballot_sync(full, on);
+#pragma unroll
+  for (int round = 0; round < 2; ++round) {
+    if (__popc(todo) < 4) break;  // uniform
+    const int leader = __ffs(todo) - 1;
+    const int32_t X0 = __shfl_sync(full, X, leader);
+    const bool mine = ((todo >> lane) & 1u) && X == X0;
+    const unsigned same = __ballot_sync(full, mine);
+    if (same == (1u << leader)) break;
+    const long long t = warp_sum(mine ? w : 0ll);
+    if (lane == leader) atomicAdd((unsigned long long *)&W[X0], (unsigned long long)t);
+    todo &= ~same;
+  }
+  if ((todo >> lane) & 1u) atomicAdd((unsigned long long *)&W[X], (unsigned long long)w);
+}
+
 // Applies the pass to one vertex per lane (full warp): a survivor leaves its
 // cluster for its destination (Algorithm 2, Update), or stays unlabelled
 // (C[v] = kEmpty) until the new-cluster ids are given out.  The records
 // still hold C and D, so other vertices' sums are not disturbed.  Lists the
 // movers' row chunks (kept tables) and the movers that are not hubs (final
-// objective) where those lists are kept, one append per warp.
+// objective) where those lists are kept, one append per warp.  used: null, or
+// the ids in use, marked from every vertex's new label.
 __device__ __forceinline__ void apply_lanes(const PassArgs &a, bool on, int32_t v, int64_t deg, const AbRec &r,
-                                            long long wv, bool keep, UpdateSums &sum) {
+                                            long long wv, bool keep, UpdateSums &sum, int32_t *used = nullptr) {
   const int lane = threadIdx.x & 31;
-  if (on && keep) {
-    atomicAdd((unsigned long long *)&a.W[r.C], (unsigned long long)(-wv));
-    if (r.D >= 0) {
-      a.C[v] = LC_IDX(r.D, a.g.n, kDbgDest);
-      atomicAdd((unsigned long long *)&a.W[LC_IDX(r.D, a.g.n, kDbgDest)], (unsigned long long)wv);
-    } else {
-      a.C[v] = kEmpty;
-      sum.empties++;
-    }
+  keep = keep && on;
+  if (keep) {
+    a.C[v] = r.D >= 0 ? LC_IDX(r.D, a.g.n, kDbgDest) : kEmpty;
+    sum.empties += r.D < 0;
     sum.moved++;
   }
+  add_weights(a.W, keep, r.C, -wv);
+  add_weights(a.W, keep && r.D >= 0, LC_IDX(keep && r.D >= 0 ? r.D : 0, a.g.n, kDbgDest), wv);
+  if (used && on && !(keep && r.D < 0)) used[keep ? r.D : r.C] = 1;
   if (on && r.D != kNone) sum.cand += deg;
   if (on && a.M) a.M[v] = keep;
   if (a.upd_list) {  // uniform over the launch
-    const int nch = on && keep ? (int)((deg + kUpdChunk - 1) / kUpdChunk) : 0;
+    const int nch = keep ? (int)((deg + kUpdChunk - 1) / kUpdChunk) : 0;
     int incl = nch;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -672,7 +909,7 @@ __device__ __forceinline__ void apply_lanes(const PassArgs &a, bool on, int32_t 
     for (int k = 0; k < nch; ++k) a.upd_list[first + k] = make_int2(v, k);
   }
   if (a.movers) {  // uniform over the launch
-    const bool listed = on && keep && deg <= a.hub_min;  // hubs: k_hub_delta_in
+    const bool listed = keep && deg <= a.hub_min;  // hubs: k_hub_delta_in
     const unsigned m = __ballot_sync(0xFFFFFFFFu, listed);
     int first = 0;
     if (lane == 0 && m) first = atomicAdd(&a.sc->n_movers, __popc(m));
@@ -707,10 +944,12 @@ __device__ __forceinline__ int stage_ab(const PassArgs &a, const VRec *__restric
 
 // Afterburner and update of a chunk: for each candidate, delta_v adjusted by
 // every adjacent candidate that precedes it; it survives iff the adjusted
-// delta is >= 0.
+// delta is >= 0.  G lanes per candidate, four edges each in flight, so that
+// a row up to 4 G edges is one chain of gathers and a warp has 32 / G chains
+// going: the walk is bound by their latency.
 template <int G>
 __device__ __forceinline__ void ab_chunk(const PassArgs &a, const VRec *__restrict__ rec, int64_t base, int m,
-                                         AbStage &st, UpdateSums &sum) {
+                                         AbStage &st, UpdateSums &sum, int32_t *used = nullptr) {
   constexpr int V = 32 / G;
   const int lane = threadIdx.x & 31, grp = lane / G, sub = lane & (G - 1);
   VRec vr{};
@@ -731,13 +970,13 @@ __device__ __forceinline__ void ab_chunk(const PassArgs &a, const VRec *__restri
   }
   __syncwarp();
   const bool keep = r.D != kNone && delta + st.sum[r.D != kNone ? pos : 0] >= 0;
-  apply_lanes(a, lane < m, vr.v, vr.deg, r, vr.w, keep, sum);
+  apply_lanes(a, lane < m, vr.v, vr.deg, r, vr.w, keep, sum, used);
   __syncwarp();
 }
 
 // Bin 0: one thread per vertex (full warp, lanes with on = false idle).
 __device__ __forceinline__ void ab_thread(const PassArgs &a, bool on, const VRec *__restrict__ rec, int64_t i,
-                                          UpdateSums &sum) {
+                                          UpdateSums &sum, int32_t *used = nullptr) {
   VRec vr{};
   AbRec r{0, kNone, 0};
   bool keep = false;
@@ -750,7 +989,46 @@ __device__ __forceinline__ void ab_thread(const PassArgs &a, bool on, const VRec
     }
   }
   __syncwarp();
-  apply_lanes(a, on, vr.v, vr.deg, r, vr.w, keep, sum);
+  apply_lanes(a, on, vr.v, vr.deg, r, vr.w, keep, sum, used);
+}
+
+// ------------------------------------------ objective after a pass
+
+// Change of IN over edges [e0, e1) of mover v (strided by GS): an edge to
+// a non-mover counts both directions, an edge between movers one (the
+// other mover counts the other).  A mover that got its own emptied id back
+// counts as a non-mover, from either end.
+template <int GS>
+__device__ __forceinline__ long long delta_in_edges(const PassArgs &a, int32_t v, int64_t e0, int64_t e1,
+                                                    int r) {
+  constexpr int U = 4;
+  const int32_t Cvn = a.C[v], Cvo = a.ab[v].C;
+  long long d = 0;
+  for (int64_t base = e0 + r; base < e1; base += (int64_t)GS * U) {
+    int32_t u[U], w[U], Cun[U], Cuo[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int64_t e = base + (int64_t)k * GS;
+      u[k] = -1;
+      w[k] = 0;
+      if (e < e1) {
+        u[k] = LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn);
+        w[k] = __ldg(a.g.ew + e);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      Cun[k] = u[k] >= 0 ? a.C[u[k]] : 0;
+      Cuo[k] = u[k] >= 0 ? a.ab[u[k]].C : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (u[k] < 0) continue;
+      const int s = (Cvn == Cun[k] ? 1 : 0) - (Cvo == Cuo[k] ? 1 : 0);
+      d += (long long)(Cun[k] != Cuo[k] ? 1 : 2) * s * w[k];
+    }
+  }
+  return d;
 }
 
 }  // namespace lc

@@ -57,51 +57,26 @@ template <int G>
 __global__ void __launch_bounds__(256) k_first_pass(PassArgs a, const VRec *__restrict__ rec, int64_t count,
                                                     int chunk) {
   __shared__ MoveStage st[8];
-  long long cntL = 0;
+  MoveState ms = move_state(a);
   const WarpChunk c = warp_chunk_of(count, chunk);
-  if (c.m > 0) first_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], cntL);
-  flush_block_sum(cntL, &a.sc->count_L);
+  if (c.m > 0) first_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], ms);
+  flush_block_sum(ms.cntL, &a.sc->count_L);
 }
 
 __global__ void __launch_bounds__(256) k_first_thread(PassArgs a, const VRec *__restrict__ rec, int64_t count) {
-  long long cntL = 0;
+  MoveState ms = move_state(a);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const VRec vr = rec[i];
-    const GraphParam P = a.gp[vr.g];
-    long long gb = LLONG_MIN;
-    int32_t xb = kNone;
-#pragma unroll 4
-    for (int64_t e = vr.beg; e < vr.beg + vr.deg; ++e) first_edge(a, P.Lam, P.mu * vr.w, e, gb, xb);
-    decide(a, P, vr.v, vr.v, 0, xb, gb, cntL);
-  }
-  flush_block_sum(cntL, &a.sc->count_L);
+       i += (int64_t)gridDim.x * blockDim.x)
+    first_thread(a, rec, i, ms);
+  flush_block_sum(ms.cntL, &a.sc->count_L);
 }
 
 __global__ void __launch_bounds__(256, 4) k_move_thread(PassArgs a, const VRec *__restrict__ rec, int64_t count) {
-  long long cntL = 0, phi = 0, nX = 0;
+  MoveState ms = move_state(a);
   // warp-uniform trip count: phi_add takes whole warps
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < count; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    const bool on = i < count;
-    VRec vr{};
-    long long gC = 0;
-    if (on) {
-      vr = rec[i];
-      const int32_t Cv = LC_IDX(a.C[vr.v], a.g.n, kDbgLabel);
-      const GraphParam P = a.gp[vr.g];
-      const long long WC = a.W[Cv];
-      long long gb;
-      int32_t xb;
-      const long long self = thread_gains(a, vr, Cv, P, gb, xb, nX);
-      gC = gain_self(P, self, vr.w, WC);
-      decide(a, P, vr.v, Cv, gC, xb, gb, cntL);
-    }
-    phi_add(a, on, vr.g, gC, phi);
-  }
-  flush_block_sum(nX, &a.sc->distinct_x);
-  flush_block_sum(cntL, &a.sc->count_L);
-  flush_block_sum(phi, &a.phi_acc[0]);
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < count; base += (int64_t)gridDim.x * blockDim.x)
+    move_thread(a, base + threadIdx.x < count, rec, base + threadIdx.x, ms);
+  flush_move(a, ms);
 }
 
 template <int G>
@@ -109,38 +84,33 @@ __global__ void __launch_bounds__(256) k_move_lanes(PassArgs a, const VRec *__re
                                                     int chunk) {
   __shared__ MoveStage st[8];
   __shared__ LaneTags tags[8];
-  long long cntL = 0, phi = 0, nX = 0;
+  MoveState ms = move_state(a);
   const WarpChunk c = warp_chunk_of(count, chunk);
-  if (c.m > 0) lanes_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], tags[threadIdx.x >> 5], cntL, phi, nX);
-  flush_block_sum(nX, &a.sc->distinct_x);
-  flush_block_sum(cntL, &a.sc->count_L);
-  flush_block_sum(phi, &a.phi_acc[0]);
+  if (c.m > 0) lanes_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], tags[threadIdx.x >> 5], ms);
+  flush_move(a, ms);
 }
 
-// Bins 3-4: one warp per vertex, a per-warp split shared table of SLOTS
+// Bins 3-4: one warp per vertex, a per-warp split shared table of kWarpSlots
 // slots.
-template <int SLOTS>
+constexpr int kWarpSlots = 512;
 __global__ void __launch_bounds__(kWarpBinWarps * 32, 4)
     k_move_warp(PassArgs a, const VRec *__restrict__ rec, int64_t count, int chunk) {
-  constexpr int U = SLOTS / 128;  // edges per lane per batch: 64 (bin 3) or 128 (bin 4)
-  __shared__ uint32_t keys[kWarpBinWarps][SLOTS];
-  __shared__ int32_t vals[kWarpBinWarps][SLOTS];
+  __shared__ uint32_t keys[kWarpBinWarps][kWarpSlots];
+  __shared__ int32_t vals[kWarpBinWarps][kWarpSlots];
   __shared__ MoveStage st[kWarpBinWarps];
-  long long cntL = 0, phi = 0, nX = 0;
+  MoveState ms = move_state(a);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const SplitTab tab{keys[wid], vals[wid]};
   const WarpChunk c = warp_chunk_of(count, chunk);
   if (c.m > 0) {
-    for (int s = lane; s < SLOTS; s += 32) {
+    for (int s = lane; s < kWarpSlots; s += 32) {
       tab.key[s] = 0u;
       tab.val[s] = 0;
     }
     __syncwarp();
-    warp_chunk<U>(a, rec, c.base, c.m, st[wid], tab, cntL, phi, nX);
+    warp_chunk(a, rec, c.base, c.m, st[wid], tab, kWarpSlots, ms);
   }
-  flush_block_sum(nX, &a.sc->distinct_x);
-  flush_block_sum(cntL, &a.sc->count_L);
-  flush_block_sum(phi, &a.phi_acc[0]);
+  flush_move(a, ms);
 }
 
 // A block's chunk of vertices, staged and decided by its first warp.
@@ -161,7 +131,7 @@ __global__ void __launch_bounds__(GS) k_first_block(PassArgs a, const VRec *__re
   __shared__ MoveStage st;
   __shared__ long long rg[GS / 32];
   __shared__ int32_t rx[GS / 32];
-  long long cntL = 0, phi = 0;
+  MoveState ms = move_state(a);
   const BlockChunk b = block_chunk_of(count, chunk);
   ChunkLane c{};
   if (threadIdx.x < 32) c = stage_move(a, rec, b.base, b.m, threadIdx.x, true, st.ctx);
@@ -176,17 +146,17 @@ __global__ void __launch_bounds__(GS) k_first_block(PassArgs a, const VRec *__re
     if (threadIdx.x == 0) st.res[k] = MoveRes{gb, xb, 0};
   }
   __syncthreads();
-  if (threadIdx.x < 32) settle_move(a, c, b.m, threadIdx.x, true, st.res, cntL, phi);
-  flush_block_sum(cntL, &a.sc->count_L);
+  if (threadIdx.x < 32) settle_move(a, c, b.m, threadIdx.x, true, st.res, ms);
+  flush_block_sum(ms.cntL, &a.sc->count_L);
 }
 
 // Bins 5-8: one block per vertex; dynamic shared memory holds the split
-// table (SLOTS keys, then SLOTS values).  A row uses min(2 deg rounded up
-// to 32, SLOTS) slots: bin 8 (deg <= 4096) has 6144 slots, a load factor of
-// at most 2/3, so that four blocks fit in an SM's shared memory.
-// BUILD: the tables use the kept-table layout (tab_cap slots) and are
-// copied out to each vertex's gtab region with S(v, C[v]) added.
-template <int GS, int SLOTS, bool BUILD>
+// table (SLOTS keys, then SLOTS values): bin 8 (deg <= 4096) has 6144 slots,
+// a load factor of at most 2/3, so that four blocks fit in an SM's shared
+// memory.  N: edges per thread of the bin's longest row.
+// BUILD: the tables use the kept-table layout (tab_cap slots), are scanned,
+// and copied out to each vertex's gtab region with S(v, C[v]) added.
+template <int GS, int SLOTS, int N, bool BUILD>
 __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__restrict__ rec,
                                                    int64_t count, int chunk) {
   extern __shared__ uint32_t smem_tab[];
@@ -198,7 +168,7 @@ __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__res
   __shared__ long long rg[2][GS / 32];
   __shared__ int32_t rx[2][GS / 32], rs[2][GS / 32];
   int par = 0;
-  long long cntL = 0, phi = 0, nX = 0;
+  MoveState ms = move_state(a);
   const BlockChunk b = block_chunk_of(count, chunk);
   ChunkLane c{};
   if (threadIdx.x < 32) c = stage_move(a, rec, b.base, b.m, threadIdx.x, false, st.ctx);
@@ -209,10 +179,13 @@ __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__res
   __syncthreads();
   for (int k = 0; k < b.m; ++k) {
     const MoveCtx x = st.ctx[k];
-    const uint32_t cap = BUILD ? tab_cap(x.deg) : min(warp_table_cap(x.deg), (uint32_t)SLOTS);
+    const uint32_t cap = BUILD ? tab_cap(x.deg) : (uint32_t)SLOTS;
     bool ok = true;
-    int32_t self =
-        (int32_t)split_insert_row<GS, 4>(a, x.beg, x.beg + x.deg, x.Cv, tab, cap, threadIdx.x, ok);
+    int32_t self, slot[N];
+    if constexpr (BUILD)
+      self = (int32_t)split_insert_row<GS, 4>(a, x.beg, x.beg + x.deg, x.Cv, tab, cap, threadIdx.x, ok);
+    else
+      self = claim_row<GS, N>(a, x.beg, x.deg, x.Cv, tab, cap, threadIdx.x, slot, ok);
     if (!ok) {
       a.sc->error = 1;
       LC_DBG_FAIL(kDbgProbe, b.base + k, a.g.n);
@@ -221,7 +194,10 @@ __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__res
     long long gb = LLONG_MIN;
     int32_t xb = kNone;
     unsigned long long *gt = a.gtab + 2 * x.beg;
-    split_argmax<GS, BUILD>(a, x.Lam, x.muw, tab, cap, threadIdx.x, gb, xb, gt, nX);
+    if constexpr (BUILD)
+      split_argmax<GS>(a, x.Lam, x.muw, tab, cap, threadIdx.x, gb, xb, gt, ms.nX);
+    else
+      claim_argmax<N>(a, x.Lam, x.muw, tab, slot, gb, xb, ms.nX);
     // one reduction of (best gain, cluster, S_self) for thread 0 only: warp
     // level, one barrier, thread 0 combines the warps
     warp_argmax(gb, xb);
@@ -249,10 +225,8 @@ __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__res
     par ^= 1;
   }
   __syncthreads();
-  if (threadIdx.x < 32) settle_move(a, c, b.m, threadIdx.x, false, st.res, cntL, phi);
-  flush_block_sum(nX, &a.sc->distinct_x);
-  flush_block_sum(cntL, &a.sc->count_L);
-  flush_block_sum(phi, &a.phi_acc[0]);
+  if (threadIdx.x < 32) settle_move(a, c, b.m, threadIdx.x, false, st.res, ms);
+  flush_move(a, ms);
 }
 
 // --------------------------------------------------------- hubs (bin 9)
@@ -278,50 +252,9 @@ __device__ __forceinline__ void hub_acc_add(const PassArgs &a, int h, long long 
 // Lanes of a warp holding the same cluster are combined first (lane_sums),
 // so a popular cluster costs one global atomic per warp.
 __global__ void __launch_bounds__(kHubThreads) k_hub_move_insert(PassArgs a) {
-  constexpr int U = 4;
   __shared__ LaneTags tags[kHubThreads / 32];
-  const int c = blockIdx.x;
-  const int h = a.hub.hub_of[c];
-  const int32_t v = a.hub.vtx[h];
-  const int64_t beg = a.g.rp[v], end = a.g.rp[v + 1];
-  const int32_t Cv = LC_IDX(a.C[v], a.g.n, kDbgLabel);
-  unsigned long long *tab = a.gtab + 2 * beg;
-  const uint32_t cap = (uint32_t)(2 * (end - beg));
-  const int lane = threadIdx.x & 31;
-  LaneTags &tg = tags[threadIdx.x >> 5];
-  const int64_t e0 = a.hub.e0[c], e1 = a.hub.e1[c];
-  long long self = 0;
-  bool ok = true;
-  for (int64_t base = e0; base < e1; base += kHubThreads * U) {
-    int32_t u[U], w[U], X[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t e = base + k * kHubThreads + threadIdx.x;
-      u[k] = -1;
-      w[k] = 0;
-      if (e < e1) {
-        u[k] = LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn);
-        w[k] = __ldg(a.g.ew + e);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < U; ++k) X[k] = u[k] >= 0 ? LC_IDX(a.C[u[k]], a.g.n, kDbgLabel) : -1;
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const bool other = u[k] >= 0 && X[k] != Cv;
-      if (u[k] >= 0 && X[k] == Cv) self += w[k];
-      int leader;
-      const int32_t S = lane_sums<32>(tg, lane, other, X[k], w[k], leader);
-      if (other && lane == leader) {
-        bool fresh = false;
-        ok &= table_add(tab, cap, X[k], S, fresh);
-      }
-    }
-  }
-  if (!ok) {
-    a.sc->error = 1;
-    LC_DBG_FAIL(kDbgProbe, v, a.g.n);
-  }
+  const int h = a.hub.hub_of[blockIdx.x];
+  const long long self = hub_insert<kHubThreads>(a, blockIdx.x, tags[threadIdx.x >> 5]);
   hub_acc_add(a, h, self);
 }
 
@@ -359,7 +292,7 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_first(PassArgs a) {
 // Final step per hub: combine chunk partials, then decide (Algorithm 2).
 // first = 1: singleton start, g(v, C[v]) = 0 and no objective term.
 __global__ void k_hub_decide(PassArgs a, int first) {
-  long long cntL = 0, phi = 0;
+  MoveState ms = move_state(a);
   for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < a.hub.H; h += gridDim.x * blockDim.x) {
     const int32_t v = a.hub.vtx[h];
     const GraphParam P = a.gp[graph_of(a, v)];
@@ -376,16 +309,16 @@ __global__ void k_hub_decide(PassArgs a, int first) {
       const long long self = a.hub.acc[h];
       a.hub.acc[h] = 0;
       gC = gain_self(P, self, a.g.vw[v], a.W[Cv]);
-      phi_add_one(a, graph_of(a, v), gC, phi);
+      phi_add_one(a, ms.acc, graph_of(a, v), gC, ms.phi);
       if (a.tab_build && self > 0) {  // the hub's kept table gets its own cluster
         const int64_t beg = a.g.rp[v];
         if (!tab_put(a.gtab + 2 * beg, tab_cap(a.g.rp[v + 1] - beg), Cv, self)) a.sc->error = 1;
       }
     }
-    decide(a, P, v, Cv, gC, xb, gb, cntL);
+    decide(a, P, v, Cv, gC, xb, gb, ms);
   }
-  flush_block_sum(cntL, &a.sc->count_L);
-  flush_block_sum(phi, &a.phi_acc[0]);
+  flush_block_sum(ms.cntL, &a.sc->count_L);
+  flush_block_sum(ms.phi, &ms.acc[0]);
 }
 
 // ------------------------------------------------ afterburner (Algorithm 3)
@@ -399,7 +332,7 @@ __global__ void __launch_bounds__(256, 4) k_ab_thread(PassArgs a, const VRec *__
   flush_update(a, sum);
 }
 
-// 16 lanes or a warp per candidate, a chunk of vertices per warp.
+// 4, 8 or 16 lanes or a warp per candidate, a chunk of vertices per warp.
 template <int G>
 __global__ void __launch_bounds__(256, 4) k_ab_warp(PassArgs a, const VRec *__restrict__ rec, int64_t count,
                                                     int chunk) {
@@ -512,9 +445,9 @@ __global__ void __launch_bounds__(GS > 32 ? GS : 256)
     const int g = owner ? graph_of(a, v) : 0;
     const long long gC = owner ? gain_self(a.gp[g], self, a.g.vw[v], a.W[Cv]) : 0;
     if constexpr (GS <= 32)
-      phi_add(a, owner, g, gC, phi);
+      phi_add(a, a.phi_acc, owner, g, gC, phi);
     else if (owner)
-      phi_add_one(a, g, gC, phi);
+      phi_add_one(a, a.phi_acc, g, gC, phi);
   });
   flush_block_sum(phi, &a.phi_acc[0]);
 }
@@ -537,7 +470,7 @@ __global__ void k_hub_obj_final(PassArgs a) {
     const long long self = a.hub.acc[h];
     a.hub.acc[h] = 0;
     const int g = graph_of(a, v);
-    phi_add_one(a, g, gain_self(a.gp[g], self, a.g.vw[v], a.W[a.C[v]]), phi);
+    phi_add_one(a, a.phi_acc, g, gain_self(a.gp[g], self, a.g.vw[v], a.W[a.C[v]]), phi);
   }
   flush_block_sum(phi, &a.phi_acc[0]);
 }
@@ -717,7 +650,7 @@ __global__ void __launch_bounds__(GS) k_tab_scan(PassArgs a, const int32_t *__re
                                                  int64_t count) {
   __shared__ long long rs[2][GS / 32], rg[2][GS / 32];
   __shared__ int32_t rx[2][GS / 32];
-  long long cntL = 0, phi = 0;
+  MoveState ms = move_state(a);
   int par = 0;
   for (int64_t i = blockIdx.x; i < count; i += gridDim.x) {
     const int32_t v = list[i];
@@ -747,13 +680,13 @@ __global__ void __launch_bounds__(GS) k_tab_scan(PassArgs a, const int32_t *__re
         }
       }
       const long long gC = gain_self(P, self, wv, a.W[Cv]);
-      phi_add_one(a, graph_of(a, v), gC, phi);
-      decide(a, P, v, Cv, gC, xb, gb, cntL);
+      phi_add_one(a, ms.acc, graph_of(a, v), gC, ms.phi);
+      decide(a, P, v, Cv, gC, xb, gb, ms);
     }
     par ^= 1;
   }
-  flush_block_sum(cntL, &a.sc->count_L);
-  flush_block_sum(phi, &a.phi_acc[0]);
+  flush_block_sum(ms.cntL, &a.sc->count_L);
+  flush_block_sum(ms.phi, &ms.acc[0]);
 }
 
 // Hubs: each chunk scans its share of the hub's table; k_hub_decide
@@ -790,7 +723,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_assign_empty(PassArgs a, Empty
   const int total = a.sc->empty_movers;  // nothing writes it during this launch
   if (total == 0) return;
   GridBarrier bar(a.sc);
-  if (!assign_empty(a, w, total, bar)) return;
+  if (!assign_empty(a, w, total, false, bar)) return;
   bar.leave();
 }
 
@@ -848,9 +781,10 @@ __global__ void k_iota(int32_t *C, int64_t n) {
 
 __global__ void k_cluster_weights(const int32_t *__restrict__ C, const int64_t *__restrict__ vw,
                                   int64_t *W, int64_t n) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd((unsigned long long *)&W[C[v]], (unsigned long long)vw[v]);
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = base + threadIdx.x;
+    add_weights(W, v < n, v < n ? C[v] : 0, v < n ? vw[v] : 0);
+  }
 }
 
 // ------------------------------------------------------------ binning
@@ -896,21 +830,21 @@ static inline unsigned blocks_for(int64_t items, int per_block) {
 static constexpr int block_table_bytes(int slots) { return slots * 8; }
 
 void configure_kernels() {
-  cudaFuncSetAttribute(k_move_block<64, 1024, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<64, 1024, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(1024));
-  cudaFuncSetAttribute(k_move_block<128, 2048, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<128, 2048, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(2048));
-  cudaFuncSetAttribute(k_move_block<256, 4096, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<256, 4096, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(4096));
-  cudaFuncSetAttribute(k_move_block<256, 6144, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<256, 6144, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(6144));
-  cudaFuncSetAttribute(k_move_block<64, 1024, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<64, 1024, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(1024));
-  cudaFuncSetAttribute(k_move_block<128, 2048, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<128, 2048, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(2048));
-  cudaFuncSetAttribute(k_move_block<256, 4096, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<256, 4096, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(4096));
-  cudaFuncSetAttribute(k_move_block<256, 6144, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_move_block<256, 6144, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(6144));
 }
 
@@ -1023,10 +957,10 @@ int launch_first_pass(const PassArgs &a, const Bins &b, cudaStream_t s) {
   return n;
 }
 
-template <int GS, int SLOTS>
+template <int GS, int SLOTS, int N>
 static int launch_move_block(const PassArgs &a, BinRange r, cudaStream_t s) {
-  return launch_block_chunks(a.tab_build ? k_move_block<GS, SLOTS, true> : k_move_block<GS, SLOTS, false>, GS,
-                             block_table_bytes(SLOTS), a, r, s);
+  return launch_block_chunks(a.tab_build ? k_move_block<GS, SLOTS, N, true> : k_move_block<GS, SLOTS, N, false>,
+                             GS, block_table_bytes(SLOTS), a, r, s);
 }
 
 // Bins 0-4 (degree <= 256): aggregation from the CSR in every pass.
@@ -1034,17 +968,16 @@ static int launch_move_low(const PassArgs &a, const Bins &b, cudaStream_t s) {
   int n = launch_threads(k_move_thread, a, bin_range(b, 0, 0), s);
   n += launch_warp_chunks(k_move_lanes<16>, a, bin_range(b, 1, 1), s);
   n += launch_warp_chunks(k_move_lanes<32>, a, bin_range(b, 2, 2), s);
-  n += launch_warp_chunks(k_move_warp<256>, a, bin_range(b, 3, 3), s);
-  n += launch_warp_chunks(k_move_warp<512>, a, bin_range(b, 4, 4), s);
+  n += launch_warp_chunks(k_move_warp, a, bin_range(b, 3, 4), s);
   return n;
 }
 
 int launch_move(const PassArgs &a, const Bins &b, cudaStream_t s) {
   int n = launch_move_low(a, b, s);
-  n += launch_move_block<64, 1024>(a, bin_range(b, 5, 5), s);
-  n += launch_move_block<128, 2048>(a, bin_range(b, 6, 6), s);
-  n += launch_move_block<256, 4096>(a, bin_range(b, 7, 7), s);
-  n += launch_move_block<256, 6144>(a, bin_range(b, 8, 8), s);
+  n += launch_move_block<64, 1024, 8>(a, bin_range(b, 5, 5), s);
+  n += launch_move_block<128, 2048, 8>(a, bin_range(b, 6, 6), s);
+  n += launch_move_block<256, 4096, 8>(a, bin_range(b, 7, 7), s);
+  n += launch_move_block<256, 6144, 16>(a, bin_range(b, 8, 8), s);
   if (a.hub.H > 0) {
     k_hub_move_insert<<<a.hub.Q, kHubThreads, 0, s>>>(a);
     k_hub_move_scan<<<a.hub.Q, kHubThreads, 0, s>>>(a);
@@ -1079,9 +1012,10 @@ int launch_table_pass(const PassArgs &a, const Bins &b, cudaStream_t s) {
 }
 
 // One of the afterburner's bin groups 2-4: 16 (group 2 only), 32, 128 or 512
-// threads per candidate (BinPlan::ab_gs).
+// threads per candidate (BinPlan::ab_gs).  Bin 2 of group 2 (rows up to 32
+// edges) always takes 8 lanes per candidate.
 static int launch_ab_group(const PassArgs &a, const Bins &b, int g, cudaStream_t s) {
-  const BinRange r = bin_range(b, kAbFirstBin[g], kAbFirstBin[g + 1] - 1);
+  const BinRange r = bin_range(b, g == 2 ? 3 : kAbFirstBin[g], kAbFirstBin[g + 1] - 1);
   if (a.ab_gs[g] == 16) return launch_warp_chunks(k_ab_warp<16>, a, r, s);
   if (a.ab_gs[g] == 32) return launch_warp_chunks(k_ab_warp<32>, a, r, s);
   if (a.ab_gs[g] == 128) return launch_block_chunks(k_ab_block<128>, 128, 0, a, r, s);
@@ -1090,7 +1024,8 @@ static int launch_ab_group(const PassArgs &a, const Bins &b, int g, cudaStream_t
 
 int launch_afterburner(const PassArgs &a, const Bins &b, cudaStream_t s) {
   int n = launch_threads(k_ab_thread, a, bin_range(b, 0, 0), s);
-  n += launch_warp_chunks(k_ab_warp<16>, a, bin_range(b, 1, 1), s);
+  n += launch_warp_chunks(k_ab_warp<4>, a, bin_range(b, 1, 1), s);
+  n += launch_warp_chunks(k_ab_warp<8>, a, bin_range(b, 2, 2), s);
   for (int g = 2; g < kAbGroups; ++g) n += launch_ab_group(a, b, g, s);
   if (a.hub.H > 0) {
     k_hub_afterburner<<<a.hub.Q, kHubThreads, 0, s>>>(a);
@@ -1165,43 +1100,6 @@ int launch_objective(const PassArgs &a, const Bins &b, cudaStream_t s) {
 // call's final state, which the best-of test of Algorithm 2 needs, costs a
 // walk over the movers' rows instead of a sweep of the whole graph:
 //   Phi' = Phi + Lam dIN - mu (Q' - Q).
-
-// Change of IN over edges [e0, e1) of mover v (strided by GS): an edge to
-// a non-mover counts both directions, an edge between movers one (the
-// other mover counts the other).  A mover that got its own emptied id back
-// counts as a non-mover, from either end.
-template <int GS>
-__device__ __forceinline__ long long delta_in_edges(const PassArgs &a, int32_t v, int64_t e0, int64_t e1,
-                                                    int r) {
-  constexpr int U = 4;
-  const int32_t Cvn = a.C[v], Cvo = a.ab[v].C;
-  long long d = 0;
-  for (int64_t base = e0 + r; base < e1; base += (int64_t)GS * U) {
-    int32_t u[U], w[U], Cun[U], Cuo[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t e = base + (int64_t)k * GS;
-      u[k] = -1;
-      w[k] = 0;
-      if (e < e1) {
-        u[k] = LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn);
-        w[k] = __ldg(a.g.ew + e);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      Cun[k] = u[k] >= 0 ? a.C[u[k]] : 0;
-      Cuo[k] = u[k] >= 0 ? a.ab[u[k]].C : 0;
-    }
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      if (u[k] < 0) continue;
-      const int s = (Cvn == Cun[k] ? 1 : 0) - (Cvo == Cuo[k] ? 1 : 0);
-      d += (long long)(Cun[k] != Cuo[k] ? 1 : 2) * s * w[k];
-    }
-  }
-  return d;
-}
 
 // The per-graph accumulators of the objective update: a.obj holds
 // [Phi entering | Q entering | Q after | dIN], G entries each.
