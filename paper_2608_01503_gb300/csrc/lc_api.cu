@@ -19,6 +19,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "lc_bins.cuh"
 #include "lc_constraint.cuh"
 #include "lc_coop.cuh"
 #include "lc_fused.cuh"
@@ -187,7 +188,7 @@ struct Run {
   int64_t *W = nullptr, *delta = nullptr, *bound = nullptr, *off = nullptr, *scan64 = nullptr;
   uint8_t *M = nullptr;  // survivors of the last pass (trace only)
   AbRec *ab = nullptr;
-  unsigned long long *eblocks = nullptr;  // per-block counts of the new-cluster ids
+  int32_t *coop = nullptr;  // per-block counts of the cooperative kernels
   int2 *upd_list = nullptr;
   unsigned long long *gtab = nullptr;
   Scalars *sc = nullptr;
@@ -200,6 +201,7 @@ struct Run {
   int *improved = nullptr;
   int32_t *gstart = nullptr, *gfree = nullptr, *gmover = nullptr;
   uint8_t *keep = nullptr;
+  int64_t *gptr = nullptr;  // [G + 1] vertex ranges of a batch
   GraphStats *st = nullptr;
   std::vector<long long> hT, hV, hsw2;
   std::vector<cudaGraphExec_t> execs;  // captured passes (opts.graphs), freed with the call
@@ -279,7 +281,7 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.W, n0));
   LC_TRY(r.ar.get(&r.delta, n0));
   LC_TRY(r.ar.get(&r.ab, n0));
-  LC_TRY(r.ar.get(&r.eblocks, kCoopBlocks));
+  LC_TRY(r.ar.get(&r.coop, kCoopScratch));
   LC_TRY(r.ar.get(&r.bound, n0 + 1));
   LC_TRY(r.ar.get(&r.off, n0 + 1));
   LC_TRY(r.ar.get(&r.scan64, scan_scratch(n0 + 1)));
@@ -331,7 +333,7 @@ static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tab
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
   b += 4 * scan_scratch(big);                                // scan32
   b += 2 * 8 * n + (int64_t)sizeof(AbRec) * n;               // W, delta, ab
-  b += 8 * kCoopBlocks;                                      // eblocks
+  b += 4 * kCoopScratch;                                     // coop
   b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + n;      // bound, off, scan64, M
   b += 8 * (2 * nnz0 > 0 ? 2 * nnz0 : 1);                    // gtab
   if (G > 1) b += 8 * (G + 1) + 4 * n;                       // graph_ptr, gid
@@ -356,40 +358,19 @@ int64_t cluster_footprint(int64_t n, int64_t nnz, int count, const lc_opts &o) {
 // than the last shared-memory bin are cut into chunks of the plan's hub_chunk edges).
 static int bins_for(Run &r, Level &L) {
   LC_TRY(r.ar.get(&L.bins.lists, L.g.n));
-  LC_TRY(r.ar.get(&L.bins.offs, kBins + 1));
+  BinOut *d_out = nullptr;
+  LC_TRY(r.ar.get(&d_out, 1));
   LC_TRY(r.ar.get(&L.bins.recs, L.g.n));
-  build_bins(L.g, r.plan, L.bins, r.scan32, r.s);
-  launch_vertex_records(L.g, L.gid, L.bins, r.s);
-  int32_t h[kBins + 1];
-  LC_CK(cudaMemcpyAsync(h, L.bins.offs, sizeof(h), cudaMemcpyDeviceToHost, r.s));
+  launch_bins(L.g, L.gid, r.plan, L.bins, d_out, r.coop, r.sc, r.s);
+  BinOut out{};
+  LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaStreamSynchronize(r.s));
-  finish_bins(L.bins, h);
-  r.res->kernel_launches[LC_K_OTHER] += 4 * kBins + 1;
+  finish_bins(L.bins, out);
+  r.res->kernel_launches[LC_K_OTHER] += 1;
   L.hub = Hubs{};
-  L.max_deg = 0;
-  const int H = (int)L.bins.count[kHubBin];
+  L.max_deg = out.max_deg;
+  const int H = (int)L.bins.count[kHubBin], Q = (int)out.chunks;
   if (H > 0) {
-    int64_t *rows = nullptr;
-    LC_TRY(r.ar.get(&rows, 2 * H));
-    launch_hub_rows(L.g.rp, L.bins.list[kHubBin], H, rows, r.s);
-    r.res->kernel_launches[LC_K_OTHER] += 1;
-    std::vector<int64_t> hrows(2 * (size_t)H);
-    LC_CK(cudaMemcpyAsync(hrows.data(), rows, 16 * (size_t)H, cudaMemcpyDeviceToHost, r.s));
-    LC_CK(cudaStreamSynchronize(r.s));
-    std::vector<int32_t> hub_of, c0(H + 1);
-    std::vector<int64_t> e0, e1;
-    for (int k = 0; k < H; ++k) {
-      L.max_deg = std::max(L.max_deg, hrows[2 * k + 1] - hrows[2 * k]);
-      c0[k] = (int32_t)hub_of.size();
-      const int64_t ch = r.plan.hub_chunk;
-      for (int64_t b = hrows[2 * k]; b < hrows[2 * k + 1]; b += ch) {
-        hub_of.push_back(k);
-        e0.push_back(b);
-        e1.push_back(b + ch < hrows[2 * k + 1] ? b + ch : hrows[2 * k + 1]);
-      }
-    }
-    const int Q = (int)hub_of.size();
-    c0[H] = Q;
     int32_t *d_hub_of, *d_c0, *d_part_x;
     int64_t *d_e0, *d_e1;
     long long *d_acc, *d_part_g;
@@ -400,12 +381,6 @@ static int bins_for(Run &r, Level &L) {
     LC_TRY(r.ar.get(&d_e1, Q));
     LC_TRY(r.ar.get(&d_acc, H));
     LC_TRY(r.ar.get(&d_part_g, Q));
-    LC_CK(cudaMemcpyAsync(d_hub_of, hub_of.data(), 4 * (size_t)Q, cudaMemcpyHostToDevice, r.s));
-    LC_CK(cudaMemcpyAsync(d_c0, c0.data(), 4 * (size_t)(H + 1), cudaMemcpyHostToDevice, r.s));
-    LC_CK(cudaMemcpyAsync(d_e0, e0.data(), 8 * (size_t)Q, cudaMemcpyHostToDevice, r.s));
-    LC_CK(cudaMemcpyAsync(d_e1, e1.data(), 8 * (size_t)Q, cudaMemcpyHostToDevice, r.s));
-    LC_CK(cudaMemsetAsync(d_acc, 0, 8 * (size_t)H, r.s));
-    LC_CK(cudaStreamSynchronize(r.s));  // host vectors are released below
     L.hub.H = H;
     L.hub.Q = Q;
     L.hub.vtx = L.bins.list[kHubBin];
@@ -416,6 +391,8 @@ static int bins_for(Run &r, Level &L) {
     L.hub.acc = d_acc;
     L.hub.part_g = d_part_g;
     L.hub.part_x = d_part_x;
+    launch_hub_plan(L.bins, r.plan, L.hub, r.s);
+    r.res->kernel_launches[LC_K_OTHER] += 1;
   }
   return launch_check();
 }
@@ -564,7 +541,8 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
   LC_TRY(upload_params(r, L, active));
   PassArgs a = pass_args(r, L);
   a.M = r.M;
-  EmptyScratch w{r.used, r.freelist, r.emovers, r.gfree, r.gmover, r.eblocks};
+  EmptyScratch w{r.used, r.freelist, r.emovers, r.gfree, r.gmover,
+                 reinterpret_cast<unsigned long long *>(r.coop)};
   if (use_fused(r, L)) {
     FusedArgs f{};
     f.rec = L.bins.recs;
@@ -939,7 +917,7 @@ static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *
   LC_CK(cudaStreamSynchronize(r.s));
   if (ends[0] != 0 || ends[1] != g.nnz) return LC_ERR_ARG;
   r.prof.begin(LC_K_OTHER);
-  launch_stats(g, r.o.validate, r.st, gid, r.Tg, r.Vg, r.sw2g, r.s);
+  launch_stats(g, r.o.validate, r.st, gid, r.gptr, r.Tg, r.Vg, r.sw2g, r.s);
   r.prof.end(16.0 * g.n + 8.0 * g.nnz);
   r.res->kernel_launches[LC_K_OTHER] += g.nnz > 0 ? 2 : 1;
   LC_CK(cudaMemcpyAsync(hst, r.st, sizeof(GraphStats), cudaMemcpyDeviceToHost, r.s));
@@ -1033,11 +1011,10 @@ static int level0(Run &r, Level &L, const LevelGraph &g0, const std::vector<int6
     L.nv[g] = gptr[g + 1] - gptr[g];
   }
   if (r.G > 1) {
-    int64_t *d_gptr = nullptr;
-    LC_TRY(r.ar.get(&d_gptr, r.G + 1));
+    LC_TRY(r.ar.get(&r.gptr, r.G + 1));
     LC_TRY(r.ar.get(&L.gid, g0.n));
-    LC_CK(cudaMemcpyAsync(d_gptr, gptr.data(), 8 * (size_t)(r.G + 1), cudaMemcpyHostToDevice, r.s));
-    launch_graph_ids(d_gptr, r.G, L.gid, g0.n, r.s);
+    LC_CK(cudaMemcpyAsync(r.gptr, gptr.data(), 8 * (size_t)(r.G + 1), cudaMemcpyHostToDevice, r.s));
+    launch_graph_ids(r.gptr, r.G, L.gid, g0.n, r.s);
     LC_CK(cudaStreamSynchronize(r.s));
     r.res->kernel_launches[LC_K_OTHER] += 1;
   }

@@ -9,6 +9,10 @@ namespace lc {
 constexpr int kCoopThreads = 1024;
 constexpr int kCoopBlocks = 152;  // at most one block per SM
 
+// int32 entries of a call's scratch for the blocks' counts: the bins' count
+// kBins per block, the new-cluster ids one 64-bit word.
+constexpr int64_t kCoopScratch = (int64_t)kBins * kCoopBlocks;
+
 // Polls before a wait gives up (about 0.6 us each): the launch then sets the
 // error flag and every block returns, so the call ends with LC_ERR_DEVICE.
 constexpr unsigned kCoopPolls = 1u << 24;

@@ -787,36 +787,6 @@ __global__ void k_cluster_weights(const int32_t *__restrict__ C, const int64_t *
   }
 }
 
-// ------------------------------------------------------------ binning
-
-struct BinFlag {
-  const int64_t *rp;
-  int64_t lo, hi;  // lo < deg <= hi
-  __device__ int32_t operator()(int64_t v) const {
-    const int64_t d = rp[v + 1] - rp[v];
-    return (d > lo && d <= hi) ? 1 : 0;
-  }
-};
-struct BinEmit {
-  int32_t *lists;
-  const int32_t *off;  // start of this bin in lists
-  __device__ void operator()(int64_t v, int32_t pos, int32_t f) const {
-    if (f) lists[*off + pos] = (int32_t)v;
-  }
-};
-
-__global__ void k_bin_next_offset(int32_t *offs, int k, const int32_t *total) {
-  offs[k + 1] = offs[k] + *total;
-}
-
-__global__ void k_hub_rows(const int64_t *__restrict__ rp, const int32_t *__restrict__ vtx, int H,
-                           int64_t *__restrict__ out) {
-  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < H; h += gridDim.x * blockDim.x) {
-    out[2 * h] = rp[vtx[h]];
-    out[2 * h + 1] = rp[vtx[h] + 1];
-  }
-}
-
 // ================================================================ host
 
 static inline unsigned blocks_for(int64_t items, int per_block) {
@@ -846,49 +816,6 @@ void configure_kernels() {
                        block_table_bytes(4096));
   cudaFuncSetAttribute(k_move_block<256, 6144, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        block_table_bytes(6144));
-}
-
-void build_bins(const LevelGraph &g, const BinPlan &plan, Bins &b, int32_t *scan_tmp, cudaStream_t s) {
-  cudaMemsetAsync(b.offs, 0, sizeof(int32_t), s);
-  int64_t lo = -1;
-  for (int k = 0; k < kBins; ++k) {
-    const int64_t hi = k < kBins - 1 ? plan.max_deg[k] : INT64_MAX;
-    scan_apply<int32_t>(g.n, BinFlag{g.rp, lo, hi}, BinEmit{b.lists, b.offs + k}, scan_tmp, s);
-    k_bin_next_offset<<<1, 1, 0, s>>>(b.offs, k, scan_tmp + scan_tiles(g.n));
-    lo = hi;
-  }
-}
-
-void finish_bins(Bins &b, const int32_t *h_offs) {
-  for (int k = 0; k < kBins; ++k) {
-    b.list[k] = b.lists + h_offs[k];
-    b.rec[k] = b.recs + h_offs[k];
-    b.count[k] = h_offs[k + 1] - h_offs[k];
-  }
-}
-
-__global__ void k_vertex_records(LevelGraph g, const int32_t *__restrict__ gid, const int32_t *__restrict__ lists,
-                                 VRec *__restrict__ recs) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t v = lists[i];
-    VRec r;
-    r.v = v;
-    r.beg = g.rp[v];
-    r.deg = (int32_t)(g.rp[v + 1] - r.beg);
-    r.g = gid ? gid[v] : 0;
-    r.pad = 0;
-    r.w = g.vw[v];
-    recs[i] = r;
-  }
-}
-
-void launch_vertex_records(const LevelGraph &g, const int32_t *gid, Bins &b, cudaStream_t s) {
-  if (g.n > 0) k_vertex_records<<<blocks_for(g.n, 256), 256, 0, s>>>(g, gid, b.lists, b.recs);
-}
-
-void launch_hub_rows(const int64_t *rp, const int32_t *vtx, int H, int64_t *out, cudaStream_t s) {
-  if (H > 0) k_hub_rows<<<blocks_for(H, 256), 256, 0, s>>>(rp, vtx, H, out);
 }
 
 // Vertices per warp of the chunked kernels: 32, so that one lane decides one

@@ -43,7 +43,6 @@ struct PassArgs {
 // Vertex lists of the degree bins of one level (stable: ascending ids).
 struct Bins {
   int32_t *lists;    // device, n entries, bin after bin
-  int32_t *offs;     // device, kBins + 1 entries
   VRec *recs;        // device, n entries: the vertex records of `lists`, same order
   const int32_t *list[kBins];
   const VRec *rec[kBins];
@@ -63,15 +62,7 @@ inline BinRange bin_range(const Bins &b, int lo, int hi) {
 }
 
 void configure_kernels();
-// Builds b.lists / b.offs on the stream; the caller copies b.offs to the host
-// and fills b.list / b.count (see finish_bins).
-void build_bins(const LevelGraph &g, const BinPlan &plan, Bins &b, int32_t *scan_tmp, cudaStream_t s);
-void finish_bins(Bins &b, const int32_t *h_offs);
-// Fills b.recs from b.lists (gid: graph of each vertex, or null for one graph).
-void launch_vertex_records(const LevelGraph &g, const int32_t *gid, Bins &b, cudaStream_t s);
-
 // Launchers return the number of kernels they launched.
-void launch_hub_rows(const int64_t *rp, const int32_t *vtx, int H, int64_t *out, cudaStream_t s);
 // Resets the pass counters; advance = 1 also loads the pass's temperature
 // from the device schedule (sc->phi_tab) and moves to the next pass.
 void launch_pass_begin(Scalars *sc, cudaStream_t s, int advance = 0);
