@@ -1,5 +1,5 @@
 // lc_empty.cuh — ids for the movers to new empty clusters, as phases of a
-// cooperative kernel (all blocks, kCoopThreads threads each).
+// cooperative kernel (all blocks, T threads each).
 #pragma once
 
 #include "lc_coop.cuh"
@@ -8,7 +8,8 @@
 namespace lc {
 
 // Exclusive scan over the block of packed counts; `total` is the block's sum.
-// red: kCoopThreads / 32 entries of shared memory.
+// red: T / 32 entries of shared memory.
+template <int T>
 __device__ __forceinline__ unsigned long long coop_scan(unsigned long long x, unsigned long long *red,
                                                         unsigned long long &total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -23,7 +24,7 @@ __device__ __forceinline__ unsigned long long coop_scan(unsigned long long x, un
   __syncthreads();
   unsigned long long before = 0;
   total = 0;
-  for (int w = 0; w < kCoopThreads / 32; ++w) {
+  for (int w = 0; w < T / 32; ++w) {
     const unsigned long long t = red[w];
     before += w < wid ? t : 0;
     total += t;
@@ -35,12 +36,13 @@ __device__ __forceinline__ unsigned long long coop_scan(unsigned long long x, un
 // are counted and listed together: packed as free << 32 | movers (both below
 // 2^31).  marked: w.used already marks the ids in use.  False if a barrier
 // ran out.
+template <int T>
 __device__ __forceinline__ bool assign_empty(const PassArgs &a, const EmptyScratch &w, int total, bool marked,
                                              GridBarrier &bar) {
-  __shared__ unsigned long long red[kCoopThreads / 32];
+  __shared__ unsigned long long red[T / 32];
   const int64_t n = a.g.n;
-  const int64_t tid = (int64_t)blockIdx.x * kCoopThreads + threadIdx.x;
-  const int64_t nt = (int64_t)gridDim.x * kCoopThreads;
+  const int64_t tid = (int64_t)blockIdx.x * T + threadIdx.x;
+  const int64_t nt = (int64_t)gridDim.x * T;
   if (!marked) {
     for (int64_t x = tid; x < n; x += nt) w.used[x] = 0;
     if (!bar.sync()) return false;
@@ -51,23 +53,23 @@ __device__ __forceinline__ bool assign_empty(const PassArgs &a, const EmptyScrat
     if (!bar.sync()) return false;
   }
   // each block its own run of ids
-  const int64_t per = ((n + gridDim.x - 1) / gridDim.x + kCoopThreads - 1) / kCoopThreads * kCoopThreads;
+  const int64_t per = ((n + gridDim.x - 1) / gridDim.x + T - 1) / T * T;
   const int64_t lo = (int64_t)blockIdx.x * per, hi = lo + per < n ? lo + per : n;
   auto flags = [&](int64_t x) {
     if (x >= hi) return 0ull;
     return (w.used[x] == 0 ? 1ull << 32 : 0ull) | (a.C[x] == kEmpty ? 1ull : 0ull);
   };
   unsigned long long mine = 0, sum;
-  for (int64_t x = lo + threadIdx.x; x < hi; x += kCoopThreads) mine += flags(x);
-  coop_scan(mine, red, sum);
+  for (int64_t x = lo + threadIdx.x; x < hi; x += T) mine += flags(x);
+  coop_scan<T>(mine, red, sum);
   if (threadIdx.x == 0) w.blocks[blockIdx.x] = sum;
   if (!bar.sync()) return false;
   unsigned long long before = 0;
-  coop_scan((int)threadIdx.x < (int)blockIdx.x ? w.blocks[threadIdx.x] : 0ull, red, before);
-  for (int64_t base = lo; base < hi; base += kCoopThreads) {
+  coop_scan<T>((int)threadIdx.x < (int)blockIdx.x ? w.blocks[threadIdx.x] : 0ull, red, before);
+  for (int64_t base = lo; base < hi; base += T) {
     const int64_t x = base + threadIdx.x;
     const unsigned long long f = flags(x);
-    const unsigned long long at = before + coop_scan(f, red, sum);
+    const unsigned long long at = before + coop_scan<T>(f, red, sum);
     before += sum;
     if (x < hi) {
       const int32_t pf = (int32_t)(at >> 32), pm = (int32_t)(uint32_t)at;

@@ -27,8 +27,11 @@ namespace lc {
 
 namespace {
 
-constexpr int kT = kCoopThreads, kW = kT / 32;
-constexpr int kWarpSlots = 512;                 // shared table of a warp (bins 3-4)
+// 512 threads with 128 registers: 1,024 with 64 spilled 1.3 KB a thread and
+// ran 15-18 % slower on SBM 10,000, R-MAT 16 and the 97^3 lattice, 768 with 80
+// 5 % slower, in spite of more warps.
+constexpr int kT = 512, kW = kT / 32;
+constexpr int kWarpSlots = 1024;                // shared table of a warp (bins 3-4)
 constexpr int kTeam = 128;                      // threads of a team (bins 5-6)
 constexpr int kTeamSlots = kWarpSlots * kTeam / 32;
 constexpr int kRowSlots = kWarpSlots * kW;      // the whole block's table
@@ -55,45 +58,54 @@ __device__ __forceinline__ void team_sync(int team) {
 // the blocks that had long rows.  Pieces are fetched one ahead.
 enum { kNextRow = 0, kNextTeam = 1, kNextChunk = 2, kNextCount = 3 };
 
-// A run of bins cut into chunks for warps.
-struct ChunkList {
-  const VRec *rec;
-  int64_t count, chunks;
-  int c;
+// The runs of bins that a phase's warps take in chunks, longest rows first:
+// kept in shared memory, so that the loop over chunks holds no registers for
+// them.
+struct ChunkLists {
+  unsigned end[5];  // chunks of the lists up to this one
+  int c[5];         // vertices per chunk
+  int lo[5];        // first bin
 };
-// One chunk of a list per warp, of at most `most` vertices (fewer where rows
-// are long, so that the last ones even out); a thread per vertex takes 32.
-__device__ __forceinline__ ChunkList chunk_list(const FusedArgs &f, int lo, int hi, int most) {
-  ChunkList l;
-  l.rec = f.rec + f.off[lo];
-  l.count = f.off[hi + 1] - f.off[lo];
-  const int64_t nw = (int64_t)gridDim.x * kW;
-  const int64_t c = (l.count + nw - 1) / nw;
-  l.c = lo == 0 ? 32 : c >= most ? most : c < 1 ? 1 : (int)c;
-  l.chunks = (l.count + l.c - 1) / l.c;
-  return l;
+// Lists of bins lo .. hi, one chunk per warp of at most `most` vertices (fewer
+// where rows are long, so that the last ones even out); a thread per vertex
+// (bin 0) takes 32.  Every thread of the block.
+template <int N>
+__device__ __forceinline__ void plan_chunks(const FusedArgs &f, ChunkLists &l, const int (&lo)[N], const int (&hi)[N],
+                                            const int (&most)[N]) {
+  __syncthreads();  // the last phase's lists are no longer read
+  if (threadIdx.x == 0) {
+    const int64_t nw = (int64_t)gridDim.x * kW;
+    unsigned end = 0;
+    for (int k = 0; k < N; ++k) {
+      const int64_t count = f.off[hi[k] + 1] - f.off[lo[k]];
+      const int64_t c = (count + nw - 1) / nw;
+      l.lo[k] = lo[k];
+      l.c[k] = lo[k] == 0 ? 32 : c >= most[k] ? most[k] : c < 1 ? 1 : (int)c;
+      end += (unsigned)((count + l.c[k] - 1) / l.c[k]);
+      l.end[k] = end;
+    }
+  }
+  __syncthreads();
 }
 
-// Calls body(list, rec, base, m) for the warp's chunks of lists[0 .. N).
+// Calls body(list, rec, m) for the warp's chunks, rec its first record.
 template <int N, typename Body>
-__device__ __forceinline__ void for_chunks(const ChunkList (&lists)[N], unsigned *next, Body body) {
-  int64_t total = 0;
-#pragma unroll
-  for (int k = 0; k < N; ++k) total += lists[k].chunks;
-  const unsigned nw = gridDim.x * kW;
+__device__ __forceinline__ void for_chunks(const FusedArgs &f, const ChunkLists &l, const int (&hi)[N],
+                                           unsigned *next, Body body) {
+  const unsigned total = l.end[N - 1], nw = gridDim.x * kW;
   const int lane = threadIdx.x & 31;
   unsigned j = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  while (j < total) {  // chunks < 2^31: n is an int32 range
+  while (j < total) {
     unsigned after = 0;
     if (total > nw && lane == 0) after = nw + atomicAdd(next, 1u);
-    int64_t at = j;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      if (at >= 0 && at < lists[k].chunks) {
-        const int64_t base = at * lists[k].c, left = lists[k].count - base;
-        body(k, lists[k].rec, base, (int)(left < lists[k].c ? left : lists[k].c));
+      const unsigned start = k > 0 ? l.end[k > 0 ? k - 1 : 0] : 0u;
+      if (j >= start && j < l.end[k]) {
+        const int c = l.c[k];
+        const int64_t from = f.off[l.lo[k]] + (int64_t)(j - start) * c, left = f.off[hi[k] + 1] - from;
+        body(k, f.rec + from, (int)(left < c ? left : c));
       }
-      at -= lists[k].chunks;
     }
     if (total <= nw) break;
     j = __shfl_sync(0xFFFFFFFFu, after, 0);
@@ -221,7 +233,7 @@ __device__ __forceinline__ long long block_total(long long x, long long *red) {
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
   __syncthreads();
   if (threadIdx.x >= 32) return 0;
-  return warp_sum(red[threadIdx.x]);
+  return warp_sum(threadIdx.x < kW ? red[threadIdx.x] : 0ll);
 }
 
 // The chunks of the hubs above kRowMaxDeg edges.
@@ -241,6 +253,7 @@ __global__ void __launch_bounds__(kT, 1)
   int32_t *vals = reinterpret_cast<int32_t *>(keys + kRowSlots);
   Stage &stage = reinterpret_cast<Stage *>(vals + kRowSlots)[threadIdx.x >> 5];
   __shared__ RowPart part;
+  __shared__ ChunkLists lists;
   __shared__ long long red[kW];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, team = threadIdx.x / kTeam;
   const SplitTab wtab{keys + wid * kWarpSlots, vals + wid * kWarpSlots};
@@ -316,15 +329,15 @@ __global__ void __launch_bounds__(kT, 1)
               a.hub.part_x[c] = xb;
             }
           });
-        const ChunkList lists[4] = {chunk_list(f, 5, 6, 1), chunk_list(f, 2, 4, 8), chunk_list(f, 1, 1, 32),
-                                    chunk_list(f, 0, 0, 32)};
-        for_chunks(lists, next + kNextChunk, [&](int k, const VRec *rec, int64_t b, int m) {
+        constexpr int lo[4] = {5, 2, 1, 0}, hi[4] = {6, 4, 1, 0}, most[4] = {1, 8, 32, 32};
+        plan_chunks(f, lists, lo, hi, most);
+        for_chunks(f, lists, hi, next + kNextChunk, [&](int k, const VRec *rec, int m) {
           if (k <= 1)
-            first_chunk<32>(a, rec, b, m, stage.move.st, ms);
+            first_chunk<32>(a, rec, 0, m, stage.move.st, ms);
           else if (k == 2)
-            first_chunk<16>(a, rec, b, m, stage.move.st, ms);
+            first_chunk<16>(a, rec, 0, m, stage.move.st, ms);
           else if (lane < m)
-            first_thread(a, rec, b + lane, ms);
+            first_thread(a, rec, lane, ms);
         });
       } else {
         if (f.big)
@@ -341,17 +354,17 @@ __global__ void __launch_bounds__(kT, 1)
           row_move<kTeam, kTeamSlots / 2 / kTeam>(a, vr, ttab, kTeamSlots, threadIdx.x % kTeam, part, tsync, ms);
         });
         __syncthreads();  // the teams' tables are clean and their partials read
-        const ChunkList lists[4] = {chunk_list(f, 3, 4, 8), chunk_list(f, 2, 2, 32), chunk_list(f, 1, 1, 32),
-                                    chunk_list(f, 0, 0, 32)};
-        for_chunks(lists, next + kNextChunk, [&](int k, const VRec *rec, int64_t b, int m) {
+        constexpr int lo[4] = {3, 2, 1, 0}, hi[4] = {4, 2, 1, 0}, most[4] = {8, 32, 32, 32};
+        plan_chunks(f, lists, lo, hi, most);
+        for_chunks(f, lists, hi, next + kNextChunk, [&](int k, const VRec *rec, int m) {
           if (k == 0)
-            warp_chunk(a, rec, b, m, stage.move.st, wtab, kWarpSlots, ms);
+            warp_chunk(a, rec, 0, m, stage.move.st, wtab, kWarpSlots, ms);
           else if (k == 1)
-            lanes_chunk<32>(a, rec, b, m, stage.move.st, stage.move.tags, ms);
+            lanes_chunk<32, 4>(a, rec, 0, m, stage.move.st, stage.move.tags, ms);
           else if (k == 2)
-            lanes_chunk<16>(a, rec, b, m, stage.move.st, stage.move.tags, ms);
+            lanes_chunk<16, 4>(a, rec, 0, m, stage.move.st, stage.move.tags, ms);
           else
-            move_thread(a, lane < m, rec, b + lane, ms);
+            move_thread(a, lane < m, rec, lane, ms);
         });
       }
       if (last)  // Q of W before the last update (see launch_final_objective)
@@ -450,17 +463,17 @@ __global__ void __launch_bounds__(kT, 1)
         }
         if (wid == 0) apply_lanes(a, lane == 0, vr.v, vr.deg, r, vr.w, keep, us, used);
       });
-      const ChunkList lists[5] = {chunk_list(f, 5, 6, 1), chunk_list(f, 3, 4, 8), chunk_list(f, 2, 2, 32),
-                                  chunk_list(f, 1, 1, 32), chunk_list(f, 0, 0, 32)};
-      for_chunks(lists, next + kNextChunk, [&](int k, const VRec *rec, int64_t b, int m) {
+      constexpr int lo[5] = {5, 3, 2, 1, 0}, hi[5] = {6, 4, 2, 1, 0}, most[5] = {1, 8, 32, 32, 32};
+      plan_chunks(f, lists, lo, hi, most);
+      for_chunks(f, lists, hi, next + kNextChunk, [&](int k, const VRec *rec, int m) {
         if (k <= 1)
-          ab_chunk<32>(a, rec, b, m, stage.ab, us, used);
+          ab_chunk<32>(a, rec, 0, m, stage.ab, us, used);
         else if (k == 2)
-          ab_chunk<8>(a, rec, b, m, stage.ab, us, used);
+          ab_chunk<8>(a, rec, 0, m, stage.ab, us, used);
         else if (k == 3)
-          ab_chunk<4>(a, rec, b, m, stage.ab, us, used);
+          ab_chunk<4>(a, rec, 0, m, stage.ab, us, used);
         else
-          ab_thread(a, lane < m, rec, b + lane, us, used);
+          ab_thread(a, lane < m, rec, lane, us, used);
       });
     }
     if (f.big) {
@@ -491,7 +504,7 @@ __global__ void __launch_bounds__(kT, 1)
     if (!bar.sync()) return;
     const int total = f.empties[i % 3];
     if (total > 0) {  // uniform over the grid
-      if (!assign_empty(a, f.empty, total, true, bar)) return;
+      if (!assign_empty<kT>(a, f.empty, total, true, bar)) return;
       if (!bar.sync()) return;
     }
   }
@@ -519,13 +532,14 @@ __global__ void __launch_bounds__(kT, 1)
         if (threadIdx.x == 0) add(vr.g, d);
       }
     }
-    const ChunkList lists[3] = {chunk_list(f, 5, 6, 1), chunk_list(f, 1, 4, 8), chunk_list(f, 0, 0, 32)};
+    constexpr int lo[3] = {5, 1, 0}, hi[3] = {6, 4, 0}, most[3] = {1, 8, 32};
+    plan_chunks(f, lists, lo, hi, most);
     // the counters of the pass after the last were zeroed by it and not used
-    for_chunks(lists, f.next + (p % 3) * 2 * kNextCount, [&](int k, const VRec *rec, int64_t b, int m) {
+    for_chunks(f, lists, hi, f.next + (p % 3) * 2 * kNextCount, [&](int k, const VRec *rec, int m) {
       VRec vr{};
       bool mover = false;
       if (lane < m) {
-        vr = rec[b + lane];
+        vr = rec[lane];
         mover = a.C[vr.v] != a.ab[vr.v].C;
       }
       if (k == 2) {

@@ -65,7 +65,7 @@ inline BinPlan default_bin_plan() {
   BinPlan p;
   for (int k = 0; k < kBins - 1; ++k) p.max_deg[k] = kBinMaxDeg[k];
   p.hub_chunk = kHubChunk;
-  const int32_t gs[5] = {1, 16, 32, 128, 512};
+  const int32_t gs[5] = {1, 16, 16, 128, 128};
   for (int k = 0; k < 5; ++k) p.ab_gs[k] = gs[k];
   return p;
 }

@@ -329,13 +329,13 @@ __device__ __forceinline__ int32_t lane_sums(LaneTags &t, int lane, bool on, int
   return S;
 }
 
-// A step takes the rows of two vertices (G = 32) or four (G = 16): their
-// label gathers are issued together, then their W gathers, while the next
+// A step takes the rows of U (G = 32) or 2 U (G = 16) vertices: their label
+// gathers are issued together, then their W gathers, while the next
 // step's columns and weights are on their way.
-template <int G>
+template <int G, int U = 2>
 __device__ __forceinline__ void lanes_chunk(const PassArgs &a, const VRec *__restrict__ rec, int64_t base, int m,
                                             MoveStage &st, LaneTags &tags, MoveState &ms) {
-  constexpr int V = 32 / G, U = 2;
+  constexpr int V = 32 / G;
   const int lane = threadIdx.x & 31, grp = lane / G, sub = lane & (G - 1);
   const ChunkLane c = stage_move(a, rec, base, m, lane, false, st.ctx);
   __syncwarp();
@@ -944,10 +944,10 @@ __device__ __forceinline__ int stage_ab(const PassArgs &a, const VRec *__restric
 
 // Afterburner and update of a chunk: for each candidate, delta_v adjusted by
 // every adjacent candidate that precedes it; it survives iff the adjusted
-// delta is >= 0.  G lanes per candidate, four edges each in flight, so that
-// a row up to 4 G edges is one chain of gathers and a warp has 32 / G chains
+// delta is >= 0.  G lanes per candidate, U edges each in flight, so that
+// a row up to U G edges is one chain of gathers and a warp has 32 / G chains
 // going: the walk is bound by their latency.
-template <int G>
+template <int G, int U = 4>
 __device__ __forceinline__ void ab_chunk(const PassArgs &a, const VRec *__restrict__ rec, int64_t base, int m,
                                          AbStage &st, UpdateSums &sum, int32_t *used = nullptr) {
   constexpr int V = 32 / G;
@@ -962,7 +962,7 @@ __device__ __forceinline__ void ab_chunk(const PassArgs &a, const VRec *__restri
     long long acc = 0;
     if (k + grp < nc) {
       const AbCtx c = st.ctx[k + grp];
-      acc = ab_edges<G, 4>(a, c, c.beg, c.beg + c.deg, sub);
+      acc = ab_edges<G, U>(a, c, c.beg, c.beg + c.deg, sub);
     }
     __syncwarp();
     if (__any_sync(0xFFFFFFFFu, acc != 0)) acc = group_sum<G>(acc);
@@ -975,6 +975,7 @@ __device__ __forceinline__ void ab_chunk(const PassArgs &a, const VRec *__restri
 }
 
 // Bin 0: one thread per vertex (full warp, lanes with on = false idle).
+template <int U = 4>
 __device__ __forceinline__ void ab_thread(const PassArgs &a, bool on, const VRec *__restrict__ rec, int64_t i,
                                           UpdateSums &sum, int32_t *used = nullptr) {
   VRec vr{};
@@ -985,7 +986,7 @@ __device__ __forceinline__ void ab_thread(const PassArgs &a, bool on, const VRec
     r = a.ab[vr.v];
     if (r.D != kNone) {
       const AbCtx c = ab_ctx(a, vr.v, r, a.gp[vr.g], vr.beg, vr.deg, vr.w);
-      keep = a.delta[vr.v] + ab_edges<1, 4>(a, c, c.beg, c.beg + c.deg, 0) >= 0;
+      keep = a.delta[vr.v] + ab_edges<1, U>(a, c, c.beg, c.beg + c.deg, 0) >= 0;
     }
   }
   __syncwarp();

@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_assign_empty(PassArgs a, Empty
   const int total = a.sc->empty_movers;  // nothing writes it during this launch
   if (total == 0) return;
   GridBarrier bar(a.sc);
-  if (!assign_empty(a, w, total, false, bar)) return;
+  if (!assign_empty<kCoopThreads>(a, w, total, false, bar)) return;
   bar.leave();
 }
 

@@ -71,7 +71,7 @@ int time_setting(const Workload &w, const lc_opts &o, int repeats, double *ms,
 }
 
 const int kDefaultMax[9] = {8, 16, 32, 128, 256, 512, 1024, 2048, 4096};
-const int kDefaultAb[5] = {1, 16, 32, 128, 512};
+const int kDefaultAb[5] = {1, 16, 16, 128, 128};
 
 }  // namespace
 
