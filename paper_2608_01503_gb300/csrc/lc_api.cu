@@ -13,6 +13,7 @@
 #include <climits>
 #include <cstdio>
 #include <cstring>
+#include <deque>
 #include <mutex>
 #include <unordered_map>
 #include <vector>
@@ -25,6 +26,7 @@
 #include "lc_fused.cuh"
 #include "lc_contract.cuh"
 #include "lc_leiden.cuh"
+#include "lc_level.cuh"
 #include "lc_internal.cuh"
 #include "lc_memory.cuh"
 #include "lc_pass.cuh"
@@ -162,6 +164,8 @@ struct Level {
   Bins bins{};
   Hubs hub{};
   int64_t max_deg = 0;               // longest hub row (0: no hub)
+  BinOut bin_out{};                  // of the full graph, if known before its bins are built
+  bool bins_known = false;
   int32_t *gid = nullptr;            // [n] graph of each vertex (nullptr: one graph)
   GraphParam *gp = nullptr;          // [G] device
   std::vector<int64_t> vbase, nv;    // [G] host
@@ -204,12 +208,15 @@ struct Run {
   int64_t *gptr = nullptr;  // [G + 1] vertex ranges of a batch
   GraphStats *st = nullptr;
   std::vector<long long> hT, hV, hsw2;
+  LevelOut *lout = nullptr;                 // level ends (lc_level.cu)
+  long long *lcounts = nullptr;             // [kLevelCounts]
+  std::deque<std::vector<GraphParam>> staged;  // sources of uploads, until the call's work is done
   std::vector<cudaGraphExec_t> execs;  // captured passes (opts.graphs), freed with the call
   explicit Run(const lc_opts &o_) : s((cudaStream_t)o_.stream), o(o_), ar((cudaStream_t)o_.stream, o_) {}
   Run(const Run &) = delete;
   ~Run() {
-    if (execs.empty()) return;
-    cudaStreamSynchronize(s);  // replays finished before their graphs go
+    if (execs.empty() && staged.empty()) return;
+    cudaStreamSynchronize(s);  // replays and uploads finished before what they read goes
     for (cudaGraphExec_t e : execs) cudaGraphExecDestroy(e);
     cudaGetLastError();
   }
@@ -282,6 +289,8 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.delta, n0));
   LC_TRY(r.ar.get(&r.ab, n0));
   LC_TRY(r.ar.get(&r.coop, kCoopScratch));
+  LC_TRY(r.ar.get(&r.lcounts, kLevelCounts));
+  LC_TRY(r.ar.get(&r.lout, 1));
   LC_TRY(r.ar.get(&r.bound, n0 + 1));
   LC_TRY(r.ar.get(&r.off, n0 + 1));
   LC_TRY(r.ar.get(&r.scan64, scan_scratch(n0 + 1)));
@@ -333,7 +342,7 @@ static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tab
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
   b += 4 * scan_scratch(big);                                // scan32
   b += 2 * 8 * n + (int64_t)sizeof(AbRec) * n;               // W, delta, ab
-  b += 4 * kCoopScratch;                                     // coop
+  b += 4 * kCoopScratch + 8 * kLevelCounts + (int64_t)sizeof(LevelOut);  // coop, lcounts, lout
   b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + n;      // bound, off, scan64, M
   b += 8 * (2 * nnz0 > 0 ? 2 * nnz0 : 1);                    // gtab
   if (G > 1) b += 8 * (G + 1) + 4 * n;                       // graph_ptr, gid
@@ -362,9 +371,12 @@ static int bins_for(Run &r, Level &L) {
   LC_TRY(r.ar.get(&d_out, 1));
   LC_TRY(r.ar.get(&L.bins.recs, L.g.n));
   launch_bins(L.g, L.gid, r.plan, L.bins, d_out, r.coop, r.sc, r.s);
-  BinOut out{};
-  LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaStreamSynchronize(r.s));
+  BinOut out = L.bin_out;
+  if (!L.bins_known) {
+    LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
+    LC_CK(cudaStreamSynchronize(r.s));
+  }
+  L.bins_known = false;  // a filtered graph's bins are built later on the same level
   finish_bins(L.bins, out);
   r.res->kernel_launches[LC_K_OTHER] += 1;
   L.hub = Hubs{};
@@ -407,9 +419,12 @@ static int upload_params(Run &r, Level &L, const std::vector<uint8_t> &active) {
     h[g].Lam = r.Lam[g];
     h[g].vbase = (int32_t)L.vbase[g];
     h[g].active = active[g];
+    h[g].nv = (int32_t)L.nv[g];
+    h[g].pad = 0;
   }
-  LC_CK(cudaMemcpyAsync(L.gp, h.data(), sizeof(GraphParam) * (size_t)r.G, cudaMemcpyHostToDevice, r.s));
-  LC_CK(cudaStreamSynchronize(r.s));
+  // no wait: the source lives as long as the call
+  r.staged.push_back(std::move(h));
+  LC_CK(cudaMemcpyAsync(L.gp, r.staged.back().data(), sizeof(GraphParam) * (size_t)r.G, cudaMemcpyHostToDevice, r.s));
   return LC_OK;
 }
 
@@ -436,13 +451,6 @@ static PassArgs pass_args(Run &r, const Level &L) {
   a.hub_min = r.plan.hub_min();
   for (int g = 0; g < kAbGroups; ++g) a.ab_gs[g] = r.plan.ab_gs[g];
   return a;
-}
-
-static int fill_per_graph(Run &r, long long *dst, long long value) {
-  std::vector<long long> h(r.G, value);
-  LC_CK(cudaMemcpyAsync(dst, h.data(), 8 * (size_t)r.G, cudaMemcpyHostToDevice, r.s));
-  LC_CK(cudaStreamSynchronize(r.s));
-  return LC_OK;
 }
 
 // Host copies for the optional trace callback (single-graph calls only).
@@ -577,7 +585,8 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
     launch_cluster_weights(r.C, L.g.vw, r.W, n, r.s);
     r.res->kernel_launches[LC_K_OTHER] += 1;
   }
-  LC_TRY(fill_per_graph(r, r.phi_out, singleton ? 0 : LLONG_MIN));  // Phi(singletons) = 0
+  launch_fill(r.phi_out, singleton ? 0 : LLONG_MIN, r.G, r.s);  // Phi(singletons) = 0
+  r.res->kernel_launches[LC_K_OTHER] += 1;
   LC_CK(cudaMemsetAsync(r.phi_acc, 0, 8 * (size_t)r.G, r.s));
   // Kept tables (opts.tables = 1, Section IV-A-3): the first aggregation
   // pass of the call writes the tables of the vertices of degree above
@@ -752,28 +761,40 @@ static int constrained_passes(Run &r, Level &L, int level, const std::vector<uin
   return rc;
 }
 
-// Per-graph number of labels used by C (host nc[G]); also leaves newid
-// (global ascending numbering) and gstart on the device.
-static int count_labels(Run &r, Level &L, const int32_t *C, std::vector<int64_t> &nc, int64_t *total) {
+// Per-graph number of labels used by C; also leaves newid (global ascending
+// numbering) and gstart on the device.  begin_count queues the work and the
+// read-back, end_count forms the numbers once the stream has been waited for.
+struct LabelCount {
+  std::vector<int32_t> gs;
+  int32_t total = 0;
+};
+static int begin_count(Run &r, Level &L, const int32_t *C, LabelCount &c) {
   const int64_t n = L.g.n;
   launch_mark_used(C, n, r.used, r.s);
   launch_number_labels(r.used, n, L.gid, L.gp, nullptr, r.newid, r.gstart, nullptr, r.scan32, r.s);
   r.res->kernel_launches[LC_K_CONTRACT] += 4;
-  std::vector<int32_t> gs(r.G);
-  int32_t tot = 0;
-  LC_CK(cudaMemcpyAsync(gs.data(), r.gstart, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaMemcpyAsync(&tot, compact_total(r.scan32, n), 4, cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaStreamSynchronize(r.s));
-  LC_TRY(launch_check());
+  c.gs.assign(r.G, 0);
+  LC_CK(cudaMemcpyAsync(c.gs.data(), r.gstart, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
+  LC_CK(cudaMemcpyAsync(&c.total, compact_total(r.scan32, n), 4, cudaMemcpyDeviceToHost, r.s));
+  return LC_OK;
+}
+static int64_t end_count(const Run &r, const Level &L, const LabelCount &c, std::vector<int64_t> &nc) {
   nc.assign(r.G, 0);
   int prev = -1;
   for (int g = 0; g < r.G; ++g) {
     if (L.nv[g] == 0) continue;
-    if (prev >= 0) nc[prev] = gs[g] - gs[prev];
+    if (prev >= 0) nc[prev] = c.gs[g] - c.gs[prev];
     prev = g;
   }
-  if (prev >= 0) nc[prev] = tot - gs[prev];
-  *total = tot;
+  if (prev >= 0) nc[prev] = c.total - c.gs[prev];
+  return c.total;
+}
+static int count_labels(Run &r, Level &L, const int32_t *C, std::vector<int64_t> &nc, int64_t *total) {
+  LabelCount c;
+  LC_TRY(begin_count(r, L, C, c));
+  LC_CK(cudaStreamSynchronize(r.s));
+  LC_TRY(launch_check());
+  *total = end_count(r, L, c, nc);
   return LC_OK;
 }
 
@@ -818,6 +839,59 @@ static int compact_level(Run &r, Level &L, Level &N, int level, bool *any) {
   LC_CK(cudaStreamSynchronize(r.s));  // L.cont is read by the copy above
   r.prof.end(24.0 * n);
   r.res->kernel_launches[LC_K_CONTRACT] += 4;
+  return launch_check();
+}
+
+// compact_level and contract_level of a small level in two cooperative
+// kernels with one read-back between them (lc_level.cu); also leaves the
+// sizes of N's bins.
+static bool use_small_level(const Run &r, const Level &L) {
+  return !r.prof.on && !r.o.event_cb && L.g.n + L.g.nnz <= kFusedMaxSize;
+}
+static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
+  Phase range("lc.contract");
+  LC_TRY(r.ar.get(&L.Cd, L.g.n));
+  const LevelScratch w{r.used, r.newid, r.cnt, r.bound, r.off, r.W, r.delta, r.gtab, r.gfree, r.lcounts};
+  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.sc, r.s);
+  LevelOut out{};
+  std::vector<int32_t> nc(r.G);
+  LC_CK(cudaMemcpyAsync(&out, r.lout, sizeof(out), cudaMemcpyDeviceToHost, r.s));
+  LC_CK(cudaMemcpyAsync(nc.data(), w.nc, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
+  LC_CK(cudaStreamSynchronize(r.s));
+  LC_TRY(launch_check());
+  r.res->kernel_launches[LC_K_CONTRACT] += 1;
+  L.cont.assign(r.G, 0);
+  N.vbase.assign(r.G, 0);
+  N.nv.assign(r.G, 0);
+  int64_t base = 0;
+  for (int g = 0; g < r.G; ++g) {
+    if (L.nv[g] == 0) continue;
+    if (nc[g] < L.nv[g]) {
+      L.cont[g] = 1;
+      N.vbase[g] = base;
+      N.nv[g] = nc[g];
+      base += nc[g];
+    } else {
+      r.top[g] = level;
+    }
+  }
+  *any = base > 0;
+  if (!*any) return LC_OK;
+  if (base != out.n_c) return LC_ERR_DEVICE;
+  int64_t *rp_c = nullptr, *vw_c = nullptr;
+  int32_t *col_c = nullptr, *ew_c = nullptr;
+  LC_TRY(r.ar.get(&rp_c, out.n_c + 1));
+  LC_TRY(r.ar.get(&vw_c, out.n_c));
+  if (r.G > 1) LC_TRY(r.ar.get(&N.gid, out.n_c));
+  LC_TRY(r.ar.get(&col_c, out.nnz_c));
+  LC_TRY(r.ar.get(&ew_c, out.nnz_c));
+  launch_level_build(L.g, L.gid, L.Cd, w, out, rp_c, col_c, ew_c, vw_c, N.gid, r.sc, r.s);
+  r.res->kernel_launches[LC_K_CONTRACT] += 1;
+  r.res->edges_contract += L.g.nnz;
+  N.g = LevelGraph{out.n_c, out.nnz_c, rp_c, col_c, ew_c, vw_c};
+  N.bin_out = out.bins;
+  for (int k = 0; k < kBins; ++k) N.bin_out.offs[k + 1] += N.bin_out.offs[k];
+  N.bins_known = true;
   return launch_check();
 }
 
@@ -908,14 +982,8 @@ static int check_graph_args(const lc_csr *g, const int64_t *vw, const int32_t *e
 // Statistics, validation and the exactness guards of the header, per graph.
 static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *hst) {
   LC_TRY(r.ar.get(&r.st, 1));
-  GraphStats z{};
-  z.err_key = ~0ull;
-  LC_CK(cudaMemcpyAsync(r.st, &z, sizeof(z), cudaMemcpyHostToDevice, r.s));
-  int64_t ends[2] = {0, 0};
-  LC_CK(cudaMemcpyAsync(&ends[0], g.rp, 8, cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaMemcpyAsync(&ends[1], g.rp + g.n, 8, cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaStreamSynchronize(r.s));
-  if (ends[0] != 0 || ends[1] != g.nnz) return LC_ERR_ARG;
+  LC_CK(cudaMemsetAsync(r.st, 0, sizeof(GraphStats), r.s));
+  LC_CK(cudaMemsetAsync(&r.st->err_key, 0xFF, sizeof(r.st->err_key), r.s));
   r.prof.begin(LC_K_OTHER);
   launch_stats(g, r.o.validate, r.st, gid, r.gptr, r.Tg, r.Vg, r.sw2g, r.s);
   r.prof.end(16.0 * g.n + 8.0 * g.nnz);
@@ -931,6 +999,7 @@ static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *
   }
   LC_CK(cudaStreamSynchronize(r.s));
   LC_TRY(launch_check());
+  if (hst->first != 0 || hst->last != g.nnz) return LC_ERR_ARG;
   if (!gid) {
     r.hT[0] = hst->T;
     r.hV[0] = hst->V;
@@ -1048,13 +1117,14 @@ static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t>
       LC_TRY(local_move_passes(r, L, true, l, 0, present));
     Level N;
     bool any = false;
-    LC_TRY(compact_level(r, lv[l], N, l, &any));
+    const bool small = use_small_level(r, lv[l]);
+    LC_TRY(small ? end_small_level(r, lv[l], N, l, &any) : compact_level(r, lv[l], N, l, &any));
     if (!any) {
       top = l;
       break;
     }
     lv.push_back(std::move(N));
-    LC_TRY(contract_level(r, lv[l], lv[l + 1], l));
+    if (!small) LC_TRY(contract_level(r, lv[l], lv[l + 1], l));
     if (lv[l].B) {  // coarse vertices carry their members' constraint label
       int32_t *Bc = nullptr;
       LC_TRY(r.ar.get(&Bc, lv[l + 1].g.n));
@@ -1082,11 +1152,11 @@ static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t>
       LC_CK(cudaMemcpyAsync(r.C_out, r.C, sizeof(int32_t) * L.g.n, cudaMemcpyDeviceToDevice, r.s));
     }
   }
-  // final dense labels per graph and the exact objective per graph
+  // final dense labels per graph and the exact objective per graph, one wait
+  // for all that is read back
   Level &L0 = lv[0];
-  std::vector<int64_t> nc;
-  int64_t total = 0;
-  LC_TRY(count_labels(r, L0, r.C_out, nc, &total));
+  LabelCount count;
+  LC_TRY(begin_count(r, L0, r.C_out, count));
   launch_relabel(r.C_out, r.newid, labels_out, L0.g.n, L0.gid, r.gstart, nullptr, 1, r.s);
   std::vector<long long> phi;
   if (r.o.uncoarsen && r.o.pass_limit >= 1 && !B0) {
@@ -1095,11 +1165,13 @@ static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t>
     // graph that stopped there), whose best-of test left its exact Phi
     phi.assign(r.G, 0);
     LC_CK(cudaMemcpyAsync(phi.data(), r.phi_final, 8 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
-    LC_CK(cudaStreamSynchronize(r.s));
   } else {
     LC_TRY(objective_of(r, L0, r.C_out, phi));
   }
-  LC_TRY(check_device_error(r));
+  LC_TRY(check_device_error(r));  // waits
+  LC_TRY(launch_check());
+  std::vector<int64_t> nc;
+  end_count(r, L0, count, nc);
   for (int g = 0; g < r.G; ++g) {
     lc_result &res = r.res[g];
     res.n_clusters = nc[g];
@@ -1308,7 +1380,8 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
     LC_CK(cudaMemcpyAsync(r.C_out, R, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, r.s));
     Level N;
     bool any = false;
-    LC_TRY(compact_level(r, L, N, l, &any));
+    const bool small = use_small_level(r, L);
+    LC_TRY(small ? end_small_level(r, L, N, l, &any) : compact_level(r, L, N, l, &any));
     if (!any) {  // the refinement merged nothing
       top = l;
       r.top[0] = l;
@@ -1316,7 +1389,7 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
       break;
     }
     lv.push_back(std::move(N));
-    LC_TRY(contract_level(r, lv[l], lv[l + 1], l));
+    if (!small) LC_TRY(contract_level(r, lv[l], lv[l + 1], l));
     launch_downsample(lv[l].Cd, Bd, Ccur, n, r.s);  // coarse vertex x: its members' cluster
     r.res->kernel_launches[LC_K_OTHER] += 1;
   }
@@ -1334,13 +1407,14 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
     }
   }
   Level &L0 = lv[0];
-  std::vector<int64_t> nc;
-  int64_t total = 0;
-  LC_TRY(count_labels(r, L0, r.C_out, nc, &total));
+  LabelCount count;
+  LC_TRY(begin_count(r, L0, r.C_out, count));
   launch_relabel(r.C_out, r.newid, labels_out, L0.g.n, nullptr, r.gstart, nullptr, 1, r.s);
   std::vector<long long> phi;
-  LC_TRY(objective_of(r, L0, r.C_out, phi));
+  LC_TRY(objective_of(r, L0, r.C_out, phi));  // waits
   LC_TRY(check_device_error(r));
+  std::vector<int64_t> nc;
+  end_count(r, L0, count, nc);
   r.res->n_clusters = nc[0];
   finish_result(r, 0, r.res, phi[0]);
   return LC_OK;

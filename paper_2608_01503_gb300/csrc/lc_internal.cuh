@@ -115,6 +115,8 @@ struct GraphParam {
   long long mu, Lam;
   int32_t vbase;
   int32_t active;
+  int32_t nv;  // its vertices at this level (0: finished below it)
+  int32_t pad;
 };
 
 // Call-wide constants of the afterburner order (Section IV-A-1).

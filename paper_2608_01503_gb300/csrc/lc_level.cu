@@ -1,0 +1,362 @@
+// lc_level.cu — the end of a small coarsening level in two cooperative
+// kernels: label compaction and Algorithm 4's contraction, which as separate
+// launches (marks, three scans of three launches each, bounds, six insert
+// kernels, a compaction, two read-backs) took 28 launches of 2-4 us and two
+// more waits of the host, whatever the level's size.  The method is
+// lc_contract.cu's: coarse vertex x owns 2 bound[x] slots of the global hash
+// scratch, every fine edge that leaves its cluster is inserted there, and
+// the occupied slots in order are the coarse rows.
+#include "lc_coop.cuh"
+#include "lc_group.cuh"
+#include "lc_level.cuh"
+#include "lc_move.cuh"
+
+namespace lc {
+
+namespace {
+
+constexpr int kT = 512, kW = kT / 32;
+static_assert(kLevelCounts >= (int64_t)kCoopBlocks * kW, "one count per warp");
+
+struct EndArgs {
+  LevelGraph g;
+  const int32_t *gid;
+  const GraphParam *gp;
+  int32_t G;
+  const VRec *rec;
+  int64_t off[kBins + 1];
+  int32_t max_deg[kBins - 1];
+  int32_t hub_chunk;
+  const int32_t *C;
+  int32_t *Cd;
+  LevelScratch w;
+  LevelOut *out;
+  Scalars *sc;
+};
+
+// Exclusive scan over the grid of in(i), i < n: out(i, prefix, value); the
+// total to every thread.  Each warp takes a run of its own.  False if a
+// barrier ran out.
+template <typename In, typename Out>
+__device__ __forceinline__ bool grid_scan(int64_t n, long long *counts, GridBarrier &bar, In in, Out out,
+                                          long long &total) {
+  __shared__ long long red[kW], red_all[kW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nw = gridDim.x * kW, me = blockIdx.x * kW + wid;
+  const int64_t per = ((n + nw - 1) / nw + 31) / 32 * 32;
+  const int64_t lo = (int64_t)me * per, hi = lo + per < n ? lo + per : n;
+  long long mine = 0;
+  for (int64_t i = lo + lane; i < hi; i += 32) mine += in(i);
+  mine = warp_sum(mine);
+  if (lane == 0) counts[me] = mine;
+  if (!bar.sync()) return false;
+  long long before = 0, all = 0;
+  for (int k = threadIdx.x; k < nw; k += kT) {
+    const long long c = counts[k];
+    all += c;
+    before += k < blockIdx.x * kW ? c : 0;
+  }
+  before = warp_sum(before);
+  all = warp_sum(all);
+  if (lane == 0) {
+    red[wid] = before;
+    red_all[wid] = all;
+  }
+  __syncthreads();
+  before = all = 0;
+  for (int k = 0; k < kW; ++k) {
+    before += red[k];
+    all += red_all[k];
+  }
+  for (int k = 0; k < wid; ++k) before += counts[blockIdx.x * kW + k];
+  total = all;
+  __syncthreads();
+  for (int64_t base = lo; base < hi; base += 32) {
+    const int64_t i = base + lane;
+    const long long x = i < hi ? in(i) : 0;
+    long long incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (i < hi) out(i, before + incl - x, x);
+    before += __shfl_sync(0xFFFFFFFFu, incl, 31);
+  }
+  return true;
+}
+
+// Inserts edges [beg + r, end) (stride GS) of a vertex of coarse id x;
+// returns the slots claimed.
+template <int GS>
+__device__ __forceinline__ int insert_row(const EndArgs &a, int32_t x, int64_t beg, int64_t end, int r, bool &ok) {
+  constexpr int U = 4;
+  const int64_t o0 = a.w.off[x];
+  const uint32_t cap = (uint32_t)(2 * (a.w.off[x + 1] - o0));
+  unsigned long long *tab = a.w.tab + 2 * o0;
+  int fresh_n = 0;
+  for (int64_t base = beg + r; base < end; base += (int64_t)GS * U) {
+    int32_t u[U], w[U], y[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int64_t e = base + (int64_t)k * GS;
+      u[k] = -1;
+      w[k] = 0;
+      if (e < end) {
+        u[k] = LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn);
+        w[k] = __ldg(a.g.ew + e);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) y[k] = u[k] >= 0 ? LC_IDX(a.Cd[u[k]], a.g.n, kDbgCoarse) : x;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (y[k] == x) continue;
+      bool fresh = false;
+      ok &= table_add(tab, cap, y[k], w[k], fresh);
+      fresh_n += fresh;
+    }
+  }
+  return fresh_n;
+}
+
+__global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ EndArgs a) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t n = a.g.n;
+  const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
+  const int64_t wbase = tid - lane;
+  GridBarrier bar(a.sc);
+  for (int64_t x = tid; x <= n; x += nt) {
+    a.w.bound[x] = 0;
+    if (x < n) {
+      a.w.used[x] = 0;
+      a.w.cnt[x] = 0;
+      a.w.vw[x] = 0;
+    }
+  }
+  for (int64_t g = tid; g < a.G; g += nt) a.w.nc[g] = 0;
+  if (!bar.sync()) return;
+  for (int64_t v = tid; v < n; v += nt) a.w.used[LC_IDX(a.C[v], n, kDbgLabel)] = 1;
+  if (!bar.sync()) return;
+  if (a.gid) {  // labels in use per graph, which tell the graphs that go on
+    for (int64_t x0 = wbase; x0 < n; x0 += nt) {
+      const int64_t x = x0 + lane;
+      const int g = x < n && a.w.used[x] ? a.gid[x] : -1;
+      const unsigned on = __ballot_sync(0xFFFFFFFFu, g >= 0);
+      if (!on) continue;
+      const int g0 = __shfl_sync(0xFFFFFFFFu, g, __ffs(on) - 1);
+      if (__all_sync(0xFFFFFFFFu, g < 0 || g == g0)) {
+        if (lane == 0) atomicAdd(&a.w.nc[g0], __popc(on));
+      } else if (g >= 0) {
+        atomicAdd(&a.w.nc[g], 1);
+      }
+    }
+    if (!bar.sync()) return;
+  }
+  // dense ids, ascending, of the labels of the graphs that go on
+  auto goes_on = [&](int64_t x) {
+    const int g = a.gid ? a.gid[x] : 0;
+    return !a.gid || a.w.nc[g] < a.gp[g].nv;
+  };
+  long long n_c = 0;
+  if (!grid_scan(
+          n, a.w.counts, bar,
+          [&](int64_t x) -> long long { return a.w.used[x] && goes_on(x) ? 1 : 0; },
+          [&](int64_t x, long long at, long long) { a.w.newid[x] = (int32_t)at; }, n_c))
+    return;
+  if (!a.gid && n_c == n) n_c = 0;  // nothing merges
+  if (tid == 0) {
+    a.out->n_c = n_c;
+    if (!a.gid) a.w.nc[0] = n_c ? (int32_t)n_c : (int32_t)n;
+  }
+  if (n_c == 0) {  // uniform: the host reads no more than this
+    bar.leave();
+    return;
+  }
+  if (!bar.sync()) return;
+  // coarse ids, edge bounds and weights
+  for (int64_t v0 = wbase; v0 < n; v0 += nt) {
+    const int64_t v = v0 + lane;
+    int32_t x = -1;
+    if (v < n) {
+      x = goes_on(v) ? a.w.newid[a.C[v]] : -1;
+      a.Cd[v] = x;
+    }
+    add_weights(a.w.bound, x >= 0, x >= 0 ? x : 0, x >= 0 ? a.g.rp[v + 1] - a.g.rp[v] : 0);
+    add_weights(a.w.vw, x >= 0, x >= 0 ? x : 0, x >= 0 ? a.g.vw[v] : 0);
+  }
+  if (!bar.sync()) return;
+  long long slots = 0;
+  if (!grid_scan(
+          n_c + 1, a.w.counts, bar, [&](int64_t x) -> long long { return a.w.bound[x]; },
+          [&](int64_t x, long long at, long long) { a.w.off[x] = at; }, slots))
+    return;
+  if (!bar.sync()) return;
+  // insert: rows of bins 7-9 by a block, bins 1-6 by a warp, bin 0 by a thread
+  bool ok = true;
+  {
+    __shared__ int s_fresh;
+    for (int64_t i = a.off[7] + blockIdx.x; i < a.off[kBins]; i += gridDim.x) {
+      const VRec vr = a.rec[i];
+      const int32_t x = a.Cd[vr.v];
+      if (x < 0) continue;  // block-uniform
+      __syncthreads();
+      if (threadIdx.x == 0) s_fresh = 0;
+      __syncthreads();
+      const int f = (int)__reduce_add_sync(
+          0xFFFFFFFFu, (unsigned)insert_row<kT>(a, x, vr.beg, vr.beg + vr.deg, threadIdx.x, ok));
+      if (lane == 0 && f) atomicAdd(&s_fresh, f);
+      __syncthreads();
+      if (threadIdx.x == 0 && s_fresh) atomicAdd(&a.w.cnt[x], s_fresh);
+    }
+    const int64_t nw = (int64_t)gridDim.x * kW;
+    for (int64_t i = a.off[1] + (int64_t)wid * gridDim.x + blockIdx.x; i < a.off[7]; i += nw) {
+      const VRec vr = a.rec[i];
+      const int32_t x = a.Cd[vr.v];
+      if (x < 0) continue;  // warp-uniform
+      const int f =
+          (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)insert_row<32>(a, x, vr.beg, vr.beg + vr.deg, lane, ok));
+      if (lane == 0 && f) atomicAdd(&a.w.cnt[x], f);
+    }
+    for (int64_t i = a.off[0] + tid; i < a.off[1]; i += nt) {
+      const VRec vr = a.rec[i];
+      const int32_t x = a.Cd[vr.v];
+      if (x < 0) continue;
+      const int f = insert_row<1>(a, x, vr.beg, vr.beg + vr.deg, 0, ok);
+      if (f) atomicAdd(&a.w.cnt[x], f);
+    }
+  }
+  if (!ok) a.sc->error = 1;
+  if (!bar.sync()) return;
+  // coarse row offsets, and the sizes of the coarse bins
+  __shared__ int s_bin[kBins], s_max;
+  __shared__ long long s_chunks;
+  if (threadIdx.x < kBins) s_bin[threadIdx.x] = 0;
+  if (threadIdx.x == 0) {
+    s_max = 0;
+    s_chunks = 0;
+  }
+  __syncthreads();
+  long long nnz_c = 0;
+  if (!grid_scan(
+          n_c, a.w.counts, bar, [&](int64_t x) -> long long { return a.w.cnt[x]; },
+          [&](int64_t x, long long at, long long deg) {
+            a.w.rp[x] = at;
+            int b = 0;
+#pragma unroll
+            for (int k = 0; k < kBins - 1; ++k) b += deg > a.max_deg[k] ? 1 : 0;
+            atomicAdd(&s_bin[b], 1);
+            if (b == kHubBin) {
+              atomicMax(&s_max, (int)deg);
+              atomicAdd((unsigned long long *)&s_chunks,
+                        (unsigned long long)((deg + a.hub_chunk - 1) / a.hub_chunk));
+            }
+          },
+          nnz_c))
+    return;
+  __syncthreads();
+  // offs[k + 1] counts bin k here; the host sums
+  if (threadIdx.x < kBins && s_bin[threadIdx.x]) atomicAdd(&a.out->bins.offs[threadIdx.x + 1], s_bin[threadIdx.x]);
+  if (threadIdx.x == 0 && s_max > 0) {
+    atomicMax(&a.out->bins.max_deg, s_max);
+    atomicAdd((unsigned long long *)&a.out->bins.chunks, (unsigned long long)s_chunks);
+  }
+  if (tid == 0) {
+    a.out->nnz_c = nnz_c;
+    a.w.rp[n_c] = nnz_c;
+  }
+  bar.leave();
+}
+
+struct BuildArgs {
+  int64_t n, n_c, slots;
+  const int32_t *gid, *Cd;
+  LevelScratch w;
+  int64_t *rp_c;
+  int32_t *col_c, *ew_c;
+  int64_t *vw_c;
+  int32_t *gid_c;
+  Scalars *sc;
+};
+
+__global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ BuildArgs a) {
+  const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
+  GridBarrier bar(a.sc);
+  for (int64_t x = tid; x <= a.n_c; x += nt) {
+    a.rp_c[x] = a.w.rp[x];
+    if (x < a.n_c) a.vw_c[x] = a.w.vw[x];
+  }
+  if (a.gid_c)
+    for (int64_t v = tid; v < a.n; v += nt) {
+      const int32_t x = a.Cd[v];
+      if (x >= 0) a.gid_c[x] = a.gid[v];
+    }
+  // the occupied slots in order; all slots in use lie below 2 off[n_c]
+  const int64_t slots = 2 * a.w.off[a.n_c];
+  long long nnz = 0;
+  if (!grid_scan(
+          slots, a.w.counts, bar, [&](int64_t s) -> long long { return a.w.tab[s] != kEmptySlot ? 1 : 0; },
+          [&](int64_t s, long long at, long long full) {
+            if (!full) return;
+            const unsigned long long t = a.w.tab[s];
+            a.col_c[at] = slot_key(t);
+            a.ew_c[at] = slot_val(t);
+            a.w.tab[s] = kEmptySlot;
+          },
+          nnz))
+    return;
+  bar.leave();
+}
+
+unsigned level_blocks(int64_t n, int64_t nnz) {
+  // a block per 64 vertices or 1,024 stored edges, at most one per SM
+  int64_t blocks = n / 64 > nnz / 1024 ? n / 64 : nnz / 1024;
+  if (blocks > coop_blocks()) blocks = coop_blocks();
+  return (unsigned)(blocks < 1 ? 1 : blocks);
+}
+
+}  // namespace
+
+void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
+                      const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
+                      Scalars *sc, cudaStream_t s) {
+  cudaMemsetAsync(out, 0, sizeof(LevelOut), s);
+  EndArgs a{};
+  a.g = g;
+  a.gid = gid;
+  a.gp = gp;
+  a.G = G;
+  a.rec = b.recs;
+  for (int k = 0; k < kBins; ++k) a.off[k] = b.list[k] - b.list[0];
+  a.off[kBins] = g.n;
+  for (int k = 0; k < kBins - 1; ++k) a.max_deg[k] = (int32_t)plan.max_deg[k];
+  a.hub_chunk = (int32_t)plan.hub_chunk;
+  a.C = C;
+  a.Cd = Cd;
+  a.w = w;
+  a.out = out;
+  a.sc = sc;
+  void *args[] = {&a};
+  cudaLaunchCooperativeKernel((const void *)k_level_end, dim3(level_blocks(g.n, g.nnz)), dim3(kT), args, 0, s);
+}
+
+void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
+                        const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
+                        int32_t *gid_c, Scalars *sc, cudaStream_t s) {
+  BuildArgs a{};
+  a.n = g.n;
+  a.n_c = out.n_c;
+  a.gid = gid;
+  a.Cd = Cd;
+  a.w = w;
+  a.rp_c = rp_c;
+  a.col_c = col_c;
+  a.ew_c = ew_c;
+  a.vw_c = vw_c;
+  a.gid_c = gid_c;
+  a.sc = sc;
+  void *args[] = {&a};
+  cudaLaunchCooperativeKernel((const void *)k_level_build, dim3(level_blocks(g.n, g.nnz)), dim3(kT), args, 0, s);
+}
+
+}  // namespace lc

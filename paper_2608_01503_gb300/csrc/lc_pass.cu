@@ -1205,6 +1205,13 @@ void launch_iota(int32_t *C, int64_t n, cudaStream_t s) {
   k_iota<<<blocks_for(n, 256), 256, 0, s>>>(C, n);
 }
 
+__global__ void k_fill(long long *a, long long value, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] = value;
+}
+void launch_fill(long long *a, long long value, int n, cudaStream_t s) {
+  if (n > 0) k_fill<<<blocks_for(n, 256), 256, 0, s>>>(a, value, n);
+}
+
 void launch_cluster_weights(const int32_t *C, const int64_t *vw, int64_t *W, int64_t n,
                             cudaStream_t s) {
   cudaMemsetAsync(W, 0, sizeof(int64_t) * (size_t)(n > 0 ? n : 1), s);

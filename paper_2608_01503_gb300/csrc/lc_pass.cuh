@@ -107,6 +107,7 @@ void launch_destinations(const PassArgs &a, int32_t *D, cudaStream_t s);
 int launch_bestof(const PassArgs &a, int32_t *C_out, cudaStream_t s);
 // phi_final[g] = phi_out[g] for every graph active in the call (gp[g].active).
 int launch_keep_phi(const PassArgs &a, long long *phi_final, cudaStream_t s);
+void launch_fill(long long *a, long long value, int n, cudaStream_t s);
 void launch_iota(int32_t *C, int64_t n, cudaStream_t s);
 void launch_cluster_weights(const int32_t *C, const int64_t *vw, int64_t *W, int64_t n,
                             cudaStream_t s);

@@ -44,6 +44,10 @@ __global__ void __launch_bounds__(256) k_stats_vertices(LevelGraph g, int valida
       graph_add(sw2g, gg, w * w);
     }
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->first = g.rp[0];
+    st->last = g.rp[g.n];
+  }
   flush_block_sum(V, &st->V);
   flush_block_sum(sw2, &st->sw2);
 }

@@ -10,6 +10,7 @@ struct GraphStats {
   long long V;    // sum of vertex weights
   long long sw2;  // sum of w(v)^2 (exact when the guards hold)
   unsigned long long fp1, fp2;  // symmetric-edge fingerprints, 0 when symmetric
+  int64_t first, last;          // row_ptr[0], row_ptr[n]
   unsigned long long err_key;   // (code << 40 | vertex), min over violations; ~0 if none
 };
 
