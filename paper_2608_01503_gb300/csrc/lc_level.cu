@@ -120,8 +120,29 @@ __device__ __forceinline__ int insert_row(const EndArgs &a, int32_t x, int64_t b
   return fresh_n;
 }
 
+// The rows of records [lo, hi) by GS lanes each.
+template <int GS>
+__device__ __forceinline__ void insert_group(const EndArgs &a, int64_t lo, int64_t hi, bool &ok) {
+  constexpr int V = 32 / GS;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, sub = lane & (GS - 1);
+  const int64_t nw = (int64_t)gridDim.x * kW;
+  for (int64_t i0 = lo + ((int64_t)wid * gridDim.x + blockIdx.x) * V; i0 < hi; i0 += nw * V) {
+    const int64_t i = i0 + lane / GS;
+    int32_t x = -1;
+    int f = 0;
+    if (i < hi) {
+      const VRec vr = a.rec[i];
+      x = a.Cd[vr.v];
+      if (x >= 0) f = insert_row<GS>(a, x, vr.beg, vr.beg + vr.deg, sub, ok);
+    }
+    __syncwarp();
+    f = group_sum<GS>(f);
+    if (sub == 0 && f) atomicAdd(&a.w.cnt[x], f);
+  }
+}
+
 __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ EndArgs a) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int64_t n = a.g.n;
   const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
   const int64_t wbase = tid - lane;
@@ -192,11 +213,23 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
           [&](int64_t x, long long at, long long) { a.w.off[x] = at; }, slots))
     return;
   if (!bar.sync()) return;
-  // insert: rows of bins 7-9 by a block, bins 1-6 by a warp, bin 0 by a thread
+  // insert: rows of bin 9 by all blocks, 7-8 by a block, 3-6 by a warp, 1-2 by eight lanes, bin 0 by a thread
   bool ok = true;
   {
     __shared__ int s_fresh;
-    for (int64_t i = a.off[7] + blockIdx.x; i < a.off[kBins]; i += gridDim.x) {
+    // hub rows by all blocks, a piece each
+    for (int64_t i = a.off[kHubBin]; i < a.off[kBins]; ++i) {
+      const VRec vr = a.rec[i];
+      const int32_t x = a.Cd[vr.v];
+      if (x < 0) continue;
+      const int64_t end = vr.beg + vr.deg;
+      int f = 0;
+      for (int64_t e = vr.beg + (int64_t)blockIdx.x * 4 * kT; e < end; e += (int64_t)gridDim.x * 4 * kT)
+        f += insert_row<kT>(a, x, e, e + 4 * kT < end ? e + 4 * kT : end, threadIdx.x, ok);
+      f = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)f);
+      if (lane == 0 && f) atomicAdd(&a.w.cnt[x], f);
+    }
+    for (int64_t i = a.off[7] + blockIdx.x; i < a.off[kHubBin]; i += gridDim.x) {
       const VRec vr = a.rec[i];
       const int32_t x = a.Cd[vr.v];
       if (x < 0) continue;  // block-uniform
@@ -209,15 +242,10 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
       __syncthreads();
       if (threadIdx.x == 0 && s_fresh) atomicAdd(&a.w.cnt[x], s_fresh);
     }
-    const int64_t nw = (int64_t)gridDim.x * kW;
-    for (int64_t i = a.off[1] + (int64_t)wid * gridDim.x + blockIdx.x; i < a.off[7]; i += nw) {
-      const VRec vr = a.rec[i];
-      const int32_t x = a.Cd[vr.v];
-      if (x < 0) continue;  // warp-uniform
-      const int f =
-          (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)insert_row<32>(a, x, vr.beg, vr.beg + vr.deg, lane, ok));
-      if (lane == 0 && f) atomicAdd(&a.w.cnt[x], f);
-    }
+    // short rows by eight lanes, four edges each in flight: the walk is bound
+    // by the latency of its gathers and probes
+    insert_group<32>(a, a.off[3], a.off[7], ok);
+    insert_group<8>(a, a.off[1], a.off[3], ok);
     for (int64_t i = a.off[0] + tid; i < a.off[1]; i += nt) {
       const VRec vr = a.rec[i];
       const int32_t x = a.Cd[vr.v];
