@@ -1,0 +1,30 @@
+"""pLeidenR's order of the trees: small forests are ranked by counting, a
+forest with a very large tree is radix-sorted; both against the oracle."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import paper_2608_01503_gb300 as lc  # noqa: E402
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# a star's tree holds about half of its leaves: 20,000 leaves stay below 2^30
+# pairs, 120,000 do not
+@pytest.mark.parametrize("leaves", [1, 31, 2_000, 20_000, 120_000])
+def test_star(leaves):
+    rp, col, ew = gg.from_edges(leaves + 1, np.zeros(leaves, np.int64), np.arange(1, leaves + 1))
+    g = gg.cpm_inputs(rp, col, ew, 1, 4 * leaves + 4)
+    labels, res = lc.lc_cluster_leiden(dev(rp), dev(col), dev(ew), dev(g.vw), g.lam_num, g.lam_den)
+    ref, orc, _ = oracle.pleiden(g)
+    assert np.array_equal(labels.cpu().numpy(), ref) and res["phi"] == orc["phi"]
