@@ -181,6 +181,7 @@ struct Run {
   Method m;
   lc_result *res;  // [G]
   int G = 1;
+  int coop_blocks = kCoopBlocks;  // blocks of a cooperative launch (a server slot's share)
   std::vector<long long> mu, Lam;
   std::vector<int> top;  // [G] last level of each graph
   Arena ar;
@@ -370,7 +371,7 @@ static int bins_for(Run &r, Level &L) {
   BinOut *d_out = nullptr;
   LC_TRY(r.ar.get(&d_out, 1));
   LC_TRY(r.ar.get(&L.bins.recs, L.g.n));
-  launch_bins(L.g, L.gid, r.plan, L.bins, d_out, r.coop, r.sc, r.s);
+  launch_bins(L.g, L.gid, r.plan, L.bins, d_out, r.coop, r.sc, r.coop_blocks, r.s);
   BinOut out = L.bin_out;
   if (!L.bins_known) {
     LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
@@ -449,6 +450,7 @@ static PassArgs pass_args(Run &r, const Level &L) {
   a.dirty_list = r.dirty_list;
   a.obj = r.obj;
   a.hub_min = r.plan.hub_min();
+  a.coop = r.coop_blocks;
   for (int g = 0; g < kAbGroups; ++g) a.ab_gs[g] = r.plan.ab_gs[g];
   return a;
 }
@@ -852,7 +854,7 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   Phase range("lc.contract");
   LC_TRY(r.ar.get(&L.Cd, L.g.n));
   const LevelScratch w{r.used, r.newid, r.cnt, r.bound, r.off, r.W, r.delta, r.gtab, r.gfree, r.lcounts};
-  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.sc, r.s);
+  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.sc, r.coop_blocks, r.s);
   LevelOut out{};
   std::vector<int32_t> nc(r.G);
   LC_CK(cudaMemcpyAsync(&out, r.lout, sizeof(out), cudaMemcpyDeviceToHost, r.s));
@@ -885,7 +887,7 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   if (r.G > 1) LC_TRY(r.ar.get(&N.gid, out.n_c));
   LC_TRY(r.ar.get(&col_c, out.nnz_c));
   LC_TRY(r.ar.get(&ew_c, out.nnz_c));
-  launch_level_build(L.g, L.gid, L.Cd, w, out, rp_c, col_c, ew_c, vw_c, N.gid, r.sc, r.s);
+  launch_level_build(L.g, L.gid, L.Cd, w, out, rp_c, col_c, ew_c, vw_c, N.gid, r.sc, r.coop_blocks, r.s);
   r.res->kernel_launches[LC_K_CONTRACT] += 1;
   r.res->edges_contract += L.g.nnz;
   N.g = LevelGraph{out.n_c, out.nnz_c, rp_c, col_c, ew_c, vw_c};
@@ -1598,12 +1600,17 @@ int lc_cluster_iterated(const lc_csr *g, const int64_t *vertex_w, const int32_t 
   return rc;
 }
 
-int lc_cluster_batch(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w, int32_t count,
+}  // extern "C"
+
+namespace lc {
+// lc_cluster_batch whose cooperative launches take at most coop_blocks blocks.
+int cluster_batch_within(int coop_blocks, const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w, int32_t count,
                      const int64_t *graph_ptr, const int64_t *lambda_num, const int64_t *lambda_den,
                      const lc_opts *opts, int32_t *labels_out, lc_result *res) {
   if (!res || count < 1 || !graph_ptr || !lambda_num || !lambda_den) return LC_ERR_ARG;
   lc_opts o = resolve_opts(opts);
   Run r(o);
+  r.coop_blocks = coop_blocks;
   int rc = begin_call(r, opts, res, count);
   if (rc == LC_OK) rc = check_graph_args(g, vertex_w, edge_w);
   std::vector<int64_t> gptr(graph_ptr, graph_ptr + count + 1);
@@ -1624,6 +1631,16 @@ int lc_cluster_batch(const lc_csr *g, const int64_t *vertex_w, const int32_t *ed
   }
   end_call(r, rc);
   return rc;
+}
+}  // namespace lc
+
+extern "C" {
+
+int lc_cluster_batch(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w, int32_t count,
+                     const int64_t *graph_ptr, const int64_t *lambda_num, const int64_t *lambda_den,
+                     const lc_opts *opts, int32_t *labels_out, lc_result *res) {
+  return cluster_batch_within(kCoopBlocks, g, vertex_w, edge_w, count, graph_ptr, lambda_num, lambda_den, opts,
+                              labels_out, res);
 }
 
 int lc_cluster_host(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w,

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kT, 1)
 }  // namespace
 
 void launch_bins(const LevelGraph &g, const int32_t *gid, const BinPlan &plan, const Bins &b, BinOut *out,
-                 int32_t *counts, Scalars *sc, cudaStream_t s) {
+                 int32_t *counts, Scalars *sc, int coop, cudaStream_t s) {
   cudaMemsetAsync(out, 0, sizeof(BinOut), s);
   if (g.n <= 0) return;
   BinArgs a{};
@@ -220,7 +220,7 @@ void launch_bins(const LevelGraph &g, const int32_t *gid, const BinPlan &plan, c
   a.counts = counts;
   a.sc = sc;
   int64_t blocks = (g.n + kT - 1) / kT;
-  if (blocks > coop_blocks()) blocks = coop_blocks();
+  if (blocks > coop_blocks(coop)) blocks = coop_blocks(coop);
   void *args[] = {&a};
   cudaLaunchCooperativeKernel((const void *)k_bins, dim3((unsigned)blocks), dim3(kT), args, 0, s);
 }

@@ -58,13 +58,15 @@ struct GridBarrier {
   }
 };
 
-// Blocks a cooperative launch of one block per SM may have on this device.
-inline int coop_blocks() {
+// Blocks a cooperative launch of one block per SM may have on this device, of
+// at most `limit` (a call's share of the SMs while others run beside it).
+inline int coop_blocks(int limit) {
   int dev = 0, sms = 1;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 1;
-  return sms < kCoopBlocks ? sms : kCoopBlocks;
+  if (sms > kCoopBlocks) sms = kCoopBlocks;
+  return limit < 1 ? 1 : limit < sms ? limit : sms;
 }
 
 }  // namespace lc

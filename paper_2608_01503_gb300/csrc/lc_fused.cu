@@ -602,7 +602,7 @@ int64_t fused_row_max() { return kRowMaxDeg; }
 int launch_fused_passes(const PassArgs &a, const FusedArgs &f, cudaStream_t s) {
   // a block per 64 vertices or 1,024 stored edges, at most one per SM
   int64_t blocks = a.g.n / 64 > a.g.nnz / 1024 ? a.g.n / 64 : a.g.nnz / 1024;
-  if (blocks > coop_blocks()) blocks = coop_blocks();
+  if (blocks > coop_blocks(a.coop)) blocks = coop_blocks(a.coop);
   if (blocks < 1) blocks = 1;
   PassArgs pa = a;
   FusedArgs fa = f;

@@ -336,10 +336,10 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
   bar.leave();
 }
 
-unsigned level_blocks(int64_t n, int64_t nnz) {
+unsigned level_blocks(int64_t n, int64_t nnz, int coop) {
   // a block per 64 vertices or 1,024 stored edges, at most one per SM
   int64_t blocks = n / 64 > nnz / 1024 ? n / 64 : nnz / 1024;
-  if (blocks > coop_blocks()) blocks = coop_blocks();
+  if (blocks > coop_blocks(coop)) blocks = coop_blocks(coop);
   return (unsigned)(blocks < 1 ? 1 : blocks);
 }
 
@@ -347,7 +347,7 @@ unsigned level_blocks(int64_t n, int64_t nnz) {
 
 void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
                       const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
-                      Scalars *sc, cudaStream_t s) {
+                      Scalars *sc, int coop, cudaStream_t s) {
   cudaMemsetAsync(out, 0, sizeof(LevelOut), s);
   EndArgs a{};
   a.g = g;
@@ -365,12 +365,12 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
   a.out = out;
   a.sc = sc;
   void *args[] = {&a};
-  cudaLaunchCooperativeKernel((const void *)k_level_end, dim3(level_blocks(g.n, g.nnz)), dim3(kT), args, 0, s);
+  cudaLaunchCooperativeKernel((const void *)k_level_end, dim3(level_blocks(g.n, g.nnz, coop)), dim3(kT), args, 0, s);
 }
 
 void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
                         const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
-                        int32_t *gid_c, Scalars *sc, cudaStream_t s) {
+                        int32_t *gid_c, Scalars *sc, int coop, cudaStream_t s) {
   BuildArgs a{};
   a.n = g.n;
   a.n_c = out.n_c;
@@ -384,7 +384,7 @@ void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *
   a.gid_c = gid_c;
   a.sc = sc;
   void *args[] = {&a};
-  cudaLaunchCooperativeKernel((const void *)k_level_build, dim3(level_blocks(g.n, g.nnz)), dim3(kT), args, 0, s);
+  cudaLaunchCooperativeKernel((const void *)k_level_build, dim3(level_blocks(g.n, g.nnz, coop)), dim3(kT), args, 0, s);
 }
 
 }  // namespace lc

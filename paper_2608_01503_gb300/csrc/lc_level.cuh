@@ -29,11 +29,11 @@ constexpr int64_t kLevelCounts = 152 * 16 + 16;
 // out->n_c = 0 when that is every graph.
 void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
                       const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
-                      Scalars *sc, cudaStream_t s);
+                      Scalars *sc, int coop, cudaStream_t s);
 // The coarse graph from the scratch into its own arrays (out as read back),
 // its graph ids (null for one graph); leaves the hash slots clean.
 void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
                         const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
-                        int32_t *gid_c, Scalars *sc, cudaStream_t s);
+                        int32_t *gid_c, Scalars *sc, int coop, cudaStream_t s);
 
 }  // namespace lc

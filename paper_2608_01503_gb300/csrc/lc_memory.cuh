@@ -75,4 +75,10 @@ struct Arena {
 // whose levels shrink more slowly can need more.
 int64_t cluster_footprint(int64_t n, int64_t nnz, int count, const lc_opts &o);
 
+// lc_cluster_batch whose cooperative launches take at most coop_blocks blocks
+// (one per SM), so that calls on other streams run beside them.
+int cluster_batch_within(int coop_blocks, const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w,
+                         int32_t count, const int64_t *graph_ptr, const int64_t *lambda_num,
+                         const int64_t *lambda_den, const lc_opts *opts, int32_t *labels_out, lc_result *res);
+
 }  // namespace lc

@@ -1170,7 +1170,7 @@ int launch_final_objective(const PassArgs &a, cudaStream_t s) {
 int launch_assign_empty(const PassArgs &a, const EmptyScratch &w, cudaStream_t s) {
   if (a.g.n <= 0) return 0;
   int64_t blocks = (a.g.n + 4 * kCoopThreads - 1) / (4 * kCoopThreads);
-  if (blocks > coop_blocks()) blocks = coop_blocks();
+  if (blocks > coop_blocks(a.coop)) blocks = coop_blocks(a.coop);
   PassArgs pa = a;
   EmptyScratch es = w;
   void *args[] = {&pa, &es};

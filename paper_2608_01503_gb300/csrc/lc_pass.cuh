@@ -37,6 +37,7 @@ struct PassArgs {
   long long *obj;            // [4 G] per graph: Phi entering the last pass, Q entering it,
                              // Q after it, change of IN by its moves (objective update)
   int64_t hub_min;           // rows longer than this are hubs (BinPlan::hub_min)
+  int32_t coop;               // blocks a cooperative launch may have
   int32_t ab_gs[kAbGroups];   // threads per candidate in group g (BinPlan)
 };
 

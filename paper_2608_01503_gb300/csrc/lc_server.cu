@@ -18,6 +18,7 @@
 // its jobs then go back to the head of the queue with twice the estimate
 // and wait for memory (a job larger than the whole budget runs alone, with
 // no limit), so callers only see LC_ERR_OOM when the device itself is out.
+#include <algorithm>
 #include <cuda_runtime.h>
 
 #include <chrono>
@@ -30,6 +31,7 @@
 #include <vector>
 
 #include "../../include/lc.h"
+#include "lc_coop.cuh"
 #include "lc_memory.cuh"
 
 namespace {
@@ -58,6 +60,7 @@ struct lc_server {
   int device = 0;
   int64_t budget = 0, claimed = 0;
   int64_t next_id = 1;
+  int busy = 0;  // admissions running
   bool stop = false;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
@@ -91,8 +94,9 @@ void add_offset(T *a, int64_t count, T add, cudaStream_t st) {
 // Packs jobs into one CSR on the device (each job copied to its offset,
 // then shifted to global ids) and clusters them in one batched call.
 // labels (host, the packed vertex range) and res[k] are filled on success.
-// scratch_limit: the clustering's scratch limit (0: none).
-int cluster_packed(lc_server *s, cudaStream_t st, Job *const *jobs, int count, int64_t scratch_limit,
+// scratch_limit: the clustering's scratch limit (0: none).  coop_blocks: its
+// cooperative launches' share of the SMs.
+int cluster_packed(lc_server *s, cudaStream_t st, Job *const *jobs, int count, int64_t scratch_limit, int coop_blocks,
                    std::vector<int32_t> &labels, std::vector<int64_t> &gptr, lc_result *res) {
   std::vector<int64_t> eptr(count + 1, 0), lam_num(count), lam_den(count);
   gptr.assign(count + 1, 0);
@@ -135,8 +139,8 @@ int cluster_packed(lc_server *s, cudaStream_t st, Job *const *jobs, int count, i
     lc_csr g{n, nnz, d_rp, d_col};
     if (cudaGetLastError() != cudaSuccess) rc = LC_ERR_CUDA;
     if (rc == LC_OK)
-      rc = lc_cluster_batch(&g, d_vw, d_ew, count, gptr.data(), lam_num.data(), lam_den.data(), &o,
-                            d_lab, res);
+      rc = lc::cluster_batch_within(coop_blocks, &g, d_vw, d_ew, count, gptr.data(), lam_num.data(),
+                                    lam_den.data(), &o, d_lab, res);
     if (rc == LC_OK && n > 0) {
       if (cudaMemcpyAsync(labels.data(), d_lab, 4 * n, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         rc = LC_ERR_CUDA;
@@ -151,7 +155,7 @@ int cluster_packed(lc_server *s, cudaStream_t st, Job *const *jobs, int count, i
 // offending ones report an error.
 // limited: the admission fits the budget, so its scratch is limited to
 // what it reserved.
-void run_batch(lc_server *s, cudaStream_t st, std::vector<Job *> &batch, bool limited) {
+void run_batch(lc_server *s, cudaStream_t st, std::vector<Job *> &batch, bool limited, int coop_blocks) {
   const int count = (int)batch.size();
   std::vector<int32_t> labels;
   std::vector<int64_t> gptr;
@@ -160,7 +164,8 @@ void run_batch(lc_server *s, cudaStream_t st, std::vector<Job *> &batch, bool li
   std::vector<std::vector<int32_t>> own(count);
   int64_t reserved = 0;
   for (Job *j : batch) reserved += j->scratch;
-  const int rc = cluster_packed(s, st, batch.data(), count, limited ? reserved : 0, labels, gptr, res.data());
+  const int rc = cluster_packed(s, st, batch.data(), count, limited ? reserved : 0, coop_blocks, labels, gptr,
+                                res.data());
   if (rc == LC_ERR_OOM && limited) {
     // the estimate was short: back to the head of the queue, in order, with
     // twice the reservation, to wait for memory
@@ -182,7 +187,8 @@ void run_batch(lc_server *s, cudaStream_t st, std::vector<Job *> &batch, bool li
     rcs[0] = rc;
   } else {
     for (int k = 0; k < count; ++k) {
-      rcs[k] = cluster_packed(s, st, &batch[k], 1, limited ? batch[k]->scratch : 0, labels, gptr, &res[k]);
+      rcs[k] = cluster_packed(s, st, &batch[k], 1, limited ? batch[k]->scratch : 0, coop_blocks, labels, gptr,
+                              &res[k]);
       if (rcs[k] == LC_OK) own[k].assign(labels.begin(), labels.begin() + batch[k]->n);
     }
   }
@@ -213,6 +219,7 @@ void worker(lc_server *s) {
   for (;;) {
     std::vector<Job *> batch;
     bool limited = true;
+    int coop_blocks = lc::kCoopBlocks;
     {
       std::unique_lock<std::mutex> lock(s->mu);
       for (;;) {
@@ -240,6 +247,12 @@ void worker(lc_server *s) {
               batch[k]->state = 1;
             }
             s->claimed += add;
+            // A small level's cooperative kernel keeps every SM it gets to
+            // itself and leaves most of it idle, waiting; slots that run at
+            // the same time split the SMs instead of taking turns.
+            s->busy++;
+            const int beside = std::min<int64_t>(s->cfg.slots, s->busy + (int64_t)s->queue.size());
+            coop_blocks = lc::kCoopBlocks / beside;
             break;
           }
         }
@@ -247,7 +260,9 @@ void worker(lc_server *s) {
       }
     }
     if (batch.empty()) break;
-    run_batch(s, st, batch, limited);
+    run_batch(s, st, batch, limited, coop_blocks);
+    std::lock_guard<std::mutex> lock(s->mu);
+    s->busy--;
   }
   cudaStreamDestroy(st);
 }
