@@ -11,6 +11,7 @@
 // All sums are integer (commutative atomics and shuffles), argmax ties go to
 // the smallest cluster id and the afterburner order is a total order, so the
 // results do not depend on scheduling.
+#include <algorithm>
 #include <climits>
 
 #include "lc_coop.cuh"
@@ -343,15 +344,14 @@ __global__ void __launch_bounds__(256, 4) k_ab_warp(PassArgs a, const VRec *__re
   flush_update(a, sum);
 }
 
-// A block per candidate, a chunk of vertices per block.  The per-warp sums
-// alternate between two buffers, so one barrier per candidate suffices (the
-// next candidate's barrier orders thread 0's reads before the buffer is
-// written again).
+// A block per candidate, a chunk of vertices per block.  Every warp walks its
+// part of all the chunk's candidates and leaves its sums, so the warps meet
+// twice a chunk and not once a candidate (half of their time, before).
 template <int GS>
 __global__ void __launch_bounds__(GS, 2048 / GS / 2) k_ab_block(PassArgs a, const VRec *__restrict__ rec,
                                                                 int64_t count, int chunk) {
   __shared__ AbStage st;
-  __shared__ long long rs[2][GS / 32];
+  __shared__ long long rs[32][GS / 32];
   __shared__ int s_nc;
   UpdateSums sum;
   const BlockChunk b = block_chunk_of(count, chunk);
@@ -365,23 +365,17 @@ __global__ void __launch_bounds__(GS, 2048 / GS / 2) k_ab_block(PassArgs a, cons
   }
   __syncthreads();
   const int nc = s_nc;
-  int par = 0;
   for (int k = 0; k < nc; ++k) {
     const AbCtx c = st.ctx[k];
     const long long acc = warp_sum(ab_edges<GS, 4>(a, c, c.beg, c.beg + c.deg, threadIdx.x));
-    if ((threadIdx.x & 31) == 0) rs[par][threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      long long t = 0;
-      for (int w = 0; w < GS / 32; ++w) t += rs[par][w];
-      st.sum[k] = t;
-    }
-    par ^= 1;
+    if ((threadIdx.x & 31) == 0) rs[k][threadIdx.x >> 5] = acc;
   }
   __syncthreads();
   if (threadIdx.x < 32) {
-    const bool keep = r.D != kNone && delta + st.sum[r.D != kNone ? pos : 0] >= 0;
-    apply_lanes(a, (int)threadIdx.x < b.m, vr.v, vr.deg, r, vr.w, keep, sum);
+    long long t = delta;
+    if (r.D != kNone)
+      for (int w = 0; w < GS / 32; ++w) t += rs[pos][w];
+    apply_lanes(a, (int)threadIdx.x < b.m, vr.v, vr.deg, r, vr.w, r.D != kNone && t >= 0, sum);
   }
   flush_update(a, sum);
 }
@@ -834,9 +828,11 @@ static inline int block_chunk_size(int64_t count) {
 }
 
 using ChunkKernel = void (*)(PassArgs, const VRec *, int64_t, int);
-static int launch_warp_chunks(ChunkKernel k, const PassArgs &a, BinRange r, cudaStream_t s) {
+// most: vertices per warp at most (fewer where rows are long: blocks that
+// end sooner even the SMs out)
+static int launch_warp_chunks(ChunkKernel k, const PassArgs &a, BinRange r, cudaStream_t s, int most = 32) {
   if (r.count <= 0) return 0;
-  const int chunk = warp_chunk_size(r.count);
+  const int chunk = std::min(warp_chunk_size(r.count), most);
   k<<<warp_chunk_blocks(r.count, chunk), 256, 0, s>>>(a, r.rec, r.count, chunk);
   return 1;
 }
@@ -895,7 +891,7 @@ static int launch_move_low(const PassArgs &a, const Bins &b, cudaStream_t s) {
   int n = launch_threads(k_move_thread, a, bin_range(b, 0, 0), s);
   n += launch_warp_chunks(k_move_lanes<16>, a, bin_range(b, 1, 1), s);
   n += launch_warp_chunks(k_move_lanes<32>, a, bin_range(b, 2, 2), s);
-  n += launch_warp_chunks(k_move_warp, a, bin_range(b, 3, 4), s);
+  n += launch_warp_chunks(k_move_warp, a, bin_range(b, 3, 4), s, 16);
   return n;
 }
 
@@ -943,8 +939,8 @@ int launch_table_pass(const PassArgs &a, const Bins &b, cudaStream_t s) {
 // edges) always takes 8 lanes per candidate.
 static int launch_ab_group(const PassArgs &a, const Bins &b, int g, cudaStream_t s) {
   const BinRange r = bin_range(b, g == 2 ? 3 : kAbFirstBin[g], kAbFirstBin[g + 1] - 1);
-  if (a.ab_gs[g] == 16) return launch_warp_chunks(k_ab_warp<16>, a, r, s);
-  if (a.ab_gs[g] == 32) return launch_warp_chunks(k_ab_warp<32>, a, r, s);
+  if (a.ab_gs[g] == 16) return launch_warp_chunks(k_ab_warp<16>, a, r, s, 16);
+  if (a.ab_gs[g] == 32) return launch_warp_chunks(k_ab_warp<32>, a, r, s, 16);
   if (a.ab_gs[g] == 128) return launch_block_chunks(k_ab_block<128>, 128, 0, a, r, s);
   return launch_block_chunks(k_ab_block<512>, 512, 0, a, r, s);
 }
