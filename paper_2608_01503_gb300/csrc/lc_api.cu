@@ -981,15 +981,25 @@ static int check_graph_args(const lc_csr *g, const int64_t *vw, const int32_t *e
   return LC_OK;
 }
 
-// Statistics, validation and the exactness guards of the header, per graph.
-static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *hst) {
+// Statistics, validation and the exactness guards of the header, per graph; C:
+// null, or the clustering whose objective is wanted (lc_objective), which the
+// same pass over the edges sums.
+static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *hst, const int32_t *C = nullptr) {
   LC_TRY(r.ar.get(&r.st, 1));
   LC_CK(cudaMemsetAsync(r.st, 0, sizeof(GraphStats), r.s));
   LC_CK(cudaMemsetAsync(&r.st->err_key, 0xFF, sizeof(r.st->err_key), r.s));
   r.prof.begin(LC_K_OTHER);
-  launch_stats(g, r.o.validate, r.st, gid, r.gptr, r.Tg, r.Vg, r.sw2g, r.s);
-  r.prof.end(16.0 * g.n + 8.0 * g.nnz);
+  launch_stats(g, r.o.validate, r.st, gid, r.gptr, r.Tg, r.Vg, r.sw2g, C, r.s);
+  r.prof.end(16.0 * g.n + (C ? 12.0 : 8.0) * g.nnz);
   r.res->kernel_launches[LC_K_OTHER] += g.nnz > 0 ? 2 : 1;
+  if (C) {
+    LC_TRY(r.ar.get(&r.W, g.n));
+    LC_TRY(r.ar.get(&r.used, g.n));
+    r.prof.begin(LC_K_OBJECTIVE);
+    launch_label_stats(g, C, r.W, r.used, r.st, r.s);
+    r.prof.end(44.0 * g.n);
+    r.res->kernel_launches[LC_K_OBJECTIVE] += 2;
+  }
   LC_CK(cudaMemcpyAsync(hst, r.st, sizeof(GraphStats), cudaMemcpyDeviceToHost, r.s));
   r.hT.assign(r.G, 0);
   r.hV.assign(r.G, 0);
@@ -1253,14 +1263,14 @@ static void end_call(Run &r, int rc) {
 
 // Single-graph set-up shared by the step-level entry points.
 static int single_graph(Run &r, const lc_csr *g, const int64_t *vw, const int32_t *ew, int64_t mu,
-                        int64_t Lam, Level &L, GraphStats *st) {
+                        int64_t Lam, Level &L, GraphStats *st, const int32_t *C = nullptr) {
   r.mu.assign(1, mu);
   r.Lam.assign(1, Lam);
   LC_TRY(alloc_per_graph(r));
   LevelGraph g0{g->n, g->nnz, g->row_ptr, g->col, ew, vw};
   std::vector<int64_t> gptr{0, g->n};
   LC_TRY(level0(r, L, g0, gptr));
-  return prepare(r, g0, nullptr, st);
+  return prepare(r, g0, nullptr, st, C);
 }
 
 static int labels_in_range(Run &r, const int32_t *labels, int64_t n, int64_t limit) {
@@ -1784,20 +1794,13 @@ int lc_objective(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w
   if (rc == LC_OK && g->n > 0) {
     Level L;
     GraphStats st{};
-    rc = single_graph(r, g, vertex_w, edge_w, lambda_num, lambda_den, L, &st);
-    if (rc == LC_OK) rc = labels_in_range(r, labels, g->n, g->n);
-    if (rc == LC_OK) rc = alloc_scratch(r, g->n, 0);
-    if (rc == LC_OK) rc = bins_for(r, L);
-    if (rc == LC_OK) rc = upload_params(r, L, std::vector<uint8_t>{1});
-    std::vector<long long> phi;
-    if (rc == LC_OK) rc = objective_of(r, L, labels, phi);
-    std::vector<int64_t> nc;
-    int64_t total = 0;
-    if (rc == LC_OK) rc = count_labels(r, L, labels, nc, &total);
+    rc = single_graph(r, g, vertex_w, edge_w, lambda_num, lambda_den, L, &st, labels);
+    if (rc == LC_OK && st.bad_labels) rc = LC_ERR_ARG;
     if (rc == LC_OK) {
-      res->n_clusters = total;
+      res->n_clusters = st.clusters;
       res->levels = 1;
-      finish_result(r, 0, res, phi[0]);
+      // Phi = Lam IN - mu Q (Eq. 1 regrouped by cluster)
+      finish_result(r, 0, res, lambda_den * st.inside - (lambda_num ? lambda_num * st.q : 0));
     }
   } else if (rc == LC_OK) {
     res->lambda_den = lambda_den;

@@ -5,6 +5,7 @@
 // entries, so a single long row does not serialise them.
 #include "lc_group.cuh"
 #include "lc_internal.cuh"
+#include "lc_move.cuh"
 #include "lc_validate.cuh"
 
 namespace lc {
@@ -137,10 +138,13 @@ __device__ __noinline__ void report_entry(GraphStats *st, int32_t v, int32_t x, 
   if (w <= 0) report(st, LC_ERR_WEIGHT, v);
 }
 
-template <bool VALIDATE>
+// INSIDE: also the weight inside the clusters of C (labels are compared, never
+// followed).
+template <bool VALIDATE, bool INSIDE>
 __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, GraphStats *st,
                                                                const int32_t *__restrict__ gid,
-                                                               const int64_t *__restrict__ gptr, long long *Tg) {
+                                                               const int64_t *__restrict__ gptr, long long *Tg,
+                                                               const int32_t *__restrict__ C) {
   constexpr unsigned full = 0xFFFFFFFFu;
   __shared__ int4 s_mark[kStatsThreads / 32][kStatsStep / 4];
   const int lane = threadIdx.x & 31;
@@ -149,7 +153,7 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
   const bool vec = ((reinterpret_cast<uintptr_t>(g.col) | reinterpret_cast<uintptr_t>(g.ew)) & 15) == 0;
   const int64_t runs = (g.nnz + kStatsRun - 1) / kStatsRun;
   const int64_t nwarps = (int64_t)gridDim.x * (kStatsThreads / 32);
-  long long T = 0;
+  long long T = 0, inside = 0;
   unsigned long long f1 = 0, f2 = 0;
   unsigned minus = 0;  // edges subtracted: -h = ~h + 1, the ones added at the end
   mark4[lane] = make_int4(0, 0, 0, 0);
@@ -159,7 +163,7 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
     Four u = load_four(g.col, e0 + 4 * lane, e1, vec), w = load_four(g.ew, e0 + 4 * lane, e1, vec);
     int64_t r0 = 0;          // row of the entry before the step (of the run's first entry at its start)
     int32_t carry = -1;      // the column before the step
-    if (VALIDATE || gid) {
+    if (VALIDATE || INSIDE || gid) {
       r0 = warp_find_row(g.rp, g.n, e0, lane);
       if (lane == 0 && __ldg(g.rp + r0) == e0) mark[0] = (int32_t)r0 + 1;
       if (e0 > 0) carry = __ldg(g.col + e0 - 1);
@@ -172,7 +176,7 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
       const int left = e1 - base < kStatsStep ? (int)(e1 - base) : kStatsStep;
 #pragma unroll
       for (int k = 0; k < 4; ++k) T += w.x[k];  // 0 past the end
-      if (!VALIDATE && !gid) {
+      if (!VALIDATE && !INSIDE && !gid) {
         u = un;
         w = wn;
         continue;
@@ -217,6 +221,15 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
       const bool first[4] = {m.x != 0, m.y != 0, m.z != 0, m.w != 0};
       const int32_t up = __shfl_up_sync(full, u.x[3], 1);
       const int32_t before[4] = {lane > 0 ? up : carry, u.x[0], u.x[1], u.x[2]};
+      if (INSIDE) {
+        int32_t cu[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          cu[k] = 4 * lane + k < left && (uint32_t)u.x[k] < (uint32_t)g.n ? C[u.x[k]] : -1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (cu[k] >= 0 && cu[k] == C[row[k]]) inside += w.x[k];
+      }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const bool on = 4 * lane + k < left;
@@ -259,10 +272,49 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
     if (gid && cur_g >= 0) graph_add(Tg, cur_g, tg);
   }
   flush_block_sum(T, &st->T);
+  if (INSIDE) flush_block_sum(inside, &st->inside);
   if (VALIDATE) {
     flush_block_sum((long long)(f1 + minus), (long long *)&st->fp1);
     flush_block_sum((long long)(f2 + minus), (long long *)&st->fp2);
   }
+}
+
+// Cluster weights and ids in use of the labels C, which are checked against
+// [0, n) before they are followed.
+__global__ void __launch_bounds__(256) k_label_sums(LevelGraph g, const int32_t *__restrict__ C, int64_t *W,
+                                                    int32_t *__restrict__ used, GraphStats *st) {
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < g.n; base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = base + threadIdx.x;
+    const int32_t x = v < g.n ? C[v] : 0;
+    const bool ok = v < g.n && x >= 0 && x < g.n;
+    if (v < g.n && !ok) atomicAdd(&st->bad_labels, 1ull);
+    if (ok) used[x] = 1;
+    add_weights(W, ok, ok ? x : 0, ok ? g.vw[v] : 0);
+  }
+}
+// Q = sum_x W(x)^2 - w(x)^2 (unsigned arithmetic: exact whenever it fits) and
+// the number of ids in use.
+__global__ void __launch_bounds__(256) k_label_squares(LevelGraph g, const int64_t *__restrict__ W,
+                                                       const int32_t *__restrict__ used, GraphStats *st) {
+  long long q = 0, k = 0;
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < g.n; x += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long a = (unsigned long long)W[x], b = (unsigned long long)g.vw[x];
+    q += (long long)(a * a - b * b);
+    k += used[x] != 0;
+  }
+  flush_block_sum(q, &st->q);
+  flush_block_sum(k, &st->clusters);
+}
+
+void launch_label_stats(const LevelGraph &g, const int32_t *C, int64_t *W, int32_t *used, GraphStats *st,
+                        cudaStream_t s) {
+  if (g.n <= 0) return;
+  int64_t b = (g.n + 255) / 256;
+  if (b > 152 * 8) b = 152 * 8;
+  cudaMemsetAsync(W, 0, sizeof(int64_t) * (size_t)g.n, s);
+  cudaMemsetAsync(used, 0, sizeof(int32_t) * (size_t)g.n, s);
+  k_label_sums<<<(unsigned)b, 256, 0, s>>>(g, C, W, used, st);
+  k_label_squares<<<(unsigned)b, 256, 0, s>>>(g, W, used, st);
 }
 
 __global__ void k_labels_in_range(const int32_t *__restrict__ C, int64_t n, int64_t limit,
@@ -273,7 +325,7 @@ __global__ void k_labels_in_range(const int32_t *__restrict__ C, int64_t n, int6
 }
 
 void launch_stats(const LevelGraph &g, int validate, GraphStats *st, const int32_t *gid, const int64_t *gptr,
-                  long long *Tg, long long *Vg, long long *sw2g, cudaStream_t s) {
+                  long long *Tg, long long *Vg, long long *sw2g, const int32_t *C, cudaStream_t s) {
   auto blocks = [](int64_t items) {
     int64_t b = (items + 255) / 256;
     if (b < 1) b = 1;
@@ -287,10 +339,9 @@ void launch_stats(const LevelGraph &g, int validate, GraphStats *st, const int32
     // would leave as a last, half-empty turn
     int64_t b = (runs + kStatsThreads / 32 - 1) / (kStatsThreads / 32);
     if (b > INT32_MAX) b = INT32_MAX;
-    if (validate)
-      k_stats_edges<true><<<(unsigned)b, kStatsThreads, 0, s>>>(g, st, gid, gptr, Tg);
-    else
-      k_stats_edges<false><<<(unsigned)b, kStatsThreads, 0, s>>>(g, st, gid, gptr, Tg);
+    auto *k = C ? (validate ? k_stats_edges<true, true> : k_stats_edges<false, true>)
+                : (validate ? k_stats_edges<true, false> : k_stats_edges<false, false>);
+    k<<<(unsigned)b, kStatsThreads, 0, s>>>(g, st, gid, gptr, Tg, C);
   }
 }
 
