@@ -351,7 +351,7 @@ static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tab
 }
 static int64_t level_bytes(int64_t n, int64_t nnz, int64_t G, const BinPlan &p) {
   const int64_t hubs = nnz / (p.hub_min() + 1) + 1, chunks = nnz / p.hub_chunk + hubs;
-  return 4 * n + (int64_t)sizeof(VRec) * n + 4 * (kBins + 1) + 40 * chunks + 36 * hubs  // bins, hub plan
+  return 4 * n + (int64_t)sizeof(VRec) * n + 4 * (kBins + 1) + 40 * chunks + 40 * hubs  // bins, hub plan
          + (int64_t)sizeof(GraphParam) * G                   // upload_params
          + 4 * n + (G > 1 ? 4 * n : 0)                      // Cd, next level's gid
          + 16 * (n + 1) + 8 * nnz;                          // coarse row_ptr, vw, col, ew
@@ -384,7 +384,7 @@ static int bins_for(Run &r, Level &L) {
   L.max_deg = out.max_deg;
   const int H = (int)L.bins.count[kHubBin], Q = (int)out.chunks;
   if (H > 0) {
-    int32_t *d_hub_of, *d_c0, *d_part_x;
+    int32_t *d_hub_of, *d_c0, *d_part_x, *d_done;
     int64_t *d_e0, *d_e1;
     long long *d_acc, *d_part_g;
     LC_TRY(r.ar.get(&d_hub_of, Q));
@@ -393,6 +393,7 @@ static int bins_for(Run &r, Level &L) {
     LC_TRY(r.ar.get(&d_e0, Q));
     LC_TRY(r.ar.get(&d_e1, Q));
     LC_TRY(r.ar.get(&d_acc, H));
+    LC_TRY(r.ar.get(&d_done, H));
     LC_TRY(r.ar.get(&d_part_g, Q));
     L.hub.H = H;
     L.hub.Q = Q;
@@ -402,6 +403,7 @@ static int bins_for(Run &r, Level &L) {
     L.hub.e1 = d_e1;
     L.hub.c0 = d_c0;
     L.hub.acc = d_acc;
+    L.hub.done = d_done;
     L.hub.part_g = d_part_g;
     L.hub.part_x = d_part_x;
     launch_hub_plan(L.bins, r.plan, L.hub, r.s);

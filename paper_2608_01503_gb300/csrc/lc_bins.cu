@@ -159,7 +159,7 @@ static_assert(kW == 32, "one lane per warp in the tile scan");
 // of hub h, and each chunk's hub and edges.  One block.
 __global__ void __launch_bounds__(kT, 1)
     k_hub_plan(const VRec *__restrict__ hubs, int H, int32_t hub_chunk, int32_t *c0, int32_t *hub_of, int64_t *e0,
-               int64_t *e1, long long *acc) {
+               int64_t *e1, long long *acc, int32_t *done) {
   __shared__ int32_t s_w[kW];
   __shared__ int32_t s_run;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(kT, 1)
     if (h < H) {
       c0[h] = before + incl - c;
       acc[h] = 0;
+      done[h] = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0) s_run += total;
@@ -236,7 +237,7 @@ void finish_bins(Bins &b, const BinOut &out) {
 void launch_hub_plan(const Bins &b, const BinPlan &plan, const Hubs &hub, cudaStream_t s) {
   k_hub_plan<<<1, kT, 0, s>>>(b.rec[kHubBin], hub.H, (int32_t)plan.hub_chunk, const_cast<int32_t *>(hub.c0),
                              const_cast<int32_t *>(hub.hub_of), const_cast<int64_t *>(hub.e0),
-                             const_cast<int64_t *>(hub.e1), hub.acc);
+                             const_cast<int64_t *>(hub.e1), hub.acc, hub.done);
 }
 
 }  // namespace lc

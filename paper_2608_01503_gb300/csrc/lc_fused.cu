@@ -17,7 +17,7 @@
 // (lc_move.cuh), so the results are identical.  Rows are taken by a thread
 // (bin 0), 16 lanes, a warp (bins 2-4), four warps (bins 5-6) or the block
 // (bins 7-8 and hubs of up to kRowSlots / 2 edges); longer hub rows go by
-// chunks over the global table, with two more barriers per pass.
+// chunks over the global table, with one more barrier per pass.
 #include "lc_coop.cuh"
 #include "lc_empty.cuh"
 #include "lc_fused.cuh"
@@ -251,6 +251,49 @@ __device__ __forceinline__ void big_chunks(const PassArgs &a, Body body) {
   }
 }
 
+// Whether this block is the last of the chunks of hub h to get here (whole
+// block; thread 0's earlier stores and atomics are then visible to the last
+// one's L2 reads).  It leaves the counter at zero for the next use.
+__device__ __forceinline__ bool last_of_hub(const PassArgs &a, int h) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const int n = a.hub.c0[h + 1] - a.hub.c0[h];
+    s_last = atomicAdd(&a.hub.done[h], 1) == n - 1;
+    if (s_last) {
+      a.hub.done[h] = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return s_last != 0;
+}
+
+// The decision for hub h from its chunks' partials (thread 0 of the last
+// block of the hub).
+__device__ __forceinline__ void decide_hub(const PassArgs &a, int h, int32_t v, bool first, MoveState &ms) {
+  const int g = graph_of(a, v);
+  const GraphParam P = a.gp[g];
+  long long gb = LLONG_MIN, gC = 0;
+  int32_t xb = kNone;
+  for (int c = a.hub.c0[h]; c < a.hub.c0[h + 1]; ++c) {
+    const long long pg = __ldcg(a.hub.part_g + c);
+    const int32_t px = __ldcg(a.hub.part_x + c);
+    if (better(pg, px, gb, xb)) {
+      gb = pg;
+      xb = px;
+    }
+  }
+  const int32_t Cv = a.C[v];
+  if (!first) {
+    const long long self = (long long)atomicExch((unsigned long long *)&a.hub.acc[h], 0ull);
+    gC = gain_self(P, self, a.g.vw[v], a.W[Cv]);
+    phi_add_one(a, ms.acc, g, gC, ms.phi);
+  }
+  decide(a, P, v, Cv, gC, xb, gb, ms);
+}
+
 __global__ void __launch_bounds__(kT, 1)
     k_passes(const __grid_constant__ PassArgs a, const __grid_constant__ FusedArgs f) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -333,6 +376,7 @@ __global__ void __launch_bounds__(kT, 1)
               a.hub.part_g[c] = gb;
               a.hub.part_x[c] = xb;
             }
+            if (last_of_hub(a, h) && threadIdx.x == 0) decide_hub(a, h, v, true, ms);
           });
         constexpr int lo[4] = {5, 2, 1, 0}, hi[4] = {6, 4, 1, 0}, most[4] = {1, 8, 32, 32};
         plan_chunks(f, lists, lo, hi, most);
@@ -345,12 +389,20 @@ __global__ void __launch_bounds__(kT, 1)
             first_thread(a, rec, lane, ms);
         });
       } else {
-        if (f.big)
-          big_chunks(a, [&](int c, int h, int32_t v) {
-            const long long s = block_total(hub_insert<kT>(a, c, stage.move.tags), red);
-            if (threadIdx.x == 0 && s != 0)
-              atomicAdd((unsigned long long *)&a.hub.acc[h], (unsigned long long)s);
-          });
+        if (f.big) {
+          // few chunks: a piece of one edge a thread each for the idle blocks,
+          // whose table inserts would follow one another in a thread
+          const int cut = gridDim.x >= 4u * (unsigned)a.hub.Q ? 4 : gridDim.x >= 2u * (unsigned)a.hub.Q ? 2 : 1;
+          for (int j = blockIdx.x; j < a.hub.Q * cut; j += gridDim.x) {
+            const int c = j / cut, h = a.hub.hub_of[c];
+            const int32_t v = a.hub.vtx[h];
+            if (a.g.rp[v + 1] - a.g.rp[v] <= kRowMaxDeg) continue;  // block-uniform
+            const int64_t e0 = a.hub.e0[c], len = a.hub.e1[c] - e0, p = j % cut;
+            const long long s =
+                block_total(hub_insert<kT>(a, v, e0 + len * p / cut, e0 + len * (p + 1) / cut, stage.move.tags), red);
+            if (threadIdx.x == 0 && s != 0) atomicAdd((unsigned long long *)&a.hub.acc[h], (unsigned long long)s);
+          }
+        }
         block_rows(f, next + kNextRow, [&](const VRec &vr) {
           row_move<kT, (int)(kRowMaxDeg / kT)>(a, vr, btab, kRowSlots, threadIdx.x, part, bsync, ms);
         });
@@ -380,44 +432,22 @@ __global__ void __launch_bounds__(kT, 1)
           graph_add(f.fin, g, g >= 0 ? (long long)((unsigned long long)a.gp[g].mu * W * W) : 0ll);
         }
     }
-    if (f.big) {
+    if (f.big && !first) {
       if (!bar.sync()) return;
-      if (!first) {
-        big_chunks(a, [&](int c, int h, int32_t v) {
-          const GraphParam P = a.gp[graph_of(a, v)];
-          const int64_t beg = a.g.rp[v];
-          long long gb = LLONG_MIN;
-          int32_t xb = kNone;
-          range_argmax<kT>(a, P.Lam, P.mu * a.g.vw[v], a.gtab + 2 * beg, (uint32_t)(2 * (a.hub.e0[c] - beg)),
-                           (uint32_t)(2 * (a.hub.e1[c] - beg)), threadIdx.x, gb, xb, ms.nX);
-          Grp<kT>::argmax(gb, xb, part.g, part.x);
-          if (threadIdx.x == 0) {
-            a.hub.part_g[c] = gb;
-            a.hub.part_x[c] = xb;
-          }
-        });
-        if (!bar.sync()) return;
-      }
-      for (int64_t h = tid; h < a.hub.H; h += nt) {
-        const int32_t v = a.hub.vtx[h];
-        if (a.g.rp[v + 1] - a.g.rp[v] <= kRowMaxDeg) continue;
-        const int g = graph_of(a, v);
-        const GraphParam P = a.gp[g];
-        long long gb = LLONG_MIN, gC = 0;
+      big_chunks(a, [&](int c, int h, int32_t v) {
+        const GraphParam P = a.gp[graph_of(a, v)];
+        const int64_t beg = a.g.rp[v];
+        long long gb = LLONG_MIN;
         int32_t xb = kNone;
-        for (int c = a.hub.c0[h]; c < a.hub.c0[h + 1]; ++c)
-          if (better(a.hub.part_g[c], a.hub.part_x[c], gb, xb)) {
-            gb = a.hub.part_g[c];
-            xb = a.hub.part_x[c];
-          }
-        const int32_t Cv = a.C[v];
-        if (!first) {
-          gC = gain_self(P, a.hub.acc[h], a.g.vw[v], a.W[Cv]);
-          a.hub.acc[h] = 0;
-          phi_add_one(a, acc, g, gC, ms.phi);
+        range_argmax<kT>(a, P.Lam, P.mu * a.g.vw[v], a.gtab + 2 * beg, (uint32_t)(2 * (a.hub.e0[c] - beg)),
+                         (uint32_t)(2 * (a.hub.e1[c] - beg)), threadIdx.x, gb, xb, ms.nX);
+        Grp<kT>::argmax(gb, xb, part.g, part.x);
+        if (threadIdx.x == 0) {
+          a.hub.part_g[c] = gb;
+          a.hub.part_x[c] = xb;
         }
-        decide(a, P, v, Cv, gC, xb, gb, ms);
-      }
+        if (last_of_hub(a, h) && threadIdx.x == 0) decide_hub(a, h, v, false, ms);
+      });
     }
     {
       const int e = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)ms.empties);
@@ -452,11 +482,20 @@ __global__ void __launch_bounds__(kT, 1)
       if (f.big)
         big_chunks(a, [&](int c, int h, int32_t v) {
           const AbRec r = a.ab[v];
-          if (r.D == kNone) return;  // block-uniform
+          const int64_t deg = a.g.rp[v + 1] - a.g.rp[v];
+          if (r.D == kNone) {  // block-uniform
+            if (wid == 0 && c == a.hub.c0[h]) apply_lanes(a, lane == 0, v, deg, r, a.g.vw[v], false, us, used);
+            return;
+          }
           const AbCtx ctx = ab_ctx(a, v, r, a.gp[graph_of(a, v)], 0, 0, a.g.vw[v]);
-          const long long s = block_total(ab_edges<kT, 2>(a, ctx, a.hub.e0[c], a.hub.e1[c], threadIdx.x), red);
+          const long long s = block_total(ab_edges<kT, 4>(a, ctx, a.hub.e0[c], a.hub.e1[c], threadIdx.x), red);
           if (threadIdx.x == 0 && s != 0)
             atomicAdd((unsigned long long *)&a.hub.acc[h], (unsigned long long)s);
+          if (last_of_hub(a, h) && wid == 0) {
+            long long t = 0;
+            if (lane == 0) t = (long long)atomicExch((unsigned long long *)&a.hub.acc[h], 0ull);
+            apply_lanes(a, lane == 0, v, deg, r, a.g.vw[v], lane == 0 && a.delta[v] + t >= 0, us, used);
+          }
         });
       block_rows(f, next + kNextRow, [&](const VRec &vr) {
         const AbRec r = a.ab[vr.v];
@@ -480,27 +519,6 @@ __global__ void __launch_bounds__(kT, 1)
         else
           ab_thread(a, lane < m, rec, lane, us, used);
       });
-    }
-    if (f.big) {
-      if (!bar.sync()) return;
-      for (int64_t h0 = wbase; h0 < a.hub.H; h0 += nt) {
-        const int64_t h = h0 + lane;
-        bool on = h < a.hub.H, keep = false;
-        int32_t v = 0;
-        int64_t deg = 0;
-        AbRec r{0, kNone, 0};
-        if (on) {
-          v = a.hub.vtx[h];
-          deg = a.g.rp[v + 1] - a.g.rp[v];
-          on = deg > kRowMaxDeg;
-        }
-        if (on) {
-          r = a.ab[v];
-          keep = r.D != kNone && a.delta[v] + a.hub.acc[h] >= 0;
-          a.hub.acc[h] = 0;
-        }
-        apply_lanes(a, on, v, deg, r, on ? a.g.vw[v] : 0, keep, us, used);
-      }
     }
     {
       const int e = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)us.empties);

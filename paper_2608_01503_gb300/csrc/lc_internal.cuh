@@ -104,6 +104,7 @@ struct Hubs {
   const int64_t *e0 = nullptr, *e1 = nullptr;  // [Q]
   const int32_t *c0 = nullptr;      // [H+1]
   long long *acc = nullptr;         // [H] per-hub sums, zero between uses
+  int32_t *done = nullptr;          // [H] chunks that have got through a phase, zero between uses
   long long *part_g = nullptr;      // [Q] per-chunk argmax partials
   int32_t *part_x = nullptr;        // [Q]
 };

@@ -710,19 +710,16 @@ __device__ __forceinline__ void warp_chunk(const PassArgs &a, const VRec *__rest
   __syncwarp();
 }
 
-// Inserts chunk c of a hub row into the hub's global table (GS threads, tg:
-// this warp's tags); returns this thread's part of S(v, C[v]).
+// Inserts edges [e0, e1) of hub v into its global table (GS threads, tg: this
+// warp's tags); returns this thread's part of S(v, C[v]).
 template <int GS>
-__device__ __forceinline__ long long hub_insert(const PassArgs &a, int c, LaneTags &tg) {
-  constexpr int U = GS > 512 ? 2 : 4;
-  const int h = a.hub.hub_of[c];
-  const int32_t v = a.hub.vtx[h];
+__device__ __forceinline__ long long hub_insert(const PassArgs &a, int32_t v, int64_t e0, int64_t e1, LaneTags &tg) {
+  constexpr int U = 4;
   const int64_t beg = a.g.rp[v], end = a.g.rp[v + 1];
   const int32_t Cv = LC_IDX(a.C[v], a.g.n, kDbgLabel);
   unsigned long long *tab = a.gtab + 2 * beg;
   const uint32_t cap = (uint32_t)(2 * (end - beg));
   const int lane = threadIdx.x & 31;
-  const int64_t e0 = a.hub.e0[c], e1 = a.hub.e1[c];
   long long self = 0;
   bool ok = true;
   for (int64_t base = e0; base < e1; base += GS * U) {
@@ -741,6 +738,7 @@ __device__ __forceinline__ long long hub_insert(const PassArgs &a, int c, LaneTa
     for (int k = 0; k < U; ++k) X[k] = u[k] >= 0 ? LC_IDX(a.C[u[k]], a.g.n, kDbgLabel) : -1;
 #pragma unroll
     for (int k = 0; k < U; ++k) {
+      if (base + k * GS >= e1) break;  // uniform
       const bool other = u[k] >= 0 && X[k] != Cv;
       if (u[k] >= 0 && X[k] == Cv) self += w[k];
       int leader;

@@ -254,8 +254,9 @@ __device__ __forceinline__ void hub_acc_add(const PassArgs &a, int h, long long 
 // so a popular cluster costs one global atomic per warp.
 __global__ void __launch_bounds__(kHubThreads) k_hub_move_insert(PassArgs a) {
   __shared__ LaneTags tags[kHubThreads / 32];
-  const int h = a.hub.hub_of[blockIdx.x];
-  const long long self = hub_insert<kHubThreads>(a, blockIdx.x, tags[threadIdx.x >> 5]);
+  const int c = blockIdx.x, h = a.hub.hub_of[c];
+  const long long self =
+      hub_insert<kHubThreads>(a, a.hub.vtx[h], a.hub.e0[c], a.hub.e1[c], tags[threadIdx.x >> 5]);
   hub_acc_add(a, h, self);
 }
 
