@@ -16,6 +16,7 @@
 #include "lc_group.cuh"
 #include "lc_internal.cuh"
 #include "lc_scan.cuh"
+#include "lc_step.cuh"
 
 namespace lc {
 
@@ -140,6 +141,7 @@ __device__ __forceinline__ int insert_edges(const InsertArgs &a, int32_t x, int6
 template <int GS>
 __global__ void __launch_bounds__(GS > 32 ? GS : 256)
     k_insert(InsertArgs a, const int32_t *__restrict__ list, int64_t count) {
+  step_begin();
   const int r = Grp<GS>::rank();
   for_each_vertex<GS>(count, [&](int64_t i, bool active) {
     if (!active) return;
@@ -154,21 +156,25 @@ __global__ void __launch_bounds__(GS > 32 ? GS : 256)
     }
     if (fresh_n) atomicAdd(&a.cnt[x], fresh_n);
   });
+  step_end();
 }
 
 // Hub rows: one block per chunk of the level's hub plan.
 __global__ void __launch_bounds__(kHubThreads) k_insert_hub(InsertArgs a, Hubs hub) {
+  step_begin();
   const int c = blockIdx.x;
   const int32_t v = hub.vtx[hub.hub_of[c]];
   const int32_t x = a.Cd[v];
-  if (x < 0) return;  // graph finished coarsening
-  bool ok = true;
-  const int fresh_n = insert_edges<kHubThreads>(a, x, hub.e0[c], hub.e1[c], threadIdx.x, ok);
-  if (!ok) {
-    *a.error = 1;
-    LC_DBG_FAIL(kDbgProbe, v, a.g.n);
+  if (x >= 0) {  // else the graph finished coarsening
+    bool ok = true;
+    const int fresh_n = insert_edges<kHubThreads>(a, x, hub.e0[c], hub.e1[c], threadIdx.x, ok);
+    if (!ok) {
+      *a.error = 1;
+      LC_DBG_FAIL(kDbgProbe, v, a.g.n);
+    }
+    if (fresh_n) atomicAdd(&a.cnt[x], fresh_n);
   }
-  if (fresh_n) atomicAdd(&a.cnt[x], fresh_n);
+  step_end();
 }
 
 struct CntIn {
@@ -267,15 +273,6 @@ void launch_contract_offsets(const LevelGraph &g, const int32_t *Cd, int64_t n_c
   scan_apply<int64_t>(n_c + 1, I64In{bound}, I64Out{off}, scan_tmp64, s);
 }
 
-template <int GS>
-static int launch_insert(const InsertArgs &a, const int32_t *list, int64_t count, cudaStream_t s) {
-  if (count <= 0) return 0;
-  const int threads = GS > 32 ? GS : 256;
-  const int per_block = GS > 32 ? 1 : threads / GS;
-  k_insert<GS><<<blocks_for(count, per_block), threads, 0, s>>>(a, list, count);
-  return 1;
-}
-
 int launch_contract_insert(const LevelGraph &g, const int32_t *Cd, const int64_t *off,
                            unsigned long long *tab, int32_t *cnt, int64_t n_c, int *error,
                            const int32_t *const *lists, const int64_t *counts, const Hubs &hub,
@@ -287,17 +284,18 @@ int launch_contract_insert(const LevelGraph &g, const int32_t *Cd, const int64_t
     for (int k = lo; k <= hi; ++k) c += counts[k];
     return c;
   };
-  int n = 0;
-  n += launch_insert<1>(a, lists[0], range(0, 0), s);
-  n += launch_insert<16>(a, lists[1], range(1, 1), s);
-  n += launch_insert<32>(a, lists[2], range(2, 4), s);
-  n += launch_insert<128>(a, lists[5], range(5, 6), s);
-  n += launch_insert<512>(a, lists[7], range(7, 8), s);
-  if (hub.H > 0) {
-    k_insert_hub<<<hub.Q, kHubThreads, 0, s>>>(a, hub);
-    n++;
-  }
-  return n;
+  Step st(s);
+  const auto insert = [&](void (*k)(InsertArgs, const int32_t *, int64_t), int threads, int rows, const int32_t *list,
+                          int64_t count) {
+    if (count > 0) st.run(false, k, blocks_for(count, rows), threads, 0, a, list, count);
+  };
+  insert(k_insert<1>, 256, 256, lists[0], range(0, 0));
+  insert(k_insert<16>, 256, 16, lists[1], range(1, 1));
+  insert(k_insert<32>, 256, 8, lists[2], range(2, 4));
+  insert(k_insert<128>, 128, 1, lists[5], range(5, 6));
+  insert(k_insert<512>, 512, 1, lists[7], range(7, 8));
+  if (hub.H > 0) st.run(false, k_insert_hub, hub.Q, kHubThreads, 0, a, hub);
+  return st.launches;
 }
 
 void launch_contract_rowptr(const int32_t *cnt, int64_t n_c, int64_t *rp_c, int64_t *scan_tmp64,

@@ -251,49 +251,6 @@ __device__ __forceinline__ void big_chunks(const PassArgs &a, Body body) {
   }
 }
 
-// Whether this block is the last of the chunks of hub h to get here (whole
-// block; thread 0's earlier stores and atomics are then visible to the last
-// one's L2 reads).  It leaves the counter at zero for the next use.
-__device__ __forceinline__ bool last_of_hub(const PassArgs &a, int h) {
-  __shared__ int s_last;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const int n = a.hub.c0[h + 1] - a.hub.c0[h];
-    s_last = atomicAdd(&a.hub.done[h], 1) == n - 1;
-    if (s_last) {
-      a.hub.done[h] = 0;
-      __threadfence();
-    }
-  }
-  __syncthreads();
-  return s_last != 0;
-}
-
-// The decision for hub h from its chunks' partials (thread 0 of the last
-// block of the hub).
-__device__ __forceinline__ void decide_hub(const PassArgs &a, int h, int32_t v, bool first, MoveState &ms) {
-  const int g = graph_of(a, v);
-  const GraphParam P = a.gp[g];
-  long long gb = LLONG_MIN, gC = 0;
-  int32_t xb = kNone;
-  for (int c = a.hub.c0[h]; c < a.hub.c0[h + 1]; ++c) {
-    const long long pg = __ldcg(a.hub.part_g + c);
-    const int32_t px = __ldcg(a.hub.part_x + c);
-    if (better(pg, px, gb, xb)) {
-      gb = pg;
-      xb = px;
-    }
-  }
-  const int32_t Cv = a.C[v];
-  if (!first) {
-    const long long self = (long long)atomicExch((unsigned long long *)&a.hub.acc[h], 0ull);
-    gC = gain_self(P, self, a.g.vw[v], a.W[Cv]);
-    phi_add_one(a, ms.acc, g, gC, ms.phi);
-  }
-  decide(a, P, v, Cv, gC, xb, gb, ms);
-}
-
 __global__ void __launch_bounds__(kT, 1)
     k_passes(const __grid_constant__ PassArgs a, const __grid_constant__ FusedArgs f) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -376,7 +333,7 @@ __global__ void __launch_bounds__(kT, 1)
               a.hub.part_g[c] = gb;
               a.hub.part_x[c] = xb;
             }
-            if (last_of_hub(a, h) && threadIdx.x == 0) decide_hub(a, h, v, true, ms);
+            if (last_of_hub(a, h) && wid == 0) decide_hub(a, h, v, true, lane, ms);
           });
         constexpr int lo[4] = {5, 2, 1, 0}, hi[4] = {6, 4, 1, 0}, most[4] = {1, 8, 32, 32};
         plan_chunks(f, lists, lo, hi, most);
@@ -446,7 +403,7 @@ __global__ void __launch_bounds__(kT, 1)
           a.hub.part_g[c] = gb;
           a.hub.part_x[c] = xb;
         }
-        if (last_of_hub(a, h) && threadIdx.x == 0) decide_hub(a, h, v, false, ms);
+        if (last_of_hub(a, h) && wid == 0) decide_hub(a, h, v, false, lane, ms);
       });
     }
     {

@@ -756,6 +756,60 @@ __device__ __forceinline__ long long hub_insert(const PassArgs &a, int32_t v, in
   return self;
 }
 
+// Whether this block is the last of the chunks of hub h to get here (whole
+// block; thread 0's earlier stores and atomics are then visible to the last
+// one's L2 reads).  It leaves the counter at zero for the next use.
+__device__ __forceinline__ bool last_of_hub(const PassArgs &a, int h) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const int n = a.hub.c0[h + 1] - a.hub.c0[h];
+    s_last = atomicAdd(&a.hub.done[h], 1) == n - 1;
+    if (s_last) {
+      a.hub.done[h] = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return s_last != 0;
+}
+
+// Takes the sum of hub h's chunks and leaves zero.
+__device__ __forceinline__ long long take_hub_acc(const PassArgs &a, int h) {
+  return (long long)atomicExch((unsigned long long *)&a.hub.acc[h], 0ull);
+}
+
+// The decision for hub h from its chunks' partials (one warp of the last
+// block of the hub; first: from singletons, S(v, C[v]) = 0).  Lane 0 returns
+// S(v, C[v]).
+__device__ __forceinline__ long long decide_hub(const PassArgs &a, int h, int32_t v, bool first, int lane,
+                                                MoveState &ms) {
+  long long gb = LLONG_MIN, gC = 0, self = 0;
+  int32_t xb = kNone;
+  for (int c = a.hub.c0[h] + lane; c < a.hub.c0[h + 1]; c += 32) {
+    const long long pg = __ldcg(a.hub.part_g + c);
+    const int32_t px = __ldcg(a.hub.part_x + c);
+    if (better(pg, px, gb, xb)) {
+      gb = pg;
+      xb = px;
+    }
+  }
+  warp_argmax(gb, xb);
+  if (lane == 0) {
+    const int g = graph_of(a, v);
+    const GraphParam P = a.gp[g];
+    const int32_t Cv = a.C[v];
+    if (!first) {
+      self = take_hub_acc(a, h);
+      gC = gain_self(P, self, a.g.vw[v], a.W[Cv]);
+      phi_add_one(a, ms.acc, g, gC, ms.phi);
+    }
+    decide(a, P, v, Cv, gC, xb, gb, ms);
+  }
+  return self;
+}
+
 // ------------------------------------------------ afterburner (Algorithm 3)
 
 // What a candidate's row walk needs, staged per chunk.

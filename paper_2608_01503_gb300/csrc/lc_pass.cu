@@ -21,6 +21,7 @@
 #include "lc_move.cuh"
 #include "lc_pass.cuh"
 #include "lc_scan.cuh"
+#include "lc_step.cuh"
 
 namespace lc {
 
@@ -57,38 +58,46 @@ __device__ __forceinline__ WarpChunk warp_chunk_of(int64_t count, int chunk) {
 template <int G>
 __global__ void __launch_bounds__(256) k_first_pass(PassArgs a, const VRec *__restrict__ rec, int64_t count,
                                                     int chunk) {
+  step_begin();
   __shared__ MoveStage st[8];
   MoveState ms = move_state(a);
   const WarpChunk c = warp_chunk_of(count, chunk);
   if (c.m > 0) first_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], ms);
   flush_block_sum(ms.cntL, &a.sc->count_L);
+  step_end();
 }
 
 __global__ void __launch_bounds__(256) k_first_thread(PassArgs a, const VRec *__restrict__ rec, int64_t count) {
+  step_begin();
   MoveState ms = move_state(a);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
        i += (int64_t)gridDim.x * blockDim.x)
     first_thread(a, rec, i, ms);
   flush_block_sum(ms.cntL, &a.sc->count_L);
+  step_end();
 }
 
 __global__ void __launch_bounds__(256, 4) k_move_thread(PassArgs a, const VRec *__restrict__ rec, int64_t count) {
+  step_begin();
   MoveState ms = move_state(a);
   // warp-uniform trip count: phi_add takes whole warps
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < count; base += (int64_t)gridDim.x * blockDim.x)
     move_thread(a, base + threadIdx.x < count, rec, base + threadIdx.x, ms);
   flush_move(a, ms);
+  step_end();
 }
 
 template <int G>
 __global__ void __launch_bounds__(256) k_move_lanes(PassArgs a, const VRec *__restrict__ rec, int64_t count,
                                                     int chunk) {
+  step_begin();
   __shared__ MoveStage st[8];
   __shared__ LaneTags tags[8];
   MoveState ms = move_state(a);
   const WarpChunk c = warp_chunk_of(count, chunk);
   if (c.m > 0) lanes_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], tags[threadIdx.x >> 5], ms);
   flush_move(a, ms);
+  step_end();
 }
 
 // Bins 3-4: one warp per vertex, a per-warp split shared table of kWarpSlots
@@ -96,6 +105,7 @@ __global__ void __launch_bounds__(256) k_move_lanes(PassArgs a, const VRec *__re
 constexpr int kWarpSlots = 512;
 __global__ void __launch_bounds__(kWarpBinWarps * 32, 4)
     k_move_warp(PassArgs a, const VRec *__restrict__ rec, int64_t count, int chunk) {
+  step_begin();
   __shared__ uint32_t keys[kWarpBinWarps][kWarpSlots];
   __shared__ int32_t vals[kWarpBinWarps][kWarpSlots];
   __shared__ MoveStage st[kWarpBinWarps];
@@ -112,6 +122,7 @@ __global__ void __launch_bounds__(kWarpBinWarps * 32, 4)
     warp_chunk(a, rec, c.base, c.m, st[wid], tab, kWarpSlots, ms);
   }
   flush_move(a, ms);
+  step_end();
 }
 
 // A block's chunk of vertices, staged and decided by its first warp.
@@ -129,6 +140,7 @@ __device__ __forceinline__ BlockChunk block_chunk_of(int64_t count, int chunk) {
 template <int GS>
 __global__ void __launch_bounds__(GS) k_first_block(PassArgs a, const VRec *__restrict__ rec, int64_t count,
                                                     int chunk) {
+  step_begin();
   __shared__ MoveStage st;
   __shared__ long long rg[GS / 32];
   __shared__ int32_t rx[GS / 32];
@@ -149,6 +161,7 @@ __global__ void __launch_bounds__(GS) k_first_block(PassArgs a, const VRec *__re
   __syncthreads();
   if (threadIdx.x < 32) settle_move(a, c, b.m, threadIdx.x, true, st.res, ms);
   flush_block_sum(ms.cntL, &a.sc->count_L);
+  step_end();
 }
 
 // Bins 5-8: one block per vertex; dynamic shared memory holds the split
@@ -160,6 +173,7 @@ __global__ void __launch_bounds__(GS) k_first_block(PassArgs a, const VRec *__re
 template <int GS, int SLOTS, int N, bool BUILD>
 __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__restrict__ rec,
                                                    int64_t count, int chunk) {
+  step_begin();
   extern __shared__ uint32_t smem_tab[];
   const SplitTab tab{smem_tab, reinterpret_cast<int32_t *>(smem_tab + SLOTS)};
   __shared__ MoveStage st;
@@ -228,6 +242,7 @@ __global__ void __launch_bounds__(GS) k_move_block(PassArgs a, const VRec *__res
   __syncthreads();
   if (threadIdx.x < 32) settle_move(a, c, b.m, threadIdx.x, false, st.res, ms);
   flush_move(a, ms);
+  step_end();
 }
 
 // --------------------------------------------------------- hubs (bin 9)
@@ -253,11 +268,13 @@ __device__ __forceinline__ void hub_acc_add(const PassArgs &a, int h, long long 
 // Lanes of a warp holding the same cluster are combined first (lane_sums),
 // so a popular cluster costs one global atomic per warp.
 __global__ void __launch_bounds__(kHubThreads) k_hub_move_insert(PassArgs a) {
+  step_begin();
   __shared__ LaneTags tags[kHubThreads / 32];
   const int c = blockIdx.x, h = a.hub.hub_of[c];
   const long long self =
       hub_insert<kHubThreads>(a, a.hub.vtx[h], a.hub.e0[c], a.hub.e1[c], tags[threadIdx.x >> 5]);
   hub_acc_add(a, h, self);
+  step_end();
 }
 
 // Move, step 2: argmax over the chunk's share of the hub table (reset as
@@ -269,80 +286,64 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_move_scan(PassArgs a) {
   const int64_t beg = a.g.rp[v];
   const long long wv = a.g.vw[v];
   const GraphParam P = a.gp[graph_of(a, v)];
-  long long gb = LLONG_MIN, nX = 0;
+  MoveState ms = move_state(a);
+  long long gb = LLONG_MIN;
   int32_t xb = kNone;
   range_argmax<kHubThreads>(a, P.Lam, P.mu * wv, a.gtab + 2 * beg, (uint32_t)(2 * (a.hub.e0[c] - beg)),
-                            (uint32_t)(2 * (a.hub.e1[c] - beg)), threadIdx.x, gb, xb, nX, a.tab_build != 0);
+                            (uint32_t)(2 * (a.hub.e1[c] - beg)), threadIdx.x, gb, xb, ms.nX, a.tab_build != 0);
   hub_part_store(a, c, gb, xb);
-  flush_block_sum(nX, &a.sc->distinct_x);
+  if (last_of_hub(a, h) && threadIdx.x < 32) {
+    const long long self = decide_hub(a, h, v, false, threadIdx.x, ms);
+    // the hub's kept table gets its own cluster
+    if (a.tab_build && self > 0 && !tab_put(a.gtab + 2 * beg, tab_cap(a.g.rp[v + 1] - beg), a.C[v], self))
+      a.sc->error = 1;
+  }
+  flush_move(a, ms);
 }
 
 // First pass: argmax over a chunk of a hub row.
 __global__ void __launch_bounds__(kHubThreads) k_hub_first(PassArgs a) {
-  const int c = blockIdx.x;
-  const int32_t v = a.hub.vtx[a.hub.hub_of[c]];
+  step_begin();
+  const int c = blockIdx.x, h = a.hub.hub_of[c];
+  const int32_t v = a.hub.vtx[h];
   const long long wv = a.g.vw[v];
   const GraphParam P = a.gp[graph_of(a, v)];
+  MoveState ms = move_state(a);
   long long gb = LLONG_MIN;
   int32_t xb = kNone;
 #pragma unroll 4
   for (int64_t e = a.hub.e0[c] + threadIdx.x; e < a.hub.e1[c]; e += kHubThreads)
     first_edge(a, P.Lam, P.mu * wv, e, gb, xb);
   hub_part_store(a, c, gb, xb);
-}
-
-// Final step per hub: combine chunk partials, then decide (Algorithm 2).
-// first = 1: singleton start, g(v, C[v]) = 0 and no objective term.
-__global__ void k_hub_decide(PassArgs a, int first) {
-  MoveState ms = move_state(a);
-  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < a.hub.H; h += gridDim.x * blockDim.x) {
-    const int32_t v = a.hub.vtx[h];
-    const GraphParam P = a.gp[graph_of(a, v)];
-    long long gb = LLONG_MIN;
-    int32_t xb = kNone;
-    for (int c = a.hub.c0[h]; c < a.hub.c0[h + 1]; ++c)
-      if (better(a.hub.part_g[c], a.hub.part_x[c], gb, xb)) {
-        gb = a.hub.part_g[c];
-        xb = a.hub.part_x[c];
-      }
-    long long gC = 0;
-    const int32_t Cv = first ? v : a.C[v];
-    if (!first) {
-      const long long self = a.hub.acc[h];
-      a.hub.acc[h] = 0;
-      gC = gain_self(P, self, a.g.vw[v], a.W[Cv]);
-      phi_add_one(a, ms.acc, graph_of(a, v), gC, ms.phi);
-      if (a.tab_build && self > 0) {  // the hub's kept table gets its own cluster
-        const int64_t beg = a.g.rp[v];
-        if (!tab_put(a.gtab + 2 * beg, tab_cap(a.g.rp[v + 1] - beg), Cv, self)) a.sc->error = 1;
-      }
-    }
-    decide(a, P, v, Cv, gC, xb, gb, ms);
-  }
+  if (last_of_hub(a, h) && threadIdx.x < 32) decide_hub(a, h, v, true, threadIdx.x, ms);
   flush_block_sum(ms.cntL, &a.sc->count_L);
-  flush_block_sum(ms.phi, &ms.acc[0]);
+  step_end();
 }
 
 // ------------------------------------------------ afterburner (Algorithm 3)
 
 // Bin 0: a thread per vertex.
 __global__ void __launch_bounds__(256, 4) k_ab_thread(PassArgs a, const VRec *__restrict__ rec, int64_t count) {
+  step_begin();
   UpdateSums sum;
   // warp-uniform trip count: the update's lists are appended per warp
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < count; base += (int64_t)gridDim.x * blockDim.x)
     ab_thread(a, base + threadIdx.x < count, rec, base + threadIdx.x, sum);
   flush_update(a, sum);
+  step_end();
 }
 
 // 4, 8 or 16 lanes or a warp per candidate, a chunk of vertices per warp.
 template <int G>
 __global__ void __launch_bounds__(256, 4) k_ab_warp(PassArgs a, const VRec *__restrict__ rec, int64_t count,
                                                     int chunk) {
+  step_begin();
   __shared__ AbStage st[8];
   UpdateSums sum;
   const WarpChunk c = warp_chunk_of(count, chunk);
   if (c.m > 0) ab_chunk<G>(a, rec, c.base, c.m, st[threadIdx.x >> 5], sum);
   flush_update(a, sum);
+  step_end();
 }
 
 // A block per candidate, a chunk of vertices per block.  Every warp walks its
@@ -351,6 +352,7 @@ __global__ void __launch_bounds__(256, 4) k_ab_warp(PassArgs a, const VRec *__re
 template <int GS>
 __global__ void __launch_bounds__(GS, 2048 / GS / 2) k_ab_block(PassArgs a, const VRec *__restrict__ rec,
                                                                 int64_t count, int chunk) {
+  step_begin();
   __shared__ AbStage st;
   __shared__ long long rs[32][GS / 32];
   __shared__ int s_nc;
@@ -379,39 +381,28 @@ __global__ void __launch_bounds__(GS, 2048 / GS / 2) k_ab_block(PassArgs a, cons
     apply_lanes(a, (int)threadIdx.x < b.m, vr.v, vr.deg, r, vr.w, r.D != kNone && t >= 0, sum);
   }
   flush_update(a, sum);
+  step_end();
 }
 
 __global__ void __launch_bounds__(kHubThreads) k_hub_afterburner(PassArgs a) {
+  step_begin();
   const int c = blockIdx.x;
   const int h = a.hub.hub_of[c];
   const int32_t v = a.hub.vtx[h];
   const AbRec r = a.ab[v];
-  if (r.D == kNone) return;  // block-uniform
-  const AbCtx ctx = ab_ctx(a, v, r, a.gp[graph_of(a, v)], 0, 0, a.g.vw[v]);
-  const long long acc = ab_edges<kHubThreads, 4>(a, ctx, a.hub.e0[c], a.hub.e1[c], threadIdx.x);
-  hub_acc_add(a, h, acc);
-}
-
-__global__ void k_hub_ab_final(PassArgs a) {
   UpdateSums sum;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.hub.H; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t h = base + threadIdx.x;
-    const bool on = h < a.hub.H;
-    int32_t v = 0;
-    int64_t deg = 0;
-    AbRec r{0, kNone, 0};
-    bool keep = false;
-    if (on) {
-      v = a.hub.vtx[h];
-      r = a.ab[v];
-      deg = a.g.rp[v + 1] - a.g.rp[v];
-      const long long acc = a.hub.acc[h];
-      a.hub.acc[h] = 0;
-      keep = r.D != kNone && a.delta[v] + acc >= 0;
-    }
-    apply_lanes(a, on, v, deg, r, on ? a.g.vw[v] : 0, keep, sum);
+  bool mine = c == a.hub.c0[h];  // no candidate: its first chunk keeps it where it is
+  long long t = -1;
+  if (r.D != kNone) {  // block-uniform
+    const AbCtx ctx = ab_ctx(a, v, r, a.gp[graph_of(a, v)], 0, 0, a.g.vw[v]);
+    hub_acc_add(a, h, ab_edges<kHubThreads, 4>(a, ctx, a.hub.e0[c], a.hub.e1[c], threadIdx.x));
+    mine = last_of_hub(a, h);
+    if (mine && threadIdx.x == 0) t = a.delta[v] + take_hub_acc(a, h);
   }
+  if (mine && threadIdx.x < 32)
+    apply_lanes(a, threadIdx.x == 0, v, a.g.rp[v + 1] - a.g.rp[v], r, a.g.vw[v], t >= 0, sum);
   flush_update(a, sum);
+  step_end();
 }
 
 // ---------------------------------------------------- objective, S_self
@@ -684,14 +675,15 @@ __global__ void __launch_bounds__(GS) k_tab_scan(PassArgs a, const int32_t *__re
   flush_block_sum(ms.phi, &ms.acc[0]);
 }
 
-// Hubs: each chunk scans its share of the hub's table; k_hub_decide
-// combines the partials and the parts of S(v, C[v]).
+// Hubs: each chunk scans its share of the hub's table; the last one combines
+// the partials and the parts of S(v, C[v]).
 __global__ void __launch_bounds__(kHubThreads) k_hub_tab_scan(PassArgs a) {
   const int c = blockIdx.x;
   const int h = a.hub.hub_of[c];
   const int32_t v = a.hub.vtx[h];
   const int64_t beg = a.g.rp[v];
   const GraphParam P = a.gp[graph_of(a, v)];
+  MoveState ms = move_state(a);
   long long self = 0, gb = LLONG_MIN;
   int32_t xb = kNone;
   // a chunk of edges [e0, e1) owns the slot pairs [e0 - beg, e1 - beg)
@@ -700,6 +692,8 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_tab_scan(PassArgs a) {
                                  a.g.vw[v], a.tab_reset != 0, self, gb, xb);
   hub_part_store(a, c, gb, xb);
   hub_acc_add(a, h, self);
+  if (last_of_hub(a, h) && threadIdx.x < 32) decide_hub(a, h, v, false, threadIdx.x, ms);
+  flush_move(a, ms);
 }
 
 // ------------------------------------------------ ids of new clusters
@@ -828,28 +822,31 @@ static inline int block_chunk_size(int64_t count) {
   return c < 1 ? 1 : c > 32 ? 32 : (int)c;
 }
 
-using ChunkKernel = void (*)(PassArgs, const VRec *, int64_t, int);
-// most: vertices per warp at most (fewer where rows are long: blocks that
-// end sooner even the SMs out)
-static int launch_warp_chunks(ChunkKernel k, const PassArgs &a, BinRange r, cudaStream_t s, int most = 32) {
-  if (r.count <= 0) return 0;
-  const int chunk = std::min(warp_chunk_size(r.count), most);
-  k<<<warp_chunk_blocks(r.count, chunk), 256, 0, s>>>(a, r.rec, r.count, chunk);
-  return 1;
-}
-static int launch_block_chunks(ChunkKernel k, int threads, size_t smem, const PassArgs &a, BinRange r,
-                               cudaStream_t s) {
-  if (r.count <= 0) return 0;
-  const int chunk = block_chunk_size(r.count);
-  k<<<(unsigned)((r.count + chunk - 1) / chunk), threads, smem, s>>>(a, r.rec, r.count, chunk);
-  return 1;
-}
-static int launch_threads(void (*k)(PassArgs, const VRec *, int64_t), const PassArgs &a, BinRange r,
-                          cudaStream_t s) {
-  if (r.count <= 0) return 0;
-  k<<<blocks_for(r.count, 256), 256, 0, s>>>(a, r.rec, r.count);
-  return 1;
-}
+// The launches of one step of a pass.  Order: short rows first, long rows
+// last.  Long rows first (so that short ones fill the last SMs) was slower:
+// the block kernels' shared memory leaves the SMs a small L1 for whatever
+// runs among them (ms, short / long rows first: R-MAT scale 22 65.1 / 73.1,
+// 256^3 lattice 50.1 / 53.2, batch 59.5 / 62.8, R-MAT 20 level 6.09 / 6.50).
+class PassStep : public Step {
+ public:
+  using Step::Step;
+  // most: vertices per warp at most (fewer where rows are long: blocks that
+  // end sooner even the SMs out)
+  void warp_chunks(void (*k)(PassArgs, const VRec *, int64_t, int), const PassArgs &a, BinRange r, int most = 32) {
+    if (r.count <= 0) return;
+    const int chunk = std::min(warp_chunk_size(r.count), most);
+    run(false, k, warp_chunk_blocks(r.count, chunk), 256, 0, a, r.rec, r.count, chunk);
+  }
+  void block_chunks(void (*k)(PassArgs, const VRec *, int64_t, int), int threads, size_t smem, const PassArgs &a,
+                    BinRange r) {
+    if (r.count <= 0) return;
+    const int chunk = block_chunk_size(r.count);
+    run(false, k, (unsigned)((r.count + chunk - 1) / chunk), threads, smem, a, r.rec, r.count, chunk);
+  }
+  void threads(void (*k)(PassArgs, const VRec *, int64_t), const PassArgs &a, BinRange r) {
+    if (r.count > 0) run(false, k, blocks_for(r.count, 256), 256, 0, a, r.rec, r.count);
+  }
+};
 
 // The same over the plain vertex list (kernels that need little of a record).
 template <int GS>
@@ -867,96 +864,85 @@ static inline unsigned hub_final_blocks(int H) { return blocks_for(H, 256); }
 // Kernels without tables take runs of bins: bin 0 -> 1 thread, 1 -> 16
 // lanes, 2..4 -> one warp, 5..6 -> 128 threads, 7..8 -> 512 threads.
 int launch_first_pass(const PassArgs &a, const Bins &b, cudaStream_t s) {
-  int n = 0;
-  n += launch_threads(k_first_thread, a, bin_range(b, 0, 0), s);
-  n += launch_warp_chunks(k_first_pass<16>, a, bin_range(b, 1, 1), s);
-  n += launch_warp_chunks(k_first_pass<32>, a, bin_range(b, 2, 4), s);
-  n += launch_block_chunks(k_first_block<128>, 128, 0, a, bin_range(b, 5, 6), s);
-  n += launch_block_chunks(k_first_block<512>, 512, 0, a, bin_range(b, 7, 8), s);
-  if (a.hub.H > 0) {
-    k_hub_first<<<a.hub.Q, kHubThreads, 0, s>>>(a);
-    k_hub_decide<<<hub_final_blocks(a.hub.H), 256, 0, s>>>(a, 1);
-    n += 2;
-  }
-  return n;
+  PassStep st(s);
+  st.threads(k_first_thread, a, bin_range(b, 0, 0));
+  st.warp_chunks(k_first_pass<16>, a, bin_range(b, 1, 1));
+  st.warp_chunks(k_first_pass<32>, a, bin_range(b, 2, 4));
+  st.block_chunks(k_first_block<128>, 128, 0, a, bin_range(b, 5, 6));
+  st.block_chunks(k_first_block<512>, 512, 0, a, bin_range(b, 7, 8));
+  if (a.hub.H > 0) st.run(false, k_hub_first, a.hub.Q, kHubThreads, 0, a);
+  return st.launches;
+}
+
+// Bins 0-4 (degree <= 256) aggregate from the CSR in every pass; hubs: their
+// inserts go among them.
+static void move_low(PassStep &st, const PassArgs &a, const Bins &b, bool hubs) {
+  st.threads(k_move_thread, a, bin_range(b, 0, 0));
+  st.warp_chunks(k_move_lanes<16>, a, bin_range(b, 1, 1));
+  st.warp_chunks(k_move_lanes<32>, a, bin_range(b, 2, 2));
+  // after the block kernels these inserts cost R-MAT scale 22 5 ms in 65
+  // (their shared memory leaves a small L1), before all others nothing
+  if (hubs) st.run(false, k_hub_move_insert, a.hub.Q, kHubThreads, 0, a);
+  st.warp_chunks(k_move_warp, a, bin_range(b, 3, 4), 16);
 }
 
 template <int GS, int SLOTS, int N>
-static int launch_move_block(const PassArgs &a, BinRange r, cudaStream_t s) {
-  return launch_block_chunks(a.tab_build ? k_move_block<GS, SLOTS, N, true> : k_move_block<GS, SLOTS, N, false>,
-                             GS, block_table_bytes(SLOTS), a, r, s);
-}
-
-// Bins 0-4 (degree <= 256): aggregation from the CSR in every pass.
-static int launch_move_low(const PassArgs &a, const Bins &b, cudaStream_t s) {
-  int n = launch_threads(k_move_thread, a, bin_range(b, 0, 0), s);
-  n += launch_warp_chunks(k_move_lanes<16>, a, bin_range(b, 1, 1), s);
-  n += launch_warp_chunks(k_move_lanes<32>, a, bin_range(b, 2, 2), s);
-  n += launch_warp_chunks(k_move_warp, a, bin_range(b, 3, 4), s, 16);
-  return n;
+static void move_block(PassStep &st, const PassArgs &a, BinRange r) {
+  st.block_chunks(a.tab_build ? k_move_block<GS, SLOTS, N, true> : k_move_block<GS, SLOTS, N, false>, GS,
+                  block_table_bytes(SLOTS), a, r);
 }
 
 int launch_move(const PassArgs &a, const Bins &b, cudaStream_t s) {
-  int n = launch_move_low(a, b, s);
-  n += launch_move_block<64, 1024, 8>(a, bin_range(b, 5, 5), s);
-  n += launch_move_block<128, 2048, 8>(a, bin_range(b, 6, 6), s);
-  n += launch_move_block<256, 4096, 8>(a, bin_range(b, 7, 7), s);
-  n += launch_move_block<256, 6144, 16>(a, bin_range(b, 8, 8), s);
-  if (a.hub.H > 0) {
-    k_hub_move_insert<<<a.hub.Q, kHubThreads, 0, s>>>(a);
-    k_hub_move_scan<<<a.hub.Q, kHubThreads, 0, s>>>(a);
-    k_hub_decide<<<hub_final_blocks(a.hub.H), 256, 0, s>>>(a, 0);
-    n += 3;
-  }
-  return n;
-}
-
-template <int GS, int V>
-static int launch_tab_scan(const PassArgs &a, BinRange r, cudaStream_t s) {
-  if (r.count <= 0) return 0;
-  k_tab_scan<GS, V><<<blocks_for(r.count, 1), GS, 0, s>>>(a, r.list, r.count);
-  return 1;
+  PassStep st(s);
+  move_low(st, a, b, a.hub.H > 0);
+  move_block<64, 1024, 8>(st, a, bin_range(b, 5, 5));
+  move_block<128, 2048, 8>(st, a, bin_range(b, 6, 6));
+  move_block<256, 4096, 8>(st, a, bin_range(b, 7, 7));
+  move_block<256, 6144, 16>(st, a, bin_range(b, 8, 8));
+  if (a.hub.H > 0) st.run(true, k_hub_move_scan, a.hub.Q, kHubThreads, 0, a);
+  return st.launches;
 }
 
 int launch_table_pass(const PassArgs &a, const Bins &b, cudaStream_t s) {
-  k_tab_update<<<152 * 8, 256, 0, s>>>(a);  // reads the last pass's records, before any is rewritten
-  k_tab_rebuild<<<152 * 4, 256, 0, s>>>(a);
-  int n = 2 + launch_move_low(a, b, s);
+  PassStep st(s);
+  st.run(true, k_tab_update, 152 * 8, 256, 0, a);  // reads the last pass's records, before any is rewritten
+  st.run(true, k_tab_rebuild, 152 * 4, 256, 0, a);
   // one 16-byte pair of slots per thread per batch of V: bin 5 has at most
   // 512 pairs, bin 6 1024, bin 7 2048, bin 8 3072
-  n += launch_tab_scan<128, 4>(a, bin_range(b, 5, 5), s);
-  n += launch_tab_scan<256, 4>(a, bin_range(b, 6, 6), s);
-  n += launch_tab_scan<512, 4>(a, bin_range(b, 7, 8), s);
-  if (a.hub.H > 0) {
-    k_hub_tab_scan<<<a.hub.Q, kHubThreads, 0, s>>>(a);
-    k_hub_decide<<<hub_final_blocks(a.hub.H), 256, 0, s>>>(a, 0);
-    n += 2;
-  }
-  return n;
+  const auto scan = [&](void (*k)(PassArgs, const int32_t *, int64_t), int threads, BinRange r) {
+    if (r.count > 0) st.run(true, k, blocks_for(r.count, 1), threads, 0, a, r.list, r.count);
+  };
+  scan(k_tab_scan<128, 4>, 128, bin_range(b, 5, 5));
+  scan(k_tab_scan<256, 4>, 256, bin_range(b, 6, 6));
+  scan(k_tab_scan<512, 4>, 512, bin_range(b, 7, 8));
+  if (a.hub.H > 0) st.run(true, k_hub_tab_scan, a.hub.Q, kHubThreads, 0, a);
+  move_low(st, a, b, false);
+  return st.launches;
 }
 
 // One of the afterburner's bin groups 2-4: 16 (group 2 only), 32, 128 or 512
 // threads per candidate (BinPlan::ab_gs).  Bin 2 of group 2 (rows up to 32
 // edges) always takes 8 lanes per candidate.
-static int launch_ab_group(const PassArgs &a, const Bins &b, int g, cudaStream_t s) {
+static void ab_group(PassStep &st, const PassArgs &a, const Bins &b, int g) {
   const BinRange r = bin_range(b, g == 2 ? 3 : kAbFirstBin[g], kAbFirstBin[g + 1] - 1);
-  if (a.ab_gs[g] == 16) return launch_warp_chunks(k_ab_warp<16>, a, r, s, 16);
-  if (a.ab_gs[g] == 32) return launch_warp_chunks(k_ab_warp<32>, a, r, s, 16);
-  if (a.ab_gs[g] == 128) return launch_block_chunks(k_ab_block<128>, 128, 0, a, r, s);
-  return launch_block_chunks(k_ab_block<512>, 512, 0, a, r, s);
+  if (a.ab_gs[g] == 16)
+    st.warp_chunks(k_ab_warp<16>, a, r, 16);
+  else if (a.ab_gs[g] == 32)
+    st.warp_chunks(k_ab_warp<32>, a, r, 16);
+  else if (a.ab_gs[g] == 128)
+    st.block_chunks(k_ab_block<128>, 128, 0, a, r);
+  else
+    st.block_chunks(k_ab_block<512>, 512, 0, a, r);
 }
 
 int launch_afterburner(const PassArgs &a, const Bins &b, cudaStream_t s) {
-  int n = launch_threads(k_ab_thread, a, bin_range(b, 0, 0), s);
-  n += launch_warp_chunks(k_ab_warp<4>, a, bin_range(b, 1, 1), s);
-  n += launch_warp_chunks(k_ab_warp<8>, a, bin_range(b, 2, 2), s);
-  for (int g = 2; g < kAbGroups; ++g) n += launch_ab_group(a, b, g, s);
-  if (a.hub.H > 0) {
-    k_hub_afterburner<<<a.hub.Q, kHubThreads, 0, s>>>(a);
-    k_hub_ab_final<<<hub_final_blocks(a.hub.H), 256, 0, s>>>(a);
-    n += 2;
-  }
-  return n;
+  PassStep st(s);
+  st.threads(k_ab_thread, a, bin_range(b, 0, 0));
+  st.warp_chunks(k_ab_warp<4>, a, bin_range(b, 1, 1));
+  st.warp_chunks(k_ab_warp<8>, a, bin_range(b, 2, 2));
+  for (int g = 2; g < kAbGroups; ++g) ab_group(st, a, b, g);
+  if (a.hub.H > 0) st.run(false, k_hub_afterburner, a.hub.Q, kHubThreads, 0, a);
+  return st.launches;
 }
 
 // ------------------------------------- symmetry-breaking ablations
