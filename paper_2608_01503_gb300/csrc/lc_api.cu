@@ -15,6 +15,7 @@
 #include <cstring>
 #include <deque>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -246,26 +247,41 @@ static cudaStream_t capture_stream() {
   return st.s[dev];
 }
 
+static int64_t per_graph_bytes(int64_t G) { return G * (17 * 8 + 4 * 4 + 1); }
+
+// The per-graph arrays, one block cut up in order of element size: a provider
+// call costs 2 to 4 us (PyTorch's allocator through a callback).
 static int alloc_per_graph(Run &r) {
-  const int G = r.G;
-  LC_TRY(r.ar.get(&r.phi_acc, G));
-  LC_TRY(r.ar.get(&r.phi_out, G));
-  LC_TRY(r.ar.get(&r.phi_trace, G));
-  LC_TRY(r.ar.get(&r.obj, 4 * (int64_t)G));
-  LC_TRY(r.ar.get(&r.fused, 6 * (int64_t)G));
-  LC_TRY(r.ar.get(&r.phi_final, G));
-  LC_CK(cudaMemsetAsync(r.phi_final, 0, 8 * (size_t)G, r.s));  // a graph with no vertices: Phi = 0
-  LC_TRY(r.ar.get(&r.Tg, G));
-  LC_TRY(r.ar.get(&r.Vg, G));
-  LC_TRY(r.ar.get(&r.sw2g, G));
-  LC_TRY(r.ar.get(&r.improved, G));
-  LC_TRY(r.ar.get(&r.gstart, G));
-  LC_TRY(r.ar.get(&r.gfree, G));
-  LC_TRY(r.ar.get(&r.gmover, G));
-  LC_TRY(r.ar.get(&r.keep, G));
-  LC_CK(cudaMemsetAsync(r.Tg, 0, 8 * (size_t)G, r.s));
-  LC_CK(cudaMemsetAsync(r.Vg, 0, 8 * (size_t)G, r.s));
-  LC_CK(cudaMemsetAsync(r.sw2g, 0, 8 * (size_t)G, r.s));
+  const int64_t G = r.G;
+  uint8_t *p = nullptr;
+  LC_TRY(r.ar.get(&p, per_graph_bytes(G)));
+  const auto cut = [&](auto **out, int64_t count) {
+    *out = reinterpret_cast<std::remove_reference_t<decltype(**out)> *>(p);
+    p += count * (int64_t)sizeof(**out);
+  };
+  cut(&r.phi_final, G);  // the first four are zeroed: a graph with no vertices has Phi = 0
+  cut(&r.Tg, G);
+  cut(&r.Vg, G);
+  cut(&r.sw2g, G);
+  LC_CK(cudaMemsetAsync(r.phi_final, 0, 4 * 8 * (size_t)G, r.s));
+  cut(&r.phi_acc, G);
+  cut(&r.phi_out, G);
+  cut(&r.phi_trace, G);
+  cut(&r.obj, 4 * G);
+  cut(&r.fused, 6 * G);
+  cut(&r.improved, G);
+  cut(&r.gstart, G);
+  cut(&r.gfree, G);
+  cut(&r.gmover, G);
+  cut(&r.keep, G);
+  return LC_OK;
+}
+
+// The counters of the cooperative kernels.
+static int alloc_counters(Run &r) {
+  LC_TRY(r.ar.get(&r.coop, kCoopScratch));
+  LC_TRY(r.ar.get(&r.sc, 1));
+  LC_CK(cudaMemsetAsync(r.sc, 0, sizeof(Scalars), r.s));
   return LC_OK;
 }
 
@@ -289,7 +305,6 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.W, n0));
   LC_TRY(r.ar.get(&r.delta, n0));
   LC_TRY(r.ar.get(&r.ab, n0));
-  LC_TRY(r.ar.get(&r.coop, kCoopScratch));
   LC_TRY(r.ar.get(&r.lcounts, kLevelCounts));
   LC_TRY(r.ar.get(&r.lout, 1));
   LC_TRY(r.ar.get(&r.bound, n0 + 1));
@@ -297,9 +312,7 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.scan64, scan_scratch(n0 + 1)));
   if (r.o.event_cb) LC_TRY(r.ar.get(&r.M, n0));
   LC_TRY(r.ar.get(&r.gtab, 2 * nnz0));
-  LC_TRY(r.ar.get(&r.sc, 1));
   LC_CK(cudaMemsetAsync(r.gtab, 0, sizeof(unsigned long long) * (size_t)(2 * nnz0 > 0 ? 2 * nnz0 : 1), r.s));
-  LC_CK(cudaMemsetAsync(r.sc, 0, sizeof(Scalars), r.s));
   return LC_OK;
 }
 
@@ -338,16 +351,17 @@ static int resolve_plan(const lc_opts &o, BinPlan *out) {
 // upload_params, compact_level, contract_level), for the footprint below.
 static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tables) {
   const int64_t n = n0 > 0 ? n0 : 1, big = 2 * nnz0 > n0 + 1 ? 2 * nnz0 : n0 + 1;
-  int64_t b = G * (17 * 8 + 4 * 4 + 1);                     // alloc_per_graph
+  int64_t b = per_graph_bytes(G);                            // alloc_per_graph
+  b += 4 * kCoopScratch + (int64_t)sizeof(Scalars);          // alloc_counters
   b += 8 * 4 * n;                                            // C .. movers
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
   b += 4 * scan_scratch(big);                                // scan32
   b += 2 * 8 * n + (int64_t)sizeof(AbRec) * n;               // W, delta, ab
-  b += 4 * kCoopScratch + 8 * kLevelCounts + (int64_t)sizeof(LevelOut);  // coop, lcounts, lout
+  b += 8 * kLevelCounts + (int64_t)sizeof(LevelOut);         // lcounts, lout
   b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + n;      // bound, off, scan64, M
   b += 8 * (2 * nnz0 > 0 ? 2 * nnz0 : 1);                    // gtab
   if (G > 1) b += 8 * (G + 1) + 4 * n;                       // graph_ptr, gid
-  return b + (int64_t)sizeof(Scalars) + (int64_t)sizeof(GraphStats);
+  return b + (int64_t)sizeof(GraphStats);
 }
 static int64_t level_bytes(int64_t n, int64_t nnz, int64_t G, const BinPlan &p) {
   const int64_t hubs = nnz / (p.hub_min() + 1) + 1, chunks = nnz / p.hub_chunk + hubs;
@@ -366,18 +380,15 @@ int64_t cluster_footprint(int64_t n, int64_t nnz, int count, const lc_opts &o) {
 
 // Degree bins of a level, and the chunk plan of its hub bin (rows longer
 // than the last shared-memory bin are cut into chunks of the plan's hub_chunk edges).
-static int bins_for(Run &r, Level &L) {
+// begin_bins queues the kernel, end_bins takes its counts.
+static int begin_bins(Run &r, Level &L, BinOut **d_out) {
   LC_TRY(r.ar.get(&L.bins.lists, L.g.n));
-  BinOut *d_out = nullptr;
-  LC_TRY(r.ar.get(&d_out, 1));
+  LC_TRY(r.ar.get(d_out, 1));
   LC_TRY(r.ar.get(&L.bins.recs, L.g.n));
-  launch_bins(L.g, L.gid, r.plan, L.bins, d_out, r.coop, r.sc, r.coop_blocks, r.s);
-  BinOut out = L.bin_out;
-  if (!L.bins_known) {
-    LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
-    LC_CK(cudaStreamSynchronize(r.s));
-  }
-  L.bins_known = false;  // a filtered graph's bins are built later on the same level
+  launch_bins(L.g, L.gid, r.plan, L.bins, *d_out, r.coop, r.sc, r.coop_blocks, r.s);
+  return LC_OK;
+}
+static int end_bins(Run &r, Level &L, const BinOut &out) {
   finish_bins(L.bins, out);
   r.res->kernel_launches[LC_K_OTHER] += 1;
   L.hub = Hubs{};
@@ -410,6 +421,17 @@ static int bins_for(Run &r, Level &L) {
     r.res->kernel_launches[LC_K_OTHER] += 1;
   }
   return launch_check();
+}
+static int bins_for(Run &r, Level &L) {
+  BinOut *d_out = nullptr;
+  LC_TRY(begin_bins(r, L, &d_out));
+  BinOut out = L.bin_out;
+  if (!L.bins_known) {
+    LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
+    LC_CK(cudaStreamSynchronize(r.s));
+  }
+  L.bins_known = false;  // a filtered graph's bins are built later on the same level
+  return end_bins(r, L, out);
 }
 
 // Uploads the per-graph constants of a level; active[g] selects the graphs
@@ -766,20 +788,23 @@ static int constrained_passes(Run &r, Level &L, int level, const std::vector<uin
 }
 
 // Per-graph number of labels used by C; also leaves newid (global ascending
-// numbering) and gstart on the device.  begin_count queues the work and the
-// read-back, end_count forms the numbers once the stream has been waited for.
+// numbering) and gstart on the device.  begin_count queues the work,
+// read_count the read-back, end_count forms the numbers once the stream has
+// been waited for.
 struct LabelCount {
   std::vector<int32_t> gs;
   int32_t total = 0;
 };
-static int begin_count(Run &r, Level &L, const int32_t *C, LabelCount &c) {
+static void begin_count(Run &r, const Level &L, const int32_t *C) {
   const int64_t n = L.g.n;
   launch_mark_used(C, n, r.used, r.s);
   launch_number_labels(r.used, n, L.gid, L.gp, nullptr, r.newid, r.gstart, nullptr, r.scan32, r.s);
   r.res->kernel_launches[LC_K_CONTRACT] += 4;
+}
+static int read_count(Run &r, const Level &L, LabelCount &c) {
   c.gs.assign(r.G, 0);
   LC_CK(cudaMemcpyAsync(c.gs.data(), r.gstart, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaMemcpyAsync(&c.total, compact_total(r.scan32, n), 4, cudaMemcpyDeviceToHost, r.s));
+  LC_CK(cudaMemcpyAsync(&c.total, compact_total(r.scan32, L.g.n), 4, cudaMemcpyDeviceToHost, r.s));
   return LC_OK;
 }
 static int64_t end_count(const Run &r, const Level &L, const LabelCount &c, std::vector<int64_t> &nc) {
@@ -795,7 +820,8 @@ static int64_t end_count(const Run &r, const Level &L, const LabelCount &c, std:
 }
 static int count_labels(Run &r, Level &L, const int32_t *C, std::vector<int64_t> &nc, int64_t *total) {
   LabelCount c;
-  LC_TRY(begin_count(r, L, C, c));
+  begin_count(r, L, C);
+  LC_TRY(read_count(r, L, c));
   LC_CK(cudaStreamSynchronize(r.s));
   LC_TRY(launch_check());
   *total = end_count(r, L, c, nc);
@@ -985,8 +1011,9 @@ static int check_graph_args(const lc_csr *g, const int64_t *vw, const int32_t *e
 
 // Statistics, validation and the exactness guards of the header, per graph; C:
 // null, or the clustering whose objective is wanted (lc_objective), which the
-// same pass over the edges sums.
-static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *hst, const int32_t *C = nullptr) {
+// same pass over the edges sums.  begin_prepare queues the kernels,
+// end_prepare waits for them and judges.
+static int begin_prepare(Run &r, const LevelGraph &g, const int32_t *gid, const int32_t *C = nullptr) {
   LC_TRY(r.ar.get(&r.st, 1));
   LC_CK(cudaMemsetAsync(r.st, 0, sizeof(GraphStats), r.s));
   LC_CK(cudaMemsetAsync(&r.st->err_key, 0xFF, sizeof(r.st->err_key), r.s));
@@ -1002,6 +1029,12 @@ static int prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *
     r.prof.end(44.0 * g.n);
     r.res->kernel_launches[LC_K_OBJECTIVE] += 2;
   }
+  return LC_OK;
+}
+// d_out, out: null, or a bin kernel's counts to read back on the way.
+static int end_prepare(Run &r, const LevelGraph &g, const int32_t *gid, GraphStats *hst, const BinOut *d_out = nullptr,
+                       BinOut *out = nullptr) {
+  if (d_out) LC_CK(cudaMemcpyAsync(out, d_out, sizeof(*out), cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaMemcpyAsync(hst, r.st, sizeof(GraphStats), cudaMemcpyDeviceToHost, r.s));
   r.hT.assign(r.G, 0);
   r.hV.assign(r.G, 0);
@@ -1098,10 +1131,33 @@ static int level0(Run &r, Level &L, const LevelGraph &g0, const std::vector<int6
     LC_TRY(r.ar.get(&L.gid, g0.n));
     LC_CK(cudaMemcpyAsync(r.gptr, gptr.data(), 8 * (size_t)(r.G + 1), cudaMemcpyHostToDevice, r.s));
     launch_graph_ids(r.gptr, r.G, L.gid, g0.n, r.s);
-    LC_CK(cudaStreamSynchronize(r.s));
     r.res->kernel_launches[LC_K_OTHER] += 1;
   }
   return LC_OK;
+}
+
+// Everything before the first pass on G_0: statistics, validation and guards,
+// the range of given labels ([0, limit)), scratch and bins.  What the call
+// needs besides is taken and the bins are built while the GPU reads the
+// graph, so that the host waits once; the bin kernel follows nothing but
+// row_ptr's length, so it may run on a graph that turns out to be refused.
+// The graph's faults are reported before a lack of memory.  gptr is read
+// until the wait.
+static int set_up(Run &r, Level &L, const LevelGraph &g0, const std::vector<int64_t> &gptr,
+                  const int32_t *labels = nullptr, int64_t limit = 0) {
+  LC_TRY(alloc_per_graph(r));
+  LC_TRY(level0(r, L, g0, gptr));
+  LC_TRY(begin_prepare(r, g0, L.gid));
+  if (labels) launch_labels_in_range(labels, g0.n, limit, r.st, r.s);
+  BinOut *d_out = nullptr, out{};
+  int rc = alloc_counters(r);
+  if (rc == LC_OK) rc = begin_bins(r, L, &d_out);
+  if (rc == LC_OK) rc = alloc_scratch(r, g0.n, g0.nnz);
+  GraphStats st{};
+  LC_TRY(end_prepare(r, g0, L.gid, &st, rc == LC_OK ? d_out : nullptr, &out));
+  if (st.bad_labels) return LC_ERR_ARG;
+  LC_TRY(rc);
+  return end_bins(r, L, out);
 }
 
 // Algorithm 1 on every graph of the call; labels_out gets each graph's dense
@@ -1109,20 +1165,16 @@ static int level0(Run &r, Level &L, const LevelGraph &g0, const std::vector<int6
 static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t> &gptr,
                         int32_t *labels_out, const int32_t *B0 = nullptr) {
   Phase call_range("lc.cluster");
-  GraphStats st{};
-  LC_TRY(alloc_per_graph(r));
   std::vector<Level> lv(1);
-  LC_TRY(level0(r, lv[0], g0, gptr));
+  LC_TRY(set_up(r, lv[0], g0, gptr));
   lv[0].B = B0;
-  LC_TRY(prepare(r, g0, lv[0].gid, &st));
-  LC_TRY(alloc_scratch(r, g0.n, g0.nnz));
   r.top.assign(r.G, 0);
   int top = 0;
   for (int l = 0;; ++l) {
     if (l >= kMaxLevels) return LC_ERR_TIMEOUT;
     Phase level_range("lc.level");
     Level &L = lv[l];
-    LC_TRY(bins_for(r, L));
+    if (l > 0) LC_TRY(bins_for(r, L));
     std::vector<uint8_t> present(r.G);
     for (int g = 0; g < r.G; ++g) present[g] = L.nv[g] > 0;
     if (L.B)
@@ -1170,10 +1222,14 @@ static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t>
   // for all that is read back
   Level &L0 = lv[0];
   LabelCount count;
-  LC_TRY(begin_count(r, L0, r.C_out, count));
+  begin_count(r, L0, r.C_out);
   launch_relabel(r.C_out, r.newid, labels_out, L0.g.n, L0.gid, r.gstart, nullptr, 1, r.s);
   std::vector<long long> phi;
-  if (r.o.uncoarsen && r.o.pass_limit >= 1 && !B0) {
+  const bool phi_known = r.o.uncoarsen && r.o.pass_limit >= 1 && !B0;
+  // the blocks go back, in stream order, while the GPU still works
+  if (phi_known) r.ar.release_all_but({r.phi_final, r.scan32, r.sc});
+  LC_TRY(read_count(r, L0, count));
+  if (phi_known) {
     // each graph's final clustering is the C_out of its last LocalMovePasses
     // call, at level 0 (the uncoarsening call, or the coarsening call of a
     // graph that stopped there), whose best-of test left its exact Phi
@@ -1263,26 +1319,6 @@ static void end_call(Run &r, int rc) {
   }
 }
 
-// Single-graph set-up shared by the step-level entry points.
-static int single_graph(Run &r, const lc_csr *g, const int64_t *vw, const int32_t *ew, int64_t mu,
-                        int64_t Lam, Level &L, GraphStats *st, const int32_t *C = nullptr) {
-  r.mu.assign(1, mu);
-  r.Lam.assign(1, Lam);
-  LC_TRY(alloc_per_graph(r));
-  LevelGraph g0{g->n, g->nnz, g->row_ptr, g->col, ew, vw};
-  std::vector<int64_t> gptr{0, g->n};
-  LC_TRY(level0(r, L, g0, gptr));
-  return prepare(r, g0, nullptr, st, C);
-}
-
-static int labels_in_range(Run &r, const int32_t *labels, int64_t n, int64_t limit) {
-  launch_labels_in_range(labels, n, limit, r.st, r.s);
-  GraphStats st2{};
-  LC_CK(cudaMemcpyAsync(&st2, r.st, sizeof(st2), cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaStreamSynchronize(r.s));
-  return st2.err_key != ~0ull ? LC_ERR_ARG : LC_OK;
-}
-
 // ----------------------------------------------------------- pLeiden
 
 static int alloc_leiden(Run &r, int64_t n0, LeidenScratch &ls) {
@@ -1322,13 +1358,8 @@ static int alloc_leiden(Run &r, int64_t n0, LeidenScratch &ls) {
 // the coarsening.
 static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t *labels_out) {
   Phase call_range("lc.pleiden");
-  GraphStats st{};
-  LC_TRY(alloc_per_graph(r));
   std::vector<Level> lv(1);
-  LC_TRY(level0(r, lv[0], g0, std::vector<int64_t>{0, g0.n}));
-  LC_TRY(prepare(r, g0, nullptr, &st));
-  if (C0) LC_TRY(labels_in_range(r, C0, g0.n, g0.n));  // initial labels must lie in [0, n)
-  LC_TRY(alloc_scratch(r, g0.n, g0.nnz));
+  LC_TRY(set_up(r, lv[0], g0, std::vector<int64_t>{0, g0.n}, C0, g0.n));  // initial labels must lie in [0, n)
   LeidenScratch ls{};
   LC_TRY(alloc_leiden(r, g0.n, ls));
   int32_t *Ccur = nullptr, *Bd = nullptr, *R = nullptr;
@@ -1347,7 +1378,7 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
     Phase level_range("lc.level");
     Level &L = lv[l];
     const int64_t n = L.g.n;
-    LC_TRY(bins_for(r, L));
+    if (l > 0) LC_TRY(bins_for(r, L));
     LC_TRY(upload_params(r, L, present));
     std::vector<long long> phi_in;
     LC_TRY(objective_of(r, L, Ccur, phi_in));  // leaves the clustering in r.C
@@ -1422,8 +1453,9 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
   }
   Level &L0 = lv[0];
   LabelCount count;
-  LC_TRY(begin_count(r, L0, r.C_out, count));
+  begin_count(r, L0, r.C_out);
   launch_relabel(r.C_out, r.newid, labels_out, L0.g.n, nullptr, r.gstart, nullptr, 1, r.s);
+  LC_TRY(read_count(r, L0, count));
   std::vector<long long> phi;
   LC_TRY(objective_of(r, L0, r.C_out, phi));  // waits
   LC_TRY(check_device_error(r));
@@ -1703,11 +1735,9 @@ int lc_local_move(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_
   if (rc == LC_OK && g->n > 0 && !labels_inout) rc = LC_ERR_ARG;
   if (rc == LC_OK && g->n > 0) {
     Level L;
-    GraphStats st{};
-    rc = single_graph(r, g, vertex_w, edge_w, lambda_num, lambda_den, L, &st);
-    if (rc == LC_OK) rc = labels_in_range(r, labels_inout, g->n, g->n);
-    if (rc == LC_OK) rc = alloc_scratch(r, g->n, g->nnz);
-    if (rc == LC_OK) rc = bins_for(r, L);
+    r.mu.assign(1, lambda_num);
+    r.Lam.assign(1, lambda_den);
+    rc = set_up(r, L, LevelGraph{g->n, g->nnz, g->row_ptr, g->col, edge_w, vertex_w}, {0, g->n}, labels_inout, g->n);
     if (rc == LC_OK) {
       cudaMemcpyAsync(r.C, labels_inout, 4 * g->n, cudaMemcpyDeviceToDevice, r.s);
       rc = local_move_passes(r, L, singleton_start != 0, 0, singleton_start ? 0 : 1,
@@ -1715,15 +1745,19 @@ int lc_local_move(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_
     }
     if (rc == LC_OK) {
       cudaMemcpyAsync(labels_inout, r.C_out, 4 * g->n, cudaMemcpyDeviceToDevice, r.s);
+      begin_count(r, L, labels_inout);
+      // the blocks go back, in stream order, while the GPU still works
+      r.ar.release_all_but({r.phi_final, r.scan32, r.sc});
       long long phi = 0;
+      LabelCount count;
       std::vector<int64_t> nc;
-      int64_t total = 0;
       if (cudaMemcpyAsync(&phi, r.phi_out, 8, cudaMemcpyDeviceToHost, r.s) != cudaSuccess)
         rc = LC_ERR_CUDA;
-      if (rc == LC_OK) rc = count_labels(r, L, labels_inout, nc, &total);
-      if (rc == LC_OK) rc = check_device_error(r);
+      if (rc == LC_OK) rc = read_count(r, L, count);
+      if (rc == LC_OK) rc = check_device_error(r);  // waits
+      if (rc == LC_OK) rc = launch_check();
       if (rc == LC_OK) {
-        res->n_clusters = total;
+        res->n_clusters = end_count(r, L, count, nc);
         res->levels = 1;
         finish_result(r, 0, res, phi);
       }
@@ -1753,11 +1787,9 @@ int lc_contract(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w,
     return cudaStreamSynchronize(r.s) == cudaSuccess ? LC_OK : LC_ERR_CUDA;
   }
   Level L;
-  GraphStats st{};
-  rc = single_graph(r, g, vertex_w, edge_w, 0, 1, L, &st);
-  if (rc == LC_OK) rc = labels_in_range(r, labels, g->n, n_c);
-  if (rc == LC_OK) rc = alloc_scratch(r, g->n, g->nnz);
-  if (rc == LC_OK) rc = bins_for(r, L);
+  r.mu.assign(1, 0);
+  r.Lam.assign(1, 1);
+  rc = set_up(r, L, LevelGraph{g->n, g->nnz, g->row_ptr, g->col, edge_w, vertex_w}, {0, g->n}, labels, n_c);
   if (rc == LC_OK) {
     L.Cd = const_cast<int32_t *>(labels);
     launch_contract_offsets(L.g, L.Cd, n_c, r.bound, r.off, c_vw, r.scan64, r.s);
@@ -1794,9 +1826,13 @@ int lc_objective(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w
   if (rc == LC_OK) rc = check_lambda(lambda_num, lambda_den);
   if (rc == LC_OK && g->n > 0 && !labels) rc = LC_ERR_ARG;
   if (rc == LC_OK && g->n > 0) {
-    Level L;
+    r.mu.assign(1, lambda_num);
+    r.Lam.assign(1, lambda_den);
+    const LevelGraph g0{g->n, g->nnz, g->row_ptr, g->col, edge_w, vertex_w};
     GraphStats st{};
-    rc = single_graph(r, g, vertex_w, edge_w, lambda_num, lambda_den, L, &st, labels);
+    rc = alloc_per_graph(r);
+    if (rc == LC_OK) rc = begin_prepare(r, g0, nullptr, labels);
+    if (rc == LC_OK) rc = end_prepare(r, g0, nullptr, &st);
     if (rc == LC_OK && st.bad_labels) rc = LC_ERR_ARG;
     if (rc == LC_OK) {
       res->n_clusters = st.clusters;

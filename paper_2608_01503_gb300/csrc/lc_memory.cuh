@@ -13,6 +13,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <initializer_list>
 #include <vector>
 
 #include "../../include/lc.h"
@@ -57,6 +59,15 @@ struct Arena {
     if (held > peak) peak = held;
     *out = (T *)p;
     return LC_OK;
+  }
+  // Gives everything back but the blocks that start at one of `keep`.
+  void release_all_but(std::initializer_list<const void *> keep) {
+    for (size_t i = 0; i < ptrs.size(); ++i) {
+      if (!ptrs[i] || std::find(keep.begin(), keep.end(), ptrs[i]) != keep.end()) continue;
+      dev_free(o, s, ptrs[i], sizes[i]);
+      ptrs[i] = nullptr;
+      held -= (int64_t)sizes[i];
+    }
   }
   void release(void *p) {
     for (size_t i = 0; i < ptrs.size(); ++i)

@@ -321,7 +321,7 @@ __global__ void k_labels_in_range(const int32_t *__restrict__ C, int64_t n, int6
                                   GraphStats *st) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x)
-    if (C[v] < 0 || C[v] >= limit) report(st, LC_ERR_ARG, v);
+    if (C[v] < 0 || C[v] >= limit) st->bad_labels = 1;  // whoever comes last, the same value
 }
 
 void launch_stats(const LevelGraph &g, int validate, GraphStats *st, const int32_t *gid, const int64_t *gptr,

@@ -29,7 +29,7 @@ void launch_stats(const LevelGraph &g, int validate, GraphStats *st, const int32
 // and the ids in use, with W and used (both [n]) as scratch.
 void launch_label_stats(const LevelGraph &g, const int32_t *C, int64_t *W, int32_t *used, GraphStats *st,
                         cudaStream_t s);
-// Reports LC_ERR_ARG for any label outside [0, limit).
+// Sets bad_labels if any label lies outside [0, limit).
 void launch_labels_in_range(const int32_t *C, int64_t n, int64_t limit, GraphStats *st,
                             cudaStream_t s);
 

@@ -1,6 +1,8 @@
 """The edge checks name the row of a fault wherever it lies: dense rows, rows
 that end on the check's step and run boundaries, and entries with thousands of
 empty rows between them; unaligned arrays take the scalar loads."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -69,3 +71,33 @@ def test_fault_is_reported_with_its_row(name, offset):
             bad = col.copy()
             bad[at] = bad[at - 1]
             assert check(rp, bad, ew, offset) == (4, row[at])  # duplicate
+
+
+@pytest.mark.parametrize("limit,code_ok", [(0, 0), (100_000, 7)])
+def test_faults_of_the_graph_and_labels_come_before_memory(limit, code_ok):
+    """Scratch is taken while the graph is still being read: a self-loop is
+    reported before bad labels, both before a scratch limit that is too low,
+    and the device holds what it held before."""
+    n = 4000
+    rp = np.arange(0, 2 * n + 2, 2)
+    ring = np.stack(((np.arange(n) - 1) % n, (np.arange(n) + 1) % n), 1)
+    col = np.sort(ring, 1).astype(np.int32).ravel()
+    loop = col.copy()
+    loop[2 * 700] = 700  # row 700: {699, 701} -> {700, 701}
+    good, bad = np.zeros(n, np.int32), np.full(n, n, np.int32)
+
+    def code(c, labels):
+        a = [torch.from_numpy(x).cuda() for x in (rp, c, np.ones(2 * n, np.int32), np.ones(n, np.int64))]
+        lab = torch.from_numpy(labels).cuda()
+        gc.collect()  # what earlier tests left must not be freed in between
+        base = torch.cuda.memory_allocated()
+        try:
+            lc.lc_local_move(*a, 1, 2, lab, opts=lc.Options(scratch_limit=limit))
+            got = 0
+        except lc.LCError as e:
+            got = e.code
+        assert torch.cuda.memory_allocated() == base
+        return got
+
+    assert code(loop, bad) == 3 and code(col, bad) == 1 and code(loop, good) == 3
+    assert code(col, good) == code_ok
