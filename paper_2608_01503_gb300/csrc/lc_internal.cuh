@@ -269,10 +269,18 @@ __device__ __forceinline__ bool better(long long g1, int32_t x1, long long g2, i
 // Lam is near the exactness guards, one 64-bit division replaces the far
 // costlier 128-bit one.  Either way the quotient is exact.
 __device__ __forceinline__ long long eps_bucket(const Method &m, long long Lam, long long delta) {
+  const long long n64 = (long long)m.eps_den * delta, d64 = (long long)m.eps_num * Lam;
+  // 32-bit operands: a third of the 64-bit division's work
+  const unsigned long long abs64 = (unsigned long long)(n64 < 0 ? -n64 : n64);
+  if (delta == (long long)(int32_t)delta && ((abs64 | (unsigned long long)d64) >> 32) == 0 &&
+      Lam == (long long)(int32_t)Lam) {
+    const uint32_t n32 = (uint32_t)abs64, d32 = (uint32_t)d64;
+    const uint32_t q = n32 / d32;
+    return n64 < 0 ? -(long long)q - (q * d32 != n32 ? 1 : 0) : (long long)q;
+  }
   const __int128 num = (__int128)m.eps_den * delta;
   const __int128 den = (__int128)m.eps_num * Lam;
-  if (num == (__int128)(long long)num && den == (__int128)(long long)den) {
-    const long long n64 = (long long)num, d64 = (long long)den;
+  if (num == (__int128)n64 && den == (__int128)d64) {
     long long q = n64 / d64;  // truncates toward zero
     if (q * d64 != n64 && n64 < 0) q -= 1;
     return q;

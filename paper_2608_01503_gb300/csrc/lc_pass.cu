@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(256, 4) k_ab_thread(PassArgs a, const VRec *__
   UpdateSums sum;
   // warp-uniform trip count: the update's lists are appended per warp
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < count; base += (int64_t)gridDim.x * blockDim.x)
-    ab_thread(a, base + threadIdx.x < count, rec, base + threadIdx.x, sum);
+    ab_thread<8>(a, base + threadIdx.x < count, rec, base + threadIdx.x, sum);
   flush_update(a, sum);
   step_end();
 }
