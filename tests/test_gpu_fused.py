@@ -93,3 +93,20 @@ def test_batch_of_mixed_graphs():
         ref, orc, _ = oracle.louvain_plus(g)
         lo, hi = p["graph_ptr"][k], p["graph_ptr"][k + 1]
         assert np.array_equal(got[lo:hi], ref) and res[k]["phi"] == orc["phi"], k
+
+
+@pytest.mark.parametrize("lam", [(1, 60_000), (7, 200_003), (1, 1_000_003)])
+def test_gains_on_both_sides_of_32_bits(lam):
+    """Edge weights up to 2^15 under lambda denominators that take the gains,
+    their differences and the epsilon buckets' operands across 2^31 and 2^32,
+    where the 32-bit forms hand over."""
+    n, m = 1500, 12_000
+    rng = np.random.default_rng(9)
+    s, t = rng.integers(0, n, m), rng.integers(0, n, m)
+    g = gg.cpm_inputs(*gg.from_edges(n, s[s != t], t[s != t], seed=9, wmin=1, wmax=1 << 15), *lam)
+    args = (dev(g.row_ptr), dev(g.col), dev(g.ew), dev(g.vw), g.lam_num, g.lam_den)
+    a, ra = lc.lc_cluster(*args)
+    b, rb = lc.lc_cluster(*args, opts=lc.Options(profile=True))
+    ref, orc, _ = oracle.louvain_plus(g)
+    assert np.array_equal(a.cpu().numpy(), ref) and ra["phi"] == orc["phi"]
+    assert torch.equal(a, b) and ra["phi"] == rb["phi"]
