@@ -3,6 +3,7 @@
 // (Algorithm 5).  LocalMovePasses and the contraction are the Louvain+
 // kernels.
 #include <climits>
+#include <type_traits>
 #include <utility>
 
 #include "lc_group.cuh"
@@ -10,6 +11,7 @@
 #include "lc_move.cuh"
 #include "lc_pass.cuh"
 #include "lc_scan.cuh"
+#include "lc_step.cuh"
 
 namespace lc {
 
@@ -154,18 +156,46 @@ __device__ __forceinline__ bool edge_ok(const GraphParam &P, int32_t w, long lon
   return P.Lam * (long long)w - P.mu * wu * wv >= 0;
 }
 
-// The per-vertex refinement kernels take the level's degree bins: one
-// thread per vertex up to degree 32 (GS = 1), one warp above (GS = 32).
+// The per-vertex refinement kernels take the level's degree bins (ref_rows
+// below): a thread, 16 lanes, a warp or a block per vertex, four edges each in
+// flight, since their walks are chains of gathers.  With a thread up to degree
+// 32 and a warp above, one edge at a time, the longest row of an R-MAT graph
+// of scale 18 kept one warp busy for most of each kernel.
 
+// The smallest (key, id) over the group.
 template <int GS>
-__device__ __forceinline__ long long grp_sum(long long x) {
-  if constexpr (GS == 1) return x;
-  else return warp_sum(x);
+__device__ __forceinline__ void grp_min_key(uint64_t &x, int32_t &h) {
+  constexpr int L = GS < 32 ? GS : 32;
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) {
+    const uint64_t ox = __shfl_xor_sync(0xFFFFFFFFu, x, o);
+    const int32_t oh = __shfl_xor_sync(0xFFFFFFFFu, h, o);
+    if (key_less(ox, oh, x, h)) {
+      x = ox;
+      h = oh;
+    }
+  }
+  if constexpr (GS > 32) {
+    __shared__ uint64_t rk[GS / 32];
+    __shared__ int32_t rh[GS / 32];
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+      rk[threadIdx.x >> 5] = x;
+      rh[threadIdx.x >> 5] = h;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < GS / 32; ++w)
+      if (key_less(rk[w], rh[w], x, h)) {
+        x = rk[w];
+        h = rh[w];
+      }
+  }
 }
 
 // S(v, B[v]), membership of U, and the key f(v).
 template <int GS>
-__global__ void __launch_bounds__(kThreads) k_ref_self(LevelGraph g, const GraphParam *gp,
+__global__ void __launch_bounds__(GS > 32 ? GS : kThreads) k_ref_self(LevelGraph g, const GraphParam *gp,
                                                        const int32_t *__restrict__ list, int64_t count,
                                                        const int32_t *__restrict__ B,
                                                        const int64_t *__restrict__ WB,
@@ -173,15 +203,18 @@ __global__ void __launch_bounds__(kThreads) k_ref_self(LevelGraph g, const Graph
                                                        uint64_t *__restrict__ f, RefRec *__restrict__ rec,
                                                        uint32_t seed, int32_t level) {
   const GraphParam P = gp[0];
+  __shared__ long long red[Grp<GS>::kWarps];
   const int r = Grp<GS>::rank();
+  step_begin();
   for_each_vertex<GS>(count, [&](int64_t i, bool active) {
     const int32_t v = active ? list[i] : 0;
     const int32_t Bv = active ? B[v] : 0;
     const int64_t beg = active ? g.rp[v] : 0, end = active ? g.rp[v + 1] : 0;
     long long sb = 0;
+#pragma unroll 4
     for (int64_t e = beg + r; e < end; e += GS)
       if (B[__ldg(g.col + e)] == Bv) sb += __ldg(g.ew + e);
-    sb = grp_sum<GS>(sb);
+    sb = Grp<GS>::sum(sb, red);
     if (active && r == 0) {
       const long long wv = g.vw[v];
       const bool inU = P.Lam * sb - P.mu * wv * (WB[Bv] - wv) >= 0;
@@ -191,19 +224,21 @@ __global__ void __launch_bounds__(kThreads) k_ref_self(LevelGraph g, const Graph
       rec[v] = RefRec{Bv, inU ? 1 : 0, wv};
     }
   });
+  step_end();
 }
 
 // ChooseRandom: among v itself and the qualifying neighbours, the
 // candidate c with the smallest (rand(v << 32 | c), c) of stream 0 --
 // uniform, and independent of the order of the row.
 template <int GS>
-__global__ void __launch_bounds__(kThreads) k_ref_choose(LevelGraph g, const GraphParam *gp,
+__global__ void __launch_bounds__(GS > 32 ? GS : kThreads) k_ref_choose(LevelGraph g, const GraphParam *gp,
                                                          const int32_t *__restrict__ list, int64_t count,
                                                          const RefRec *__restrict__ rec,
                                                          int32_t *__restrict__ H, uint32_t seed,
                                                          int32_t level) {
   const GraphParam P = gp[0];
   const int r = Grp<GS>::rank();
+  step_begin();
   for_each_vertex<GS>(count, [&](int64_t i, bool active) {
     const int32_t v = active ? list[i] : 0;
     const RefRec rv = active ? rec[v] : RefRec{0, 0, 0};
@@ -212,7 +247,9 @@ __global__ void __launch_bounds__(kThreads) k_ref_choose(LevelGraph g, const Gra
     int32_t h = v;
     if (inU) {
       best = stream_rand(seed, level, 0, ((int64_t)v << 32) | v);
-      for (int64_t e = g.rp[v] + r; e < g.rp[v + 1]; e += GS) {
+      const int64_t end = g.rp[v + 1];
+#pragma unroll 4
+      for (int64_t e = g.rp[v] + r; e < end; e += GS) {
         const int32_t u = __ldg(g.col + e);
         const RefRec ru = rec[u];  // one gather: B[u], u in U, w(u)
         if (ru.inU && ru.B == rv.B && edge_ok(P, __ldg(g.ew + e), ru.w, rv.w)) {
@@ -224,19 +261,10 @@ __global__ void __launch_bounds__(kThreads) k_ref_choose(LevelGraph g, const Gra
         }
       }
     }
-    if constexpr (GS > 1) {
-#pragma unroll
-      for (int o = GS / 2; o > 0; o >>= 1) {
-        const uint64_t ob = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-        const int32_t oh = __shfl_xor_sync(0xFFFFFFFFu, h, o);
-        if (ob < best || (ob == best && oh < h)) {
-          best = ob;
-          h = oh;
-        }
-      }
-    }
+    grp_min_key<GS>(best, h);
     if (active && r == 0) H[v] = inU ? h : v;
   });
+  step_end();
 }
 
 __global__ void k_ref_keep(const int32_t *__restrict__ H, const uint64_t *__restrict__ f,
@@ -312,27 +340,31 @@ __global__ void k_ref_check_roots(const int32_t *__restrict__ root, const uint64
 // Weight to the earlier vertices of the tree (same root, smaller key) and
 // the vertex's term of w(C, B minus C) along the tree order.
 template <int GS>
-__global__ void __launch_bounds__(kThreads) k_ref_sv(LevelGraph g, const int32_t *__restrict__ list,
+__global__ void __launch_bounds__(GS > 32 ? GS : kThreads) k_ref_sv(LevelGraph g, const int32_t *__restrict__ list,
                                                      int64_t count, const KeyRec *__restrict__ krec,
                                                      const int64_t *__restrict__ SB,
                                                      int64_t *__restrict__ Sv, int64_t *__restrict__ tv) {
+  __shared__ long long red[Grp<GS>::kWarps];
   const int r = Grp<GS>::rank();
+  step_begin();
   for_each_vertex<GS>(count, [&](int64_t i, bool active) {
     const int32_t v = active ? list[i] : 0;
     const KeyRec kv = active ? krec[v] : KeyRec{0, 0, 0};
     const int64_t beg = active ? g.rp[v] : 0, end = active ? g.rp[v + 1] : 0;
     long long s = 0;
+#pragma unroll 4
     for (int64_t e = beg + r; e < end; e += GS) {
       const int32_t u = __ldg(g.col + e);
       const KeyRec ku = krec[u];  // one gather: root and key of u
       if (ku.root == kv.root && key_less(ku.f, u, kv.f, v)) s += __ldg(g.ew + e);
     }
-    s = grp_sum<GS>(s);
+    s = Grp<GS>::sum(s, red);
     if (active && r == 0) {
       Sv[v] = s;
       tv[v] = SB[v] - 2 * s;
     }
   });
+  step_end();
 }
 
 // ------------------------------------------- LSD radix sort (8-bit digits)
@@ -603,25 +635,44 @@ void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C
 
 int64_t radix_hist_len(int64_t n) { return 256 * ((n + kRadixTile - 1) / kRadixTile) + 256; }
 
+// One refinement kernel over all rows: launch(threads per vertex, step, range,
+// blocks, threads per block) for each group of bins that has rows.
+template <typename Launch>
+static void ref_rows(const Bins &bins, cudaStream_t s, Launch launch) {
+  Step st(s);
+  const auto group = [&](auto gs, int lo, int hi) {
+    const BinRange r = bin_range(bins, lo, hi);
+    if (r.count > 0)
+      launch(gs, st, r, ld_grid(r.count, gs() > 32 ? 1 : kThreads / gs()), gs() > 32 ? gs() : kThreads);
+  };
+  group(std::integral_constant<int, 1>{}, 0, 0);
+  group(std::integral_constant<int, 16>{}, 1, 2);
+  group(std::integral_constant<int, 32>{}, 3, 4);
+  group(std::integral_constant<int, 128>{}, 5, 6);
+  group(std::integral_constant<int, 512>{}, 7, kBins - 1);
+}
+
 void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphParam *gp, const int32_t *B,
                            uint32_t seed, int32_t level, int32_t *R, LeidenScratch &ls, int *error,
                            cudaStream_t s) {
   const int64_t n = g.n;
   if (n == 0) return;
   const unsigned gt = ld_grid(n, 256);
-  const BinRange lo = bin_range(bins, 0, 2), hi = bin_range(bins, 3, kBins - 1);
-  const unsigned glo = ld_grid(lo.count, 256), ghi = ld_grid(hi.count, kWarps);
-  if (lo.count) k_ref_self<1><<<glo, kThreads, 0, s>>>(g, gp, lo.list, lo.count, B, ls.WB, ls.SB, ls.flags, ls.f, ls.rec, seed, level);
-  if (hi.count) k_ref_self<32><<<ghi, kThreads, 0, s>>>(g, gp, hi.list, hi.count, B, ls.WB, ls.SB, ls.flags, ls.f, ls.rec, seed, level);
-  if (lo.count) k_ref_choose<1><<<glo, kThreads, 0, s>>>(g, gp, lo.list, lo.count, ls.rec, ls.H, seed, level);
-  if (hi.count) k_ref_choose<32><<<ghi, kThreads, 0, s>>>(g, gp, hi.list, hi.count, ls.rec, ls.H, seed, level);
+  ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
+    st.run(false, k_ref_self<gs()>, blocks, threads, 0, g, gp, r.list, r.count, B, ls.WB, ls.SB, ls.flags, ls.f,
+           ls.rec, seed, level);
+  });
+  ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
+    st.run(false, k_ref_choose<gs()>, blocks, threads, 0, g, gp, r.list, r.count, ls.rec, ls.H, seed, level);
+  });
   k_ref_keep<<<gt, 256, 0, s>>>(ls.H, ls.f, ls.flags, n);
   k_ref_fix<<<gt, 256, 0, s>>>(ls.H, ls.f, ls.flags, n);
   k_ref_parent<<<gt, 256, 0, s>>>(ls.H, ls.f, ls.flags, ls.first_bad, n);  // parents
   k_ref_roots<<<gt, 256, 0, s>>>(ls.first_bad, ls.root, n, error);
   k_ref_check_roots<<<gt, 256, 0, s>>>(ls.root, ls.f, ls.krec, n, error);
-  if (lo.count) k_ref_sv<1><<<glo, kThreads, 0, s>>>(g, lo.list, lo.count, ls.krec, ls.SB, ls.Sv, ls.tv);
-  if (hi.count) k_ref_sv<32><<<ghi, kThreads, 0, s>>>(g, hi.list, hi.count, ls.krec, ls.SB, ls.Sv, ls.tv);
+  ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
+    st.run(false, k_ref_sv<gs()>, blocks, threads, 0, g, r.list, r.count, ls.krec, ls.SB, ls.Sv, ls.tv);
+  });
   // the vertices of multi-vertex trees, ordered by (f, id) and then by
   // (root, rank): trees contiguous, keys ascending within each tree
   cudaMemsetAsync(ls.size, 0, sizeof(int32_t) * (size_t)n, s);

@@ -72,7 +72,7 @@ void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C
                            cudaStream_t s);
 // pLeidenR (Algorithm 6) with constraint B (dense labels in [0, n)): refined
 // labels R (tree root ids, or the vertex itself).  bins: the level's degree
-// bins (per-vertex kernels use a thread up to degree 32, a warp above).
+// bins.
 struct Bins;
 void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphParam *gp, const int32_t *B,
                            uint32_t seed, int32_t level, int32_t *R, LeidenScratch &ls, int *error,

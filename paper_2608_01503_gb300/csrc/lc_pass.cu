@@ -412,6 +412,7 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_afterburner(PassArgs a) {
 template <int GS>
 __global__ void __launch_bounds__(GS > 32 ? GS : 256)
     k_objective(PassArgs a, const int32_t *__restrict__ list, int64_t count) {
+  step_begin();
   __shared__ long long rs[GS > 32 ? GS / 32 : 1];
   long long phi = 0;
   const int r = Grp<GS>::rank();
@@ -436,9 +437,11 @@ __global__ void __launch_bounds__(GS > 32 ? GS : 256)
       phi_add_one(a, a.phi_acc, g, gC, phi);
   });
   flush_block_sum(phi, &a.phi_acc[0]);
+  step_end();
 }
 
 __global__ void __launch_bounds__(kHubThreads) k_hub_objective(PassArgs a) {
+  step_begin();
   const int c = blockIdx.x;
   const int h = a.hub.hub_of[c];
   const int32_t Cv = a.C[a.hub.vtx[h]];
@@ -447,6 +450,7 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_objective(PassArgs a) {
   for (int64_t e = a.hub.e0[c] + threadIdx.x; e < a.hub.e1[c]; e += kHubThreads)
     if (a.C[LC_IDX(__ldg(a.g.col + e), a.g.n, kDbgColumn)] == Cv) self += __ldg(a.g.ew + e);
   hub_acc_add(a, h, self);
+  step_end();
 }
 
 __global__ void k_hub_obj_final(PassArgs a) {
@@ -848,17 +852,6 @@ class PassStep : public Step {
   }
 };
 
-// The same over the plain vertex list (kernels that need little of a record).
-template <int GS>
-static int launch_list_kernel(void (*k)(PassArgs, const int32_t *, int64_t), const PassArgs &a, BinRange r,
-                              cudaStream_t s) {
-  if (r.count <= 0) return 0;
-  const int threads = GS > 32 ? GS : 256;
-  const int per_block = GS > 32 ? 1 : threads / GS;
-  k<<<blocks_for(r.count, per_block), threads, 0, s>>>(a, r.list, r.count);
-  return 1;
-}
-
 static inline unsigned hub_final_blocks(int H) { return blocks_for(H, 256); }
 
 // Kernels without tables take runs of bins: bin 0 -> 1 thread, 1 -> 16
@@ -986,18 +979,20 @@ int launch_symmetry_ablation(const PassArgs &a, bool mlh, int32_t *size, cudaStr
 }
 
 int launch_objective(const PassArgs &a, const Bins &b, cudaStream_t s) {
-  int n = 0;
-  n += launch_list_kernel<1>(k_objective<1>, a, bin_range(b, 0, 0), s);
-  n += launch_list_kernel<16>(k_objective<16>, a, bin_range(b, 1, 1), s);
-  n += launch_list_kernel<32>(k_objective<32>, a, bin_range(b, 2, 4), s);
-  n += launch_list_kernel<128>(k_objective<128>, a, bin_range(b, 5, 6), s);
-  n += launch_list_kernel<512>(k_objective<512>, a, bin_range(b, 7, 8), s);
+  PassStep st(s);
+  const auto rows = [&](void (*k)(PassArgs, const int32_t *, int64_t), int threads, int per_block, BinRange r) {
+    if (r.count > 0) st.run(false, k, blocks_for(r.count, per_block), threads, 0, a, r.list, r.count);
+  };
+  rows(k_objective<1>, 256, 256, bin_range(b, 0, 0));
+  rows(k_objective<16>, 256, 16, bin_range(b, 1, 1));
+  rows(k_objective<32>, 256, 8, bin_range(b, 2, 4));
+  rows(k_objective<128>, 128, 1, bin_range(b, 5, 6));
+  rows(k_objective<512>, 512, 1, bin_range(b, 7, 8));
   if (a.hub.H > 0) {
-    k_hub_objective<<<a.hub.Q, kHubThreads, 0, s>>>(a);
-    k_hub_obj_final<<<hub_final_blocks(a.hub.H), 256, 0, s>>>(a);
-    n += 2;
+    st.run(false, k_hub_objective, a.hub.Q, kHubThreads, 0, a);
+    st.run(true, k_hub_obj_final, hub_final_blocks(a.hub.H), 256, 0, a);
   }
-  return n;
+  return st.launches;
 }
 
 // ------------------------- objective after the last pass (one graph)
