@@ -15,7 +15,6 @@
 #include <cstring>
 #include <deque>
 #include <mutex>
-#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -165,7 +164,7 @@ struct Level {
   Bins bins{};
   Hubs hub{};
   int64_t max_deg = 0;               // longest hub row (0: no hub)
-  BinOut bin_out{};                  // of the full graph, if known before its bins are built
+  BinOut bin_out{};                  // of the full graph, whose lists a small level's end has built
   bool bins_known = false;
   int32_t *gid = nullptr;            // [n] graph of each vertex (nullptr: one graph)
   GraphParam *gp = nullptr;          // [G] device
@@ -249,31 +248,36 @@ static cudaStream_t capture_stream() {
 
 static int64_t per_graph_bytes(int64_t G) { return G * (17 * 8 + 4 * 4 + 1); }
 
+// The next `count` elements of a block that p walks through (largest
+// alignment first).
+template <typename T>
+static T *cut(uint8_t *&p, int64_t count) {
+  T *at = reinterpret_cast<T *>(p);
+  p += count * (int64_t)sizeof(T);
+  return at;
+}
+
 // The per-graph arrays, one block cut up in order of element size: a provider
 // call costs 2 to 4 us (PyTorch's allocator through a callback).
 static int alloc_per_graph(Run &r) {
   const int64_t G = r.G;
   uint8_t *p = nullptr;
   LC_TRY(r.ar.get(&p, per_graph_bytes(G)));
-  const auto cut = [&](auto **out, int64_t count) {
-    *out = reinterpret_cast<std::remove_reference_t<decltype(**out)> *>(p);
-    p += count * (int64_t)sizeof(**out);
-  };
-  cut(&r.phi_final, G);  // the first four are zeroed: a graph with no vertices has Phi = 0
-  cut(&r.Tg, G);
-  cut(&r.Vg, G);
-  cut(&r.sw2g, G);
+  r.phi_final = cut<long long>(p, G);  // the first four are zeroed: a graph with no vertices has Phi = 0
+  r.Tg = cut<long long>(p, G);
+  r.Vg = cut<long long>(p, G);
+  r.sw2g = cut<long long>(p, G);
   LC_CK(cudaMemsetAsync(r.phi_final, 0, 4 * 8 * (size_t)G, r.s));
-  cut(&r.phi_acc, G);
-  cut(&r.phi_out, G);
-  cut(&r.phi_trace, G);
-  cut(&r.obj, 4 * G);
-  cut(&r.fused, 6 * G);
-  cut(&r.improved, G);
-  cut(&r.gstart, G);
-  cut(&r.gfree, G);
-  cut(&r.gmover, G);
-  cut(&r.keep, G);
+  r.phi_acc = cut<long long>(p, G);
+  r.phi_out = cut<long long>(p, G);
+  r.phi_trace = cut<long long>(p, G);
+  r.obj = cut<long long>(p, 4 * G);
+  r.fused = cut<long long>(p, 6 * G);
+  r.improved = cut<int>(p, G);
+  r.gstart = cut<int32_t>(p, G);
+  r.gfree = cut<int32_t>(p, G);
+  r.gmover = cut<int32_t>(p, G);
+  r.keep = cut<uint8_t>(p, G);
   return LC_OK;
 }
 
@@ -423,14 +427,14 @@ static int end_bins(Run &r, Level &L, const BinOut &out) {
   return launch_check();
 }
 static int bins_for(Run &r, Level &L) {
-  BinOut *d_out = nullptr;
-  LC_TRY(begin_bins(r, L, &d_out));
-  BinOut out = L.bin_out;
-  if (!L.bins_known) {
-    LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
-    LC_CK(cudaStreamSynchronize(r.s));
+  if (L.bins_known) {
+    L.bins_known = false;  // a filtered graph's bins are built later on the same level
+    return end_bins(r, L, L.bin_out);
   }
-  L.bins_known = false;  // a filtered graph's bins are built later on the same level
+  BinOut *d_out = nullptr, out{};
+  LC_TRY(begin_bins(r, L, &d_out));
+  LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
+  LC_CK(cudaStreamSynchronize(r.s));
   return end_bins(r, L, out);
 }
 
@@ -881,14 +885,17 @@ static bool use_small_level(const Run &r, const Level &L) {
 static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   Phase range("lc.contract");
   LC_TRY(r.ar.get(&L.Cd, L.g.n));
-  const LevelScratch w{r.used, r.newid, r.cnt, r.bound, r.off, r.W, r.delta, r.gtab, r.gfree, r.lcounts};
+  // the passes are over: their records' space holds the labels' weights
+  const LevelScratch w{r.used,  r.newid, r.cnt,  r.bound, reinterpret_cast<int64_t *>(r.ab), r.off, r.W,
+                       r.delta, r.gtab,  r.gfree, r.lcounts};
   launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.sc, r.coop_blocks, r.s);
   LevelOut out{};
   std::vector<int32_t> nc(r.G);
   LC_CK(cudaMemcpyAsync(&out, r.lout, sizeof(out), cudaMemcpyDeviceToHost, r.s));
-  LC_CK(cudaMemcpyAsync(nc.data(), w.nc, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
+  if (r.G > 1) LC_CK(cudaMemcpyAsync(nc.data(), w.nc, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaStreamSynchronize(r.s));
   LC_TRY(launch_check());
+  if (r.G == 1) nc[0] = (int32_t)(out.n_c > 0 ? out.n_c : L.g.n);
   r.res->kernel_launches[LC_K_CONTRACT] += 1;
   L.cont.assign(r.G, 0);
   N.vbase.assign(r.G, 0);
@@ -908,14 +915,18 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   *any = base > 0;
   if (!*any) return LC_OK;
   if (base != out.n_c) return LC_ERR_DEVICE;
-  int64_t *rp_c = nullptr, *vw_c = nullptr;
+  // the GPU waits for these: one block for what is sized by the vertices
+  uint8_t *p = nullptr;
+  LC_TRY(r.ar.get(&p, (int64_t)(sizeof(VRec) + 8 + 8 + 4 + (r.G > 1 ? 4 : 0)) * out.n_c + 8));
+  N.bins.recs = cut<VRec>(p, out.n_c);
+  int64_t *rp_c = cut<int64_t>(p, out.n_c + 1), *vw_c = cut<int64_t>(p, out.n_c);
+  N.bins.lists = cut<int32_t>(p, out.n_c);
+  if (r.G > 1) N.gid = cut<int32_t>(p, out.n_c);
   int32_t *col_c = nullptr, *ew_c = nullptr;
-  LC_TRY(r.ar.get(&rp_c, out.n_c + 1));
-  LC_TRY(r.ar.get(&vw_c, out.n_c));
-  if (r.G > 1) LC_TRY(r.ar.get(&N.gid, out.n_c));
   LC_TRY(r.ar.get(&col_c, out.nnz_c));
   LC_TRY(r.ar.get(&ew_c, out.nnz_c));
-  launch_level_build(L.g, L.gid, L.Cd, w, out, rp_c, col_c, ew_c, vw_c, N.gid, r.sc, r.coop_blocks, r.s);
+  launch_level_build(L.g, L.gid, L.Cd, w, out, rp_c, col_c, ew_c, vw_c, N.gid, bin_work(r.plan, N.bins, r.coop), r.sc,
+                     r.coop_blocks, r.s);
   r.res->kernel_launches[LC_K_CONTRACT] += 1;
   r.res->edges_contract += L.g.nnz;
   N.g = LevelGraph{out.n_c, out.nnz_c, rp_c, col_c, ew_c, vw_c};

@@ -1,8 +1,7 @@
 // lc_bins.cu — the degree bins of a level (Section IV-C-2's buckets): the
 // vertices of each bin in ascending order with their records, and the chunk
 // plan of the hub bin.
-#include "lc_bins.cuh"
-#include "lc_coop.cuh"
+#include "lc_bins_dev.cuh"
 
 namespace lc {
 
@@ -12,22 +11,11 @@ constexpr int kT = kCoopThreads, kW = kT / 32;
 
 struct BinArgs {
   LevelGraph g;
-  const int32_t *gid;         // graph of each vertex (nullptr: one graph)
-  int32_t max_deg[kBins - 1];
-  int32_t hub_chunk;
-  VRec *recs;
-  int32_t *lists;
+  const int32_t *gid;  // graph of each vertex (nullptr: one graph)
+  BinWork w;
   BinOut *out;
-  int32_t *counts;            // [kBins][kCoopBlocks]
   Scalars *sc;
 };
-
-__device__ __forceinline__ int bin_of(const BinArgs &a, int64_t deg) {
-  int b = 0;
-#pragma unroll
-  for (int k = 0; k < kBins - 1; ++k) b += deg > a.max_deg[k] ? 1 : 0;
-  return b;
-}
 
 // One cooperative launch: every block counts the bins of its run of vertices,
 // and once all have met, places them.  Bound by the records it writes: 52
@@ -35,125 +23,21 @@ __device__ __forceinline__ int bin_of(const BinArgs &a, int64_t deg) {
 // separate pass for the records took 0.35 ms at 912,673 vertices and 70 us,
 // all launches, on 10,000; this takes 30 us and 8 us.
 __global__ void __launch_bounds__(kT, 1) k_bins(const __grid_constant__ BinArgs a) {
-  __shared__ int32_t s_cnt[kBins], s_run[kBins];
-  __shared__ int32_t s_w[kW][kBins + 1];
-  __shared__ long long s_chunks;
-  __shared__ int32_t s_max;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t n = a.g.n;
-  const int64_t per = ((n + gridDim.x - 1) / gridDim.x + kT - 1) / kT * kT;
-  const int64_t lo = (int64_t)blockIdx.x * per, hi = lo + per < n ? lo + per : n;
+  const int64_t *__restrict__ rp = a.g.rp;
   GridBarrier bar(a.sc);
-  if (threadIdx.x < kBins) s_cnt[threadIdx.x] = 0;
-  if (threadIdx.x == 0) {
-    s_chunks = 0;
-    s_max = 0;
-  }
-  __syncthreads();
-  {
-    int cnt[kBins] = {};
-    long long chunks = 0;
-    int32_t longest = 0;
-    for (int64_t v = lo + threadIdx.x; v < hi; v += kT) {
-      const int64_t deg = a.g.rp[v + 1] - a.g.rp[v];
-      const int b = bin_of(a, deg);
-#pragma unroll
-      for (int k = 0; k < kBins; ++k) cnt[k] += b == k;
-      if (b == kHubBin) {
-        chunks += (deg + a.hub_chunk - 1) / a.hub_chunk;
-        longest = deg > longest ? (int32_t)deg : longest;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kBins; ++k) {
-      const int t = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)cnt[k]);
-      if (lane == 0 && t) atomicAdd(&s_cnt[k], t);
-    }
-    if (longest > 0) {
-      atomicAdd((unsigned long long *)&s_chunks, (unsigned long long)chunks);
-      atomicMax(&s_max, longest);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < kBins) a.counts[threadIdx.x * kCoopBlocks + blockIdx.x] = s_cnt[threadIdx.x];
-  if (threadIdx.x == 0 && s_max > 0) {
-    atomicAdd((unsigned long long *)&a.out->chunks, (unsigned long long)s_chunks);
-    atomicMax(&a.out->max_deg, s_max);
-  }
+  bins_count<kT>(a.w, a.g.n, a.out, [&](int64_t v) { return rp[v + 1] - rp[v]; });
   if (!bar.sync()) return;
-  // a bin per warp: its total and what the blocks before this one hold
-  if (wid < kBins) {
-    int total = 0, before = 0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) {
-      const int c = a.counts[wid * kCoopBlocks + b];
-      total += c;
-      before += b < (int)blockIdx.x ? c : 0;
-    }
-    total = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)total);
-    before = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)before);
-    if (lane == 0) {
-      s_cnt[wid] = total;
-      s_run[wid] = before;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int at = 0;
-    for (int k = 0; k < kBins; ++k) {
-      s_run[k] += at;
-      if (blockIdx.x == 0) a.out->offs[k] = at;
-      at += s_cnt[k];
-    }
-    if (blockIdx.x == 0) a.out->offs[kBins] = at;
-  }
-  __syncthreads();
-  for (int64_t base = lo; base < hi; base += kT) {
-    const int64_t v = base + threadIdx.x;
+  bins_place<kT>(a.w, a.g.n, a.out, [&](int64_t v) {
     VRec r{};
-    int b = kBins;
-    if (v < hi) {
-      r.v = (int32_t)v;
-      r.beg = a.g.rp[v];
-      const int64_t deg = a.g.rp[v + 1] - r.beg;
-      r.deg = (int32_t)deg;
-      r.g = a.gid ? a.gid[v] : 0;
-      r.w = a.g.vw[v];
-      b = bin_of(a, deg);
-    }
-    // rank within the tile: in the warp by ballots, then over the warps
-    int rank = 0, mine = 0;
-#pragma unroll
-    for (int k = 0; k < kBins; ++k) {
-      const unsigned m = __ballot_sync(0xFFFFFFFFu, b == k);
-      if (b == k) rank = __popc(m & ((1u << lane) - 1u));
-      if (lane == k) mine = __popc(m);
-    }
-    if (lane < kBins) s_w[wid][lane] = mine;
-    __syncthreads();
-    if (wid < kBins) {
-      const int c = s_w[lane][wid];  // kW == 32 warps
-      int incl = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int run = s_run[wid];
-      s_w[lane][wid] = run + incl - c;
-      __syncwarp();
-      if (lane == 31) s_run[wid] = run + incl;
-    }
-    __syncthreads();
-    if (b < kBins) {
-      const int at = s_w[wid][b] + rank;
-      a.lists[at] = r.v;
-      a.recs[at] = r;
-    }
-    __syncthreads();
-  }
+    r.v = (int32_t)v;
+    r.beg = rp[v];
+    r.deg = (int32_t)(rp[v + 1] - r.beg);
+    r.g = a.gid ? a.gid[v] : 0;
+    r.w = a.g.vw[v];
+    return r;
+  });
   bar.leave();
 }
-static_assert(kW == 32, "one lane per warp in the tile scan");
 
 // Cuts the hub rows into chunks of hub_chunk edges: c0[h] = the first chunk
 // of hub h, and each chunk's hub and edges.  One block.
@@ -213,12 +97,8 @@ void launch_bins(const LevelGraph &g, const int32_t *gid, const BinPlan &plan, c
   BinArgs a{};
   a.g = g;
   a.gid = gid;
-  for (int k = 0; k < kBins - 1; ++k) a.max_deg[k] = (int32_t)plan.max_deg[k];
-  a.hub_chunk = (int32_t)plan.hub_chunk;
-  a.recs = b.recs;
-  a.lists = b.lists;
+  a.w = bin_work(plan, b, counts);
   a.out = out;
-  a.counts = counts;
   a.sc = sc;
   int64_t blocks = (g.n + kT - 1) / kT;
   if (blocks > coop_blocks(coop)) blocks = coop_blocks(coop);

@@ -6,6 +6,7 @@
 // lc_contract.cu's: coarse vertex x owns 2 bound[x] slots of the global hash
 // scratch, every fine edge that leaves its cluster is inserted there, and
 // the occupied slots in order are the coarse rows.
+#include "lc_bins_dev.cuh"
 #include "lc_coop.cuh"
 #include "lc_group.cuh"
 #include "lc_level.cuh"
@@ -147,17 +148,23 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
   const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
   const int64_t wbase = tid - lane;
   GridBarrier bar(a.sc);
-  for (int64_t x = tid; x <= n; x += nt) {
+  for (int64_t x = tid; x < n; x += nt) {
+    a.w.used[x] = 0;
+    a.w.cnt[x] = 0;
     a.w.bound[x] = 0;
-    if (x < n) {
-      a.w.used[x] = 0;
-      a.w.cnt[x] = 0;
-      a.w.vw[x] = 0;
-    }
+    a.w.label_w[x] = 0;
   }
   for (int64_t g = tid; g < a.G; g += nt) a.w.nc[g] = 0;
   if (!bar.sync()) return;
-  for (int64_t v = tid; v < n; v += nt) a.w.used[LC_IDX(a.C[v], n, kDbgLabel)] = 1;
+  // labels in use, their edge bounds and weights
+  for (int64_t v0 = wbase; v0 < n; v0 += nt) {
+    const int64_t v = v0 + lane;
+    const bool on = v < n;
+    const int32_t X = on ? LC_IDX(a.C[v], n, kDbgLabel) : 0;
+    if (on) a.w.used[X] = 1;
+    add_weights(a.w.bound, on, X, on ? a.g.rp[v + 1] - a.g.rp[v] : 0);
+    add_weights(a.w.label_w, on, X, on ? a.g.vw[v] : 0);
+  }
   if (!bar.sync()) return;
   if (a.gid) {  // labels in use per graph, which tell the graphs that go on
     for (int64_t x0 = wbase; x0 < n; x0 += nt) {
@@ -174,44 +181,37 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
     }
     if (!bar.sync()) return;
   }
-  // dense ids, ascending, of the labels of the graphs that go on
+  // dense ids, ascending, of the labels of the graphs that go on, and where
+  // their slots start: one scan of (edge bound, 1), both below 2^31 here
   auto goes_on = [&](int64_t x) {
     const int g = a.gid ? a.gid[x] : 0;
     return !a.gid || a.w.nc[g] < a.gp[g].nv;
   };
-  long long n_c = 0;
+  long long all = 0;
   if (!grid_scan(
           n, a.w.counts, bar,
-          [&](int64_t x) -> long long { return a.w.used[x] && goes_on(x) ? 1 : 0; },
-          [&](int64_t x, long long at, long long) { a.w.newid[x] = (int32_t)at; }, n_c))
+          [&](int64_t x) -> long long { return a.w.used[x] && goes_on(x) ? (a.w.bound[x] << 32) | 1 : 0; },
+          [&](int64_t x, long long at, long long here) {
+            if (!here) return;
+            const int32_t id = (int32_t)at;
+            a.w.newid[x] = id;
+            a.w.off[id] = at >> 32;
+            a.w.vw[id] = a.w.label_w[x];
+          },
+          all))
     return;
+  long long n_c = all & 0xFFFFFFFFll;
   if (!a.gid && n_c == n) n_c = 0;  // nothing merges
   if (tid == 0) {
     a.out->n_c = n_c;
-    if (!a.gid) a.w.nc[0] = n_c ? (int32_t)n_c : (int32_t)n;
+    a.w.off[n_c] = all >> 32;
   }
   if (n_c == 0) {  // uniform: the host reads no more than this
     bar.leave();
     return;
   }
   if (!bar.sync()) return;
-  // coarse ids, edge bounds and weights
-  for (int64_t v0 = wbase; v0 < n; v0 += nt) {
-    const int64_t v = v0 + lane;
-    int32_t x = -1;
-    if (v < n) {
-      x = goes_on(v) ? a.w.newid[a.C[v]] : -1;
-      a.Cd[v] = x;
-    }
-    add_weights(a.w.bound, x >= 0, x >= 0 ? x : 0, x >= 0 ? a.g.rp[v + 1] - a.g.rp[v] : 0);
-    add_weights(a.w.vw, x >= 0, x >= 0 ? x : 0, x >= 0 ? a.g.vw[v] : 0);
-  }
-  if (!bar.sync()) return;
-  long long slots = 0;
-  if (!grid_scan(
-          n_c + 1, a.w.counts, bar, [&](int64_t x) -> long long { return a.w.bound[x]; },
-          [&](int64_t x, long long at, long long) { a.w.off[x] = at; }, slots))
-    return;
+  for (int64_t v = tid; v < n; v += nt) a.Cd[v] = goes_on(v) ? a.w.newid[a.C[v]] : -1;
   if (!bar.sync()) return;
   // insert: rows of bin 9 by all blocks, 7-8 by a block, 3-6 by a warp, 1-2 by eight lanes, bin 0 by a thread
   bool ok = true;
@@ -270,9 +270,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
           n_c, a.w.counts, bar, [&](int64_t x) -> long long { return a.w.cnt[x]; },
           [&](int64_t x, long long at, long long deg) {
             a.w.rp[x] = at;
-            int b = 0;
-#pragma unroll
-            for (int k = 0; k < kBins - 1; ++k) b += deg > a.max_deg[k] ? 1 : 0;
+            const int b = bin_of(a.max_deg, deg);
             atomicAdd(&s_bin[b], 1);
             if (b == kHubBin) {
               atomicMax(&s_max, (int)deg);
@@ -304,8 +302,12 @@ struct BuildArgs {
   int32_t *col_c, *ew_c;
   int64_t *vw_c;
   int32_t *gid_c;
+  BinWork bins;
   Scalars *sc;
 };
+
+// The coarse graph into its own arrays, and its bins: the row offsets are
+// known, so both of the bins' phases run beside those of the compaction.
 
 __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ BuildArgs a) {
   const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
@@ -319,6 +321,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
       const int32_t x = a.Cd[v];
       if (x >= 0) a.gid_c[x] = a.gid[v];
     }
+  bins_count<kT>(a.bins, a.n_c, nullptr, [&](int64_t x) { return a.w.rp[x + 1] - a.w.rp[x]; });
   // the occupied slots in order; all slots in use lie below 2 off[n_c]
   const int64_t slots = 2 * a.w.off[a.n_c];
   long long nnz = 0;
@@ -333,6 +336,15 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
           },
           nnz))
     return;
+  bins_place<kT>(a.bins, a.n_c, nullptr, [&](int64_t x) {
+    VRec r{};
+    r.v = (int32_t)x;
+    r.beg = a.w.rp[x];
+    r.deg = (int32_t)(a.w.rp[x + 1] - r.beg);
+    r.g = a.gid_c ? a.gid_c[x] : 0;
+    r.w = a.w.vw[x];
+    return r;
+  });
   bar.leave();
 }
 
@@ -370,7 +382,7 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
 
 void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
                         const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
-                        int32_t *gid_c, Scalars *sc, int coop, cudaStream_t s) {
+                        int32_t *gid_c, const BinWork &bins, Scalars *sc, int coop, cudaStream_t s) {
   BuildArgs a{};
   a.n = g.n;
   a.n_c = out.n_c;
@@ -382,6 +394,7 @@ void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *
   a.ew_c = ew_c;
   a.vw_c = vw_c;
   a.gid_c = gid_c;
+  a.bins = bins;
   a.sc = sc;
   void *args[] = {&a};
   cudaLaunchCooperativeKernel((const void *)k_level_build, dim3(level_blocks(g.n, g.nnz, coop)), dim3(kT), args, 0, s);

@@ -1,7 +1,7 @@
 // lc_level.cuh — launch interface of lc_level.cu.
 #pragma once
 
-#include "lc_bins.cuh"
+#include "lc_bins_dev.cuh"
 
 namespace lc {
 
@@ -14,7 +14,8 @@ struct LevelOut {
 // Scratch of a level's end, all sized for the level (int32 [n] unless said).
 struct LevelScratch {
   int32_t *used, *newid, *cnt;
-  int64_t *bound, *off;       // [n + 1]
+  int64_t *bound, *label_w;   // [n] edge bound and weight by label
+  int64_t *off;               // [n + 1] where a coarse vertex's slots start
   int64_t *vw, *rp;           // [n], [n + 1]: the coarse weights and row offsets
   unsigned long long *tab;    // [2 nnz] clean hash slots
   int32_t *nc;                // [G] labels in use per graph
@@ -31,9 +32,9 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
                       const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
                       Scalars *sc, int coop, cudaStream_t s);
 // The coarse graph from the scratch into its own arrays (out as read back),
-// its graph ids (null for one graph); leaves the hash slots clean.
+// its graph ids (null for one graph) and its bins; leaves the hash slots clean.
 void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
                         const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
-                        int32_t *gid_c, Scalars *sc, int coop, cudaStream_t s);
+                        int32_t *gid_c, const BinWork &bins, Scalars *sc, int coop, cudaStream_t s);
 
 }  // namespace lc
