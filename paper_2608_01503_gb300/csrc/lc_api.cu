@@ -246,8 +246,6 @@ static cudaStream_t capture_stream() {
   return st.s[dev];
 }
 
-static int64_t per_graph_bytes(int64_t G) { return G * (17 * 8 + 4 * 4 + 1); }
-
 // The next `count` elements of a block that p walks through (largest
 // alignment first).
 template <typename T>
@@ -256,6 +254,8 @@ static T *cut(uint8_t *&p, int64_t count) {
   p += count * (int64_t)sizeof(T);
   return at;
 }
+
+static int64_t per_graph_bytes(int64_t G) { return G * (17 * 8 + 4 * 4 + 1); }
 
 // The per-graph arrays, one block cut up in order of element size: a provider
 // call costs 2 to 4 us (PyTorch's allocator through a callback).
@@ -399,28 +399,19 @@ static int end_bins(Run &r, Level &L, const BinOut &out) {
   L.max_deg = out.max_deg;
   const int H = (int)L.bins.count[kHubBin], Q = (int)out.chunks;
   if (H > 0) {
-    int32_t *d_hub_of, *d_c0, *d_part_x, *d_done;
-    int64_t *d_e0, *d_e1;
-    long long *d_acc, *d_part_g;
-    LC_TRY(r.ar.get(&d_hub_of, Q));
-    LC_TRY(r.ar.get(&d_c0, H + 1));
-    LC_TRY(r.ar.get(&d_part_x, Q));
-    LC_TRY(r.ar.get(&d_e0, Q));
-    LC_TRY(r.ar.get(&d_e1, Q));
-    LC_TRY(r.ar.get(&d_acc, H));
-    LC_TRY(r.ar.get(&d_done, H));
-    LC_TRY(r.ar.get(&d_part_g, Q));
+    uint8_t *p = nullptr;  // one block: the GPU waits for it
+    LC_TRY(r.ar.get(&p, 32 * (int64_t)Q + 16 * (int64_t)H + 4));
     L.hub.H = H;
     L.hub.Q = Q;
     L.hub.vtx = L.bins.list[kHubBin];
-    L.hub.hub_of = d_hub_of;
-    L.hub.e0 = d_e0;
-    L.hub.e1 = d_e1;
-    L.hub.c0 = d_c0;
-    L.hub.acc = d_acc;
-    L.hub.done = d_done;
-    L.hub.part_g = d_part_g;
-    L.hub.part_x = d_part_x;
+    L.hub.e0 = cut<int64_t>(p, Q);
+    L.hub.e1 = cut<int64_t>(p, Q);
+    L.hub.part_g = cut<long long>(p, Q);
+    L.hub.acc = cut<long long>(p, H);
+    L.hub.hub_of = cut<int32_t>(p, Q);
+    L.hub.part_x = cut<int32_t>(p, Q);
+    L.hub.c0 = cut<int32_t>(p, H + 1);
+    L.hub.done = cut<int32_t>(p, H);
     launch_hub_plan(L.bins, r.plan, L.hub, r.s);
     r.res->kernel_launches[LC_K_OTHER] += 1;
   }
