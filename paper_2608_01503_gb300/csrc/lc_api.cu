@@ -952,9 +952,9 @@ static int contract_level(Run &r, Level &L, Level &N, int level) {
   LC_TRY(r.ar.get(&col_c, nnz_c));
   LC_TRY(r.ar.get(&ew_c, nnz_c));
   r.prof.begin(LC_K_CONTRACT);
-  launch_contract_compact(r.gtab, 2 * L.g.nnz, col_c, ew_c, r.scan32, r.s);
+  launch_contract_compact(r.gtab, 2 * L.g.nnz, r.off, rp_c, r.cnt, n_c, col_c, ew_c, r.s);
   r.prof.end(16.0 * L.g.nnz + 8.0 * nnz_c);
-  r.res->kernel_launches[LC_K_CONTRACT] += 11 + ni;
+  r.res->kernel_launches[LC_K_CONTRACT] += 9 + ni;
   LC_TRY(launch_check());
   r.res->edges_contract += L.g.nnz;
   N.g.nnz = nnz_c;
@@ -1817,7 +1817,7 @@ int lc_contract(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w,
       r.res->error_detail = nnz_c;
     }
     if (rc == LC_OK) {
-      launch_contract_compact(r.gtab, 2 * g->nnz, c_col, c_ew, r.scan32, r.s);
+      launch_contract_compact(r.gtab, 2 * g->nnz, r.off, c_row_ptr, r.cnt, n_c, c_col, c_ew, r.s);
       rc = launch_check();
     }
     if (rc == LC_OK) rc = check_device_error(r);

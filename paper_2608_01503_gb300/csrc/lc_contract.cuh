@@ -31,9 +31,10 @@ int launch_contract_insert(const LevelGraph &g, const int32_t *Cd, const int64_t
 // Coarse row offsets from the unique counts; rp_c[n_c] = nnz_c.
 void launch_contract_rowptr(const int32_t *cnt, int64_t n_c, int64_t *rp_c, int64_t *scan_tmp64,
                             cudaStream_t s);
-// Algorithm 4, line 13: stream compaction of all table slots into the coarse CSR.
-void launch_contract_compact(unsigned long long *tab, int64_t slots, int32_t *col_c, int32_t *ew_c,
-                             int32_t *scan_tmp, cudaStream_t s);
+// Algorithm 4, line 13: the table's slots (2 off[n_c] of at most `slots`) into
+// the coarse CSR; leaves the table clean and uses cnt up.
+void launch_contract_compact(unsigned long long *tab, int64_t slots, const int64_t *off, const int64_t *rp_c,
+                             int32_t *cnt, int64_t n_c, int32_t *col_c, int32_t *ew_c, cudaStream_t s);
 // gid[v] for a packed batch with vertex ranges gptr[0..G] (device).
 void launch_graph_ids(const int64_t *gptr, int G, int32_t *gid, int64_t n, cudaStream_t s);
 // C[v] = vbase_fine(g) + Cnext[Cd[v]] - vbase_coarse(g) (Cd[v] < 0: C[v] = v)
