@@ -133,7 +133,8 @@ typedef struct {
   uint32_t seed;            /* salt of the ordering hash; default 0 */
   int32_t uncoarsen;        /* 1 = Louvain+ (default), 0 = Louvain (Algorithm 1 line 12 off) */
   int32_t validate;         /* 1 = check the CSR preconditions on the device (default) */
-  int32_t profile;          /* 1 = time each kernel class with CUDA events into lc_result */
+  int32_t profile;          /* 1 = time each kernel class with CUDA events into lc_result;
+                               small levels then run as separate kernels too (slower) */
   void *stream;             /* cudaStream_t */
   lc_event_fn event_cb;     /* optional per-pass / per-level trace (slow: syncs and copies) */
   void *event_ctx;
@@ -176,7 +177,8 @@ typedef struct {
   int32_t graphs;           /* 1 = the passes of a LocalMovePasses call that repeat the same
                                launches (all but a first pass from singletons and the last)
                                are captured once per call into a CUDA graph and replayed,
-                               which removes most per-kernel launch costs on small graphs.
+                               on levels above 4 M vertices and stored edges (smaller ones
+                               run all passes in one kernel).
                                Ignored with profile, event_cb or tables = 1.  Results are
                                identical.  Default 0. */
 } lc_opts;
