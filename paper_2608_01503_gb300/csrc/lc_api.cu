@@ -203,7 +203,6 @@ struct Run {
   long long *fused = nullptr;  // [6 G] accumulators of the fused passes (FusedArgs)
   long long *phi_final = nullptr;  // [G] Phi of C_out after each graph's last LocalMovePasses call
   long long *Tg = nullptr, *Vg = nullptr, *sw2g = nullptr;
-  int *improved = nullptr;
   int32_t *gstart = nullptr, *gfree = nullptr, *gmover = nullptr;
   uint8_t *keep = nullptr;
   int64_t *gptr = nullptr;  // [G + 1] vertex ranges of a batch
@@ -255,7 +254,7 @@ static T *cut(uint8_t *&p, int64_t count) {
   return at;
 }
 
-static int64_t per_graph_bytes(int64_t G) { return G * (17 * 8 + 4 * 4 + 1); }
+static int64_t per_graph_bytes(int64_t G) { return G * (17 * 8 + 3 * 4 + 1); }
 
 // The per-graph arrays, one block cut up in order of element size: a provider
 // call costs 2 to 4 us (PyTorch's allocator through a callback).
@@ -273,7 +272,6 @@ static int alloc_per_graph(Run &r) {
   r.phi_trace = cut<long long>(p, G);
   r.obj = cut<long long>(p, 4 * G);
   r.fused = cut<long long>(p, 6 * G);
-  r.improved = cut<int>(p, G);
   r.gstart = cut<int32_t>(p, G);
   r.gfree = cut<int32_t>(p, G);
   r.gmover = cut<int32_t>(p, G);
@@ -461,7 +459,6 @@ static PassArgs pass_args(Run &r, const Level &L) {
   a.G = r.G;
   a.phi_acc = r.phi_acc;
   a.phi_out = r.phi_out;
-  a.improved = r.improved;
   a.C = r.C;
   a.W = r.W;
   a.delta = r.delta;
@@ -530,7 +527,7 @@ static int capture_pass(Run &r, Level &L, const PassArgs &a, const EmptyScratch 
   for (int k = 0; k < LC_K_COUNT; ++k) counts[k] = 0;
   launch_pass_begin(r.sc, cs, 1);
   counts[LC_K_MOVE] += launch_move(a, L.bins, cs);
-  counts[LC_K_APPLY] += launch_bestof(a, r.C_out, cs);
+  counts[LC_K_APPLY] += launch_bestof(a, r.C_out, false, cs);
   counts[LC_K_AFTERBURNER] += launch_afterburner(a, L.bins, cs);
   counts[LC_K_APPLY] += launch_assign_empty(a, w, cs) + 1;
   cudaGraph_t g = nullptr;
@@ -659,7 +656,9 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
         continue;
       }
     }
-    launch_pass_begin(r.sc, r.s, a.phi_live ? 1 : 0);
+    // later plain passes count from zero without a launch for it (k_bestof)
+    const bool begin = i == 1 || a.phi_live || tables || r.o.event_cb;
+    if (begin) launch_pass_begin(r.sc, r.s, a.phi_live ? 1 : 0);
     a.movers = incremental && last ? r.movers : nullptr;  // listed by this pass's update step
     if (incremental && last) {
       r.prof.begin(LC_K_OBJECTIVE);
@@ -694,7 +693,7 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
       r.prof.begin(LC_K_APPLY);
       // Phi entering the last pass, per graph, before the best-of test resets it
       if (incremental && last) r.res->kernel_launches[LC_K_OBJECTIVE] += launch_save_phi_enter(a, r.s);
-      r.res->kernel_launches[LC_K_APPLY] += launch_bestof(a, r.C_out, r.s);
+      r.res->kernel_launches[LC_K_APPLY] += launch_bestof(a, r.C_out, !begin, r.s);
       r.prof.end(8.0 * n);
     }
     r.prof.begin(LC_K_AFTERBURNER);
@@ -718,11 +717,11 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
   // the state entering the last pass and that pass's moves
   r.prof.begin(LC_K_OBJECTIVE);
   if (incremental) {
-    r.res->kernel_launches[LC_K_OBJECTIVE] += launch_final_objective(a, r.s) + launch_bestof(a, r.C_out, r.s);
+    r.res->kernel_launches[LC_K_OBJECTIVE] += launch_final_objective(a, r.s) + launch_final_bestof(a, r.C_out, r.s);
     r.prof.end(17.0 * n);  // W, w(v) and M per vertex (+ 13 B per mover edge, added at the end)
   } else {
     r.res->kernel_launches[LC_K_OBJECTIVE] +=
-        launch_objective(a, L.bins, r.s) + launch_bestof(a, r.C_out, r.s);
+        launch_objective(a, L.bins, r.s) + launch_final_bestof(a, r.C_out, r.s);
     r.prof.end(12.0 * nnz + 32.0 * n);
   }
   r.res->kernel_launches[LC_K_OTHER] += launch_keep_phi(a, r.phi_final, r.s);

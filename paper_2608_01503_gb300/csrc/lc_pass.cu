@@ -700,6 +700,14 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_tab_scan(PassArgs a) {
   flush_move(a, ms);
 }
 
+// Takes over the objectives of the graphs that improved (k_bestof).
+__device__ __forceinline__ void settle_bestof(const PassArgs &a) {
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.G; g += gridDim.x * blockDim.x) {
+    const long long p = a.phi_acc[g];
+    if (p > a.phi_out[g]) a.phi_out[g] = p;
+    a.phi_acc[g] = 0;
+  }
+}
 // ------------------------------------------------ ids of new clusters
 
 // The movers to new empty clusters, ascending, take the ascending ids that
@@ -711,8 +719,10 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_tab_scan(PassArgs a) {
 //
 // One cooperative launch whose blocks meet between the phases, in place of
 // nine launches per pass that mostly found nothing to do (2 us each): it
-// returns at once when the pass has no such mover.
+// returns at once when the pass has no such mover.  It also settles the
+// pass's best-of test, which as a launch of its own took 4 us a pass.
 __global__ void __launch_bounds__(kCoopThreads) k_assign_empty(PassArgs a, EmptyScratch w) {
+  settle_bestof(a);
   const int total = a.sc->empty_movers;  // nothing writes it during this launch
   if (total == 0) return;
   GridBarrier bar(a.sc);
@@ -744,25 +754,24 @@ __global__ void k_pass_begin(Scalars *sc, int advance) {
 }
 
 // Algorithm 2's best-of test, per graph, on the objective accumulated in
-// phi_acc (strict improvement keeps the earliest maximum).
-__global__ void k_bestof_test(long long *phi_acc, long long *phi_out, int *improved, int G) {
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-    const long long p = phi_acc[g];
-    if (p > phi_out[g]) {
-      phi_out[g] = p;
-      improved[g] = 1;
-    } else {
-      improved[g] = 0;
-    }
-    phi_acc[g] = 0;
+// phi_acc (strict improvement keeps the earliest maximum): the labels of the
+// graphs that improved are copied; settle_bestof, in a later kernel, takes the
+// values over.  reset: the pass has no k_pass_begin (the update step counts
+// from zero here).
+__global__ void k_bestof(PassArgs a, int32_t *__restrict__ C_out, int reset) {
+  if (reset && blockIdx.x == 0 && threadIdx.x == 0) {
+    a.sc->empty_movers = 0;
+    a.sc->n_movers = 0;
+  }
+  if (!a.gid && a.phi_acc[0] <= a.phi_out[0]) return;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < a.g.n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int g = graph_of(a, (int32_t)v);
+    if (a.phi_acc[g] > a.phi_out[g]) C_out[v] = a.C[v];
   }
 }
 
-__global__ void k_bestof_copy(PassArgs a, int32_t *__restrict__ C_out) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < a.g.n;
-       v += (int64_t)gridDim.x * blockDim.x)
-    if (a.improved[graph_of(a, (int32_t)v)]) C_out[v] = a.C[v];
-}
+__global__ void k_bestof_settle(PassArgs a) { settle_bestof(a); }
 
 // ------------------------------------------------------------ helpers
 
@@ -1173,9 +1182,13 @@ int launch_keep_phi(const PassArgs &a, long long *phi_final, cudaStream_t s) {
   return 1;
 }
 
-int launch_bestof(const PassArgs &a, int32_t *C_out, cudaStream_t s) {
-  k_bestof_test<<<blocks_for(a.G, 256), 256, 0, s>>>(a.phi_acc, a.phi_out, a.improved, a.G);
-  k_bestof_copy<<<blocks_for(a.g.n, 256), 256, 0, s>>>(a, C_out);
+int launch_bestof(const PassArgs &a, int32_t *C_out, bool reset, cudaStream_t s) {
+  k_bestof<<<blocks_for(a.g.n, 256), 256, 0, s>>>(a, C_out, reset ? 1 : 0);
+  return 1;
+}
+int launch_final_bestof(const PassArgs &a, int32_t *C_out, cudaStream_t s) {
+  k_bestof<<<blocks_for(a.g.n, 256), 256, 0, s>>>(a, C_out, 0);
+  k_bestof_settle<<<blocks_for(a.G, 256), 256, 0, s>>>(a);
   return 2;
 }
 

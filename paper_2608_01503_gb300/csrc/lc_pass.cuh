@@ -14,7 +14,6 @@ struct PassArgs {
   int32_t G;
   long long *phi_acc;     // [G] objective of the clustering entering the pass
   long long *phi_out;     // [G] objective of C_out
-  int *improved;          // [G] last best-of test
   int32_t *C;       // clustering entering the pass (updated by the apply step)
   int64_t *W;       // W(X) for X in [0, n)
   AbRec *ab;        // per pass: {C, D, epsilon bucket of delta} (Section IV-A-1 order)
@@ -104,8 +103,12 @@ struct EmptyScratch {
 int launch_assign_empty(const PassArgs &a, const EmptyScratch &w, cudaStream_t s);
 // Splits the records into destinations (for the trace).
 void launch_destinations(const PassArgs &a, int32_t *D, cudaStream_t s);
-// Per-graph best-of test and copy of improved graphs' labels into C_out.
-int launch_bestof(const PassArgs &a, int32_t *C_out, cudaStream_t s);
+// Per-graph best-of test: improved graphs' labels into C_out.  Within a pass
+// the objectives are taken over by launch_assign_empty; reset: the pass was
+// not begun by launch_pass_begin.
+int launch_bestof(const PassArgs &a, int32_t *C_out, bool reset, cudaStream_t s);
+// The same after a call's last pass, objectives included.
+int launch_final_bestof(const PassArgs &a, int32_t *C_out, cudaStream_t s);
 // phi_final[g] = phi_out[g] for every graph active in the call (gp[g].active).
 int launch_keep_phi(const PassArgs &a, long long *phi_final, cudaStream_t s);
 void launch_fill(long long *a, long long value, int n, cudaStream_t s);
