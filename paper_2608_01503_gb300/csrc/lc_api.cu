@@ -549,12 +549,12 @@ static int capture_pass(Run &r, Level &L, const PassArgs &a, const EmptyScratch 
 
 // Whether a level's passes run as one cooperative kernel (lc_fused.cu): the
 // plain passes of a level small enough that the separate launches, not their
-// work, set the time.  Measured by moving the line (ms per call, separate
-// kernels / line at 2 M / 4 M / 16 M / 40 M vertices and stored edges): 256^3
-// lattice 64.0 / 64.0 / 60.1 / 61.0 / 66.6, 512-graph batch 79.2 / 78.3 /
-// 77.8 / 78.4 / 80.7, an SBM of 100,000 vertices and 2 M stored edges 8.4 /
-// 6.8 / 6.5 / 6.5 / 6.5, one of 1 M vertices and 16 M stored edges 3.2 / 3.2 /
-// 3.2 / 3.2 / 3.8: a large level wants the separate kernels' occupancy.
+// work, set the time.  Measured by moving the line (ms per call, line at 1 M /
+// 2 M / 4 M / 8 M / 16 M vertices and stored edges): 97^3 lattice, iterated,
+// 16.3 / 15.7 / 15.2 / 15.8 / 16.7, pLeiden of R-MAT scale 18 22.2 / 23.4 /
+// 22.8 / 29.0 / 29.5, an SBM of 100,000 vertices and 2 M stored edges 4.95 /
+// 4.12 / 3.91 / 3.94 / 3.96, R-MAT scale 22 and a 512-graph batch the same
+// within 2 %: a large level wants the separate kernels' occupancy.
 constexpr int64_t kFusedMaxSize = 4000000;
 static bool use_fused(const Run &r, const Level &L) {
   return r.o.pass_limit >= 1 && r.o.tables == 0 && r.o.symmetry == 0 && !r.prof.on && !r.o.event_cb &&

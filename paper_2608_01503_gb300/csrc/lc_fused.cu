@@ -5,8 +5,9 @@
 // (up to nine move kernels, the best-of test and copy, up to seven
 // afterburner kernels, the counters and the new-cluster ids) cost 2-4 us each
 // whatever they find to do.  Here all passes of a call run in one cooperative
-// launch of one 1,024-thread block per SM; the phases of a pass are separated
-// by grid barriers (1.2 us over 152 blocks, measured):
+// launch of one 512-thread block per SM; the phases of a pass are separated
+// by grid barriers (1.2 us over 152 blocks on their own, 2.2-2.6 us behind a
+// phase's stores):
 //
 //   move:    gains, argmax, candidate test of every vertex; records written
 //   barrier
@@ -18,6 +19,14 @@
 // (bin 0), 16 lanes, a warp (bins 2-4), four warps (bins 5-6) or the block
 // (bins 7-8 and hubs of up to kRowSlots / 2 edges); longer hub rows go by
 // chunks over the global table, with one more barrier per pass.
+//
+// What bounds it: on small levels the barrier and one chain of gathers per
+// phase (4-10 us, also for a few thousand vertices), on the largest the
+// gathers, a clock per lane and SM (an SBM of 100,000 vertices and 2 M stored
+// edges: 35 us to move, 29 us to update).  Calls, ms, separate kernels / this
+// when it was built: SBM of 10,000 vertices 5.1 / 3.8, R-MAT scale 16 21.9 /
+// 13.5, SBM of 100,000 8.4 / 6.5; with later changes here and between the
+// levels 1.45, 4.8 and 3.8.
 #include "lc_coop.cuh"
 #include "lc_empty.cuh"
 #include "lc_fused.cuh"

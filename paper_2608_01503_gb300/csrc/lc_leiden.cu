@@ -160,7 +160,8 @@ __device__ __forceinline__ bool edge_ok(const GraphParam &P, int32_t w, long lon
 // below): a thread, 16 lanes, a warp or a block per vertex, four edges each in
 // flight, since their walks are chains of gathers.  With a thread up to degree
 // 32 and a warp above, one edge at a time, the longest row of an R-MAT graph
-// of scale 18 kept one warp busy for most of each kernel.
+// of scale 18 kept one warp busy for most of each kernel (pLeiden of that
+// graph 26.1 / 22.8 ms).
 
 // The smallest (key, id) over the group.
 template <int GS>

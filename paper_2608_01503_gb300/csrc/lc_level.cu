@@ -1,8 +1,12 @@
 // lc_level.cu — the end of a small coarsening level in two cooperative
-// kernels: label compaction and Algorithm 4's contraction, which as separate
-// launches (marks, three scans of three launches each, bounds, six insert
-// kernels, a compaction, two read-backs) took 28 launches of 2-4 us and two
-// more waits of the host, whatever the level's size.  The method is
+// kernels: label compaction and Algorithm 4's contraction (and the bins of the
+// next level), which as separate launches (marks, three scans of three
+// launches each, bounds, six insert kernels, a compaction, two read-backs)
+// took 28 launches of 2-4 us and two more waits of the host, whatever the
+// level's size: a call on an SBM of 10,000 vertices, four such level ends,
+// went from 2.14 to 1.60 ms, and with the bins, one scan by label and two
+// barriers less from 1.48 to 1.40.  Bound by seven grid barriers on small
+// levels, by the inserts' probes on the largest.  The method is
 // lc_contract.cu's: coarse vertex x owns 2 bound[x] slots of the global hash
 // scratch, every fine edge that leaves its cluster is inserted there, and
 // the occupied slots in order are the coarse rows.
