@@ -3,6 +3,7 @@
 // both directions; vertex weights may also be zero, the weighted degree of an
 // isolated vertex under modularity).  The edge checks are load-balanced over
 // entries, so a single long row does not serialise them.
+#include "lc_edge_print.cuh"
 #include "lc_group.cuh"
 #include "lc_internal.cuh"
 #include "lc_move.cuh"
@@ -13,13 +14,6 @@ namespace lc {
 __device__ __forceinline__ void report(GraphStats *st, int code, int64_t v) {
   const unsigned long long key = ((unsigned long long)code << 40) | (unsigned long long)(v & 0xFFFFFFFFFFll);
   atomicMin(&st->err_key, key);
-}
-
-// SplitMix64 output mix, used as an edge fingerprint.
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
 }
 
 // Per-vertex part: vertex-weight sums and checks, row-pointer sanity.
@@ -252,15 +246,11 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
         if (on && ((uint32_t)x >= (uint32_t)g.n || x == v || (!first[k] && before[k] >= x) || w.x[k] <= 0))
           report_entry(st, v, x, (int32_t)g.n, !first[k] && before[k] >= x, w.x[k]);
         const uint32_t lo = (uint32_t)min(v, x), hi = (uint32_t)max(v, x);
-        // two fingerprints of the undirected edge; the second is another
-        // (nonlinear) function of the first
-        const unsigned long long h1 = mix64((((unsigned long long)lo << 32) | hi) ^
-                                            ((unsigned long long)(uint32_t)w.x[k] * 0x9E3779B97F4A7C15ull));
-        const unsigned long long h2 = (h1 ^ (h1 >> 32)) * 0xD6E8FEB86659FD93ull;
+        const EdgePrint h = edge_print(lo, hi, (uint32_t)w.x[k]);
         const unsigned long long neg = v < x ? 0ull : ~0ull;
         if (on) {
-          f1 += h1 ^ neg;
-          f2 += h2 ^ neg;
+          f1 += h.a ^ neg;
+          f2 += h.b ^ neg;
           minus += (unsigned)(neg & 1ull);
         }
       }
