@@ -1144,8 +1144,9 @@ static int level0(Run &r, Level &L, const LevelGraph &g0, const std::vector<int6
 // Everything before the first pass on G_0: statistics, validation and guards,
 // the range of given labels ([0, limit)), scratch and bins.  What the call
 // needs besides is taken and the bins are built while the GPU reads the
-// graph, so that the host waits once; the bin kernel follows nothing but
-// row_ptr's length, so it may run on a graph that turns out to be refused.
+// graph, so that the host waits once; the bin kernel reads row_ptr alone and
+// places every vertex once whatever it finds there (lc_bin_rule.cuh), so it
+// may run on a graph that turns out to be refused.
 // The graph's faults are reported before a lack of memory.  gptr is read
 // until the wait.  passes_only: the call contracts nothing.
 static int set_up(Run &r, Level &L, const LevelGraph &g0, const std::vector<int64_t> &gptr,

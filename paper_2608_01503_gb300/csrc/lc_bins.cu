@@ -25,13 +25,13 @@ struct BinArgs {
 __global__ void __launch_bounds__(kT, 1) k_bins(const __grid_constant__ BinArgs a) {
   const int64_t *__restrict__ rp = a.g.rp;
   GridBarrier bar(a.sc);
-  bins_count<kT>(a.w, a.g.n, a.out, [&](int64_t v) { return rp[v + 1] - rp[v]; });
+  bins_count<kT>(a.w, a.g.n, a.out, [&](int64_t v) { return row_degree(rp[v], rp[v + 1]); });
   if (!bar.sync()) return;
   bins_place<kT>(a.w, a.g.n, a.out, [&](int64_t v) {
     VRec r{};
     r.v = (int32_t)v;
     r.beg = rp[v];
-    r.deg = (int32_t)(rp[v + 1] - r.beg);
+    r.deg = row_degree(r.beg, rp[v + 1]);
     r.g = a.gid ? a.gid[v] : 0;
     r.w = a.g.vw[v];
     return r;
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kT, 1)
   if (threadIdx.x == 0) s_run = 0;
   for (int base = 0; base < H; base += kT) {
     const int h = base + threadIdx.x;
-    const int c = h < H ? (hubs[h].deg + hub_chunk - 1) / hub_chunk : 0;
+    const int c = h < H ? (int)(((int64_t)hubs[h].deg + hub_chunk - 1) / hub_chunk) : 0;
     int incl = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

@@ -2,6 +2,9 @@
 // kernel (lc_bins.cu, and lc_level.cu for a level built on the device).
 #pragma once
 
+#include <type_traits>
+
+#include "lc_bin_rule.cuh"
 #include "lc_bins.cuh"
 #include "lc_coop.cuh"
 
@@ -26,13 +29,6 @@ inline BinWork bin_work(const BinPlan &plan, const Bins &b, int32_t *counts) {
   return w;
 }
 
-__device__ __forceinline__ int bin_of(const int32_t *max_deg, int64_t deg) {
-  int b = 0;
-#pragma unroll
-  for (int k = 0; k < kBins - 1; ++k) b += deg > max_deg[k] ? 1 : 0;
-  return b;
-}
-
 // Every block takes a run of vertices of its own.
 struct BinRun {
   int64_t lo, hi;
@@ -45,12 +41,14 @@ __device__ __forceinline__ BinRun bin_run(int64_t n) {
 }
 
 // Phase 1 (T threads): the bins of the block's run into w.counts; out: null,
-// or where the hub figures are summed.  A grid barrier follows.
+// or where the hub figures are summed.  A grid barrier follows.  deg_of: the
+// row_degree that the records of phase 2 hold.
 template <int T, typename Deg>
 __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *out, Deg deg_of) {
   __shared__ int32_t s_cnt[kBins];
   __shared__ long long s_chunks;
   __shared__ int32_t s_max;
+  static_assert(std::is_same<decltype(deg_of(int64_t())), int32_t>::value, "the degree as phase 2 bins it");
   const int lane = threadIdx.x & 31;
   const BinRun run = bin_run<T>(n);
   if (threadIdx.x < kBins) s_cnt[threadIdx.x] = 0;
@@ -63,13 +61,13 @@ __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *
   long long chunks = 0;
   int32_t longest = 0;
   for (int64_t v = run.lo + threadIdx.x; v < run.hi; v += T) {
-    const int64_t deg = deg_of(v);
+    const int32_t deg = deg_of(v);
     const int b = bin_of(w.max_deg, deg);
 #pragma unroll
     for (int k = 0; k < kBins; ++k) cnt[k] += b == k;
     if (b == kHubBin) {
-      chunks += (deg + w.hub_chunk - 1) / w.hub_chunk;
-      longest = deg > longest ? (int32_t)deg : longest;
+      chunks += ((int64_t)deg + w.hub_chunk - 1) / w.hub_chunk;
+      longest = deg > longest ? deg : longest;
     }
   }
 #pragma unroll
@@ -90,7 +88,8 @@ __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *
 }
 
 // Phase 2: the run's vertices into the lists and records, ascending within
-// each bin; out: null, or where block 0 leaves the bins' starts.
+// each bin; out: null, or where block 0 leaves the bins' starts.  A place past
+// the arrays (row_ptr written to between the phases) is not taken.
 template <int T, typename Rec>
 __device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, BinOut *out, Rec rec_of) {
   constexpr int W = T / 32;
@@ -160,8 +159,10 @@ __device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, BinOut *
     __syncthreads();
     if (b < kBins) {
       const int at = s_w[wid][b] + rank;
-      w.lists[at] = r.v;
-      w.recs[at] = r;
+      if (at < n) {
+        w.lists[at] = r.v;
+        w.recs[at] = r;
+      }
     }
     __syncthreads();
   }

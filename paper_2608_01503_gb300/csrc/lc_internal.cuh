@@ -10,6 +10,7 @@
 #include <stdint.h>
 
 #include "../../include/lc.h"
+#include "lc_bin_rule.cuh"
 #include "lc_debug.cuh"
 
 namespace lc {
@@ -39,7 +40,6 @@ constexpr int kMaxLevels = 256;
 // A vertex's table holds 2d slots at most, so the shared memory a bin
 // reserves per vertex tracks its degree and many vertices stay in flight.
 // Kernels without tables launch once over a contiguous range of bins.
-constexpr int kBins = 10;
 constexpr int kHubBin = kBins - 1;
 // The largest degree each bin's kernel can take (its registers or shared
 // table), which is also the default bin boundary.

@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
           n_c, a.w.counts, bar, [&](int64_t x) -> long long { return a.w.cnt[x]; },
           [&](int64_t x, long long at, long long deg) {
             a.w.rp[x] = at;
-            const int b = bin_of(a.max_deg, deg);
+            const int b = bin_of(a.max_deg, (int32_t)deg);
             atomicAdd(&s_bin[b], 1);
             if (b == kHubBin) {
               atomicMax(&s_max, (int)deg);
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
       const int32_t x = a.Cd[v];
       if (x >= 0) a.gid_c[x] = a.gid[v];
     }
-  bins_count<kT>(a.bins, a.n_c, nullptr, [&](int64_t x) { return a.w.rp[x + 1] - a.w.rp[x]; });
+  bins_count<kT>(a.bins, a.n_c, nullptr, [&](int64_t x) { return row_degree(a.w.rp[x], a.w.rp[x + 1]); });
   // the occupied slots in order; all slots in use lie below 2 off[n_c]
   const int64_t slots = 2 * a.w.off[a.n_c];
   long long nnz = 0;
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
     VRec r{};
     r.v = (int32_t)x;
     r.beg = a.w.rp[x];
-    r.deg = (int32_t)(a.w.rp[x + 1] - r.beg);
+    r.deg = row_degree(r.beg, a.w.rp[x + 1]);
     r.g = a.gid_c ? a.gid_c[x] : 0;
     r.w = a.w.vw[x];
     return r;
