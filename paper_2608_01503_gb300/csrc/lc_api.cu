@@ -1008,7 +1008,8 @@ static int check_lambda(int64_t mu, int64_t Lam) {
 }
 
 static int check_graph_args(const lc_csr *g, const int64_t *vw, const int32_t *ew) {
-  if (!g || g->n < 0 || g->n > INT32_MAX || g->nnz < 0) return LC_ERR_ARG;
+  // 2^40 entries are more than any device holds: sizes below never overflow
+  if (!g || g->n < 0 || g->n > INT32_MAX || g->nnz < 0 || g->nnz > (1ll << 40)) return LC_ERR_ARG;
   if (g->n > 0 && (!g->row_ptr || !vw)) return LC_ERR_ARG;
   if (g->nnz > 0 && (!g->col || !ew)) return LC_ERR_ARG;
   return LC_OK;
@@ -1016,8 +1017,8 @@ static int check_graph_args(const lc_csr *g, const int64_t *vw, const int32_t *e
 
 // Statistics, validation and the exactness guards of the header, per graph; C:
 // null, or the clustering whose objective is wanted (lc_objective), which the
-// same pass over the edges sums.  begin_prepare queues the kernels,
-// end_prepare waits for them and judges.
+// same pass over the edges sums.  begin_prepare queues the kernels, which read
+// no edge unless row_ptr ends at nnz; end_prepare waits for them and judges.
 static int begin_prepare(Run &r, const LevelGraph &g, const int32_t *gid, const int32_t *C = nullptr) {
   LC_TRY(r.ar.get(&r.st, 1));
   LC_CK(cudaMemsetAsync(r.st, 0, sizeof(GraphStats), r.s));

@@ -139,6 +139,9 @@ __global__ void __launch_bounds__(kStatsThreads, 4) k_stats_edges(LevelGraph g, 
                                                                const int32_t *__restrict__ gid,
                                                                const int64_t *__restrict__ gptr, long long *Tg,
                                                                const int32_t *__restrict__ C) {
+  // col and ew are as long as row_ptr says, and the caller's nnz has not been
+  // compared with it yet (uniform; the vertex part reports both ends)
+  if (__ldg(g.rp) != 0 || __ldg(g.rp + g.n) != g.nnz) return;
   constexpr unsigned full = 0xFFFFFFFFu;
   __shared__ int4 s_mark[kStatsThreads / 32][kStatsStep / 4];
   const int lane = threadIdx.x & 31;

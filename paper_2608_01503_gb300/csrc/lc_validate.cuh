@@ -16,7 +16,8 @@ struct GraphStats {
   unsigned long long err_key;   // (code << 40 | vertex), min over violations; ~0 if none
 };
 
-// Sums T, V, sum w^2; with validate: row structure, ranges, loops, weights,
+// Sums T, V, sum w^2 (T and all else about the edges only if row_ptr runs from
+// 0 to nnz); with validate: row structure, ranges, loops, weights,
 // strictly increasing rows and the symmetry fingerprints.  *st must be
 // zeroed with err_key = ~0 beforehand.
 // With a packed batch (gid non-null, gptr its vertex ranges) also per-graph
