@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <deque>
 #include <mutex>
@@ -284,6 +285,16 @@ static int alloc_counters(Run &r) {
   LC_TRY(r.ar.get(&r.coop, kCoopScratch));
   LC_TRY(r.ar.get(&r.sc, 1));
   LC_CK(cudaMemsetAsync(r.sc, 0, sizeof(Scalars), r.s));
+#if LC_DEBUG
+  // "K:P": the K-th grid barrier of the call is one that a block never reaches,
+  // and every wait gives up after P polls
+  unsigned skip[2] = {0, 0};
+  const char *e = getenv("LC_DEBUG_BARRIER");
+  if (e && sscanf(e, "%u:%u", &skip[0], &skip[1]) == 2) {
+    LC_CK(cudaMemcpyAsync(&r.sc->dbg_skip, skip, sizeof(skip), cudaMemcpyHostToDevice, r.s));
+    LC_CK(cudaStreamSynchronize(r.s));
+  }
+#endif
   return LC_OK;
 }
 
@@ -395,6 +406,7 @@ static int begin_bins(Run &r, Level &L, BinOut **d_out) {
   return LC_OK;
 }
 static int end_bins(Run &r, Level &L, const BinOut &out) {
+  if (L.g.n > 0 && !out.done) return LC_ERR_DEVICE;
   finish_bins(L.bins, out);
   r.res->kernel_launches[LC_K_OTHER] += 1;
   L.hub = Hubs{};
@@ -816,10 +828,13 @@ static int64_t end_count(const Run &r, const Level &L, const LabelCount &c, std:
   if (prev >= 0) nc[prev] = c.total - c.gs[prev];
   return c.total;
 }
-static int count_labels(Run &r, Level &L, const int32_t *C, std::vector<int64_t> &nc, int64_t *total) {
+// err: null, or the passes' error flag to read back on the way.
+static int count_labels(Run &r, Level &L, const int32_t *C, std::vector<int64_t> &nc, int64_t *total,
+                        int *err = nullptr) {
   LabelCount c;
   begin_count(r, L, C);
   LC_TRY(read_count(r, L, c));
+  if (err) LC_CK(cudaMemcpyAsync(err, &r.sc->error, sizeof(*err), cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaStreamSynchronize(r.s));
   LC_TRY(launch_check());
   *total = end_count(r, L, c, nc);
@@ -833,7 +848,9 @@ static int compact_level(Run &r, Level &L, Level &N, int level, bool *any) {
   std::vector<int64_t> nc;
   int64_t total = 0;
   r.prof.begin(LC_K_CONTRACT);
-  LC_TRY(count_labels(r, L, r.C_out, nc, &total));
+  int err = 0;  // the contraction trusts the passes' tables and counters
+  LC_TRY(count_labels(r, L, r.C_out, nc, &total, &err));
+  if (err) return LC_ERR_DEVICE;
   L.cont.assign(r.G, 0);
   *any = false;
   for (int g = 0; g < r.G; ++g) {
@@ -870,8 +887,8 @@ static int compact_level(Run &r, Level &L, Level &N, int level, bool *any) {
   return launch_check();
 }
 
-// compact_level and contract_level of a small level in two cooperative
-// kernels with one read-back between them (lc_level.cu); also leaves the
+// compact_level and contract_level of a small level in three kernels with one
+// read-back between them (lc_level.cu); also leaves the
 // sizes of N's bins.
 static bool use_small_level(const Run &r, const Level &L) {
   return !r.prof.on && !r.o.event_cb && L.g.n + L.g.nnz <= kFusedMaxSize;
@@ -880,15 +897,16 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   Phase range("lc.contract");
   LC_TRY(r.ar.get(&L.Cd, L.g.n));
   // the passes are over: their records' space holds the labels' weights
-  const LevelScratch w{r.used,  r.newid, r.cnt,  r.bound, reinterpret_cast<int64_t *>(r.ab), r.off, r.W,
-                       r.delta, r.gtab,  r.gfree, r.lcounts};
-  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.sc, r.coop_blocks, r.s);
+  const LevelScratch w{r.used,  r.newid, r.cnt,   r.bound,   reinterpret_cast<int64_t *>(r.ab), r.off, r.W,
+                       r.delta, r.gtab,  r.gfree, r.freelist, r.lcounts};
+  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.coop, r.sc, r.coop_blocks, r.s);
   LevelOut out{};
   std::vector<int32_t> nc(r.G);
   LC_CK(cudaMemcpyAsync(&out, r.lout, sizeof(out), cudaMemcpyDeviceToHost, r.s));
   if (r.G > 1) LC_CK(cudaMemcpyAsync(nc.data(), w.nc, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaStreamSynchronize(r.s));
   LC_TRY(launch_check());
+  if (!out.bins.done) return LC_ERR_DEVICE;
   if (r.G == 1) nc[0] = (int32_t)(out.n_c > 0 ? out.n_c : L.g.n);
   r.res->kernel_launches[LC_K_CONTRACT] += 1;
   L.cont.assign(r.G, 0);
@@ -919,9 +937,8 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   int32_t *col_c = nullptr, *ew_c = nullptr;
   LC_TRY(r.ar.get(&col_c, out.nnz_c));
   LC_TRY(r.ar.get(&ew_c, out.nnz_c));
-  launch_level_build(L.g, L.gid, L.Cd, w, out, rp_c, col_c, ew_c, vw_c, N.gid, bin_work(r.plan, N.bins, r.coop), r.sc,
-                     r.coop_blocks, r.s);
-  r.res->kernel_launches[LC_K_CONTRACT] += 1;
+  r.res->kernel_launches[LC_K_CONTRACT] += launch_level_build(
+      L.g, w, out, rp_c, col_c, ew_c, vw_c, N.gid, bin_work(r.plan, N.bins, r.coop), r.coop_blocks, r.s);
   r.res->edges_contract += L.g.nnz;
   N.g = LevelGraph{out.n_c, out.nnz_c, rp_c, col_c, ew_c, vw_c};
   N.bin_out = out.bins;
@@ -951,7 +968,8 @@ static int contract_level(Run &r, Level &L, Level &N, int level) {
   LC_TRY(r.ar.get(&col_c, nnz_c));
   LC_TRY(r.ar.get(&ew_c, nnz_c));
   r.prof.begin(LC_K_CONTRACT);
-  launch_contract_compact(r.gtab, 2 * L.g.nnz, r.off, rp_c, r.cnt, n_c, col_c, ew_c, r.s);
+  Step compact(r.s);
+  launch_contract_compact(compact, r.gtab, 2 * L.g.nnz, r.off, rp_c, r.cnt, n_c, col_c, ew_c);
   r.prof.end(16.0 * L.g.nnz + 8.0 * nnz_c);
   r.res->kernel_launches[LC_K_CONTRACT] += 9 + ni;
   LC_TRY(launch_check());
@@ -1396,8 +1414,11 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
     LC_TRY(objective_of(r, L, Ccur, phi_in));  // leaves the clustering in r.C
     LC_TRY(local_move_passes(r, L, false, l, 0, present));
     long long phi_out = 0;
+    int err = 0;  // what follows trusts the passes' tables and counters
     LC_CK(cudaMemcpyAsync(&phi_out, r.phi_out, sizeof(long long), cudaMemcpyDeviceToHost, r.s));
+    LC_CK(cudaMemcpyAsync(&err, &r.sc->error, sizeof(err), cudaMemcpyDeviceToHost, r.s));
     LC_CK(cudaStreamSynchronize(r.s));
+    if (err) return LC_ERR_DEVICE;
     if (phi_out == phi_in[0]) {  // LocalMoveAlt (Section V-A)
       LC_CK(cudaMemcpyAsync(r.C, r.C_out, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, r.s));
       launch_cluster_weights(r.C, L.g.vw, r.W, n, r.s);
@@ -1818,7 +1839,8 @@ int lc_contract(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w,
       r.res->error_detail = nnz_c;
     }
     if (rc == LC_OK) {
-      launch_contract_compact(r.gtab, 2 * g->nnz, r.off, c_row_ptr, r.cnt, n_c, c_col, c_ew, r.s);
+      Step compact(r.s);
+      launch_contract_compact(compact, r.gtab, 2 * g->nnz, r.off, c_row_ptr, r.cnt, n_c, c_col, c_ew);
       rc = launch_check();
     }
     if (rc == LC_OK) rc = check_device_error(r);

@@ -10,6 +10,7 @@ struct BinOut {
   int32_t offs[kBins + 1];  // start of each bin in the lists
   int32_t max_deg;          // longest hub row (0: no hub)
   int64_t chunks;           // chunks of all hub rows
+  int32_t done;             // 1: complete (no barrier's wait ran out)
 };
 
 // Fills b.lists and b.recs (ascending ids within each bin) and *out, all on

@@ -1,5 +1,5 @@
-// lc_bins_dev.cuh — the two phases of the degree bins inside a cooperative
-// kernel (lc_bins.cu, and lc_level.cu for a level built on the device).
+// lc_bins_dev.cuh — the two phases of the degree bins (both in lc_bins.cu; the
+// second in lc_level.cu for a level built on the device).
 #pragma once
 
 #include <type_traits>
@@ -40,9 +40,9 @@ __device__ __forceinline__ BinRun bin_run(int64_t n) {
   return BinRun{lo, lo + per < n ? lo + per : n};
 }
 
-// Phase 1 (T threads): the bins of the block's run into w.counts; out: null,
-// or where the hub figures are summed.  A grid barrier follows.  deg_of: the
-// row_degree that the records of phase 2 hold.
+// Phase 1 (T threads): the bins of the block's run into w.counts; the hub
+// figures are summed in *out.  A grid barrier follows.  deg_of: the row_degree
+// that the records of phase 2 hold.
 template <int T, typename Deg>
 __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *out, Deg deg_of) {
   __shared__ int32_t s_cnt[kBins];
@@ -75,29 +75,29 @@ __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *
     const int t = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)cnt[k]);
     if (lane == 0 && t) atomicAdd(&s_cnt[k], t);
   }
-  if (out && longest > 0) {
+  if (longest > 0) {
     atomicAdd((unsigned long long *)&s_chunks, (unsigned long long)chunks);
     atomicMax(&s_max, longest);
   }
   __syncthreads();
   if (threadIdx.x < kBins) w.counts[threadIdx.x * kCoopBlocks + blockIdx.x] = s_cnt[threadIdx.x];
-  if (out && threadIdx.x == 0 && s_max > 0) {
+  if (threadIdx.x == 0 && s_max > 0) {
     atomicAdd((unsigned long long *)&out->chunks, (unsigned long long)s_chunks);
     atomicMax(&out->max_deg, s_max);
   }
 }
 
-// Phase 2: the run's vertices into the lists and records, ascending within
-// each bin; out: null, or where block 0 leaves the bins' starts.  A place past
-// the arrays (row_ptr written to between the phases) is not taken.
+// Phase 2, by a grid of the same size: the vertices of the run that the block
+// counted in phase 1 into the lists and records, ascending within each bin;
+// out: null, or where block 0 leaves the bins' starts.  A place past the
+// arrays (row_ptr written to between the phases) is not taken.
 template <int T, typename Rec>
-__device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, BinOut *out, Rec rec_of) {
+__device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, const BinRun run, BinOut *out, Rec rec_of) {
   constexpr int W = T / 32;
   static_assert(W >= kBins && W <= 32, "a warp per bin, a lane per warp");
   __shared__ int32_t s_cnt[kBins], s_run[kBins];
   __shared__ int32_t s_w[W][kBins + 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const BinRun run = bin_run<T>(n);
   // a bin per warp: its total and what the blocks before this one hold
   if (wid < kBins) {
     int total = 0, before = 0;

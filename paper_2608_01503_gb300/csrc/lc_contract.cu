@@ -259,7 +259,7 @@ __device__ __forceinline__ void emit_slots(const CompactArgs &a, int64_t beg, in
 // batch 59.2 / 57.9).  2,048 slots: the two row searches are 10 probes against
 // 32 loads of 16 bytes per lane.
 constexpr int kCompactRun = 2048;
-__global__ void __launch_bounds__(256) k_compact(CompactArgs a) {
+__device__ __forceinline__ void compact_run(const CompactArgs &a) {
   const int lane = threadIdx.x & 31;
   const int64_t used = 2 * a.off[a.n_c];
   const int64_t s0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kCompactRun;
@@ -277,6 +277,11 @@ __global__ void __launch_bounds__(256) k_compact(CompactArgs a) {
   const int64_t cut = 2 * a.off[last + 1] > s1 ? 2 * a.off[last] : s1;  // the last row goes on after the run
   if (beg < cut) emit_slots(a, beg, cut, a.rp[x], -1, lane);
   if (cut < s1) emit_slots(a, cut, s1, 0, last, lane);
+}
+__global__ void __launch_bounds__(256) k_compact(CompactArgs a) {
+  step_begin();
+  compact_run(a);
+  step_end();
 }
 
 // ProjectCluster.  Labels of a graph live in its own vertex range at every
@@ -384,11 +389,11 @@ void launch_contract_rowptr(const int32_t *cnt, int64_t n_c, int64_t *rp_c, int6
                   cudaMemcpyDeviceToDevice, s);
 }
 
-void launch_contract_compact(unsigned long long *tab, int64_t slots, const int64_t *off, const int64_t *rp_c,
-                             int32_t *cnt, int64_t n_c, int32_t *col_c, int32_t *ew_c, cudaStream_t s) {
+void launch_contract_compact(Step &st, unsigned long long *tab, int64_t slots, const int64_t *off,
+                             const int64_t *rp_c, int32_t *cnt, int64_t n_c, int32_t *col_c, int32_t *ew_c) {
   if (slots <= 0 || n_c <= 0) return;
   const int64_t warps = (slots + kCompactRun - 1) / kCompactRun;
-  k_compact<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(CompactArgs{tab, off, rp_c, cnt, n_c, col_c, ew_c});
+  st.run(false, k_compact, (unsigned)((warps + 7) / 8), 256, 0, CompactArgs{tab, off, rp_c, cnt, n_c, col_c, ew_c});
 }
 
 void launch_graph_ids(const int64_t *gptr, int G, int32_t *gid, int64_t n, cudaStream_t s) {

@@ -13,13 +13,24 @@ constexpr int kCoopBlocks = 152;  // at most one block per SM
 // kBins per block, the new-cluster ids one 64-bit word.
 constexpr int64_t kCoopScratch = (int64_t)kBins * kCoopBlocks;
 
-// Polls before a wait gives up (about 0.6 us each): the launch then sets the
-// error flag and every block returns, so the call ends with LC_ERR_DEVICE.
+// Polls before a wait gives up (about 0.6 us each): the call then ends with
+// LC_ERR_DEVICE (see GridBarrier).
 constexpr unsigned kCoopPolls = 1u << 24;
+
+// Set in bar_arrived, above every count, when a wait ran out.
+constexpr unsigned kBarDead = 1u << 31;
 
 // Arrivals are counted monotonically within a launch; the last block to
 // leave zeroes both counters for the next one.  1.2 us per barrier over 152
 // blocks, measured; a block of its own only synchronises its threads.
+//
+// A wait that ran out marks the counter, which no block zeroes then: the other
+// blocks' waits end at once, and so does the first sync() of every later
+// cooperative kernel of the call.  No phase behind a barrier starts unless all
+// blocks have arrived at it, so what is lost is the kernel's result, and the
+// kernels see to it that what may be followed before the host looks is in
+// range: the bins and a level's end say that they are complete (leave), the
+// passes leave singleton labels, new-cluster ids leave no vertex unlabelled.
 struct GridBarrier {
   Scalars *sc;
   unsigned target = 0;
@@ -31,30 +42,51 @@ struct GridBarrier {
     __shared__ int ok;
     const unsigned nb = gridDim.x;
     __syncthreads();
-    if (nb == 1) return true;
+    if (nb == 1) {
+      if (target != 0) return true;
+      target = 1;
+      if (threadIdx.x == 0) ok = (*(volatile unsigned *)&sc->bar_arrived & kBarDead) == 0;
+      __syncthreads();
+      return ok != 0;
+    }
     target += nb;
     if (threadIdx.x == 0) {
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sc->bar_arrived) : "memory");
+#if LC_DEBUG
+      const unsigned most = sc->dbg_skip ? sc->dbg_polls : kCoopPolls;
+      const bool skip = sc->dbg_skip && blockIdx.x == nb - 1 && ++sc->dbg_syncs == sc->dbg_skip;
+#else
+      constexpr unsigned most = kCoopPolls;
+      constexpr bool skip = false;
+#endif
       unsigned seen = 0, polls = 0;
-      do {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&sc->bar_arrived) : "memory");
-      } while (seen < target && ++polls < kCoopPolls);
-      ok = seen >= target;
-      if (!ok) sc->error = 1;
+      if (!skip) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sc->bar_arrived) : "memory");
+        do {
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&sc->bar_arrived) : "memory");
+        } while (seen < target && ++polls < most);
+      }
+      ok = seen >= target && seen < kBarDead;
+      if (!ok) {
+        sc->error = 1;
+        if (!skip && seen < kBarDead) atomicOr(&sc->bar_arrived, kBarDead);
+      }
     }
     __syncthreads();
     return ok != 0;
   }
 
-  // Once per block after its last sync().
-  __device__ void leave() {
-    if (gridDim.x == 1) return;
+  // Once per block after its last sync(); done: null, or set to 1 once every
+  // block has got here.
+  __device__ void leave(int32_t *done = nullptr) {
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&sc->bar_left, 1u) == gridDim.x - 1) {
+    if (threadIdx.x != 0) return;
+    if (gridDim.x > 1) {
+      if (atomicAdd(&sc->bar_left, 1u) != gridDim.x - 1) return;
       sc->bar_arrived = 0;
       sc->bar_left = 0;
-      __threadfence();
     }
+    if (done) *done = 1;
+    __threadfence();
   }
 };
 

@@ -280,6 +280,10 @@ __global__ void __launch_bounds__(kT, 1)
   const int64_t wbase = tid - lane;  // whole-warp loops start here
   const int G = a.G;
   GridBarrier bar(a.sc);
+  // a barrier's wait ran out: labels that whatever follows may index with
+  auto give_up = [&] {
+    for (int64_t v = threadIdx.x; v < n; v += kT) f.C_out[v] = (int32_t)v;
+  };
 
   for (int s = threadIdx.x; s < kRowSlots; s += kT) {
     keys[s] = 0u;
@@ -302,13 +306,13 @@ __global__ void __launch_bounds__(kT, 1)
   }
   if (tid < 6) f.empties[tid] = 0;
   if (tid < 2 * kNextCount) f.next[tid] = 0;
-  if (!bar.sync()) return;
+  if (!bar.sync()) return give_up();
   if (!f.singleton) {
     for (int64_t v0 = wbase; v0 < n; v0 += nt) {
       const int64_t v = v0 + lane;
       add_weights(a.W, v < n, v < n ? a.C[v] : 0, v < n ? a.g.vw[v] : 0);
     }
-    if (!bar.sync()) return;
+    if (!bar.sync()) return give_up();
   }
 
   for (int i = 0; i < f.passes; ++i) {
@@ -399,7 +403,7 @@ __global__ void __launch_bounds__(kT, 1)
         }
     }
     if (f.big && !first) {
-      if (!bar.sync()) return;
+      if (!bar.sync()) return give_up();
       big_chunks(a, [&](int c, int h, int32_t v) {
         const GraphParam P = a.gp[graph_of(a, v)];
         const int64_t beg = a.g.rp[v];
@@ -423,7 +427,7 @@ __global__ void __launch_bounds__(kT, 1)
       const long long t = block_total(ms.phi, red);
       if (threadIdx.x == 0 && t != 0) atomicAdd((unsigned long long *)acc, (unsigned long long)t);
     }
-    if (!bar.sync()) return;
+    if (!bar.sync()) return give_up();
 
     // ---------------------------------------------------------- update
     // best-of test (Algorithm 2) on the state entering the pass: its labels
@@ -490,11 +494,11 @@ __global__ void __launch_bounds__(kT, 1)
       const int e = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)us.empties);
       if (lane == 0 && e) atomicAdd(&f.empties[i % 3], e);
     }
-    if (!bar.sync()) return;
+    if (!bar.sync()) return give_up();
     const int total = f.empties[i % 3];
     if (total > 0) {  // uniform over the grid
-      if (!assign_empty<kT>(a, f.empty, total, true, bar)) return;
-      if (!bar.sync()) return;
+      if (!assign_empty<kT>(a, f.empty, total, true, bar)) return give_up();
+      if (!bar.sync()) return give_up();
     }
   }
 
@@ -555,7 +559,7 @@ __global__ void __launch_bounds__(kT, 1)
       if (threadIdx.x == 0 && t != 0) atomicAdd((unsigned long long *)f.fin, (unsigned long long)t);
     }
   }
-  if (!bar.sync()) return;
+  if (!bar.sync()) return give_up();
   const long long *acc = f.acc + (int64_t)((p - 1) % 3) * G;
   const long long *best = f.best + (int64_t)(p & 1) * G;
   {

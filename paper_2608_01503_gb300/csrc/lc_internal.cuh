@@ -165,9 +165,10 @@ struct Scalars {
   long long distinct_x;  // (vertex, adjacent cluster) pairs whose W(X) the move step read,
                          // summed over the call (the argmax's gathers, for the profile)
   // barrier of the cooperative kernels: arrivals and blocks that have left,
-  // both zero between launches; on a line of their own
+  // both zero between launches unless a wait ran out; on a line of their own
   alignas(128) unsigned bar_arrived;
   unsigned bar_left;
+  unsigned dbg_skip, dbg_polls, dbg_syncs;  // checked build: the sync() that its last block skips, ...
   int fused_empties[6];      // FusedArgs::empties
   unsigned fused_next[18];   // FusedArgs::next
   // device-side temperature schedule (graph replays): k_pass_begin loads

@@ -1,5 +1,5 @@
-// lc_level.cu — the end of a small coarsening level in two cooperative
-// kernels: label compaction and Algorithm 4's contraction (and the bins of the
+// lc_level.cu — the end of a small coarsening level in one cooperative kernel
+// and two plain ones that run side by side: label compaction and Algorithm 4's contraction (and the bins of the
 // next level), which as separate launches (marks, three scans of three
 // launches each, bounds, six insert kernels, a compaction, two read-backs)
 // took 28 launches of 2-4 us and two more waits of the host, whatever the
@@ -11,6 +11,7 @@
 // scratch, every fine edge that leaves its cluster is inserted there, and
 // the occupied slots in order are the coarse rows.
 #include "lc_bins_dev.cuh"
+#include "lc_contract.cuh"
 #include "lc_coop.cuh"
 #include "lc_group.cuh"
 #include "lc_level.cuh"
@@ -36,19 +37,27 @@ struct EndArgs {
   int32_t *Cd;
   LevelScratch w;
   LevelOut *out;
+  int32_t *bin_counts;  // [kBins][kCoopBlocks]
   Scalars *sc;
 };
 
 // Exclusive scan over the grid of in(i), i < n: out(i, prefix, value); the
-// total to every thread.  Each warp takes a run of its own.  False if a
-// barrier ran out.
+// total to every thread.  Each warp takes a run of its own, a block's warps
+// one after the other.  False if a barrier ran out.
+struct WarpRuns {
+  int64_t per;  // of a warp
+  __device__ explicit WarpRuns(int64_t n) {
+    const int nw = gridDim.x * kW;
+    per = ((n + nw - 1) / nw + 31) / 32 * 32;
+  }
+};
 template <typename In, typename Out>
 __device__ __forceinline__ bool grid_scan(int64_t n, long long *counts, GridBarrier &bar, In in, Out out,
                                           long long &total) {
   __shared__ long long red[kW], red_all[kW];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = gridDim.x * kW, me = blockIdx.x * kW + wid;
-  const int64_t per = ((n + nw - 1) / nw + 31) / 32 * 32;
+  const int64_t per = WarpRuns(n).per;
   const int64_t lo = (int64_t)me * per, hi = lo + per < n ? lo + per : n;
   long long mine = 0;
   for (int64_t i = lo + lane; i < hi; i += 32) mine += in(i);
@@ -201,6 +210,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
             a.w.newid[x] = id;
             a.w.off[id] = at >> 32;
             a.w.vw[id] = a.w.label_w[x];
+            if (a.gid) a.w.gid[id] = a.gid[x];  // a label is a vertex of its graph
           },
           all))
     return;
@@ -211,7 +221,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
     a.w.off[n_c] = all >> 32;
   }
   if (n_c == 0) {  // uniform: the host reads no more than this
-    bar.leave();
+    bar.leave(&a.out->bins.done);
     return;
   }
   if (!bar.sync()) return;
@@ -285,7 +295,8 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
           nnz_c))
     return;
   __syncthreads();
-  // offs[k + 1] counts bin k here; the host sums
+  // the block's run for k_level_build; offs[k + 1] counts bin k here, the host sums
+  if (threadIdx.x < kBins) a.bin_counts[threadIdx.x * kCoopBlocks + blockIdx.x] = s_bin[threadIdx.x];
   if (threadIdx.x < kBins && s_bin[threadIdx.x]) atomicAdd(&a.out->bins.offs[threadIdx.x + 1], s_bin[threadIdx.x]);
   if (threadIdx.x == 0 && s_max > 0) {
     atomicMax(&a.out->bins.max_deg, s_max);
@@ -295,61 +306,42 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
     a.out->nnz_c = nnz_c;
     a.w.rp[n_c] = nnz_c;
   }
-  bar.leave();
+  bar.leave(&a.out->bins.done);
 }
 
 struct BuildArgs {
-  int64_t n, n_c, slots;
-  const int32_t *gid, *Cd;
+  int64_t n_c;
   LevelScratch w;
-  int64_t *rp_c;
-  int32_t *col_c, *ew_c;
-  int64_t *vw_c;
+  int64_t *rp_c, *vw_c;
   int32_t *gid_c;
   BinWork bins;
-  Scalars *sc;
 };
 
-// The coarse graph into its own arrays, and its bins: the row offsets are
-// known, so both of the bins' phases run beside those of the compaction.
-
+// The coarse vertices into their own arrays, and their bins (counted by
+// k_level_end over runs of the same blocks).  A plain kernel, like the
+// compaction of the slots beside it: what follows reads the coarse graph
+// before the host looks at the error flag, so neither may stop half way, as a
+// cooperative kernel's wait can.
 __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ BuildArgs a) {
+  step_begin();
   const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
-  GridBarrier bar(a.sc);
   for (int64_t x = tid; x <= a.n_c; x += nt) {
     a.rp_c[x] = a.w.rp[x];
-    if (x < a.n_c) a.vw_c[x] = a.w.vw[x];
+    if (x == a.n_c) break;
+    a.vw_c[x] = a.w.vw[x];
+    if (a.gid_c) a.gid_c[x] = a.w.gid[x];
   }
-  if (a.gid_c)
-    for (int64_t v = tid; v < a.n; v += nt) {
-      const int32_t x = a.Cd[v];
-      if (x >= 0) a.gid_c[x] = a.gid[v];
-    }
-  bins_count<kT>(a.bins, a.n_c, nullptr, [&](int64_t x) { return row_degree(a.w.rp[x], a.w.rp[x + 1]); });
-  // the occupied slots in order; all slots in use lie below 2 off[n_c]
-  const int64_t slots = 2 * a.w.off[a.n_c];
-  long long nnz = 0;
-  if (!grid_scan(
-          slots, a.w.counts, bar, [&](int64_t s) -> long long { return a.w.tab[s] != kEmptySlot ? 1 : 0; },
-          [&](int64_t s, long long at, long long full) {
-            if (!full) return;
-            const unsigned long long t = a.w.tab[s];
-            a.col_c[at] = slot_key(t);
-            a.ew_c[at] = slot_val(t);
-            a.w.tab[s] = kEmptySlot;
-          },
-          nnz))
-    return;
-  bins_place<kT>(a.bins, a.n_c, nullptr, [&](int64_t x) {
+  const int64_t per = WarpRuns(a.n_c).per * kW, lo = blockIdx.x * per;
+  bins_place<kT>(a.bins, a.n_c, BinRun{lo, lo + per < a.n_c ? lo + per : a.n_c}, nullptr, [&](int64_t x) {
     VRec r{};
     r.v = (int32_t)x;
     r.beg = a.w.rp[x];
     r.deg = row_degree(r.beg, a.w.rp[x + 1]);
-    r.g = a.gid_c ? a.gid_c[x] : 0;
+    r.g = a.gid_c ? a.w.gid[x] : 0;
     r.w = a.w.vw[x];
     return r;
   });
-  bar.leave();
+  step_end();
 }
 
 unsigned level_blocks(int64_t n, int64_t nnz, int coop) {
@@ -363,7 +355,7 @@ unsigned level_blocks(int64_t n, int64_t nnz, int coop) {
 
 void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
                       const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
-                      Scalars *sc, int coop, cudaStream_t s) {
+                      int32_t *bin_counts, Scalars *sc, int coop, cudaStream_t s) {
   cudaMemsetAsync(out, 0, sizeof(LevelOut), s);
   EndArgs a{};
   a.g = g;
@@ -379,29 +371,18 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
   a.Cd = Cd;
   a.w = w;
   a.out = out;
+  a.bin_counts = bin_counts;
   a.sc = sc;
   void *args[] = {&a};
   cudaLaunchCooperativeKernel((const void *)k_level_end, dim3(level_blocks(g.n, g.nnz, coop)), dim3(kT), args, 0, s);
 }
 
-void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
-                        const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
-                        int32_t *gid_c, const BinWork &bins, Scalars *sc, int coop, cudaStream_t s) {
-  BuildArgs a{};
-  a.n = g.n;
-  a.n_c = out.n_c;
-  a.gid = gid;
-  a.Cd = Cd;
-  a.w = w;
-  a.rp_c = rp_c;
-  a.col_c = col_c;
-  a.ew_c = ew_c;
-  a.vw_c = vw_c;
-  a.gid_c = gid_c;
-  a.bins = bins;
-  a.sc = sc;
-  void *args[] = {&a};
-  cudaLaunchCooperativeKernel((const void *)k_level_build, dim3(level_blocks(g.n, g.nnz, coop)), dim3(kT), args, 0, s);
+int launch_level_build(const LevelGraph &g, const LevelScratch &w, const LevelOut &out, int64_t *rp_c, int32_t *col_c,
+                       int32_t *ew_c, int64_t *vw_c, int32_t *gid_c, const BinWork &bins, int coop, cudaStream_t s) {
+  Step st(s);
+  launch_contract_compact(st, w.tab, 2 * g.nnz, w.off, w.rp, w.cnt, out.n_c, col_c, ew_c);
+  st.run(false, k_level_build, level_blocks(g.n, g.nnz, coop), kT, 0, BuildArgs{out.n_c, w, rp_c, vw_c, gid_c, bins});
+  return st.launches;
 }
 
 }  // namespace lc

@@ -5,10 +5,10 @@
 
 namespace lc {
 
-// What the host reads back between the two kernels of a level's end.
+// What the host reads back between the kernels of a level's end.
 struct LevelOut {
   int64_t n_c, nnz_c;  // coarse vertices and stored edges
-  BinOut bins;         // of the coarse graph (offs and hub figures only)
+  BinOut bins;         // of the coarse graph (offs and hub figures only); done: of all of this
 };
 
 // Scratch of a level's end, all sized for the level (int32 [n] unless said).
@@ -19,6 +19,7 @@ struct LevelScratch {
   int64_t *vw, *rp;           // [n], [n + 1]: the coarse weights and row offsets
   unsigned long long *tab;    // [2 nnz] clean hash slots
   int32_t *nc;                // [G] labels in use per graph
+  int32_t *gid;               // [n] graph of a coarse vertex (batches)
   long long *counts;          // [kLevelCounts] per-warp counts
 };
 constexpr int64_t kLevelCounts = 152 * 16 + 16;
@@ -30,11 +31,11 @@ constexpr int64_t kLevelCounts = 152 * 16 + 16;
 // out->n_c = 0 when that is every graph.
 void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
                       const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
-                      Scalars *sc, int coop, cudaStream_t s);
+                      int32_t *bin_counts, Scalars *sc, int coop, cudaStream_t s);
 // The coarse graph from the scratch into its own arrays (out as read back),
 // its graph ids (null for one graph) and its bins; leaves the hash slots clean.
-void launch_level_build(const LevelGraph &g, const int32_t *gid, const int32_t *Cd, const LevelScratch &w,
-                        const LevelOut &out, int64_t *rp_c, int32_t *col_c, int32_t *ew_c, int64_t *vw_c,
-                        int32_t *gid_c, const BinWork &bins, Scalars *sc, int coop, cudaStream_t s);
+// Returns the number of kernels launched.
+int launch_level_build(const LevelGraph &g, const LevelScratch &w, const LevelOut &out, int64_t *rp_c, int32_t *col_c,
+                       int32_t *ew_c, int64_t *vw_c, int32_t *gid_c, const BinWork &bins, int coop, cudaStream_t s);
 
 }  // namespace lc

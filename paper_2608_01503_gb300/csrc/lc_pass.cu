@@ -726,7 +726,13 @@ __global__ void __launch_bounds__(kCoopThreads) k_assign_empty(PassArgs a, Empty
   const int total = a.sc->empty_movers;  // nothing writes it during this launch
   if (total == 0) return;
   GridBarrier bar(a.sc);
-  if (!assign_empty<kCoopThreads>(a, w, total, false, bar)) return;
+  if (!assign_empty<kCoopThreads>(a, w, total, false, bar)) {
+    // every block that gives up labels whatever is still without: the pass's
+    // followers index by the labels, and the host looks later
+    for (int64_t v = threadIdx.x; v < a.g.n; v += kCoopThreads)
+      if (a.C[v] == kEmpty) a.C[v] = (int32_t)v;
+    return;
+  }
   bar.leave();
 }
 

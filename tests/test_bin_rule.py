@@ -64,10 +64,11 @@ def test_degree_is_the_difference_within_its_range(name, bins):
 def test_both_phases_take_the_degree_from_the_rule():
     """Counting and placing bin the one 32-bit degree (the counting phase's
     functor is held to that type; the records store it)."""
+    src = open(os.path.join(_build.CSRC, "lc_bins.cu")).read()
+    count = src[src.index("bins_count<kT>("):]
+    assert "row_degree(" in count[:count.index(";")]
     for name in ("lc_bins.cu", "lc_level.cu"):
         src = open(os.path.join(_build.CSRC, name)).read()
-        count = src[src.index("bins_count<kT>("):]
-        assert "row_degree(" in count[:count.index(";")], name
         place = src[src.index("bins_place<kT>("):]
         assert "r.deg = row_degree(" in place[:place.index("});")], name
 
