@@ -568,9 +568,20 @@ static int capture_pass(Run &r, Level &L, const PassArgs &a, const EmptyScratch 
 // 4.12 / 3.91 / 3.94 / 3.96, R-MAT scale 22 and a 512-graph batch the same
 // within 2 %: a large level wants the separate kernels' occupancy.
 constexpr int64_t kFusedMaxSize = 4000000;
+// Their kernels give a row of bins 5-6 to four warps and one of bins 7-9 to a
+// block of 512 threads, one row after the other on each SM, so such rows have
+// to be long; plans that send shorter ones there (bin_max_deg) run as separate
+// kernels, whose small blocks share an SM.  Measured (ms, separate / fused; an
+// SBM of 100,000 vertices, mean degree 32): bins 5-6 above 32 edges 4.72 /
+// 6.75, above 64 3.89 / 3.55, above 128 3.58 / 3.08 (at mean degree 100, above
+// 64 2.43 / 3.34); bins 7-9 above 64 edges 4.55 / 7.37, above 128 3.78 / 4.33,
+// above 256 3.57 / 3.31 (R-MAT scale 16: 4.86 / 7.28, 4.30 / 4.68, 4.00 / 3.50).
+static bool small_size(const Run &r, const Level &L) {
+  return L.g.n + L.g.nnz <= kFusedMaxSize && r.plan.max_deg[4] >= 128 && r.plan.max_deg[6] >= 256;
+}
 static bool use_fused(const Run &r, const Level &L) {
   return r.o.pass_limit >= 1 && r.o.tables == 0 && r.o.symmetry == 0 && !r.prof.on && !r.o.event_cb &&
-         L.g.n + L.g.nnz <= kFusedMaxSize;
+         small_size(r, L);
 }
 
 // Algorithm 2: `pass_limit` synchronous passes from r.C for the graphs with
@@ -891,7 +902,7 @@ static int compact_level(Run &r, Level &L, Level &N, int level, bool *any) {
 // read-back between them (lc_level.cu); also leaves the
 // sizes of N's bins.
 static bool use_small_level(const Run &r, const Level &L) {
-  return !r.prof.on && !r.o.event_cb && L.g.n + L.g.nnz <= kFusedMaxSize;
+  return !r.prof.on && !r.o.event_cb && small_size(r, L);
 }
 static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   Phase range("lc.contract");
@@ -899,7 +910,7 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   // the passes are over: their records' space holds the labels' weights
   const LevelScratch w{r.used,  r.newid, r.cnt,   r.bound,   reinterpret_cast<int64_t *>(r.ab), r.off, r.W,
                        r.delta, r.gtab,  r.gfree, r.freelist, r.lcounts};
-  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, r.plan, r.C_out, L.Cd, w, r.lout, r.coop, r.sc, r.coop_blocks, r.s);
+  launch_level_end(L.g, L.gid, L.gp, r.G, L.bins, L.hub, r.plan, r.C_out, L.Cd, w, r.lout, r.coop, r.sc, r.coop_blocks, r.s);
   LevelOut out{};
   std::vector<int32_t> nc(r.G);
   LC_CK(cudaMemcpyAsync(&out, r.lout, sizeof(out), cudaMemcpyDeviceToHost, r.s));

@@ -31,6 +31,7 @@ struct EndArgs {
   int32_t G;
   const VRec *rec;
   int64_t off[kBins + 1];
+  Hubs hub;
   int32_t max_deg[kBins - 1];
   int32_t hub_chunk;
   const int32_t *C;
@@ -227,19 +228,16 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
   if (!bar.sync()) return;
   for (int64_t v = tid; v < n; v += nt) a.Cd[v] = goes_on(v) ? a.w.newid[a.C[v]] : -1;
   if (!bar.sync()) return;
-  // insert: rows of bin 9 by all blocks, 7-8 by a block, 3-6 by a warp, 1-2 by eight lanes, bin 0 by a thread
+  // insert: the chunks of bin 9 and the rows of bins 7-8 by a block, 3-6 by a warp, 1-2 by eight lanes, bin 0 by a thread
   bool ok = true;
   {
     __shared__ int s_fresh;
-    // hub rows by all blocks, a piece each
-    for (int64_t i = a.off[kHubBin]; i < a.off[kBins]; ++i) {
-      const VRec vr = a.rec[i];
-      const int32_t x = a.Cd[vr.v];
+    // hub rows by their chunks: with all blocks at one row after the other, the
+    // rows of a few thousand edges kept two of them busy
+    for (int c = blockIdx.x; c < a.hub.Q; c += gridDim.x) {
+      const int32_t x = a.Cd[a.hub.vtx[a.hub.hub_of[c]]];
       if (x < 0) continue;
-      const int64_t end = vr.beg + vr.deg;
-      int f = 0;
-      for (int64_t e = vr.beg + (int64_t)blockIdx.x * 4 * kT; e < end; e += (int64_t)gridDim.x * 4 * kT)
-        f += insert_row<kT>(a, x, e, e + 4 * kT < end ? e + 4 * kT : end, threadIdx.x, ok);
+      int f = insert_row<kT>(a, x, a.hub.e0[c], a.hub.e1[c], threadIdx.x, ok);
       f = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)f);
       if (lane == 0 && f) atomicAdd(&a.w.cnt[x], f);
     }
@@ -354,7 +352,7 @@ unsigned level_blocks(int64_t n, int64_t nnz, int coop) {
 }  // namespace
 
 void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
-                      const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
+                      const Hubs &hub, const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
                       int32_t *bin_counts, Scalars *sc, int coop, cudaStream_t s) {
   cudaMemsetAsync(out, 0, sizeof(LevelOut), s);
   EndArgs a{};
@@ -365,6 +363,7 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
   a.rec = b.recs;
   for (int k = 0; k < kBins; ++k) a.off[k] = b.list[k] - b.list[0];
   a.off[kBins] = g.n;
+  a.hub = hub;
   for (int k = 0; k < kBins - 1; ++k) a.max_deg[k] = (int32_t)plan.max_deg[k];
   a.hub_chunk = (int32_t)plan.hub_chunk;
   a.C = C;

@@ -30,7 +30,7 @@ constexpr int64_t kLevelCounts = 152 * 16 + 16;
 // whose labels all differ is finished: its vertices get Cd = -1, and
 // out->n_c = 0 when that is every graph.
 void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam *gp, int G, const Bins &b,
-                      const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
+                      const Hubs &hub, const BinPlan &plan, const int32_t *C, int32_t *Cd, const LevelScratch &w, LevelOut *out,
                       int32_t *bin_counts, Scalars *sc, int coop, cudaStream_t s);
 // The coarse graph from the scratch into its own arrays (out as read back),
 // its graph ids (null for one graph) and its bins; leaves the hash slots clean.
