@@ -210,7 +210,7 @@ struct Run {
   GraphStats *st = nullptr;
   std::vector<long long> hT, hV, hsw2;
   LevelOut *lout = nullptr;                 // level ends (lc_level.cu)
-  long long *lcounts = nullptr;             // [kLevelCounts]
+  long long *lcounts = nullptr;             // [level_counts]
   std::deque<std::vector<GraphParam>> staged;  // sources of uploads, until the call's work is done
   std::vector<cudaGraphExec_t> execs;  // captured passes (opts.graphs), freed with the call
   explicit Run(const lc_opts &o_) : s((cudaStream_t)o_.stream), o(o_), ar((cudaStream_t)o_.stream, o_) {}
@@ -281,8 +281,8 @@ static int alloc_per_graph(Run &r) {
 }
 
 // The counters of the cooperative kernels.
-static int alloc_counters(Run &r) {
-  LC_TRY(r.ar.get(&r.coop, kCoopScratch));
+static int alloc_counters(Run &r, int64_t n0, int64_t nnz0) {
+  LC_TRY(r.ar.get(&r.coop, coop_scratch(n0, nnz0)));
   LC_TRY(r.ar.get(&r.sc, 1));
   LC_CK(cudaMemsetAsync(r.sc, 0, sizeof(Scalars), r.s));
 #if LC_DEBUG
@@ -318,7 +318,7 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
   LC_TRY(r.ar.get(&r.W, n0));
   LC_TRY(r.ar.get(&r.delta, n0));
   LC_TRY(r.ar.get(&r.ab, n0));
-  LC_TRY(r.ar.get(&r.lcounts, kLevelCounts));
+  LC_TRY(r.ar.get(&r.lcounts, level_counts(n0, nnz0)));
   LC_TRY(r.ar.get(&r.lout, 1));
   LC_TRY(r.ar.get(&r.bound, n0 + 1));
   LC_TRY(r.ar.get(&r.off, n0 + 1));
@@ -369,12 +369,12 @@ static int resolve_plan(const lc_opts &o, BinPlan *out) {
 static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tables) {
   const int64_t n = n0 > 0 ? n0 : 1, big = 2 * nnz0 > n0 + 1 ? 2 * nnz0 : n0 + 1;
   int64_t b = per_graph_bytes(G);                            // alloc_per_graph
-  b += 4 * kCoopScratch + (int64_t)sizeof(Scalars);          // alloc_counters
+  b += 4 * coop_scratch(n0, nnz0) + (int64_t)sizeof(Scalars);  // alloc_counters
   b += 8 * 4 * n;                                            // C .. movers
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
   b += 4 * scan_scratch(big);                                // scan32
   b += 2 * 8 * n + (int64_t)sizeof(AbRec) * n;               // W, delta, ab
-  b += 8 * kLevelCounts + (int64_t)sizeof(LevelOut);         // lcounts, lout
+  b += 8 * level_counts(n0, nnz0) + (int64_t)sizeof(LevelOut);  // lcounts, lout
   b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + n;      // bound, off, scan64, M
   b += 8 * (2 * nnz0 > 0 ? 2 * nnz0 : 1);                    // gtab
   if (G > 1) b += 8 * (G + 1) + 4 * n;                       // graph_ptr, gid
@@ -1186,7 +1186,7 @@ static int set_up(Run &r, Level &L, const LevelGraph &g0, const std::vector<int6
   LC_TRY(begin_prepare(r, g0, L.gid));
   if (labels) launch_labels_in_range(labels, g0.n, limit, r.st, r.s);
   BinOut *d_out = nullptr, out{};
-  int rc = alloc_counters(r);
+  int rc = alloc_counters(r, g0.n, g0.nnz);
   if (rc == LC_OK) rc = begin_bins(r, L, &d_out);
   if (rc == LC_OK) rc = alloc_scratch(r, g0.n, g0.nnz);
   if (rc == LC_OK && !passes_only) rc = clear_table(r, g0.nnz);

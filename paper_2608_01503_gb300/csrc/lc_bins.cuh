@@ -15,8 +15,8 @@ struct BinOut {
 
 // Fills b.lists and b.recs (ascending ids within each bin) and *out, all on
 // the device; gid: graph of each vertex, or null for one graph.  counts:
-// int32[kBins * kCoopBlocks] scratch; coop: blocks the launch may have.  The caller copies *out to the host
-// and passes it to finish_bins.
+// int32[coop_scratch] scratch; coop: blocks the launch may have.  The caller
+// copies *out to the host and passes it to finish_bins.
 void launch_bins(const LevelGraph &g, const int32_t *gid, const BinPlan &plan, const Bins &b, BinOut *out,
                  int32_t *counts, Scalars *sc, int coop, cudaStream_t s);
 void finish_bins(Bins &b, const BinOut &out);

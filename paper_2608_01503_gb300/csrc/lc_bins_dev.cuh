@@ -16,7 +16,7 @@ struct BinWork {
   int32_t hub_chunk;
   VRec *recs;
   int32_t *lists;
-  int32_t *counts;  // [kBins][kCoopBlocks]
+  int32_t *counts;  // [kBins][blocks of the launch]
 };
 
 inline BinWork bin_work(const BinPlan &plan, const Bins &b, int32_t *counts) {
@@ -80,7 +80,7 @@ __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *
     atomicMax(&s_max, longest);
   }
   __syncthreads();
-  if (threadIdx.x < kBins) w.counts[threadIdx.x * kCoopBlocks + blockIdx.x] = s_cnt[threadIdx.x];
+  if (threadIdx.x < kBins) w.counts[threadIdx.x * gridDim.x + blockIdx.x] = s_cnt[threadIdx.x];
   if (threadIdx.x == 0 && s_max > 0) {
     atomicAdd((unsigned long long *)&out->chunks, (unsigned long long)s_chunks);
     atomicMax(&out->max_deg, s_max);
@@ -102,7 +102,7 @@ __device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, const Bi
   if (wid < kBins) {
     int total = 0, before = 0;
     for (int b = lane; b < (int)gridDim.x; b += 32) {
-      const int c = w.counts[wid * kCoopBlocks + b];
+      const int c = w.counts[wid * gridDim.x + b];
       total += c;
       before += b < (int)blockIdx.x ? c : 0;
     }

@@ -9,9 +9,22 @@ namespace lc {
 constexpr int kCoopThreads = 1024;
 constexpr int kCoopBlocks = 152;  // at most one block per SM
 
-// int32 entries of a call's scratch for the blocks' counts: the bins' count
-// kBins per block, the new-cluster ids one 64-bit word.
-constexpr int64_t kCoopScratch = (int64_t)kBins * kCoopBlocks;
+// Blocks of the passes' and a level end's launches for n vertices and nnz
+// stored edges: one per 64 vertices or 1,024 edges, at most one per SM.
+inline int64_t level_grid(int64_t n, int64_t nnz) {
+  const int64_t b = n / 64 > nnz / 1024 ? n / 64 : nnz / 1024;
+  return b < 1 ? 1 : b > kCoopBlocks ? kCoopBlocks : b;
+}
+// The most blocks any cooperative launch of a call on such a graph has (the
+// bins take one per kCoopThreads vertices, new-cluster ids fewer); its scratch
+// is sized by it, so that a graph of a few vertices takes little.
+inline int64_t coop_most(int64_t n, int64_t nnz) {
+  const int64_t b = level_grid(n, nnz), bins = (n + kCoopThreads - 1) / kCoopThreads;
+  return bins > kCoopBlocks ? kCoopBlocks : b > bins ? b : bins;
+}
+// int32 entries for the blocks' counts: kBins a block for the bins, one 64-bit
+// word for the new-cluster ids.
+inline int64_t coop_scratch(int64_t n, int64_t nnz) { return (int64_t)kBins * coop_most(n, nnz); }
 
 // Polls before a wait gives up (about 0.6 us each): the call then ends with
 // LC_ERR_DEVICE (see GridBarrier).

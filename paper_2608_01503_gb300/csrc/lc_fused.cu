@@ -588,10 +588,8 @@ void configure_fused() {
 int64_t fused_row_max() { return kRowMaxDeg; }
 
 int launch_fused_passes(const PassArgs &a, const FusedArgs &f, cudaStream_t s) {
-  // a block per 64 vertices or 1,024 stored edges, at most one per SM
-  int64_t blocks = a.g.n / 64 > a.g.nnz / 1024 ? a.g.n / 64 : a.g.nnz / 1024;
+  int64_t blocks = level_grid(a.g.n, a.g.nnz);
   if (blocks > coop_blocks(a.coop)) blocks = coop_blocks(a.coop);
-  if (blocks < 1) blocks = 1;
   PassArgs pa = a;
   FusedArgs fa = f;
   void *args[] = {&pa, &fa};

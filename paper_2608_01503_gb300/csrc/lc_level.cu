@@ -22,7 +22,7 @@ namespace lc {
 namespace {
 
 constexpr int kT = 512, kW = kT / 32;
-static_assert(kLevelCounts >= (int64_t)kCoopBlocks * kW, "one count per warp");
+static_assert(kLevelWarps == kW, "one count per warp");
 
 struct EndArgs {
   LevelGraph g;
@@ -38,7 +38,7 @@ struct EndArgs {
   int32_t *Cd;
   LevelScratch w;
   LevelOut *out;
-  int32_t *bin_counts;  // [kBins][kCoopBlocks]
+  int32_t *bin_counts;  // [kBins][blocks]
   Scalars *sc;
 };
 
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
     return;
   __syncthreads();
   // the block's run for k_level_build; offs[k + 1] counts bin k here, the host sums
-  if (threadIdx.x < kBins) a.bin_counts[threadIdx.x * kCoopBlocks + blockIdx.x] = s_bin[threadIdx.x];
+  if (threadIdx.x < kBins) a.bin_counts[threadIdx.x * gridDim.x + blockIdx.x] = s_bin[threadIdx.x];
   if (threadIdx.x < kBins && s_bin[threadIdx.x]) atomicAdd(&a.out->bins.offs[threadIdx.x + 1], s_bin[threadIdx.x]);
   if (threadIdx.x == 0 && s_max > 0) {
     atomicMax(&a.out->bins.max_deg, s_max);
@@ -343,10 +343,8 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
 }
 
 unsigned level_blocks(int64_t n, int64_t nnz, int coop) {
-  // a block per 64 vertices or 1,024 stored edges, at most one per SM
-  int64_t blocks = n / 64 > nnz / 1024 ? n / 64 : nnz / 1024;
-  if (blocks > coop_blocks(coop)) blocks = coop_blocks(coop);
-  return (unsigned)(blocks < 1 ? 1 : blocks);
+  const int64_t blocks = level_grid(n, nnz), most = coop_blocks(coop);
+  return (unsigned)(blocks < most ? blocks : most);
 }
 
 }  // namespace

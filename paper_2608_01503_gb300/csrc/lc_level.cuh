@@ -20,9 +20,10 @@ struct LevelScratch {
   unsigned long long *tab;    // [2 nnz] clean hash slots
   int32_t *nc;                // [G] labels in use per graph
   int32_t *gid;               // [n] graph of a coarse vertex (batches)
-  long long *counts;          // [kLevelCounts] per-warp counts
+  long long *counts;          // [level_counts] per-warp counts
 };
-constexpr int64_t kLevelCounts = 152 * 16 + 16;
+constexpr int kLevelWarps = 16;  // of a block
+inline int64_t level_counts(int64_t n, int64_t nnz) { return kLevelWarps * level_grid(n, nnz); }
 
 // The labels C (ids in [0, n)) of a level numbered densely per graph that
 // merges something, the contraction's offsets, inserts and coarse row
