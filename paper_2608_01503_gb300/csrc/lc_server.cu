@@ -170,6 +170,7 @@ void run_batch(lc_server *s, cudaStream_t st, std::vector<Job *> &batch, bool li
     // the estimate was short: back to the head of the queue, in order, with
     // twice the reservation, to wait for memory
     std::lock_guard<std::mutex> lock(s->mu);
+    s->busy--;
     for (int k = count - 1; k >= 0; --k) {
       Job &j = *batch[k];
       s->claimed -= j.footprint;
@@ -194,6 +195,7 @@ void run_batch(lc_server *s, cudaStream_t st, std::vector<Job *> &batch, bool li
   }
   const auto now = Clock::now();
   std::lock_guard<std::mutex> lock(s->mu);
+  s->busy--;  // before anybody is told: a waiter's next request is not beside this one
   for (int k = 0; k < count; ++k) {
     Job &j = *batch[k];
     j.rc = rcs[k];
@@ -249,7 +251,8 @@ void worker(lc_server *s) {
             s->claimed += add;
             // A small level's cooperative kernel keeps every SM it gets to
             // itself and leaves most of it idle, waiting; slots that run at
-            // the same time split the SMs instead of taking turns.
+            // the same time split the SMs instead of taking turns.  The share is
+            // what admission finds and stays for the admission.
             s->busy++;
             const int beside = std::min<int64_t>(s->cfg.slots, s->busy + (int64_t)s->queue.size());
             coop_blocks = lc::kCoopBlocks / beside;
@@ -261,8 +264,6 @@ void worker(lc_server *s) {
     }
     if (batch.empty()) break;
     run_batch(s, st, batch, limited, coop_blocks);
-    std::lock_guard<std::mutex> lock(s->mu);
-    s->busy--;
   }
   cudaStreamDestroy(st);
 }
