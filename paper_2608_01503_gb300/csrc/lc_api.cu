@@ -440,6 +440,7 @@ static int bins_for(Run &r, Level &L) {
   LC_TRY(begin_bins(r, L, &d_out));
   LC_CK(cudaMemcpyAsync(&out, d_out, sizeof(out), cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaStreamSynchronize(r.s));
+  r.ar.release(d_out);
   return end_bins(r, L, out);
 }
 
@@ -793,7 +794,8 @@ static int constrained_passes(Run &r, Level &L, int level, const std::vector<uin
   r.res->kernel_launches[LC_K_OTHER] += 5;
   L.g = LevelGraph{full.n, nnz_f, rp_f, col_f, ew_f, full.vw};
   int rc = bins_for(r, L);
-  int32_t *lists_f = L.bins.lists;
+  const Bins bins_f = L.bins;
+  const void *hub_f = L.hub.e0;  // the start of the hub plan's block
   if (rc == LC_OK) rc = local_move_passes(r, L, true, level, 0, present);
   L.g = full;
   L.bins = full_bins;
@@ -803,7 +805,9 @@ static int constrained_passes(Run &r, Level &L, int level, const std::vector<uin
     r.ar.release(col_f);
     r.ar.release(ew_f);
     r.ar.release(rp_f);
-    if (lists_f != full_bins.lists) r.ar.release(lists_f);
+    r.ar.release(bins_f.lists);
+    r.ar.release(bins_f.recs);
+    r.ar.release(const_cast<void *>(hub_f));
   }
   return rc;
 }

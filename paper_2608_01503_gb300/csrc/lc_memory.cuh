@@ -70,6 +70,7 @@ struct Arena {
     }
   }
   void release(void *p) {
+    if (!p) return;
     for (size_t i = 0; i < ptrs.size(); ++i)
       if (ptrs[i] == p) {
         dev_free(o, s, p, sizes[i]);
