@@ -902,7 +902,7 @@ static int compact_level(Run &r, Level &L, Level &N, int level, bool *any) {
   return launch_check();
 }
 
-// compact_level and contract_level of a small level in three kernels with one
+// compact_level and contract_level of a small level in two kernels with one
 // read-back between them (lc_level.cu); also leaves the
 // sizes of N's bins.
 static bool use_small_level(const Run &r, const Level &L) {
@@ -952,8 +952,8 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   int32_t *col_c = nullptr, *ew_c = nullptr;
   LC_TRY(r.ar.get(&col_c, out.nnz_c));
   LC_TRY(r.ar.get(&ew_c, out.nnz_c));
-  r.res->kernel_launches[LC_K_CONTRACT] += launch_level_build(
-      L.g, w, out, rp_c, col_c, ew_c, vw_c, N.gid, bin_work(r.plan, N.bins, r.coop), r.coop_blocks, r.s);
+  launch_level_build(L.g, w, out, rp_c, col_c, ew_c, vw_c, N.gid, bin_work(r.plan, N.bins, r.coop), r.coop_blocks, r.s);
+  r.res->kernel_launches[LC_K_CONTRACT] += 1;
   r.res->edges_contract += L.g.nnz;
   N.g = LevelGraph{out.n_c, out.nnz_c, rp_c, col_c, ew_c, vw_c};
   N.bin_out = out.bins;
@@ -983,8 +983,7 @@ static int contract_level(Run &r, Level &L, Level &N, int level) {
   LC_TRY(r.ar.get(&col_c, nnz_c));
   LC_TRY(r.ar.get(&ew_c, nnz_c));
   r.prof.begin(LC_K_CONTRACT);
-  Step compact(r.s);
-  launch_contract_compact(compact, r.gtab, 2 * L.g.nnz, r.off, rp_c, r.cnt, n_c, col_c, ew_c);
+  launch_contract_compact(r.gtab, 2 * L.g.nnz, r.off, rp_c, r.cnt, n_c, col_c, ew_c, r.s);
   r.prof.end(16.0 * L.g.nnz + 8.0 * nnz_c);
   r.res->kernel_launches[LC_K_CONTRACT] += 9 + ni;
   LC_TRY(launch_check());
@@ -1854,8 +1853,7 @@ int lc_contract(const lc_csr *g, const int64_t *vertex_w, const int32_t *edge_w,
       r.res->error_detail = nnz_c;
     }
     if (rc == LC_OK) {
-      Step compact(r.s);
-      launch_contract_compact(compact, r.gtab, 2 * g->nnz, r.off, c_row_ptr, r.cnt, n_c, c_col, c_ew);
+      launch_contract_compact(r.gtab, 2 * g->nnz, r.off, c_row_ptr, r.cnt, n_c, c_col, c_ew, r.s);
       rc = launch_check();
     }
     if (rc == LC_OK) rc = check_device_error(r);

@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kT, 1) k_bins(const __grid_constant__ BinArgs 
   GridBarrier bar(a.sc);
   bins_count<kT>(a.w, a.g.n, a.out, [&](int64_t v) { return row_degree(rp[v], rp[v + 1]); });
   if (!bar.sync()) return;
-  bins_place<kT>(a.w, a.g.n, bin_run<kT>(a.g.n), a.out, [&](int64_t v) {
+  bins_place<kT>(a.w, a.g.n, bin_run<kT>(a.g.n), gridDim.x, a.out, [&](int64_t v) {
     VRec r{};
     r.v = (int32_t)v;
     r.beg = rp[v];

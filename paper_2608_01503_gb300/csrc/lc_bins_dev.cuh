@@ -87,12 +87,13 @@ __device__ __forceinline__ void bins_count(const BinWork &w, int64_t n, BinOut *
   }
 }
 
-// Phase 2, by a grid of the same size: the vertices of the run that the block
-// counted in phase 1 into the lists and records, ascending within each bin;
+// Phase 2, by as many blocks: the vertices of the run that the block of this
+// number counted in phase 1 into the lists and records, ascending in each bin;
 // out: null, or where block 0 leaves the bins' starts.  A place past the
 // arrays (row_ptr written to between the phases) is not taken.
 template <int T, typename Rec>
-__device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, const BinRun run, BinOut *out, Rec rec_of) {
+__device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, const BinRun run, int blocks, BinOut *out,
+                                           Rec rec_of) {
   constexpr int W = T / 32;
   static_assert(W >= kBins && W <= 32, "a warp per bin, a lane per warp");
   __shared__ int32_t s_cnt[kBins], s_run[kBins];
@@ -101,8 +102,8 @@ __device__ __forceinline__ void bins_place(const BinWork &w, int64_t n, const Bi
   // a bin per warp: its total and what the blocks before this one hold
   if (wid < kBins) {
     int total = 0, before = 0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) {
-      const int c = w.counts[wid * gridDim.x + b];
+    for (int b = lane; b < blocks; b += 32) {
+      const int c = w.counts[wid * blocks + b];
       total += c;
       before += b < (int)blockIdx.x ? c : 0;
     }

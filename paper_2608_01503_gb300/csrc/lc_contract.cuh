@@ -2,7 +2,6 @@
 #pragma once
 
 #include "lc_internal.cuh"
-#include "lc_step.cuh"
 
 namespace lc {
 
@@ -34,8 +33,8 @@ void launch_contract_rowptr(const int32_t *cnt, int64_t n_c, int64_t *rp_c, int6
                             cudaStream_t s);
 // Algorithm 4, line 13: the table's slots (2 off[n_c] of at most `slots`) into
 // the coarse CSR; leaves the table clean and uses cnt up.
-void launch_contract_compact(Step &st, unsigned long long *tab, int64_t slots, const int64_t *off,
-                             const int64_t *rp_c, int32_t *cnt, int64_t n_c, int32_t *col_c, int32_t *ew_c);
+void launch_contract_compact(unsigned long long *tab, int64_t slots, const int64_t *off, const int64_t *rp_c,
+                             int32_t *cnt, int64_t n_c, int32_t *col_c, int32_t *ew_c, cudaStream_t s);
 // gid[v] for a packed batch with vertex ranges gptr[0..G] (device).
 void launch_graph_ids(const int64_t *gptr, int G, int32_t *gid, int64_t n, cudaStream_t s);
 // C[v] = vbase_fine(g) + Cnext[Cd[v]] - vbase_coarse(g) (Cd[v] < 0: C[v] = v)

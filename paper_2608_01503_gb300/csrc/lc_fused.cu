@@ -260,6 +260,12 @@ __device__ __forceinline__ void big_chunks(const PassArgs &a, Body body) {
   }
 }
 
+// A barrier's wait ran out: labels that whatever follows may index with.  Not
+// inlined at the barriers: that cost the passes 1 %.
+__device__ __noinline__ void give_up(int32_t *C_out, int64_t n) {
+  for (int64_t v = threadIdx.x; v < n; v += kT) C_out[v] = (int32_t)v;
+}
+
 __global__ void __launch_bounds__(kT, 1)
     k_passes(const __grid_constant__ PassArgs a, const __grid_constant__ FusedArgs f) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -280,10 +286,6 @@ __global__ void __launch_bounds__(kT, 1)
   const int64_t wbase = tid - lane;  // whole-warp loops start here
   const int G = a.G;
   GridBarrier bar(a.sc);
-  // a barrier's wait ran out: labels that whatever follows may index with
-  auto give_up = [&] {
-    for (int64_t v = threadIdx.x; v < n; v += kT) f.C_out[v] = (int32_t)v;
-  };
 
   for (int s = threadIdx.x; s < kRowSlots; s += kT) {
     keys[s] = 0u;
@@ -306,13 +308,13 @@ __global__ void __launch_bounds__(kT, 1)
   }
   if (tid < 6) f.empties[tid] = 0;
   if (tid < 2 * kNextCount) f.next[tid] = 0;
-  if (!bar.sync()) return give_up();
+  if (!bar.sync()) return give_up(f.C_out, n);
   if (!f.singleton) {
     for (int64_t v0 = wbase; v0 < n; v0 += nt) {
       const int64_t v = v0 + lane;
       add_weights(a.W, v < n, v < n ? a.C[v] : 0, v < n ? a.g.vw[v] : 0);
     }
-    if (!bar.sync()) return give_up();
+    if (!bar.sync()) return give_up(f.C_out, n);
   }
 
   for (int i = 0; i < f.passes; ++i) {
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kT, 1)
         }
     }
     if (f.big && !first) {
-      if (!bar.sync()) return give_up();
+      if (!bar.sync()) return give_up(f.C_out, n);
       big_chunks(a, [&](int c, int h, int32_t v) {
         const GraphParam P = a.gp[graph_of(a, v)];
         const int64_t beg = a.g.rp[v];
@@ -427,7 +429,7 @@ __global__ void __launch_bounds__(kT, 1)
       const long long t = block_total(ms.phi, red);
       if (threadIdx.x == 0 && t != 0) atomicAdd((unsigned long long *)acc, (unsigned long long)t);
     }
-    if (!bar.sync()) return give_up();
+    if (!bar.sync()) return give_up(f.C_out, n);
 
     // ---------------------------------------------------------- update
     // best-of test (Algorithm 2) on the state entering the pass: its labels
@@ -494,11 +496,11 @@ __global__ void __launch_bounds__(kT, 1)
       const int e = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)us.empties);
       if (lane == 0 && e) atomicAdd(&f.empties[i % 3], e);
     }
-    if (!bar.sync()) return give_up();
+    if (!bar.sync()) return give_up(f.C_out, n);
     const int total = f.empties[i % 3];
     if (total > 0) {  // uniform over the grid
-      if (!assign_empty<kT>(a, f.empty, total, true, bar)) return give_up();
-      if (!bar.sync()) return give_up();
+      if (!assign_empty<kT>(a, f.empty, total, true, bar)) return give_up(f.C_out, n);
+      if (!bar.sync()) return give_up(f.C_out, n);
     }
   }
 
@@ -559,7 +561,7 @@ __global__ void __launch_bounds__(kT, 1)
       if (threadIdx.x == 0 && t != 0) atomicAdd((unsigned long long *)f.fin, (unsigned long long)t);
     }
   }
-  if (!bar.sync()) return give_up();
+  if (!bar.sync()) return give_up(f.C_out, n);
   const long long *acc = f.acc + (int64_t)((p - 1) % 3) * G;
   const long long *best = f.best + (int64_t)(p & 1) * G;
   {

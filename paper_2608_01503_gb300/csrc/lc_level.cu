@@ -1,5 +1,5 @@
-// lc_level.cu — the end of a small coarsening level in one cooperative kernel
-// and two plain ones that run side by side: label compaction and Algorithm 4's contraction (and the bins of the
+// lc_level.cu — the end of a small coarsening level in a cooperative kernel and
+// a plain one: label compaction and Algorithm 4's contraction (and the bins of the
 // next level), which as separate launches (marks, three scans of three
 // launches each, bounds, six insert kernels, a compaction, two read-backs)
 // took 28 launches of 2-4 us and two more waits of the host, whatever the
@@ -11,7 +11,7 @@
 // scratch, every fine edge that leaves its cluster is inserted there, and
 // the occupied slots in order are the coarse rows.
 #include "lc_bins_dev.cuh"
-#include "lc_contract.cuh"
+#include "lc_compact_dev.cuh"
 #include "lc_coop.cuh"
 #include "lc_group.cuh"
 #include "lc_level.cuh"
@@ -45,20 +45,17 @@ struct EndArgs {
 // Exclusive scan over the grid of in(i), i < n: out(i, prefix, value); the
 // total to every thread.  Each warp takes a run of its own, a block's warps
 // one after the other.  False if a barrier ran out.
-struct WarpRuns {
-  int64_t per;  // of a warp
-  __device__ explicit WarpRuns(int64_t n) {
-    const int nw = gridDim.x * kW;
-    per = ((n + nw - 1) / nw + 31) / 32 * 32;
-  }
-};
+__device__ __forceinline__ int64_t warp_run(int64_t n, int blocks) {
+  const int nw = blocks * kW;
+  return ((n + nw - 1) / nw + 31) / 32 * 32;
+}
 template <typename In, typename Out>
 __device__ __forceinline__ bool grid_scan(int64_t n, long long *counts, GridBarrier &bar, In in, Out out,
                                           long long &total) {
   __shared__ long long red[kW], red_all[kW];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = gridDim.x * kW, me = blockIdx.x * kW + wid;
-  const int64_t per = WarpRuns(n).per;
+  const int64_t per = warp_run(n, gridDim.x);
   const int64_t lo = (int64_t)me * per, hi = lo + per < n ? lo + per : n;
   long long mine = 0;
   for (int64_t i = lo + lane; i < hi; i += 32) mine += in(i);
@@ -308,29 +305,40 @@ __global__ void __launch_bounds__(kT, 1) k_level_end(const __grid_constant__ End
 }
 
 struct BuildArgs {
-  int64_t n_c;
+  CompactArgs slots;
   LevelScratch w;
   int64_t *rp_c, *vw_c;
   int32_t *gid_c;
   BinWork bins;
 };
 
-// The coarse vertices into their own arrays, and their bins (counted by
-// k_level_end over runs of the same blocks).  A plain kernel, like the
-// compaction of the slots beside it: what follows reads the coarse graph
-// before the host looks at the error flag, so neither may stop half way, as a
-// cooperative kernel's wait can.
-__global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ BuildArgs a) {
-  step_begin();
-  const int64_t tid = (int64_t)blockIdx.x * kT + threadIdx.x, nt = (int64_t)gridDim.x * kT;
-  for (int64_t x = tid; x <= a.n_c; x += nt) {
+// The coarse graph into its own arrays, and its bins (counted by k_level_end
+// over runs of half as many blocks): the first half of the blocks takes the
+// vertices, the other the edges.  A plain kernel: what follows reads the
+// coarse graph before the host looks at the error flag, so it may not stop
+// half way, as a cooperative kernel's wait can.  All levels of an SBM of 10,000
+// vertices: 51 us as one cooperative kernel with a scan over the slots, 65 us
+// with all blocks at the edges and then the vertices, 31 us like this.
+__global__ void __launch_bounds__(kT, 2) k_level_build(const __grid_constant__ BuildArgs a) {
+  const int64_t n_c = a.slots.n_c;
+  const int blocks = gridDim.x / 2, me = (int)blockIdx.x - blocks;
+  if (me >= 0) {
+    // short runs where there are warps for them: a run's 256 slots a step are a chain
+    const int64_t used = 2 * a.w.off[n_c], nw = (int64_t)blocks * kW;
+    int64_t run = (used + 256 * nw - 1) / (256 * nw) * 256;
+    run = run > kCompactRun ? kCompactRun : run;
+    for (int64_t s = ((int64_t)(threadIdx.x >> 5) * blocks + me) * run; s < used; s += nw * run)
+      compact_run(a.slots, s, run, used);
+    return;
+  }
+  for (int64_t x = (int64_t)blockIdx.x * kT + threadIdx.x; x <= n_c; x += (int64_t)blocks * kT) {
     a.rp_c[x] = a.w.rp[x];
-    if (x == a.n_c) break;
+    if (x == n_c) break;
     a.vw_c[x] = a.w.vw[x];
     if (a.gid_c) a.gid_c[x] = a.w.gid[x];
   }
-  const int64_t per = WarpRuns(a.n_c).per * kW, lo = blockIdx.x * per;
-  bins_place<kT>(a.bins, a.n_c, BinRun{lo, lo + per < a.n_c ? lo + per : a.n_c}, nullptr, [&](int64_t x) {
+  const int64_t per = warp_run(n_c, blocks) * kW, lo = blockIdx.x * per;
+  bins_place<kT>(a.bins, n_c, BinRun{lo, lo + per < n_c ? lo + per : n_c}, blocks, nullptr, [&](int64_t x) {
     VRec r{};
     r.v = (int32_t)x;
     r.beg = a.w.rp[x];
@@ -339,7 +347,6 @@ __global__ void __launch_bounds__(kT, 1) k_level_build(const __grid_constant__ B
     r.w = a.w.vw[x];
     return r;
   });
-  step_end();
 }
 
 unsigned level_blocks(int64_t n, int64_t nnz, int coop) {
@@ -374,12 +381,10 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
   cudaLaunchCooperativeKernel((const void *)k_level_end, dim3(level_blocks(g.n, g.nnz, coop)), dim3(kT), args, 0, s);
 }
 
-int launch_level_build(const LevelGraph &g, const LevelScratch &w, const LevelOut &out, int64_t *rp_c, int32_t *col_c,
-                       int32_t *ew_c, int64_t *vw_c, int32_t *gid_c, const BinWork &bins, int coop, cudaStream_t s) {
-  Step st(s);
-  launch_contract_compact(st, w.tab, 2 * g.nnz, w.off, w.rp, w.cnt, out.n_c, col_c, ew_c);
-  st.run(false, k_level_build, level_blocks(g.n, g.nnz, coop), kT, 0, BuildArgs{out.n_c, w, rp_c, vw_c, gid_c, bins});
-  return st.launches;
+void launch_level_build(const LevelGraph &g, const LevelScratch &w, const LevelOut &out, int64_t *rp_c, int32_t *col_c,
+                        int32_t *ew_c, int64_t *vw_c, int32_t *gid_c, const BinWork &bins, int coop, cudaStream_t s) {
+  const CompactArgs slots{w.tab, w.off, w.rp, w.cnt, out.n_c, col_c, ew_c};
+  k_level_build<<<2 * level_blocks(g.n, g.nnz, coop), kT, 0, s>>>(BuildArgs{slots, w, rp_c, vw_c, gid_c, bins});
 }
 
 }  // namespace lc

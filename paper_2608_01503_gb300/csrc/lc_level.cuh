@@ -35,8 +35,7 @@ void launch_level_end(const LevelGraph &g, const int32_t *gid, const GraphParam 
                       int32_t *bin_counts, Scalars *sc, int coop, cudaStream_t s);
 // The coarse graph from the scratch into its own arrays (out as read back),
 // its graph ids (null for one graph) and its bins; leaves the hash slots clean.
-// Returns the number of kernels launched.
-int launch_level_build(const LevelGraph &g, const LevelScratch &w, const LevelOut &out, int64_t *rp_c, int32_t *col_c,
-                       int32_t *ew_c, int64_t *vw_c, int32_t *gid_c, const BinWork &bins, int coop, cudaStream_t s);
+void launch_level_build(const LevelGraph &g, const LevelScratch &w, const LevelOut &out, int64_t *rp_c, int32_t *col_c,
+                        int32_t *ew_c, int64_t *vw_c, int32_t *gid_c, const BinWork &bins, int coop, cudaStream_t s);
 
 }  // namespace lc
