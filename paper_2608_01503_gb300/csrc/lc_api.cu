@@ -313,8 +313,7 @@ static int alloc_scratch(Run &r, int64_t n0, int64_t nnz0) {
     LC_TRY(r.ar.get(&r.upd_list, upd_list_size(n0, nnz0)));
     LC_CK(cudaMemsetAsync(r.dirty, 0, sizeof(int32_t) * (size_t)(n0 > 0 ? n0 : 1), r.s));
   }
-  const int64_t big = 2 * nnz0 > n0 + 1 ? 2 * nnz0 : n0 + 1;
-  LC_TRY(r.ar.get(&r.scan32, scan_scratch(big)));
+  LC_TRY(r.ar.get(&r.scan32, scan_scratch(n0)));
   LC_TRY(r.ar.get(&r.W, n0));
   LC_TRY(r.ar.get(&r.delta, n0));
   LC_TRY(r.ar.get(&r.ab, n0));
@@ -367,12 +366,12 @@ static int resolve_plan(const lc_opts &o, BinPlan *out) {
 // bins, hub plan, parameters, dense ids and coarse graph (bins_for,
 // upload_params, compact_level, contract_level), for the footprint below.
 static int64_t level0_scratch_bytes(int64_t n0, int64_t nnz0, int64_t G, int tables) {
-  const int64_t n = n0 > 0 ? n0 : 1, big = 2 * nnz0 > n0 + 1 ? 2 * nnz0 : n0 + 1;
+  const int64_t n = n0 > 0 ? n0 : 1;
   int64_t b = per_graph_bytes(G);                            // alloc_per_graph
   b += 4 * coop_scratch(n0, nnz0) + (int64_t)sizeof(Scalars);  // alloc_counters
   b += 8 * 4 * n;                                            // C .. movers
   if (tables == 1) b += 2 * 4 * n + 8 * upd_list_size(n0, nnz0);
-  b += 4 * scan_scratch(big);                                // scan32
+  b += 4 * scan_scratch(n0);                                 // scan32
   b += 2 * 8 * n + (int64_t)sizeof(AbRec) * n;               // W, delta, ab
   b += 8 * level_counts(n0, nnz0) + (int64_t)sizeof(LevelOut);  // lcounts, lout
   b += 2 * 8 * (n0 + 1) + 8 * scan_scratch(n0 + 1) + n;      // bound, off, scan64, M
@@ -403,12 +402,12 @@ static int begin_bins(Run &r, Level &L, BinOut **d_out) {
   LC_TRY(r.ar.get(d_out, 1));
   LC_TRY(r.ar.get(&L.bins.recs, L.g.n));
   launch_bins(L.g, L.gid, r.plan, L.bins, *d_out, r.coop, r.sc, r.coop_blocks, r.s);
+  r.res->kernel_launches[LC_K_OTHER] += 1;
   return LC_OK;
 }
 static int end_bins(Run &r, Level &L, const BinOut &out) {
   if (L.g.n > 0 && !out.done) return LC_ERR_DEVICE;
   finish_bins(L.bins, out);
-  r.res->kernel_launches[LC_K_OTHER] += 1;
   L.hub = Hubs{};
   L.max_deg = out.max_deg;
   const int H = (int)L.bins.count[kHubBin], Q = (int)out.chunks;
@@ -682,7 +681,10 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
     }
     // later plain passes count from zero without a launch for it (k_bestof)
     const bool begin = i == 1 || a.phi_live || tables || r.o.event_cb;
-    if (begin) launch_pass_begin(r.sc, r.s, a.phi_live ? 1 : 0);
+    if (begin) {
+      launch_pass_begin(r.sc, r.s, a.phi_live ? 1 : 0);
+      r.res->kernel_launches[LC_K_OTHER] += 1;
+    }
     a.movers = incremental && last ? r.movers : nullptr;  // listed by this pass's update step
     if (incremental && last) {
       r.prof.begin(LC_K_OBJECTIVE);
@@ -726,7 +728,7 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
     else  // ablations: no filter, or the minimum label heuristic in odd passes
       r.res->kernel_launches[LC_K_AFTERBURNER] +=
           launch_symmetry_ablation(a, r.o.symmetry == 2 && i % 2 == 1, r.cnt, r.s);
-    // records, vertices and labels (+ 24 B per candidate edge, added from sc->cand_edges at the end)
+    // records, vertices and labels (+ 16 B per candidate edge, added from sc->cand_edges at the end)
     r.prof.end(56.0 * n);
     r.prof.begin(LC_K_APPLY);
     r.res->kernel_launches[LC_K_APPLY] += launch_assign_empty(a, w, r.s);
@@ -742,7 +744,7 @@ static int local_move_passes(Run &r, Level &L, bool singleton, int level, int ph
   r.prof.begin(LC_K_OBJECTIVE);
   if (incremental) {
     r.res->kernel_launches[LC_K_OBJECTIVE] += launch_final_objective(a, r.s) + launch_final_bestof(a, r.C_out, r.s);
-    r.prof.end(17.0 * n);  // W, w(v) and M per vertex (+ 13 B per mover edge, added at the end)
+    r.prof.end(16.0 * n);  // W and w(v) per vertex (+ 16 B per mover edge, added at the end)
   } else {
     r.res->kernel_launches[LC_K_OBJECTIVE] +=
         launch_objective(a, L.bins, r.s) + launch_final_bestof(a, r.C_out, r.s);
@@ -985,7 +987,7 @@ static int contract_level(Run &r, Level &L, Level &N, int level) {
   r.prof.begin(LC_K_CONTRACT);
   launch_contract_compact(r.gtab, 2 * L.g.nnz, r.off, rp_c, r.cnt, n_c, col_c, ew_c, r.s);
   r.prof.end(16.0 * L.g.nnz + 8.0 * nnz_c);
-  r.res->kernel_launches[LC_K_CONTRACT] += 9 + ni;
+  r.res->kernel_launches[LC_K_CONTRACT] += 8 + ni;
   LC_TRY(launch_check());
   r.res->edges_contract += L.g.nnz;
   N.g.nnz = nnz_c;
@@ -1187,7 +1189,10 @@ static int set_up(Run &r, Level &L, const LevelGraph &g0, const std::vector<int6
   LC_TRY(alloc_per_graph(r));
   LC_TRY(level0(r, L, g0, gptr));
   LC_TRY(begin_prepare(r, g0, L.gid));
-  if (labels) launch_labels_in_range(labels, g0.n, limit, r.st, r.s);
+  if (labels) {
+    launch_labels_in_range(labels, g0.n, limit, r.st, r.s);
+    r.res->kernel_launches[LC_K_OTHER] += 1;
+  }
   BinOut *d_out = nullptr, out{};
   int rc = alloc_counters(r, g0.n, g0.nnz);
   if (rc == LC_OK) rc = begin_bins(r, L, &d_out);
@@ -1250,6 +1255,7 @@ static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t>
   // uncoarsening; at the top level every present graph has the singleton
   // clustering its last local-move call returned
   launch_iota(r.C_out, lv[top].g.n, r.s);
+  r.res->kernel_launches[LC_K_OTHER] += 1;
   for (int l = top - 1; l >= 0; --l) {
     Phase up_range("lc.uncoarsen");
     Level &L = lv[l];
@@ -1268,6 +1274,7 @@ static int cluster_impl(Run &r, const LevelGraph &g0, const std::vector<int64_t>
   LabelCount count;
   begin_count(r, L0, r.C_out);
   launch_relabel(r.C_out, r.newid, labels_out, L0.g.n, L0.gid, r.gstart, nullptr, 1, r.s);
+  r.res->kernel_launches[LC_K_CONTRACT] += 1;
   std::vector<long long> phi;
   const bool phi_known = r.o.uncoarsen && r.o.pass_limit >= 1 && !B0;
   // the blocks go back, in stream order, while the GPU still works
@@ -1332,11 +1339,11 @@ static void end_call(Run &r, int rc) {
   if (r.prof.on) {
     cudaStreamSynchronize(r.s);
     r.prof.finish(r.res);
-    long long cand = 0;  // afterburner: col, ew and the 16-byte record of each candidate edge
+    long long cand = 0;  // afterburner: col, ew, C and D of each candidate edge
     if (r.sc &&
         cudaMemcpyAsync(&cand, &r.sc->cand_edges, sizeof(cand), cudaMemcpyDeviceToHost, r.s) == cudaSuccess &&
         cudaStreamSynchronize(r.s) == cudaSuccess)
-      r.res->kernel_bytes[LC_K_AFTERBURNER] += 24.0 * (double)cand;
+      r.res->kernel_bytes[LC_K_AFTERBURNER] += 16.0 * (double)cand;
     long long upd = 0;  // kept tables: col, ew, the neighbour's row bounds, two slot updates
     if (r.sc &&
         cudaMemcpyAsync(&upd, &r.sc->tab_upd_edges, sizeof(upd), cudaMemcpyDeviceToHost, r.s) == cudaSuccess &&
@@ -1347,11 +1354,11 @@ static void end_call(Run &r, int rc) {
         cudaMemcpyAsync(&nx, &r.sc->distinct_x, sizeof(nx), cudaMemcpyDeviceToHost, r.s) == cudaSuccess &&
         cudaStreamSynchronize(r.s) == cudaSuccess)
       r.res->kernel_bytes[LC_K_MOVE] += 8.0 * (double)nx;
-    long long dph = 0;  // final objective: col, ew, C[u], M[u] of each mover edge
+    long long dph = 0;  // final objective: col, ew, C[u] and its previous label of each mover edge
     if (r.sc &&
         cudaMemcpyAsync(&dph, &r.sc->dphi_edges, sizeof(dph), cudaMemcpyDeviceToHost, r.s) == cudaSuccess &&
         cudaStreamSynchronize(r.s) == cudaSuccess)
-      r.res->kernel_bytes[LC_K_OBJECTIVE] += 13.0 * (double)dph;
+      r.res->kernel_bytes[LC_K_OBJECTIVE] += 16.0 * (double)dph;
     cudaGetLastError();
   }
   if (rc != LC_OK) {
@@ -1412,8 +1419,10 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
   LC_TRY(r.ar.get(&R, g0.n));
   if (C0)
     LC_CK(cudaMemcpyAsync(Ccur, C0, sizeof(int32_t) * (size_t)g0.n, cudaMemcpyDeviceToDevice, r.s));
-  else
+  else {
     launch_iota(Ccur, g0.n, r.s);
+    r.res->kernel_launches[LC_K_OTHER] += 1;
+  }
   r.top.assign(1, 0);
   const std::vector<uint8_t> present{1};
   int top = 0;
@@ -1446,7 +1455,7 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
       r.prof.begin(LC_K_ALT);
       launch_local_move_alt(L.g, L.gp, r.C, r.ab, r.delta, r.W, ls, &r.sc->error, r.s);
       r.prof.end(24.0 * n);
-      r.res->kernel_launches[LC_K_ALT] += 6;
+      r.res->kernel_launches[LC_K_ALT] += 7;  // weights, counters, a scan of three, sizes, the moves
       LC_CK(cudaMemcpyAsync(r.C_out, r.C, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, r.s));
       LC_TRY(launch_check());
     }
@@ -1461,13 +1470,14 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
     // B = C_l with dense ids (ascending), its cluster weights, the refinement
     launch_relabel(r.C_out, r.newid, Bd, n, nullptr, r.gstart, nullptr, 0, r.s);
     launch_cluster_weights(Bd, L.g.vw, ls.WB, n, r.s);
+    r.res->kernel_launches[LC_K_OTHER] += 2;
     {
       Phase refine_range("lc.refine");
       r.prof.begin(LC_K_REFINE);
-      launch_pleiden_refine(L.g, L.bins, L.gp, Bd, r.o.seed, l, R, ls, &r.sc->error, r.s);
+      r.res->kernel_launches[LC_K_REFINE] +=
+          launch_pleiden_refine(L.g, L.bins, L.gp, Bd, r.o.seed, l, R, ls, &r.sc->error, r.s);
       r.prof.end(64.0 * L.g.nnz + 200.0 * n);
     }
-    r.res->kernel_launches[LC_K_REFINE] += 40;
     LC_TRY(launch_check());
     LC_CK(cudaMemcpyAsync(r.C_out, R, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, r.s));
     Level N;
@@ -1502,6 +1512,7 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
   LabelCount count;
   begin_count(r, L0, r.C_out);
   launch_relabel(r.C_out, r.newid, labels_out, L0.g.n, nullptr, r.gstart, nullptr, 1, r.s);
+  r.res->kernel_launches[LC_K_CONTRACT] += 1;
   LC_TRY(read_count(r, L0, count));
   std::vector<long long> phi;
   LC_TRY(objective_of(r, L0, r.C_out, phi));  // waits

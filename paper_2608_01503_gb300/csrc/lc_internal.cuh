@@ -27,7 +27,7 @@ constexpr int kMaxLevels = 256;
 //   bin 0: d <= 8       one thread (aggregation in registers)
 //   bin 1: d <= 16      16 lanes, one neighbour per lane (2 vertices per warp)
 //   bin 2: d <= 32      one warp, one neighbour per lane
-//   bin 3: d <= 128     one warp, shared table of 256 slots
+//   bin 3: d <= 128     one warp, shared table of 512 slots
 //   bin 4: d <= 256     one warp, shared table of 512 slots
 //   bin 5: d <= 512     64 threads, shared table of 1024 slots
 //   bin 6: d <= 1024    128 threads, shared table of 2048 slots
@@ -95,7 +95,7 @@ struct LevelGraph {
   const int64_t *vw;
 };
 
-// Hub chunks of one level (bin 6).  Chunk c covers edges [e0[c], e1[c]) of
+// Hub chunks of one level (bin 9).  Chunk c covers edges [e0[c], e1[c]) of
 // hub hub_of[c]; the chunks of hub h are [c0[h], c0[h+1]).
 struct Hubs {
   int32_t H = 0, Q = 0;

@@ -637,9 +637,10 @@ void launch_local_move_alt(const LevelGraph &g, const GraphParam *gp, int32_t *C
 int64_t radix_hist_len(int64_t n) { return 256 * ((n + kRadixTile - 1) / kRadixTile) + 256; }
 
 // One refinement kernel over all rows: launch(threads per vertex, step, range,
-// blocks, threads per block) for each group of bins that has rows.
+// blocks, threads per block) for each group of bins that has rows.  Returns
+// the number of launches.
 template <typename Launch>
-static void ref_rows(const Bins &bins, cudaStream_t s, Launch launch) {
+static int ref_rows(const Bins &bins, cudaStream_t s, Launch launch) {
   Step st(s);
   const auto group = [&](auto gs, int lo, int hi) {
     const BinRange r = bin_range(bins, lo, hi);
@@ -651,19 +652,20 @@ static void ref_rows(const Bins &bins, cudaStream_t s, Launch launch) {
   group(std::integral_constant<int, 32>{}, 3, 4);
   group(std::integral_constant<int, 128>{}, 5, 6);
   group(std::integral_constant<int, 512>{}, 7, kBins - 1);
+  return st.launches;
 }
 
-void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphParam *gp, const int32_t *B,
-                           uint32_t seed, int32_t level, int32_t *R, LeidenScratch &ls, int *error,
-                           cudaStream_t s) {
+int launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphParam *gp, const int32_t *B,
+                          uint32_t seed, int32_t level, int32_t *R, LeidenScratch &ls, int *error, cudaStream_t s) {
   const int64_t n = g.n;
-  if (n == 0) return;
+  if (n == 0) return 0;
+  int launches = 12;  // those that every call makes; a scan is three
   const unsigned gt = ld_grid(n, 256);
-  ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
+  launches += ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
     st.run(false, k_ref_self<gs()>, blocks, threads, 0, g, gp, r.list, r.count, B, ls.WB, ls.SB, ls.flags, ls.f,
            ls.rec, seed, level);
   });
-  ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
+  launches += ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
     st.run(false, k_ref_choose<gs()>, blocks, threads, 0, g, gp, r.list, r.count, ls.rec, ls.H, seed, level);
   });
   k_ref_keep<<<gt, 256, 0, s>>>(ls.H, ls.f, ls.flags, n);
@@ -671,7 +673,7 @@ void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphPar
   k_ref_parent<<<gt, 256, 0, s>>>(ls.H, ls.f, ls.flags, ls.first_bad, n);  // parents
   k_ref_roots<<<gt, 256, 0, s>>>(ls.first_bad, ls.root, n, error);
   k_ref_check_roots<<<gt, 256, 0, s>>>(ls.root, ls.f, ls.krec, n, error);
-  ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
+  launches += ref_rows(bins, s, [&](auto gs, Step &st, BinRange r, unsigned blocks, unsigned threads) {
     st.run(false, k_ref_sv<gs()>, blocks, threads, 0, g, r.list, r.count, ls.krec, ls.SB, ls.Sv, ls.tv);
   });
   // the vertices of multi-vertex trees, ordered by (f, id) and then by
@@ -695,6 +697,7 @@ void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphPar
     if (pairs <= kMaxTreePairs) {
       k_tree_gather<<<gt, 256, 0, s>>>(ls.root, ls.size, ls.f, ls.ps_t, ls.list, ls.key, n);
       k_tree_rank<<<gm, 256, 0, s>>>(ls.root, ls.pos, ls.ps_w, ls.list, ls.key, ls.list2, m);
+      launches += 2;
     } else {
       scan_apply<int64_t>(n, MarkIn{ls.size}, MarkOut{ls.list}, ls.scan64, s);
       k_tree_sort_keys<<<gm, 256, 0, s>>>(ls.list, ls.f, ls.key, ls.scan64 + scan_tiles(n));
@@ -703,7 +706,9 @@ void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphPar
       int bits = 1;
       while (bits < 64 && (((unsigned __int128)1) << bits) < (unsigned __int128)n * (unsigned __int128)m) ++bits;
       radix_sort(ls.key2, ls.list2, ls.key, ls.list, m, bits, ls.hist, ls.scan64, s);
+      launches += 5 + 5 * (8 + (bits + 7) / 8);  // five per digit
     }
+    launches += 8;
     k_positions<<<gm, 256, 0, s>>>(order, ls.pos, ls.first_bad, m);
     scan_apply<int64_t>(m, OrderIn{order, g.vw}, PosOut{ls.ps_w}, ls.scan64, s);
     scan_apply<int64_t>(m, OrderIn{order, ls.tv}, PosOut{ls.ps_t}, ls.scan64, s);
@@ -711,6 +716,7 @@ void launch_pleiden_refine(const LevelGraph &g, const Bins &bins, const GraphPar
                                   ls.first_bad, m);
   }
   k_ref_label<<<gt, 256, 0, s>>>(ls.root, ls.size, ls.pos, ls.first_bad, R, n);
+  return launches;
 }
 
 void launch_downsample(const int32_t *Cd, const int32_t *C, int32_t *Cc, int64_t n, cudaStream_t s) {

@@ -804,7 +804,7 @@ static inline unsigned blocks_for(int64_t items, int per_block) {
   return (unsigned)b;
 }
 
-// table (8 bytes per slot) + claimed-slot list (2 bytes per half slot)
+// a key and a sum per slot
 static constexpr int block_table_bytes(int slots) { return slots * 8; }
 
 void configure_kernels() {

@@ -80,7 +80,7 @@ int launch_objective(const PassArgs &a, const Bins &b, cudaStream_t s);
 // state entering it.  launch_last_pass_enter runs at the start of the last
 // pass (Q of W before its update), launch_save_phi_enter after its move step
 // and per-graph sums (Phi entering), launch_final_objective after its update
-// (the movers' edges, Q after; needs the pass's M and Cprev): Phi into
+// (the movers' edges, Q after; needs the pass's records and mover list): Phi into
 // phi_acc[g].
 int launch_last_pass_enter(const PassArgs &a, cudaStream_t s);
 int launch_save_phi_enter(const PassArgs &a, cudaStream_t s);

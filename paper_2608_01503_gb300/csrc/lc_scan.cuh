@@ -4,10 +4,9 @@
 // the tile totals, then a per-tile block scan that hands every input its
 // exclusive prefix.  Inputs and outputs are functors, so the flag of a
 // compaction and the scatter it feeds are fused into the scan instead of
-// materialising an index array.  Used for: label compaction (ids in use),
-// new-singleton ids (free ids, empty-cluster movers), coarse CSR offsets and
-// the stream compaction of the contraction tables (Algorithm 4's
-// ExclusivePrefixSum and StreamCompaction).
+// materialising an index array.  Used for label compaction (ids in use), coarse
+// CSR offsets (Algorithm 4's ExclusivePrefixSum), and pLeiden's lists and
+// prefix sums along the tree order.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -55,9 +54,7 @@ __device__ __forceinline__ T block_exclusive(T x, T *warp_tot, T &total) {
 }
 
 template <typename T, typename In>
-__global__ void __launch_bounds__(kScanThreads) k_scan_tile_totals(In in, int64_t n, T *tile_tot,
-                                                                   const int *skip) {
-  if (skip && *skip == 0) return;
+__global__ void __launch_bounds__(kScanThreads) k_scan_tile_totals(In in, int64_t n, T *tile_tot) {
   __shared__ T wt[kScanThreads / 32 + 1];
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
   T s = 0;
@@ -73,9 +70,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tile_totals(In in, int64_
 
 // Single block: exclusive scan of tile totals in place; tile_tot[tiles] = grand total.
 template <typename T>
-__global__ void __launch_bounds__(kScanThreads) k_scan_tile_prefix(T *tile_tot, int64_t tiles,
-                                                                   const int *skip) {
-  if (skip && *skip == 0) return;
+__global__ void __launch_bounds__(kScanThreads) k_scan_tile_prefix(T *tile_tot, int64_t tiles) {
   __shared__ T wt[kScanThreads / 32 + 1];
   T carry = 0;
   for (int64_t b = 0; b < tiles; b += kScanThreads) {
@@ -92,8 +87,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tile_prefix(T *tile_tot, 
 // out(i, prefix, value) is called for every i < n with the exclusive prefix.
 template <typename T, typename In, typename Out>
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(In in, Out out, int64_t n,
-                                                             const T *tile_tot, const int *skip) {
-  if (skip && *skip == 0) return;
+                                                             const T *tile_tot) {
   __shared__ T wt[kScanThreads / 32 + 1];
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
   T carry = tile_tot[blockIdx.x];
@@ -108,18 +102,17 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(In in, Out out, int
 }
 
 // Runs the scan.  scratch: scan_scratch(n) elements of T; the grand total is
-// left in scratch[scan_tiles(n)].  If `skip` is non-null and *skip == 0 on
-// the device when a launch starts, the launch does nothing.
+// left in scratch[scan_tiles(n)].
 template <typename T, typename In, typename Out>
-void scan_apply(int64_t n, In in, Out out, T *scratch, cudaStream_t s, const int *skip = nullptr) {
+void scan_apply(int64_t n, In in, Out out, T *scratch, cudaStream_t s) {
   const int64_t tiles = scan_tiles(n);
   if (tiles == 0) {
     cudaMemsetAsync(scratch, 0, sizeof(T), s);
     return;
   }
-  k_scan_tile_totals<T, In><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, scratch, skip);
-  k_scan_tile_prefix<T><<<1, kScanThreads, 0, s>>>(scratch, tiles, skip);
-  k_scan_apply<T, In, Out><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, out, n, scratch, skip);
+  k_scan_tile_totals<T, In><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, scratch);
+  k_scan_tile_prefix<T><<<1, kScanThreads, 0, s>>>(scratch, tiles);
+  k_scan_apply<T, In, Out><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, out, n, scratch);
 }
 
 }  // namespace lc

@@ -27,8 +27,8 @@ def graphs():
 
 
 def replayed(res, plain):
-    """Passes that were replayed: a captured pass holds, and counts, the kernel
-    that loads its temperature, which direct launches do not count."""
+    """Passes that were replayed: a captured pass counts the kernel that loads its
+    temperature in the class "apply", a direct one in "other"."""
     return res["kernel_launches"]["apply"] - plain["kernel_launches"]["apply"]
 
 
