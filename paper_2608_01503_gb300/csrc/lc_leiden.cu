@@ -477,7 +477,11 @@ __global__ void k_mark_trees(const int32_t *__restrict__ root, int32_t *__restri
 // the rank that comparing (f, id) with the whole tree gives it.  That is the
 // sum of the squared tree sizes in comparisons, a few microseconds for the
 // usual forests, against two radix sorts of up to 14 digit passes and five
-// launches each; forests with a very large tree still take those.
+// launches each; forests with a very large tree still take those.  The line
+// lies where the two meet for one large tree, whose every thread walks all of
+// it (ms of a call on a star, whose tree holds half of its leaves, counting /
+// sorting: 2,000 leaves 6.2 / 10.4, 20,000 8.8 / 12.3, 40,000 11.4 / 13.7,
+// 64,000, the last below the line, 13.6 / 14.4; R-MAT scale 17 16.4 / 22.7).
 constexpr long long kMaxTreePairs = 1ll << 30;
 
 __global__ void k_tree_sizes(const int32_t *__restrict__ root, const int32_t *__restrict__ mark,
