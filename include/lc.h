@@ -85,7 +85,7 @@ enum {
 /* Graph topology: n vertices, nnz stored (directed) entries. */
 typedef struct {
   int64_t n;
-  int64_t nnz;
+  int64_t nnz;            /* at most 2^40; row_ptr[n], or the call is refused unread */
   const int64_t *row_ptr; /* [n+1] */
   const int32_t *col;     /* [nnz] */
 } lc_csr;
@@ -178,7 +178,8 @@ typedef struct {
                                launches (all but a first pass from singletons and the last)
                                are captured once per call into a CUDA graph and replayed,
                                on levels above 4 M vertices and stored edges (smaller ones
-                               run all passes in one kernel).
+                               run all passes in one kernel, unless bin_max_deg[4] < 128 or
+                               bin_max_deg[6] < 256 sends short rows to its blocks).
                                Ignored with profile, event_cb or tables = 1.  Results are
                                identical.  Default 0. */
 } lc_opts;
@@ -472,7 +473,9 @@ LC_API int64_t lc_objective_static_max_vertices(void);
  * records are per process: calls running concurrently in the checked build
  * (server slots, several threads) may report one another's failures.  On
  * valid inputs both builds compute identical results; the checked build is
- * slower.
+ * slower.  It can also leave a block out of a grid barrier, to test that a wait
+ * that runs out ends the call with LC_ERR_DEVICE: LC_DEBUG_BARRIER=K:P in the
+ * environment, the K-th barrier of each call and P polls a wait.
  *
  * lc_debug_enabled: 1 in the checked build, else 0.
  * lc_debug_selftest: checked build only (else LC_ERR_ARG): launches one
