@@ -767,14 +767,16 @@ __device__ __forceinline__ long long hub_insert(const PassArgs &a, int32_t v, in
 __device__ __forceinline__ bool last_of_hub(const PassArgs &a, int h) {
   __shared__ int s_last;
   __syncthreads();
-  const int n = a.hub.c0[h + 1] - a.hub.c0[h];
-  if (n == 1) return true;  // what thread 0 stored, it reads itself
   if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atomicAdd(&a.hub.done[h], 1) == n - 1;
-    if (s_last) {
-      a.hub.done[h] = 0;
+    const int n = a.hub.c0[h + 1] - a.hub.c0[h];
+    s_last = 1;  // of one chunk: what thread 0 stored, it reads itself
+    if (n > 1) {
       __threadfence();
+      s_last = atomicAdd(&a.hub.done[h], 1) == n - 1;
+      if (s_last) {
+        a.hub.done[h] = 0;
+        __threadfence();
+      }
     }
   }
   __syncthreads();
