@@ -39,7 +39,7 @@ def test_columns_longer_than_the_weights():
     torch.cuda.synchronize()
 
 
-@pytest.mark.parametrize("nnz", [2 * N - 1, 2 * N + 1, 1 << 24, 1 << 41, 1 << 62])
+@pytest.mark.parametrize("nnz", [2 * N - 1, 2 * N + 1, 1 << 24, 1 << 36, 1 << 41, 1 << 62])
 def test_count_beyond_the_arrays(nnz):
     rp, col, ew, vw = ring()
     lab, res = torch.zeros(N, dtype=torch.int32, device="cuda"), lc._Result()
