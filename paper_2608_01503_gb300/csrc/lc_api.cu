@@ -416,6 +416,7 @@ static int end_bins(Run &r, Level &L, const BinOut &out) {
     LC_TRY(r.ar.get(&p, 32 * (int64_t)Q + 16 * (int64_t)H + 4));
     L.hub.H = H;
     L.hub.Q = Q;
+    L.hub.settle = r.plan.hub_min() < r.plan.hub_chunk;
     L.hub.vtx = L.bins.list[kHubBin];
     L.hub.e0 = cut<int64_t>(p, Q);
     L.hub.e1 = cut<int64_t>(p, Q);
@@ -425,8 +426,7 @@ static int end_bins(Run &r, Level &L, const BinOut &out) {
     L.hub.part_x = cut<int32_t>(p, Q);
     L.hub.c0 = cut<int32_t>(p, H + 1);
     L.hub.done = cut<int32_t>(p, H);
-    launch_hub_plan(L.bins, r.plan, L.hub, r.s);
-    r.res->kernel_launches[LC_K_OTHER] += 1;
+    r.res->kernel_launches[LC_K_OTHER] += launch_hub_plan(L.bins, r.plan, L.hub, r.s);
   }
   return launch_check();
 }

@@ -39,8 +39,23 @@ __global__ void __launch_bounds__(kT, 1) k_bins(const __grid_constant__ BinArgs 
   bar.leave(&a.out->done);
 }
 
+// The chunks of hub h, by `lanes` threads of rank `lane`.
+__device__ __forceinline__ void cut_hub(const VRec &r, int h, int first, int32_t hub_chunk, int32_t *hub_of, int64_t *e0,
+                                        int64_t *e1, int lane, int lanes) {
+  const int64_t end = r.beg + r.deg;
+  for (int k = lane; r.beg + (int64_t)k * hub_chunk < end; k += lanes) {
+    const int64_t b = r.beg + (int64_t)k * hub_chunk;
+    hub_of[first + k] = h;
+    e0[first + k] = b;
+    e1[first + k] = b + hub_chunk < end ? b + hub_chunk : end;
+  }
+}
+
 // Cuts the hub rows into chunks of hub_chunk edges: c0[h] = the first chunk
-// of hub h, and each chunk's hub and edges.  One block.
+// of hub h, and each chunk's hub and edges (up to kPlanHubs hubs; more are cut
+// by k_hub_chunks, a thread each: with 100,000 hubs the one block took 0.48 ms).
+// One block.
+constexpr int kPlanHubs = 8192;
 __global__ void __launch_bounds__(kT, 1)
     k_hub_plan(const VRec *__restrict__ hubs, int H, int32_t hub_chunk, int32_t *c0, int32_t *hub_of, int64_t *e0,
                int64_t *e1, long long *acc, int32_t *done) {
@@ -75,17 +90,14 @@ __global__ void __launch_bounds__(kT, 1)
   }
   __syncthreads();
   if (threadIdx.x == 0) c0[H] = s_run;
-  for (int h = wid; h < H; h += kW) {  // a hub's chunks by a warp
-    const VRec r = hubs[h];
-    const int first = c0[h];
-    const int64_t end = r.beg + r.deg;
-    for (int k = lane; r.beg + (int64_t)k * hub_chunk < end; k += 32) {
-      const int64_t b = r.beg + (int64_t)k * hub_chunk;
-      hub_of[first + k] = h;
-      e0[first + k] = b;
-      e1[first + k] = b + hub_chunk < end ? b + hub_chunk : end;
-    }
-  }
+  if (H > kPlanHubs) return;
+  for (int h = wid; h < H; h += kW) cut_hub(hubs[h], h, c0[h], hub_chunk, hub_of, e0, e1, lane, 32);  // by a warp
+}
+__global__ void __launch_bounds__(256) k_hub_chunks(const VRec *__restrict__ hubs, int H, int32_t hub_chunk,
+                                                    const int32_t *__restrict__ c0, int32_t *hub_of, int64_t *e0,
+                                                    int64_t *e1) {
+  const int h = blockIdx.x * blockDim.x + threadIdx.x;
+  if (h < H) cut_hub(hubs[h], h, c0[h], hub_chunk, hub_of, e0, e1, 0, 1);
 }
 
 }  // namespace
@@ -114,10 +126,15 @@ void finish_bins(Bins &b, const BinOut &out) {
   }
 }
 
-void launch_hub_plan(const Bins &b, const BinPlan &plan, const Hubs &hub, cudaStream_t s) {
-  k_hub_plan<<<1, kT, 0, s>>>(b.rec[kHubBin], hub.H, (int32_t)plan.hub_chunk, const_cast<int32_t *>(hub.c0),
-                             const_cast<int32_t *>(hub.hub_of), const_cast<int64_t *>(hub.e0),
-                             const_cast<int64_t *>(hub.e1), hub.acc, hub.done);
+int launch_hub_plan(const Bins &b, const BinPlan &plan, const Hubs &hub, cudaStream_t s) {
+  const VRec *hubs = b.rec[kHubBin];
+  const int32_t chunk = (int32_t)plan.hub_chunk;
+  int32_t *c0 = const_cast<int32_t *>(hub.c0), *hub_of = const_cast<int32_t *>(hub.hub_of);
+  int64_t *e0 = const_cast<int64_t *>(hub.e0), *e1 = const_cast<int64_t *>(hub.e1);
+  k_hub_plan<<<1, kT, 0, s>>>(hubs, hub.H, chunk, c0, hub_of, e0, e1, hub.acc, hub.done);
+  if (hub.H <= kPlanHubs) return 1;
+  k_hub_chunks<<<(unsigned)((hub.H + 255) / 256), 256, 0, s>>>(hubs, hub.H, chunk, c0, hub_of, e0, e1);
+  return 2;
 }
 
 }  // namespace lc

@@ -20,7 +20,8 @@ struct BinOut {
 void launch_bins(const LevelGraph &g, const int32_t *gid, const BinPlan &plan, const Bins &b, BinOut *out,
                  int32_t *counts, Scalars *sc, int coop, cudaStream_t s);
 void finish_bins(Bins &b, const BinOut &out);
-// Fills the arrays of a hub plan (H >= 1 hubs, Q chunks) and zeroes acc.
-void launch_hub_plan(const Bins &b, const BinPlan &plan, const Hubs &hub, cudaStream_t s);
+// Fills the arrays of a hub plan (H >= 1 hubs, Q chunks) and zeroes acc; returns
+// the number of kernels launched.
+int launch_hub_plan(const Bins &b, const BinPlan &plan, const Hubs &hub, cudaStream_t s);
 
 }  // namespace lc

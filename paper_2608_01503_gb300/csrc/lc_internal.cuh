@@ -99,6 +99,7 @@ struct LevelGraph {
 // hub hub_of[c]; the chunks of hub h are [c0[h], c0[h+1]).
 struct Hubs {
   int32_t H = 0, Q = 0;
+  int32_t settle = 0;               // the plan has hubs of one chunk: see k_hub_settle
   const int32_t *vtx = nullptr;     // [H] hub vertex ids
   const int32_t *hub_of = nullptr;  // [Q]
   const int64_t *e0 = nullptr, *e1 = nullptr;  // [Q]

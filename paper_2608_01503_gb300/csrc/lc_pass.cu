@@ -264,6 +264,65 @@ __device__ __forceinline__ void hub_acc_add(const PassArgs &a, int h, long long 
   if (threadIdx.x == 0 && x != 0) atomicAdd((unsigned long long *)&a.hub.acc[h], (unsigned long long)x);
 }
 
+// Hubs of one chunk are settled by a lane each in a kernel after the step, if
+// the bin plan can have any (hub_chunk above the longest row of bin 8): a block
+// to itself, a short row's decision is a chain of loads that nothing hides
+// (ms a call, SBM of 100,000 vertices with every row above 8 edges a hub, block
+// / lane: 29.1 / 22.5, 2.4 of them by k_hub_chunks).  Longer hubs are decided by their last chunk.
+__device__ __forceinline__ bool left_to_settle(const PassArgs &a, int h) {
+  return a.hub.settle && a.hub.c0[h + 1] - a.hub.c0[h] == 1;
+}
+
+__global__ void __launch_bounds__(256) k_hub_settle(PassArgs a, int first) {
+  MoveState ms = move_state(a);
+  for (int base = blockIdx.x * blockDim.x; base < a.hub.H; base += gridDim.x * blockDim.x) {
+    const int h = base + threadIdx.x;
+    const bool on = h < a.hub.H && left_to_settle(a, h);
+    int g = 0;
+    long long gC = 0;
+    if (on) {
+      const int32_t v = a.hub.vtx[h], c = a.hub.c0[h];
+      g = graph_of(a, v);
+      const GraphParam P = a.gp[g];
+      const int32_t Cv = a.C[v];
+      if (!first) {
+        gC = gain_self(P, a.hub.acc[h], a.g.vw[v], a.W[Cv]);
+        a.hub.acc[h] = 0;
+      }
+      decide(a, P, v, Cv, gC, a.hub.part_x[c], a.hub.part_g[c], ms);
+    }
+    if (!first) phi_add(a, ms.acc, on, g, gC, ms.phi);
+  }
+  if (first)
+    flush_block_sum(ms.cntL, &a.sc->count_L);
+  else
+    flush_move(a, ms);
+}
+
+// The update of the same hubs from their chunk's sum.
+__global__ void __launch_bounds__(256) k_hub_settle_update(PassArgs a) {
+  UpdateSums sum;
+  for (int base = blockIdx.x * blockDim.x; base < a.hub.H; base += gridDim.x * blockDim.x) {
+    const int h = base + threadIdx.x;
+    const bool on = h < a.hub.H && left_to_settle(a, h);
+    int32_t v = 0;
+    AbRec r{0, kNone, 0};
+    int64_t deg = 0;
+    bool keep = false;
+    if (on) {
+      v = a.hub.vtx[h];
+      r = a.ab[v];
+      deg = a.g.rp[v + 1] - a.g.rp[v];
+      if (r.D != kNone) {
+        keep = a.delta[v] + a.hub.acc[h] >= 0;
+        a.hub.acc[h] = 0;
+      }
+    }
+    apply_lanes(a, on, v, deg, r, on ? a.g.vw[v] : 0, keep, sum);
+  }
+  flush_update(a, sum);
+}
+
 // Move, step 1: insert a chunk of a hub row into the hub's global table.
 // Lanes of a warp holding the same cluster are combined first (lane_sums),
 // so a popular cluster costs one global atomic per warp.
@@ -292,7 +351,7 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_move_scan(PassArgs a) {
   range_argmax<kHubThreads>(a, P.Lam, P.mu * wv, a.gtab + 2 * beg, (uint32_t)(2 * (a.hub.e0[c] - beg)),
                             (uint32_t)(2 * (a.hub.e1[c] - beg)), threadIdx.x, gb, xb, ms.nX, a.tab_build != 0);
   hub_part_store(a, c, gb, xb);
-  if (last_of_hub(a, h) && threadIdx.x < 32) {
+  if (!left_to_settle(a, h) && last_of_hub(a, h) && threadIdx.x < 32) {
     const long long self = decide_hub(a, h, v, false, threadIdx.x, ms);
     // the hub's kept table gets its own cluster
     if (a.tab_build && self > 0 && !tab_put(a.gtab + 2 * beg, tab_cap(a.g.rp[v + 1] - beg), a.C[v], self))
@@ -315,7 +374,7 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_first(PassArgs a) {
   for (int64_t e = a.hub.e0[c] + threadIdx.x; e < a.hub.e1[c]; e += kHubThreads)
     first_edge(a, P.Lam, P.mu * wv, e, gb, xb);
   hub_part_store(a, c, gb, xb);
-  if (last_of_hub(a, h) && threadIdx.x < 32) decide_hub(a, h, v, true, threadIdx.x, ms);
+  if (!left_to_settle(a, h) && last_of_hub(a, h) && threadIdx.x < 32) decide_hub(a, h, v, true, threadIdx.x, ms);
   flush_block_sum(ms.cntL, &a.sc->count_L);
   step_end();
 }
@@ -391,12 +450,12 @@ __global__ void __launch_bounds__(kHubThreads) k_hub_afterburner(PassArgs a) {
   const int32_t v = a.hub.vtx[h];
   const AbRec r = a.ab[v];
   UpdateSums sum;
-  bool mine = c == a.hub.c0[h];  // no candidate: its first chunk keeps it where it is
+  bool mine = c == a.hub.c0[h] && !left_to_settle(a, h);  // no candidate: its first chunk keeps it where it is
   long long t = -1;
   if (r.D != kNone) {  // block-uniform
     const AbCtx ctx = ab_ctx(a, v, r, a.gp[graph_of(a, v)], 0, 0, a.g.vw[v]);
     hub_acc_add(a, h, ab_edges<kHubThreads, 4>(a, ctx, a.hub.e0[c], a.hub.e1[c], threadIdx.x));
-    mine = last_of_hub(a, h);
+    mine = !left_to_settle(a, h) && last_of_hub(a, h);
     if (mine && threadIdx.x == 0) t = a.delta[v] + take_hub_acc(a, h);
   }
   if (mine && threadIdx.x < 32)
@@ -879,6 +938,7 @@ int launch_first_pass(const PassArgs &a, const Bins &b, cudaStream_t s) {
   st.block_chunks(k_first_block<128>, 128, 0, a, bin_range(b, 5, 6));
   st.block_chunks(k_first_block<512>, 512, 0, a, bin_range(b, 7, 8));
   if (a.hub.H > 0) st.run(false, k_hub_first, a.hub.Q, kHubThreads, 0, a);
+  if (a.hub.settle) st.run(true, k_hub_settle, blocks_for(a.hub.H, 256), 256, 0, a, 1);
   return st.launches;
 }
 
@@ -908,6 +968,7 @@ int launch_move(const PassArgs &a, const Bins &b, cudaStream_t s) {
   move_block<256, 4096, 8>(st, a, bin_range(b, 7, 7));
   move_block<256, 6144, 16>(st, a, bin_range(b, 8, 8));
   if (a.hub.H > 0) st.run(true, k_hub_move_scan, a.hub.Q, kHubThreads, 0, a);
+  if (a.hub.settle) st.run(true, k_hub_settle, blocks_for(a.hub.H, 256), 256, 0, a, 0);
   return st.launches;
 }
 
@@ -950,6 +1011,7 @@ int launch_afterburner(const PassArgs &a, const Bins &b, cudaStream_t s) {
   st.warp_chunks(k_ab_warp<8>, a, bin_range(b, 2, 2));
   for (int g = 2; g < kAbGroups; ++g) ab_group(st, a, b, g);
   if (a.hub.H > 0) st.run(false, k_hub_afterburner, a.hub.Q, kHubThreads, 0, a);
+  if (a.hub.settle) st.run(true, k_hub_settle_update, blocks_for(a.hub.H, 256), 256, 0, a);
   return st.launches;
 }
 
