@@ -394,6 +394,13 @@ int64_t cluster_footprint(int64_t n, int64_t nnz, int count, const lc_opts &o) {
   return level0_scratch_bytes(n, nnz, count, o.tables) + 2 * level_bytes(n, nnz, count, p) + (1 << 20);
 }
 
+// A kernel has reported a failure before the call's end.
+static int check_device_error(Run &r);
+static int device_error(Run &r) {
+  check_device_error(r);  // the checked build's record
+  return LC_ERR_DEVICE;
+}
+
 // Degree bins of a level, and the chunk plan of its hub bin (rows longer
 // than the last shared-memory bin are cut into chunks of the plan's hub_chunk edges).
 // begin_bins queues the kernel, end_bins takes its counts.
@@ -406,7 +413,7 @@ static int begin_bins(Run &r, Level &L, BinOut **d_out) {
   return LC_OK;
 }
 static int end_bins(Run &r, Level &L, const BinOut &out) {
-  if (L.g.n > 0 && !out.done) return LC_ERR_DEVICE;
+  if (L.g.n > 0 && !out.done) return device_error(r);
   finish_bins(L.bins, out);
   L.hub = Hubs{};
   L.max_deg = out.max_deg;
@@ -867,7 +874,7 @@ static int compact_level(Run &r, Level &L, Level &N, int level, bool *any) {
   r.prof.begin(LC_K_CONTRACT);
   int err = 0;  // the contraction trusts the passes' tables and counters
   LC_TRY(count_labels(r, L, r.C_out, nc, &total, &err));
-  if (err) return LC_ERR_DEVICE;
+  if (err) return device_error(r);
   L.cont.assign(r.G, 0);
   *any = false;
   for (int g = 0; g < r.G; ++g) {
@@ -923,7 +930,7 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   if (r.G > 1) LC_CK(cudaMemcpyAsync(nc.data(), w.nc, 4 * (size_t)r.G, cudaMemcpyDeviceToHost, r.s));
   LC_CK(cudaStreamSynchronize(r.s));
   LC_TRY(launch_check());
-  if (!out.bins.done) return LC_ERR_DEVICE;
+  if (!out.bins.done) return device_error(r);
   if (r.G == 1) nc[0] = (int32_t)(out.n_c > 0 ? out.n_c : L.g.n);
   r.res->kernel_launches[LC_K_CONTRACT] += 1;
   L.cont.assign(r.G, 0);
@@ -943,7 +950,7 @@ static int end_small_level(Run &r, Level &L, Level &N, int level, bool *any) {
   }
   *any = base > 0;
   if (!*any) return LC_OK;
-  if (base != out.n_c) return LC_ERR_DEVICE;
+  if (base != out.n_c) return device_error(r);
   // the GPU waits for these: one block for what is sized by the vertices
   uint8_t *p = nullptr;
   LC_TRY(r.ar.get(&p, (int64_t)(sizeof(VRec) + 8 + 8 + 4 + (r.G > 1 ? 4 : 0)) * out.n_c + 8));
@@ -1441,7 +1448,7 @@ static int pleiden_impl(Run &r, const LevelGraph &g0, const int32_t *C0, int32_t
     LC_CK(cudaMemcpyAsync(&phi_out, r.phi_out, sizeof(long long), cudaMemcpyDeviceToHost, r.s));
     LC_CK(cudaMemcpyAsync(&err, &r.sc->error, sizeof(err), cudaMemcpyDeviceToHost, r.s));
     LC_CK(cudaStreamSynchronize(r.s));
-    if (err) return LC_ERR_DEVICE;
+    if (err) return device_error(r);
     if (phi_out == phi_in[0]) {  // LocalMoveAlt (Section V-A)
       LC_CK(cudaMemcpyAsync(r.C, r.C_out, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, r.s));
       launch_cluster_weights(r.C, L.g.vw, r.W, n, r.s);
